@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(FIN ? 448 : 320, 1) k_ana_tc(TcAnaArgs a) {
     const int ib = a.item_off[blockIdx.x], nI = a.item_off[blockIdx.x + 1] - ib;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // the tables do not depend on the predecessor: stream them right away
             const uint64_t pol = policy_evict_first();
             int it = 0;
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(FIN ? 448 : 320, 1) k_ana_tc(TcAnaArgs a) {
                 if (k >= 0) mbar_wait(&a_full[k % ANS], (k / ANS) & 1, abort, a.status);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             int it = 0;
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = a.items[ib + i];
@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(192, 1) k_ana_tc_b(TcAnaBArgs a) {
             for (int k = it - TC_ANAB_NS; k < it; ++k)
                 if (k >= 0) mbar_wait(&a_full[k % TC_ANAB_NS], (k / TC_ANAB_NS) & 1, abort, a.status);
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             int it = 0;
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = a.items[ib + i];
@@ -908,7 +908,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
     pdl_launch();
 
     if (warp == 0 && SINGLE) {
-        if (lane == 0) {
+        if (elect_one()) {
             // the table does not depend on the predecessor (no wait); the
             // builder warps write every stage's coefficient tile. Only the
             // first stage is requested before its data lands: the builders'
@@ -940,7 +940,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
                 if (k >= 0) mbar_wait(&a_full[k % ns], (k / ns) & 1, abort, a.status);
         }
     } else if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // the table tiles of the first ns stages do not depend on the
             // predecessor (the B tiles do): they are requested before the wait,
             // overlapping the coefficient prep, and their B tiles right after it.
@@ -1004,7 +1004,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
                 if (k >= 0) mbar_wait(&a_full[k % ns], (k / ns) & 1, abort, a.status);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_bf16(TC_TILE_M, brows);
             int it = 0;
             for (int i = 0; i < nI; ++i) {

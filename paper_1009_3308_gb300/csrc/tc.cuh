@@ -29,6 +29,18 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// One lane of a converged warp.  The single-thread loops of the tcgen05 and
+// TMA roles are entered through it: behind a lane-index test the compiler
+// cannot know that one thread runs them, and guards every tcgen05.mma for a
+// possibly divergent warp.  Back-to-back M = 128, K = 16 MMAs then issue every
+// 72 cycles (N <= 128; 162 in the loops of the Legendre kernels), against 39
+// at N = 16, 48 at N = 64 and 64 at N = 128 here.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
+
 // ---- MMA ------------------------------------------------------------------
 // D(tmem) (+)= A(smem desc) x B(smem desc), kind::f16 (BF16 in, FP32 accumulate)
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
