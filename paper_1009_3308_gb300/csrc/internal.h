@@ -43,7 +43,7 @@ __host__ __device__ inline void packed_lm(int N, int i, int& L, int& m) {
 // order-major [f][m][row], or latitude-pair-major [f][row / 2][m][row % 2]
 // (pairs != 0), the layout the four-step ring kernel reads contiguously.
 __host__ __device__ inline size_t gsyn_index(int pairs, int f, int m, int row, int N, int nlat) {
-    return pairs ? ((size_t(f) * (nlat / 2) + row / 2) * size_t(N + 1) + m) * 2 + (row & 1)
+    return pairs ? ((size_t(f) * ((nlat + 1) / 2) + row / 2) * size_t(N + 1) + m) * 2 + (row & 1)
                  : (size_t(f) * (N + 1) + m) * size_t(nlat) + row;
 }
 
@@ -233,8 +233,8 @@ struct sphnse_plan {
     double* d_s = nullptr;       // sin(theta_p), nlat
     float* d_isin32 = nullptr;   // 1 / sin(theta_p) rounded to FP32, nlat
     double* d_rw = nullptr;      // (2 pi / M) w_p / sin(theta_p), nlat
-    double* d_tw = nullptr;      // e^{-2 pi i t / M}, M complex (FP64)
-    float* d_tw32 = nullptr;     // same in FP32
+    float* d_tw32 = nullptr;     // e^{-2 pi i t / M}, M complex (FP32)
+    int4* d_fxtw = nullptr;      // fixed-point twiddles of the FP64 ring kernel, M split Q62 pairs
     float* d_ftw = nullptr;      // four-step ring kernel twiddles (M = 24 M2), FP32
     int2* d_lm = nullptr;        // (L, m) of each packed entry
     double4_32a* d_prepc = nullptr;  // per ext row (m, K): (lam_K^{1/2}, lam_K^{-1/2}, c_down, c_up)
@@ -251,7 +251,7 @@ struct sphnse_plan {
     void* d_gsyn = nullptr;      // [5][N+1][nlat] complex (m-major)
     void* d_gana = nullptr;      // [3][N+1][nlat] complex (m-major)
     void* d_hana = nullptr;      // [n_ext][2 * 3]
-    void* d_gsyn_r = nullptr;    // latitude-major copies for the ring kernel: [5][nlat][N+1]
+    void* d_gsyn_r = nullptr;    // FP32 latitude-major copies for the general ring kernel: [5][nlat][N+1]
     void* d_gana_r = nullptr;    //                                             [3][nlat][N+1]
     double* d_work = nullptr;    // NDF / adjoint vectors (16 x n_coeff complex)
     double* d_grid = nullptr;    // objective: two grid fields (allocated on first use)
@@ -313,11 +313,15 @@ enum RingMode { RING_RHS = 0, RING_GRID = 1, RING_PROJECT = 2, RING_ADJOINT = 3 
 int launch_prep(sphnse_plan* P, const double* alpha, const double* beta, int prec);
 // pairs != 0: write the latitude-pair-major layout of gsyn_index
 int launch_synthesis(sphnse_plan* P, int nfields, int prec, int pairs = 0);
-int launch_ring(sphnse_plan* P, int mode, int prec, const double* gin0, const double* gin1,
+int launch_ring(sphnse_plan* P, int mode, const double* gin0, const double* gin1,
                 double* gout0, double* gout1, double* gout2);
-int launch_analysis(sphnse_plan* P, int nfields, int prec);
-// in [nf][R][Cn] -> out [nf][Cn][R] (complex entries of the precision's type)
-int launch_transpose(sphnse_plan* P, const void* in, void* out, int R, int Cn, int nf, int prec);
+int launch_analysis(sphnse_plan* P, int nfields, int prec, int pairs = 0);
+// the FP64 ring kernel (64-bit fixed point) on the latitude-pair-major buffers
+std::vector<int> ring_fx_twiddles(int nlon);
+int launch_ring_fx(sphnse_plan* P, int mode, const double* gin0, const double* gin1, double* gout0, double* gout1,
+                   double* gout2);
+// in [nf][R][Cn] -> out [nf][Cn][R] (complex FP32 entries)
+int launch_transpose(sphnse_plan* P, const void* in, void* out, int R, int Cn, int nf);
 // finish: kind 0 = RHS (F = f - nu lam alpha - N), 1 = projection (N),
 // 2 = adjoint (out = -nu lam w - s_m (N_X + lam^{1/2} H_rho))
 int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha,
@@ -367,7 +371,7 @@ int launch_finish32_batch(sphnse_plan* P, int nb, const float* hana, size_t hstr
                           double* out, const double* nu_inst);
 void tc_free(sphnse_plan* P);
 void host_io_free(sphnse_plan* P);
-int launch_analysis_stream(sphnse_plan* P, int nfields, int prec);
+int launch_analysis_stream(sphnse_plan* P, int nfields, int prec, int pairs = 0);
 void stage_begin(sphnse_plan* P, int stage);
 void stage_end(sphnse_plan* P, int stage);
 int check_cuda(cudaError_t e);

@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(128) k_synthesis(const T* __restrict__ psyn, c
 // (and sin(theta_p) for the scalar adjoint field).
 template <typename T, int NF>
 __global__ void __launch_bounds__(128) k_analysis(const T* __restrict__ pana, const T* __restrict__ gana,
-                                                   T* __restrict__ hana, int N, int nh, int nlat) {
+                                                   T* __restrict__ hana, int N, int nh, int nlat, int pairs) {
     pdl_launch();
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -198,14 +198,13 @@ __global__ void __launch_bounds__(128) k_analysis(const T* __restrict__ pana, co
     const int nrows = par ? no : ne;
     if (int(blockIdx.x * blockDim.x) >= nrows) return;
     const int rowstart = ext_off(N, m) + (par ? ne : 0);
-    const size_t ld = size_t(N + 1);
     for (int i = threadIdx.x; i < nh * NF; i += blockDim.x) {
         const int p = i / NF, f = i % NF;
         const int pr = nlat - 1 - p;
-        const T* a = gana + ((size_t(f) * ld + m) * nlat + p) * 2;
+        const T* a = gana + gsyn_index(pairs, f, m, p, N, nlat) * 2;
         T ar = a[0], ai = a[1], br = T(0), bi = T(0);
         if (pr != p) {
-            const T* b = gana + ((size_t(f) * ld + m) * nlat + pr) * 2;
+            const T* b = gana + gsyn_index(pairs, f, m, pr, N, nlat) * 2;
             br = b[0];
             bi = b[1];
         }
@@ -391,7 +390,7 @@ int launch_synthesis(sphnse_plan* P, int nfields, int prec, int pairs) {
 }
 
 template <typename T, int NF>
-static int anal_t(sphnse_plan* P) {
+static int anal_t(sphnse_plan* P, int pairs) {
     const int maxrows = ext_even(P->N, 0);
     dim3 blk(128), grd((maxrows + 127) / 128, P->N + 1, 2);
     size_t sm = size_t(P->nh) * 2 * NF * sizeof(T);
@@ -401,18 +400,18 @@ static int anal_t(sphnse_plan* P) {
     stage_begin(P, SPHNSE_STAGE_ANALYSIS);
     launch_pdl_small(P->n_cta, k_analysis<T, NF>, grd, blk, sm, P->stream,
                reinterpret_cast<const T*>(P->tab[sizeof(T) == 8 ? SPHNSE_FP64 : SPHNSE_FP32].ana),
-               reinterpret_cast<const T*>(P->d_gana), reinterpret_cast<T*>(P->d_hana), P->N, P->nh, P->nlat);
+               reinterpret_cast<const T*>(P->d_gana), reinterpret_cast<T*>(P->d_hana), P->N, P->nh, P->nlat, pairs);
     stage_end(P, SPHNSE_STAGE_ANALYSIS);
     return check_cuda(cudaGetLastError());
 }
 
-int launch_analysis(sphnse_plan* P, int nfields, int prec) {
+int launch_analysis(sphnse_plan* P, int nfields, int prec, int pairs) {
     if (stream_ok(P, prec)) {
-        int rc = launch_analysis_stream(P, nfields, prec);
+        int rc = launch_analysis_stream(P, nfields, prec, pairs);
         if (rc != SPHNSE_E_UNSUPPORTED) return rc;
     }
-    if (prec == SPHNSE_FP64) return nfields == 3 ? anal_t<double, 3>(P) : anal_t<double, 2>(P);
-    return nfields == 3 ? anal_t<float, 3>(P) : anal_t<float, 2>(P);
+    if (prec == SPHNSE_FP64) return nfields == 3 ? anal_t<double, 3>(P, pairs) : anal_t<double, 2>(P, pairs);
+    return nfields == 3 ? anal_t<float, 3>(P, pairs) : anal_t<float, 2>(P, pairs);
 }
 
 int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha, const double* forcing,

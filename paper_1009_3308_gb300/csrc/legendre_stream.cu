@@ -56,7 +56,7 @@ struct StreamArgs {
     // batches: an item v stands for instance v / (N+1) and order v % (N+1);
     // per-instance strides (elements) of bsyn, gsyn, gana, hana
     size_t sb, sg, sa, sh;
-    int pairs;           // gsyn layout (gsyn_index)
+    int pairs;           // gsyn and gana layout (gsyn_index)
 };
 
 // chunk c of order m: rows [c HR, c HR + HR) of the even and of the odd block
@@ -298,10 +298,10 @@ __global__ void __launch_bounds__(288, 1) k_ana_stream(StreamArgs a) {
         T* S = Ssm + size_t(ii & 1) * 2 * nh * 2 * NF;
         for (int i = ct; i < nh * NF; i += ncons) {
             const int f = i / nh, p = i % nh, pr = nlat - 1 - p;
-            const T* ga = gsrc + ((size_t(f) * (N + 1) + m) * nlat + p) * 2;
+            const T* ga = gsrc + gsyn_index(a.pairs, f, m, p, N, nlat) * 2;
             T ar = ga[0], ai = ga[1], br = T(0), bi = T(0);
             if (pr != p) {
-                const T* gb = gsrc + ((size_t(f) * (N + 1) + m) * nlat + pr) * 2;
+                const T* gb = gsrc + gsyn_index(a.pairs, f, m, pr, N, nlat) * 2;
                 br = gb[0];
                 bi = gb[1];
             }
@@ -392,7 +392,7 @@ static int syn_stream_t(sphnse_plan* P, int pairs) {
 }
 
 template <typename T, int NF>
-static int ana_stream_t(sphnse_plan* P) {
+static int ana_stream_t(sphnse_plan* P, int pairs) {
     constexpr int HR = half_rows<T>();
     constexpr int QPS = 2 * HR / 4;
     constexpr int NTEAM = 8 / QPS;
@@ -402,7 +402,7 @@ static int ana_stream_t(sphnse_plan* P) {
     if (sm > 227 * 1024) return SPHNSE_E_UNSUPPORTED;
     allow_dynamic_smem(reinterpret_cast<const void*>(k_ana_stream<T, NF, HR, NTEAM>), sm);
     StreamArgs a{P->tab[sizeof(T) == 8 ? SPHNSE_FP64 : SPHNSE_FP32].syn, nullptr, nullptr, P->d_gana, P->d_hana,
-                 P->d_s, P->d_items, P->d_item_off, P->d_status, P->N, P->nh, P->nlat, 0, 0, 0, 0, 0};
+                 P->d_s, P->d_items, P->d_item_off, P->d_status, P->N, P->nh, P->nlat, 0, 0, 0, 0, pairs};
     stage_begin(P, SPHNSE_STAGE_ANALYSIS);
     launch_pdl(k_ana_stream<T, NF, HR, NTEAM>, dim3(P->n_cta), dim3(threads), sm, P->stream, a);
     stage_end(P, SPHNSE_STAGE_ANALYSIS);
@@ -415,9 +415,9 @@ int launch_synthesis_stream(sphnse_plan* P, int nfields, int prec, int pairs) {
     return nfields == 5 ? syn_stream_t<float, 5>(P, pairs) : syn_stream_t<float, 3>(P, pairs);
 }
 
-int launch_analysis_stream(sphnse_plan* P, int nfields, int prec) {
-    if (prec == SPHNSE_FP64) return nfields == 3 ? ana_stream_t<double, 3>(P) : ana_stream_t<double, 2>(P);
-    return nfields == 3 ? ana_stream_t<float, 3>(P) : ana_stream_t<float, 2>(P);
+int launch_analysis_stream(sphnse_plan* P, int nfields, int prec, int pairs) {
+    if (prec == SPHNSE_FP64) return nfields == 3 ? ana_stream_t<double, 3>(P, pairs) : ana_stream_t<double, 2>(P, pairs);
+    return nfields == 3 ? ana_stream_t<float, 3>(P, pairs) : ana_stream_t<float, 2>(P, pairs);
 }
 
 // FP32 batched streaming passes over instances (items = inst * (N+1) + m)

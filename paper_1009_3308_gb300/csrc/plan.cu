@@ -146,7 +146,14 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     int rc;
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);
-    const bool ring4 = prec == SPHNSE_FP32 && ring4_ok(P);
+    if (prec == SPHNSE_FP64) {
+        if ((rc = launch_prep(P, alpha, nullptr, prec))) return rc;
+        if ((rc = launch_synthesis(P, 3, prec, 1))) return rc;
+        if ((rc = launch_ring_fx(P, RING_RHS, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
+        if ((rc = launch_analysis(P, 2, prec, 1))) return rc;
+        return launch_finish(P, 0, prec, alpha, forcing, out);
+    }
+    const bool ring4 = ring4_ok(P);
     // the tensor-core synthesis writes the latitude-pair-major layout the
     // four-step ring kernel reads contiguously (its epilogue warps are off the
     // streaming path); the FP32 streaming synthesis keeps the order-major one
@@ -162,9 +169,9 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
                                pairs)))
             return rc;
     } else {
-        if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 3, prec))) return rc;
-        if ((rc = launch_ring(P, RING_RHS, prec, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-        if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 2, prec))) return rc;
+        if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 3))) return rc;
+        if ((rc = launch_ring(P, RING_RHS, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
+        if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 2))) return rc;
     }
     if (tc) {
         // the finish step runs in the analysis epilogue where its shared
@@ -183,10 +190,16 @@ int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, dou
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     int rc;
     if ((rc = launch_prep(P, alpha, w, prec))) return rc;
+    if (prec == SPHNSE_FP64) {
+        if ((rc = launch_synthesis(P, 5, prec, 1))) return rc;
+        if ((rc = launch_ring_fx(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
+        if ((rc = launch_analysis(P, 3, prec, 1))) return rc;
+        return launch_finish(P, 2, prec, w, nullptr, out);
+    }
     if ((rc = launch_synthesis(P, 5, prec))) return rc;
-    if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 5, prec))) return rc;
-    if ((rc = launch_ring(P, RING_ADJOINT, prec, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-    if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 3, prec))) return rc;
+    if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 5))) return rc;
+    if ((rc = launch_ring(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
+    if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 3))) return rc;
     if ((rc = launch_analysis(P, 3, prec))) return rc;
     return launch_finish(P, 2, prec, w, nullptr, out);
 }
@@ -214,7 +227,7 @@ static void destroy_plan(sphnse_plan* P) {
     if (P->d_info) cudaFree(P->d_info);
     if (P->h_info) cudaFreeHost(P->h_info);
     void* ptrs[] = {P->d_items, P->d_item_off, P->d_status,
-                    P->d_x, P->d_s, P->d_isin32, P->d_rw, P->d_tw, P->d_tw32, P->d_ftw, P->d_lm, P->d_finc, P->d_prepc, P->d_finc32, P->d_prepc32, P->d_bsyn,
+                    P->d_x, P->d_s, P->d_isin32, P->d_rw, P->d_tw32, P->d_ftw, P->d_fxtw, P->d_lm, P->d_finc, P->d_prepc, P->d_finc32, P->d_prepc32, P->d_bsyn,
                     P->d_gsyn, P->d_gana, P->d_hana, P->d_gsyn_r, P->d_gana_r, P->d_grid, P->d_theta, P->d_w, P->d_work, P->d_tmp, P->d_norms};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -294,15 +307,13 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
         rc = SPHNSE_E_NOMEM;
     }
     // device constants
-    std::vector<double> rw(nlat), tw(2 * size_t(nlon));
+    std::vector<double> rw(nlat);
     std::vector<float> tw32(2 * size_t(nlon));
     for (int p = 0; p < nlat; ++p) rw[p] = (2.0 * M_PI / nlon) * P->w[p] / P->s[p];
     for (int t = 0; t < nlon; ++t) {
         const double ang = 2.0 * M_PI * double(t) / double(nlon);
-        tw[2 * t] = std::cos(ang);
-        tw[2 * t + 1] = -std::sin(ang);
-        tw32[2 * t] = float(tw[2 * t]);
-        tw32[2 * t + 1] = float(tw[2 * t + 1]);
+        tw32[2 * t] = float(std::cos(ang));
+        tw32[2 * t + 1] = float(-std::sin(ang));
     }
     std::vector<int2> lm(P->n_coeff);
     std::vector<double4_32a> finc(P->n_coeff), prepc(P->n_ext);
@@ -329,14 +340,15 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
         }
     }
     const size_t nc = size_t(P->n_coeff);
-    const size_t sz_g = size_t(nlat) * (L + 1) * 2 * sizeof(double);
+    const size_t sz_g = size_t(nlat + (nlat & 1)) * (L + 1) * 2 * sizeof(double);   // whole latitude pairs
     if (!rc) rc = dalloc(&P->d_x, nlat * sizeof(double));
     if (!rc) rc = dalloc(&P->d_s, nlat * sizeof(double));
     if (!rc) rc = dalloc(&P->d_isin32, nlat * sizeof(float));
     if (!rc) rc = dalloc(&P->d_rw, nlat * sizeof(double));
-    if (!rc) rc = dalloc(&P->d_tw, tw.size() * sizeof(double));
     if (!rc) rc = dalloc(&P->d_tw32, tw32.size() * sizeof(float));
     const std::vector<float> ftw = ring4_twiddles(nlon);
+    const std::vector<int> fxtw = ring_fx_twiddles(nlon);
+    if (!rc) rc = dalloc(&P->d_fxtw, fxtw.size() * sizeof(int));
     if (!rc && !ftw.empty()) rc = dalloc(&P->d_ftw, ftw.size() * sizeof(float));
     if (!rc) rc = dalloc(&P->d_lm, nc * sizeof(int2));
     if (!rc) rc = dalloc(&P->d_finc, nc * sizeof(double4_32a));
@@ -347,8 +359,8 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
     if (!rc) rc = dalloc(&P->d_gsyn, 5 * sz_g);
     if (!rc) rc = dalloc(&P->d_gana, 3 * sz_g);
     if (!rc) rc = dalloc(&P->d_hana, size_t(P->n_ext) * 6 * sizeof(double));
-    if (!rc) rc = dalloc(&P->d_gsyn_r, 5 * sz_g);
-    if (!rc) rc = dalloc(&P->d_gana_r, 3 * sz_g);
+    if (!rc) rc = dalloc(&P->d_gsyn_r, 5 * sz_g / 2);   // FP32 only
+    if (!rc) rc = dalloc(&P->d_gana_r, 3 * sz_g / 2);
     if (!rc) rc = dalloc(&P->d_work, 16 * nc * 2 * sizeof(double));
     if (!rc) rc = dalloc(&P->d_tmp, 2 * nc * 2 * sizeof(double));
     if (!rc) rc = dalloc(&P->d_norms, 16 * sizeof(unsigned long long));
@@ -365,8 +377,8 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
         up(P->d_isin32, isin.data(), nlat * sizeof(float));
     }
     up(P->d_rw, rw.data(), nlat * sizeof(double));
-    up(P->d_tw, tw.data(), tw.size() * sizeof(double));
     up(P->d_tw32, tw32.data(), tw32.size() * sizeof(float));
+    up(P->d_fxtw, fxtw.data(), fxtw.size() * sizeof(int));
     if (!ftw.empty()) up(P->d_ftw, ftw.data(), ftw.size() * sizeof(float));
     up(P->d_lm, lm.data(), nc * sizeof(int2));
     up(P->d_finc, finc.data(), nc * sizeof(double4_32a));
@@ -511,18 +523,24 @@ int sphnse_grid_fields(sphnse_plan* P, const double* alpha, double* zeta, double
         if ((rc = launch_synthesis_tc(P, alpha, 0))) return rc;
     } else {
         if ((rc = launch_prep(P, alpha, nullptr, prec))) return rc;
-        if ((rc = launch_synthesis(P, 3, prec))) return rc;
+        if ((rc = launch_synthesis(P, 3, prec, prec == SPHNSE_FP64))) return rc;
     }
-    if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 3, prec))) return rc;
-    return launch_ring(P, RING_GRID, prec, nullptr, nullptr, zeta, uth, uph);
+    if (prec == SPHNSE_FP64) return launch_ring_fx(P, RING_GRID, nullptr, nullptr, zeta, uth, uph);
+    if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 3))) return rc;
+    return launch_ring(P, RING_GRID, nullptr, nullptr, zeta, uth, uph);
 }
 
 int sphnse_project(sphnse_plan* P, const double* vth, const double* vph, double* out) {
     if (!P || !vth || !vph || !out) return SPHNSE_E_ARG;
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     int rc;
-    if ((rc = launch_ring(P, RING_PROJECT, prec, vth, vph, nullptr, nullptr, nullptr))) return rc;
-    if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 2, prec))) return rc;
+    if (prec == SPHNSE_FP64) {
+        if ((rc = launch_ring_fx(P, RING_PROJECT, vth, vph, nullptr, nullptr, nullptr))) return rc;
+        if ((rc = launch_analysis(P, 2, prec, 1))) return rc;
+        return launch_finish(P, 1, prec, nullptr, nullptr, out);
+    }
+    if ((rc = launch_ring(P, RING_PROJECT, vth, vph, nullptr, nullptr, nullptr))) return rc;
+    if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 2))) return rc;
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);
     if ((rc = tc ? launch_analysis_tc(P, 2) : launch_analysis(P, 2, prec))) return rc;
     return launch_finish(P, 1, prec, nullptr, nullptr, out);

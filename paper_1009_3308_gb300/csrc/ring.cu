@@ -1,4 +1,5 @@
-// Longitude ("ring") kernel: one CTA per Gauss latitude theta_p.
+// Longitude ("ring") kernels of the FP32 and BF16x3 paths (the FP64 path's
+// kernel is in ring_fx.cu).  General kernel: one CTA per Gauss latitude theta_p.
 //
 // RHS mode (Sec. 4.2: the phi sums of Eqs. (app_soln_rep), (eval_nonlin1)
 // are Fourier sums, evaluated by FFT):
@@ -10,9 +11,8 @@
 //      truncation to m = 0..N, scaling by (2 pi / M) w_p / sin(theta_p)
 //      (the quadrature weight of Eq. (quadrule) and the 1/sin of the basis).
 // M = nlon = 2^a 3^b; Stockham autosort radix-8/4/2/3 stages in shared memory
-// (radix 3 last, so every stride Ns before it is a power of two), FP64
-// twiddles e^{-2 pi i t / M} from the host (FP32 copy for FP32 mode) staged in
-// shared memory.
+// (radix 3 last, so every stride Ns before it is a power of two), twiddles
+// e^{-2 pi i t / M} computed in FP64 on the host, staged in shared memory.
 // Products keep |m| <= 2N and M >= 3N + 2 > 3N, so the truncated m <= N
 // coefficients are alias-free.
 //
@@ -251,7 +251,7 @@ static void ring_mode(sphnse_plan* P, int mode, const RingArgs& a, const TW* tw,
     }
 }
 
-int launch_ring(sphnse_plan* P, int mode, int prec, const double* gin0, const double* gin1,
+int launch_ring(sphnse_plan* P, int mode, const double* gin0, const double* gin1,
                 double* gout0, double* gout1, double* gout2) {
     RingArgs a;
     a.N = P->N;
@@ -274,8 +274,7 @@ int launch_ring(sphnse_plan* P, int mode, int prec, const double* gin0, const do
     int threads = ((P->nlon / 6 + 31) / 32) * 32;
     if (threads < 32) threads = 32;
     stage_begin(P, SPHNSE_STAGE_RING);
-    if (prec == SPHNSE_FP64) ring_mode<double, double>(P, mode, a, P->d_tw, threads);
-    else ring_mode<float, float>(P, mode, a, P->d_tw32, threads);
+    ring_mode<float, float>(P, mode, a, P->d_tw32, threads);
     stage_end(P, SPHNSE_STAGE_RING);
     return check_cuda(cudaGetLastError());
 }
@@ -415,14 +414,10 @@ __global__ void __launch_bounds__(256) k_transpose(const C* __restrict__ in, C* 
 }
 
 // in: [nf][R][Cn] -> out: [nf][Cn][R]
-int launch_transpose(sphnse_plan* P, const void* in, void* out, int R, int Cn, int nf, int prec) {
+int launch_transpose(sphnse_plan* P, const void* in, void* out, int R, int Cn, int nf) {
     dim3 blk(32, 8), grd((Cn + 31) / 32, (R + 31) / 32, nf);
     stage_begin(P, SPHNSE_STAGE_TRANSPOSE);
-    if (prec == SPHNSE_FP64)
-        launch_pdl_small(P->n_cta, k_transpose<double2>, grd, blk, 0, P->stream, reinterpret_cast<const double2*>(in),
-                   reinterpret_cast<double2*>(out), R, Cn);
-    else
-        launch_pdl_small(P->n_cta, k_transpose<float2>, grd, blk, 0, P->stream, reinterpret_cast<const float2*>(in),
+    launch_pdl_small(P->n_cta, k_transpose<float2>, grd, blk, 0, P->stream, reinterpret_cast<const float2*>(in),
                    reinterpret_cast<float2*>(out), R, Cn);
     stage_end(P, SPHNSE_STAGE_TRANSPOSE);
     return check_cuda(cudaGetLastError());
