@@ -82,9 +82,8 @@ bool make_fft_plan(int n, FFTPlan* p);
 // ---- device tables ----------------------------------------------------------
 struct Tables {
     void* syn = nullptr;     // [n_ext][nh]: rows of Pt over northern nodes (synthesis)
-    void* ana = nullptr;     // per (m, parity) block [nh][rows] (analysis)
+    void* ana = nullptr;     // FP32: per (m, parity) block [nh][rows] (analysis fallback)
     void* syn_lo = nullptr;  // BF16X3: low parts
-    void* ana_lo = nullptr;
     size_t bytes = 0;
     bool built = false;
 };
@@ -146,6 +145,25 @@ struct StepCtl {
     double A[SPHNSE_MAXK * SPHNSE_MAXK];     // difference rescaling matrix (do_rescale)
     double g[SPHNSE_MAXK];                   // predictor weights of psi
     NewtonCtl nc;
+};
+
+// One direction of the FP64 digit-split Legendre sums (legendre_dig.cu)
+struct DigSide {
+    unsigned char* blocks = nullptr;   // table digits in the order the kernel streams them
+    int* ea = nullptr;                 // row exponents
+    int4* items = nullptr;             // CTA c's items at c * istride
+    int* cnt = nullptr;
+    int4* pieces = nullptr;            // analysis: (m, parity, first ext row, rows) x 4 per tile
+    int ncta = 0, istride = 0;
+    size_t bytes = 0;
+};
+struct DigState {
+    DigSide syn, ana;
+    short4* eoff = nullptr;            // exponents of the coefficient sets per packed entry
+    double* isin = nullptr;            // 1 / sin(theta_p)
+    int* emax = nullptr;               // [3][N+1] largest biased exponents of the ring output; zero
+                                       // between calls (the finish kernel clears them)
+    bool ready = false;
 };
 
 // staging of sphnse_rhs_host: two slots, an upload and a download stream
@@ -245,9 +263,10 @@ struct sphnse_plan {
 
     sph::Tables tab[3];
     sph::TcState tc;
+    sph::DigState dig;
 
     // workspaces (sized for the largest field counts: 5 synthesis, 3 analysis)
-    void* d_bsyn = nullptr;      // [n_ext][2 * 5] (re, im) per field, precision type
+    void* d_bsyn = nullptr;      // [n_ext][2 * 5] (re, im) per field, FP32
     void* d_gsyn = nullptr;      // [5][N+1][nlat] complex (m-major)
     void* d_gana = nullptr;      // [3][N+1][nlat] complex (m-major)
     void* d_hana = nullptr;      // [n_ext][2 * 3]
@@ -308,14 +327,18 @@ namespace sph {
 // ---- launchers (kernels in *.cu) ------------------------------------------
 enum RingMode { RING_RHS = 0, RING_GRID = 1, RING_PROJECT = 2, RING_ADJOINT = 3 };
 
-// prep: coefficient sets for synthesis.  nsets fields from alpha (3: zeta,
+// FP32 prep: coefficient sets for synthesis.  nsets fields from alpha (3: zeta,
 // theta, phi) and optionally 2 more (theta, phi) from beta scaled by 1/s_m.
-int launch_prep(sphnse_plan* P, const double* alpha, const double* beta, int prec);
-// pairs != 0: write the latitude-pair-major layout of gsyn_index
-int launch_synthesis(sphnse_plan* P, int nfields, int prec, int pairs = 0);
+int launch_prep(sphnse_plan* P, const double* alpha, const double* beta);
+int launch_synthesis(sphnse_plan* P, int nfields);   // FP32, order-major
 int launch_ring(sphnse_plan* P, int mode, const double* gin0, const double* gin1,
                 double* gout0, double* gout1, double* gout2);
-int launch_analysis(sphnse_plan* P, int nfields, int prec, int pairs = 0);
+int launch_analysis(sphnse_plan* P, int nfields);
+// FP64 Legendre sums on the tensor cores (beta: the adjoint's fields 3, 4; nf analysis fields)
+int dig_setup(sphnse_plan* P, const double* d_tab);
+void dig_free(sphnse_plan* P);
+int launch_synthesis_dig(sphnse_plan* P, const double* alpha, const double* beta);
+int launch_analysis_dig(sphnse_plan* P, int nf);
 // the FP64 ring kernel (64-bit fixed point) on the latitude-pair-major buffers
 std::vector<int> ring_fx_twiddles(int nlon);
 int launch_ring_fx(sphnse_plan* P, int mode, const double* gin0, const double* gin1, double* gout0, double* gout1,
@@ -328,8 +351,8 @@ int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha,
                   const double* forcing, double* out);
 
 int ensure_tables(sphnse_plan* P, int prec);
-bool stream_ok(const sphnse_plan* P, int prec);
-int launch_synthesis_stream(sphnse_plan* P, int nfields, int prec, int pairs = 0);
+bool stream_ok(const sphnse_plan* P);
+int launch_synthesis_stream(sphnse_plan* P, int nfields);
 bool tc_supported(const sphnse_plan* P);
 int launch_analysis_tc(sphnse_plan* P, int nfields);
 // the RHS's analysis (two product fields) with the recombination and update
@@ -371,7 +394,7 @@ int launch_finish32_batch(sphnse_plan* P, int nb, const float* hana, size_t hstr
                           double* out, const double* nu_inst);
 void tc_free(sphnse_plan* P);
 void host_io_free(sphnse_plan* P);
-int launch_analysis_stream(sphnse_plan* P, int nfields, int prec, int pairs = 0);
+int launch_analysis_stream(sphnse_plan* P, int nfields);
 void stage_begin(sphnse_plan* P, int stage);
 void stage_end(sphnse_plan* P, int stage);
 int check_cuda(cudaError_t e);

@@ -6,8 +6,9 @@
 //              profiles (Eq. (disc_vec_orth_proj))
 //   finish     degree-shift recombination and the diagonal Stokes update
 //              (Sec. 4.2: nu lambda_L alpha_{L,m}) plus forcing.
-// Templated on the contraction type T (double for SPHNSE_FP64, float for
-// SPHNSE_FP32); the coefficient state in and out is always FP64.
+// Prep, synthesis and analysis serve the FP32 path (the FP64 sums are in
+// legendre_dig.cu), the finish both; the coefficient state in and out is
+// always FP64.
 #include <cuda_runtime.h>
 
 #include "finish.cuh"
@@ -22,46 +23,9 @@ namespace sph {
 //   field 1 (theta): a_K = lambda_K^{-1/2} alpha_K
 //   field 2 (phi):   (K-1) eps_{K,m} a_{K-1} - (K+2) eps_{K+1,m} a_{K+1}
 // (sin(theta) d/dtheta Pt_L^m = L eps_{L+1,m} Pt_{L+1}^m - (L+1) eps_{L,m} Pt_{L-1}^m
-//  regrouped by degree).  The FP64 coefficients come precomputed per row
-// (c = (lam^{1/2}, lam^{-1/2}, c_down, c_up)) so that the kernel does no
-// FP64 square roots or divisions.  With beta (adjoint): fields 3, 4 are the
-// theta/phi sets of beta / s_m, s_m = 1 (m = 0) or 2.
-template <typename T>
-__global__ void k_prep(const double2* __restrict__ alpha, const double2* __restrict__ beta,
-                       const double4_32a* __restrict__ prepc, T* __restrict__ bsyn, int N, int nf) {
-    // no early trigger: at large L this grid has several waves, and the
-    // streaming synthesis after it (programmatic launch, one CTA per SM)
-    // would hold SMs its later waves need
-    pdl_wait();   // alpha may be the predecessor's output
-    const int m = blockIdx.y;
-    const int K = m + blockIdx.x * blockDim.x + threadIdx.x;
-    if (K > N + 1) return;
-    const int lo = m > 0 ? m : 1;
-    const int row = ext_row(N, m, K);
-    const double4_32a c = prepc[row];
-    auto A = [&](const double2* v, int Kp) -> double2 {
-        return (Kp < lo || Kp > N) ? make_double2(0.0, 0.0) : v[packed_index(N, m, Kp)];
-    };
-    T* out = bsyn + size_t(row) * (2 * nf);
-    {
-        const double2 a0 = A(alpha, K), am = A(alpha, K - 1), ap = A(alpha, K + 1);
-        out[0] = T(c.x * a0.x);
-        out[1] = T(c.x * a0.y);
-        out[2] = T(c.y * a0.x);
-        out[3] = T(c.y * a0.y);
-        out[4] = T(c.z * am.x + c.w * ap.x);
-        out[5] = T(c.z * am.y + c.w * ap.y);
-    }
-    if (nf == 5) {
-        const double sc = m == 0 ? 1.0 : 0.5;
-        const double2 b0 = A(beta, K), bm = A(beta, K - 1), bp = A(beta, K + 1);
-        out[6] = T(sc * (c.y * b0.x));
-        out[7] = T(sc * (c.y * b0.y));
-        out[8] = T(sc * (c.z * bm.x + c.w * bp.x));
-        out[9] = T(sc * (c.z * bm.y + c.w * bp.y));
-    }
-}
-
+//  regrouped by degree).  The coefficients come precomputed per row, c =
+// (lam^{1/2}, lam^{-1/2}, c_down, c_up).  With beta (adjoint): fields 3, 4 are
+// the theta/phi sets of beta / s_m, s_m = 1 (m = 0) or 2.
 // FP32-path prep: alpha_K is converted once per row and its degree
 // neighbours come from shared memory; the arithmetic is FP32 (the FP32 path
 // contracts in FP32 anyway), keeping the weak FP64 pipe for the state only.
@@ -122,7 +86,7 @@ __global__ void __launch_bounds__(128) k_prep32(const double2* __restrict__ alph
 template <typename T, int NF>
 __global__ void __launch_bounds__(128) k_synthesis(const T* __restrict__ psyn, const T* __restrict__ bsyn,
                                                     T* __restrict__ gsyn, const double* __restrict__ sinth,
-                                                    int N, int nh, int nlat, int pairs) {
+                                                    int N, int nh, int nlat) {
     pdl_launch();
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -173,7 +137,7 @@ __global__ void __launch_bounds__(128) k_synthesis(const T* __restrict__ psyn, c
                 outr = -gr * inv_s;
                 outi = -gi * inv_s;
             }
-            T* dst = gsyn + gsyn_index(pairs, f, m, row, N, nlat) * 2;
+            T* dst = gsyn + gsyn_index(0, f, m, row, N, nlat) * 2;
             dst[0] = outr;
             dst[1] = outi;
         }
@@ -188,7 +152,7 @@ __global__ void __launch_bounds__(128) k_synthesis(const T* __restrict__ psyn, c
 // (and sin(theta_p) for the scalar adjoint field).
 template <typename T, int NF>
 __global__ void __launch_bounds__(128) k_analysis(const T* __restrict__ pana, const T* __restrict__ gana,
-                                                   T* __restrict__ hana, int N, int nh, int nlat, int pairs) {
+                                                   T* __restrict__ hana, int N, int nh, int nlat) {
     pdl_launch();
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -201,10 +165,10 @@ __global__ void __launch_bounds__(128) k_analysis(const T* __restrict__ pana, co
     for (int i = threadIdx.x; i < nh * NF; i += blockDim.x) {
         const int p = i / NF, f = i % NF;
         const int pr = nlat - 1 - p;
-        const T* a = gana + gsyn_index(pairs, f, m, p, N, nlat) * 2;
+        const T* a = gana + gsyn_index(0, f, m, p, N, nlat) * 2;
         T ar = a[0], ai = a[1], br = T(0), bi = T(0);
         if (pr != p) {
-            const T* b = gana + gsyn_index(pairs, f, m, pr, N, nlat) * 2;
+            const T* b = gana + gsyn_index(0, f, m, pr, N, nlat) * 2;
             br = b[0];
             bi = b[1];
         }
@@ -245,10 +209,12 @@ template <typename T>
 __global__ void k_finish(int kind, const T* __restrict__ hana, int nf, const double2* __restrict__ alpha,
                          const double2* __restrict__ forcing, double2* __restrict__ out,
                          const int2* __restrict__ lm, const double4_32a* __restrict__ finc, int N, double nu,
-                         int n, double omega_d) {
+                         int n, double omega_d, int* __restrict__ emax) {
     pdl_launch();
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    // the analysis is done with the column exponents: zero for the next ring
+    for (int j = i; j < 3 * (N + 1); j += gridDim.x * blockDim.x) emax[j] = 0;
     if (i >= n) return;
     const int L = lm[i].x, m = lm[i].y;
     const double4_32a c = finc[i];
@@ -341,20 +307,7 @@ __global__ void k_finish32(int kind, const float* __restrict__ hana, int nf, con
 // ---------------------------------------------------------------------------
 // launchers
 
-template <typename T>
-static int prep_t(sphnse_plan* P, const double* alpha, const double* beta) {
-    const int nf = beta ? 5 : 3;
-    dim3 blk(128), grd((P->N + 2 + 127) / 128, P->N + 1);
-    stage_begin(P, SPHNSE_STAGE_PREP);
-    launch_pdl_small(P->n_cta, k_prep<T>, grd, blk, 0, P->stream, reinterpret_cast<const double2*>(alpha),
-               reinterpret_cast<const double2*>(beta), static_cast<const double4_32a*>(P->d_prepc),
-               reinterpret_cast<T*>(P->d_bsyn), P->N, nf);
-    stage_end(P, SPHNSE_STAGE_PREP);
-    return check_cuda(cudaGetLastError());
-}
-
-int launch_prep(sphnse_plan* P, const double* alpha, const double* beta, int prec) {
-    if (prec == SPHNSE_FP64) return prep_t<double>(P, alpha, beta);
+int launch_prep(sphnse_plan* P, const double* alpha, const double* beta) {
     const int nf = beta ? 5 : 3;
     dim3 blk(128), grd((P->N + 2 + 127) / 128, P->N + 1);
     stage_begin(P, SPHNSE_STAGE_PREP);
@@ -366,31 +319,30 @@ int launch_prep(sphnse_plan* P, const double* alpha, const double* beta, int pre
 }
 
 template <typename T, int NF>
-static int synth_t(sphnse_plan* P, int pairs) {
+static int synth_t(sphnse_plan* P) {
     dim3 blk(128), grd((P->nh + 127) / 128, P->N + 1);
     size_t sm = size_t(P->N + 2) * 2 * NF * sizeof(T);
     if (sm > 48 * 1024)
         allow_dynamic_smem(reinterpret_cast<const void*>(k_synthesis<T, NF>), sm);
     stage_begin(P, SPHNSE_STAGE_SYNTHESIS);
     launch_pdl_small(P->n_cta, k_synthesis<T, NF>, grd, blk, sm, P->stream,
-               reinterpret_cast<const T*>(P->tab[sizeof(T) == 8 ? SPHNSE_FP64 : SPHNSE_FP32].syn),
+               reinterpret_cast<const T*>(P->tab[SPHNSE_FP32].syn),
                reinterpret_cast<const T*>(P->d_bsyn), reinterpret_cast<T*>(P->d_gsyn),
-               static_cast<const double*>(P->d_s), P->N, P->nh, P->nlat, pairs);
+               static_cast<const double*>(P->d_s), P->N, P->nh, P->nlat);
     stage_end(P, SPHNSE_STAGE_SYNTHESIS);
     return check_cuda(cudaGetLastError());
 }
 
-int launch_synthesis(sphnse_plan* P, int nfields, int prec, int pairs) {
-    if (stream_ok(P, prec)) {
-        int rc = launch_synthesis_stream(P, nfields, prec, pairs);
+int launch_synthesis(sphnse_plan* P, int nfields) {
+    if (stream_ok(P)) {
+        int rc = launch_synthesis_stream(P, nfields);
         if (rc != SPHNSE_E_UNSUPPORTED) return rc;
     }
-    if (prec == SPHNSE_FP64) return nfields == 5 ? synth_t<double, 5>(P, pairs) : synth_t<double, 3>(P, pairs);
-    return nfields == 5 ? synth_t<float, 5>(P, pairs) : synth_t<float, 3>(P, pairs);
+    return nfields == 5 ? synth_t<float, 5>(P) : synth_t<float, 3>(P);
 }
 
 template <typename T, int NF>
-static int anal_t(sphnse_plan* P, int pairs) {
+static int anal_t(sphnse_plan* P) {
     const int maxrows = ext_even(P->N, 0);
     dim3 blk(128), grd((maxrows + 127) / 128, P->N + 1, 2);
     size_t sm = size_t(P->nh) * 2 * NF * sizeof(T);
@@ -399,19 +351,18 @@ static int anal_t(sphnse_plan* P, int pairs) {
     }
     stage_begin(P, SPHNSE_STAGE_ANALYSIS);
     launch_pdl_small(P->n_cta, k_analysis<T, NF>, grd, blk, sm, P->stream,
-               reinterpret_cast<const T*>(P->tab[sizeof(T) == 8 ? SPHNSE_FP64 : SPHNSE_FP32].ana),
-               reinterpret_cast<const T*>(P->d_gana), reinterpret_cast<T*>(P->d_hana), P->N, P->nh, P->nlat, pairs);
+               reinterpret_cast<const T*>(P->tab[SPHNSE_FP32].ana),
+               reinterpret_cast<const T*>(P->d_gana), reinterpret_cast<T*>(P->d_hana), P->N, P->nh, P->nlat);
     stage_end(P, SPHNSE_STAGE_ANALYSIS);
     return check_cuda(cudaGetLastError());
 }
 
-int launch_analysis(sphnse_plan* P, int nfields, int prec, int pairs) {
-    if (stream_ok(P, prec)) {
-        int rc = launch_analysis_stream(P, nfields, prec, pairs);
+int launch_analysis(sphnse_plan* P, int nfields) {
+    if (stream_ok(P)) {
+        int rc = launch_analysis_stream(P, nfields);
         if (rc != SPHNSE_E_UNSUPPORTED) return rc;
     }
-    if (prec == SPHNSE_FP64) return nfields == 3 ? anal_t<double, 3>(P, pairs) : anal_t<double, 2>(P, pairs);
-    return nfields == 3 ? anal_t<float, 3>(P, pairs) : anal_t<float, 2>(P, pairs);
+    return nfields == 3 ? anal_t<float, 3>(P) : anal_t<float, 2>(P);
 }
 
 int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha, const double* forcing,
@@ -425,7 +376,7 @@ int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha, const
                                                      reinterpret_cast<const double2*>(alpha),
                                                      reinterpret_cast<const double2*>(forcing),
                                                      reinterpret_cast<double2*>(out), P->d_lm, P->d_finc, P->N, P->nu, n,
-                                                     kind == 0 && P->coriolis_split ? P->Omega : 0.0);
+                                                     kind == 0 && P->coriolis_split ? P->Omega : 0.0, P->dig.emax);
     else
         launch_pdl(k_finish32, grd, blk, 0, P->stream, kind, static_cast<const float*>(P->d_hana), nf,
                    reinterpret_cast<const double2*>(alpha), reinterpret_cast<const double2*>(forcing),

@@ -1,0 +1,831 @@
+// FP64 Legendre synthesis and analysis on the tcgen05 tensor cores, by exact
+// digit splitting (the error-free splitting of matrix products of Ozaki,
+// Ogita, Oishi and Rump, Numer. Algorithms 59 (2012)).
+//
+// Every table row is scaled by a power of two to |a| < 1 and cut into seven
+// balanced base-256 digits, every coefficient (or profile) column to |b| <=
+// 1/2 and eight digits:  a = sum_i a_i 2^(1 - 8 i),  b = sum_j b_j 2^(1 - 8 j),
+// |a_i|, |b_j| <= 128.  Digits are exact in BF16, their products are integers
+// of at most 2^14, and sums over the contracted index stay below 2^24 in the
+// leading groups, so the tensor core's FP32 accumulators hold them exactly.
+// The products of i + j = s share one accumulator group, s = 2 .. 9 (synthesis:
+// .. 10):
+//     sum_k a b = sum_s 2^(2 - 8 s) D_s,   D_s = sum_{i + j = s} sum_k a_i b_j,
+// and the epilogue adds the groups in integers.  What is left out (the eighth
+// digit of a, products with larger i + j) is about 2^-57 of max|a| |b| per term;
+// an FP64 multiply-add chain over 256 terms rounds to about 2^-50 of max|a| max|b|.
+//
+// Per K = 16 step one tile of 128 table rows takes seven MMAs, digit i of the
+// table against digits 1 .. 9 - i (10 - i) of the columns (N = G (9 - i), G
+// columns per group): with the columns of a group adjacent, those digits are a prefix of
+// the B rows and land on the groups from i + 1 on, a contiguous run of accumulator
+// columns.  The table digits are laid out once per plan in the order the
+// kernels consume them: one 28 KB block per (tile, K step) = 7 planes of 128 x
+// 16 in the un-swizzled core-matrix layout, so a stage is one bulk copy and
+// blocks whose digits are all zero (polar latitudes at high order) are left
+// out.
+//
+// Bound: HBM.  14 bytes per table entry against 8 of the FP64 table, but the
+// FP64 pipe (two operations per clock per SM) needs 10 multiply-adds per entry
+// and RHS: 0.8 ms at L = 511, where the two digit streams take 0.22 ms.
+// Measured (event pairs, GB300) against the FP64 multiply-add kernels and their
+// prep: L = 511 synthesis 558 -> 137 us, analysis 429 -> 111 us; L = 255 96 ->
+// 35, 74 -> 27; L = 100 41 -> 16, 22 -> 12; L = 31 21 -> 13, 10 -> 10.  Errors
+// against 64-bit references are those of the multiply-add kernels or smaller
+// for F, the fields and the projection at 23 sizes (mean over 24 states: u_phi
+// 3.3e-15 and u_theta 8.5e-16 at L = 255, before 3.4e-15 and 1.1e-15).
+//
+// Synthesis tiles: rows 0 .. 63 the even, rows 64 .. 127 the odd degrees of one
+// order on 64 northern latitudes (columns 0 .. G/2-1 of a group belong to the
+// even, the others to the odd degrees), so north = E + O and south = E - O
+// meet in one epilogue.  Analysis tiles: four pieces of up to 32 rows of one
+// (order, parity), one per epilogue warp, each with its own G / 4 columns.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "fx64.cuh"
+#include "internal.h"
+#include "tc.cuh"
+
+namespace sph {
+
+constexpr int DG_PLANE = 128 * 16 * 2;       // 4 KB: 128 rows x 16 of the contracted index
+constexpr int DG_ABYTES = 7 * DG_PLANE;      // one stage of table digits
+constexpr int DG_NB = 6;                     // builder warps
+constexpr int DG_MINEXP = -30;               // row scales are at least 2^-30 (smaller rows lose digits below 2^-86)
+// Orders below DG_SEGM take their first K step (the lowest degrees) apart,
+// with its own row exponents and with the remainder that its seven digits
+// leave of the table as a second block of digits; the epilogue adds the parts.
+// At the poles Pt_K^m grows like K^(m + 1/2), so with one exponent per row the
+// largest coefficients, at the lowest degrees, would meet table entries 2^13
+// below the row's maximum (L = 511, m = 1); at m = 0 the degree-shift sum of
+// u_phi cancels there; and the division by sin(theta) carries these errors
+// into u (u_theta 2.4e-15 against 1.3e-15 of the FP64 sums at L = 511).
+constexpr int DG_SEGM = 8;
+constexpr int DG_NAN = 1 << 20;              // exponent of a column with a non-finite entry
+
+// byte offset of element (row, k) of a K = 16 tile: 8 x 8 core matrices of 128
+// bytes, the two of a row group adjacent
+__host__ __device__ constexpr int dg_off(int row, int k) {
+    return (row >> 3) * 256 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
+}
+// shared-memory descriptor of that layout: K-major, no swizzle
+__device__ __forceinline__ uint64_t dg_desc(const void* smem_ptr) {
+    uint64_t d = 0;
+    d |= uint64_t((smem_u32(smem_ptr) & 0x3FFFF) >> 4);
+    d |= uint64_t(128 >> 4) << 16;   // to the next core matrix along K
+    d |= uint64_t(256 >> 4) << 32;   // to the next 8 rows
+    d |= uint64_t(1) << 46;
+    return d;
+}
+
+__device__ __forceinline__ int dg_steps(int n) { return (n + 15) / 16; }
+
+// ---------------------------------------------------------------------------
+// table digits (once per plan)
+
+// row exponents: |P| < 2^e over a row.  Synthesis rows are (m, latitude p)
+// over all degrees of the order, analysis rows are the ext rows over p.
+__global__ void k_dig_syn_scale(const double* __restrict__ tab, int* __restrict__ ea, int N, int nh) {
+    const int m = blockIdx.y, p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= nh) return;
+    const int ne = ext_even(N, m), cnt = ext_count(N, m);
+    const double* t = tab + size_t(ext_off(N, m)) * nh + p;
+    int e0 = 0, e1 = 0;   // first step, later steps
+    for (int r = 0; r < cnt; ++r) {
+        const int b = f64_bexp(t[size_t(r) * nh]);
+        if ((r < ne ? r : r - ne) < 16) e0 = max(e0, b);
+        else e1 = max(e1, b);
+    }
+    if (m >= DG_SEGM) e0 = e1 = max(e0, e1);
+    ea[m * nh + p] = max(e0 - 1022, DG_MINEXP);
+    if (m < DG_SEGM) ea[(N + 1 + m) * nh + p] = max(e1 - 1022, DG_MINEXP);
+}
+__global__ void k_dig_ana_scale(const double* __restrict__ tab, int* __restrict__ ea, int n_ext, int nh) {
+    const int r = blockIdx.x * 4 + threadIdx.x / 32;
+    if (r >= n_ext) return;
+    int e = 0;
+    for (int p = threadIdx.x & 31; p < nh; p += 32) e = max(e, f64_bexp(tab[size_t(r) * nh + p]));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) ea[r] = max(e - 1022, DG_MINEXP);
+}
+
+// seven digits of eight scaled entries -> one 16-byte chunk per plane; returns whether any is nonzero
+__device__ __forceinline__ bool dig_store(const double (&x)[8], const int (&e)[8], unsigned char* dst) {
+    long long u[8];
+    bool any = false;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const long long v = f64_to_fx(x[i], 55 - e[i]);
+        any = any || v != 0;
+        u[i] = v + 0x0080808080808080LL;
+    }
+#pragma unroll
+    for (int d = 0; d < 7; ++d) {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            // the top digit may reach +128: not masked to a byte
+            const int a = int(u[2 * i] >> (48 - 8 * d)), b = int(u[2 * i + 1] >> (48 - 8 * d));
+            const float fa = float((d == 0 ? a : a & 255) - 128), fb = float((d == 0 ? b : b & 255) - 128);
+            const __nv_bfloat162 h = __floats2bfloat162_rn(fa, fb);
+            w[i] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        *reinterpret_cast<uint4*>(dst + d * DG_PLANE) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    return any;
+}
+
+// block = (step, latitude tile, order): thread = (row, half of the step)
+__global__ void __launch_bounds__(256) k_dig_syn(const double* __restrict__ tab, const int* __restrict__ ea,
+                                                 const int* __restrict__ base, unsigned char* __restrict__ out,
+                                                 int* __restrict__ used, int N, int nh, int ntile, int remainder) {
+    const int m = blockIdx.z, t = blockIdx.y, ks = blockIdx.x, ne = ext_even(N, m);
+    if (ks >= dg_steps(ne)) return;
+    const int row = threadIdx.x & 127, h = threadIdx.x >> 7, par = row >> 6, p = t * 64 + (row & 63);
+    const int n = par ? ext_odd(N, m) : ne;
+    const double* src = tab + size_t(ext_off(N, m) + (par ? ne : 0)) * nh + p;
+    const int mr = m < DG_SEGM && ks > 0 ? N + 1 + m : m;   // row of exponents
+    double x[8];
+    int e[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int j = ks * 16 + h * 8 + i;
+        x[i] = j < n && p < nh ? src[size_t(j) * nh] : 0.0;
+        e[i] = p < nh ? ea[mr * nh + p] : 0;
+        if (remainder) {   // what the seven digits leave (exact: x has 53 bits)
+            x[i] -= scalbn(double(f64_to_fx(x[i], 55 - e[i])), e[i] - 55);
+            e[i] -= 55;
+        }
+    }
+    const int blk = base[m * ntile + t] + ks;
+    const bool any = dig_store(x, e, out + size_t(blk) * DG_ABYTES + dg_off(row, h * 8));
+    if (__syncthreads_or(any) && threadIdx.x == 0) used[blk] = 1;
+}
+__global__ void __launch_bounds__(256) k_dig_ana(const double* __restrict__ tab, const int* __restrict__ ea,
+                                                 const int4* __restrict__ pieces, unsigned char* __restrict__ out,
+                                                 int* __restrict__ used, int nh) {
+    const int tile = blockIdx.y, ks = blockIdx.x, nks = gridDim.x;
+    const int h = threadIdx.x & 1, row = threadIdx.x >> 1;
+    const int4 pc = pieces[4 * tile + (row >> 5)];
+    const bool in = (row & 31) < pc.w;
+    const int r = pc.z + (row & 31);
+    double x[8];
+    int e[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int p = ks * 16 + h * 8 + i;
+        x[i] = in && p < nh ? tab[size_t(r) * nh + p] : 0.0;
+        e[i] = in ? ea[r] : 0;
+    }
+    const int blk = tile * nks + ks;
+    const bool any = dig_store(x, e, out + size_t(blk) * DG_ABYTES + dg_off(row, h * 8));
+    if (__syncthreads_or(any) && threadIdx.x == 0) used[blk] = 1;
+}
+
+// ---------------------------------------------------------------------------
+
+struct DigArgs {
+    const unsigned char* blocks;  // table digits, DG_ABYTES per (tile, step)
+    const int4* items;            // (m | flags (or analysis tile), latitude tile, first step | end
+                                  //  step << 16, first block); flags of the parts of a split item: bit 16
+                                  //  another part follows, 17 exponents of the later steps, 18 a part
+                                  //  precedes, 19 remainder of the first step (exponents lower by 55)
+    const int* cnt;               // items of every CTA, at c * istride
+    int istride;
+    int evict_first;              // the digits exceed what L2 can keep
+    const int* ea;                // row exponents
+    unsigned* status;
+    int N, nh, nlat;
+    // synthesis
+    const double2* alpha;
+    const double2* beta;          // adjoint: fields 3, 4
+    const double4_32a* prepc;
+    const short4* eoff;           // exponents of the coefficient sets per packed entry
+    double* gsyn;                 // [nf][pair][N+1][2] complex
+    const double* isin;           // 1 / sin(theta_p)
+    // analysis
+    const int4* pieces;           // (m, parity, first ext row, rows) x 4 per tile
+    const double* gana;           // [nf][pair][N+1][2] complex
+    const int* emax;              // largest biased exponent of gana per (field, order)
+    double* hana;                 // [n_ext][2 nf]
+};
+
+// two scaled values of a column (contracted indexes 2 w, 2 w + 1) -> word w of the column's
+// rows of all eight digits; stride: bytes between the digits
+__device__ __forceinline__ void dig_put(unsigned char* dst, int stride, long long b0, long long b1) {
+    const unsigned long long u0 = (unsigned long long)b0 + 0x8080808080808080ULL;
+    const unsigned long long u1 = (unsigned long long)b1 + 0x8080808080808080ULL;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const uint32_t s0 = j < 4 ? uint32_t(u0 >> 32) : uint32_t(u0), s1 = j < 4 ? uint32_t(u1 >> 32) : uint32_t(u1);
+        // 2^23 + byte, minus 2^23 + 128
+        const int sel = 0x7650 | (3 - (j & 3));
+        const float f0 = __uint_as_float(__byte_perm(s0, 0x4B000000u, sel)) - 8388736.f;
+        const float f1 = __uint_as_float(__byte_perm(s1, 0x4B000000u, sel)) - 8388736.f;
+        const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
+        *reinterpret_cast<uint32_t*>(dst + j * stride) = *reinterpret_cast<const uint32_t*>(&h);
+    }
+}
+
+// sum_s D_s 2^(2 - 8 s) 2^e: the groups of one output added exactly, as
+// h 2^-54 + r 2^-70, and rounded once to binary64
+template <int NG>
+__device__ __forceinline__ double dig_val(const uint32_t* d, int stride, int e) {
+    int g[NG];
+#pragma unroll
+    for (int s = 0; s < NG; ++s) g[s] = __float2int_rn(__uint_as_float(d[s * stride]));
+    const long long h = ((long long)g[0] << 40) + ((long long)g[1] << 32) + ((long long)g[2] << 24) +
+                        ((long long)g[3] << 16) + ((long long)g[4] << 8) + g[5];
+    long long r = (long long)g[6] * 256 + g[7];
+    if constexpr (NG > 8) r += (g[8] + 128) >> 8;
+    if (e >= DG_NAN / 2) return __longlong_as_double(0x7FF8000000000000LL);
+    // as many of r's bits as fit below h (|h| <= 2^61)
+    const int sh = min(16, max(0, __clzll(h ^ (h >> 63)) - 3));
+    const long long v = (h << sh) + (r >> (16 - sh));
+    return v == 0 ? 0.0 : f64_scale(__ll2double_rn(v), e - 54 - sh);
+}
+
+template <bool SYN, int NF> struct DigShape {
+    // columns of one order and parity, padded; group width; pipeline stages
+    static constexpr int C = 2 * NF;
+    static constexpr int CP = SYN ? (C <= 8 ? 8 : 16) : (C <= 4 ? 4 : 8);
+    static constexpr int G = SYN ? 2 * CP : 4 * CP;
+    // accumulator groups i + j = 2 .. NG + 1.  The synthesis takes one more:
+    // near the poles the rows of the lowest orders grow like K^(m + 1/2), so a
+    // row's maximum meets the small high-degree coefficients, and the sum that
+    // matters is well below max|a| max|b| (and is then divided by sin(theta))
+    static constexpr int NG = SYN ? 9 : 8;
+    static constexpr int BBYTES = NG * G * 32;               // eight digits of the columns, SYN: a zero digit
+    static constexpr int NACC = 2 * NG * G <= 512 ? 2 : 1;   // accumulator buffers
+    static constexpr int TCOLS = NACC * NG * G <= 256 ? 256 : 512;
+    static constexpr int NS = G == 16 ? 6 : 5;
+    static constexpr int XCH = SYN ? 2 * 128 * C * 8 : 0;   // even and odd sums meet here
+    static constexpr int WARPS = 6 + DG_NB + (SYN ? 1 : 0);
+    static constexpr size_t smem(int istride) {
+        return 1024 + size_t(NS) * (DG_ABYTES + BBYTES) + XCH + 512 + size_t(istride) * (16 + 8 + 20);
+    }
+};
+
+template <bool SYN, int NF>
+__global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArgs a) {
+    using Q = DigShape<SYN, NF>;
+    constexpr int NS = Q::NS, G = Q::G, C = Q::C, CP = Q::CP, NG = Q::NG, NACC = Q::NACC;
+    static_assert(DG_NB >= NS, "every stage of the ring has a builder");
+    constexpr int NBW = NS;   // builders may not run a full ring ahead (one stage each)
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                           ~uintptr_t(1023));
+    unsigned char* As = smem;
+    unsigned char* Bs = As + NS * DG_ABYTES;
+    double* xch = reinterpret_cast<double*>(Bs + NS * Q::BBYTES);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(xch) + Q::XCH);
+    uint64_t* a_full = bars;
+    uint64_t* b_full = a_full + NS;
+    uint64_t* empty = b_full + NS;
+    uint64_t* acc_full = empty + NS;
+    uint64_t* acc_empty = acc_full + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    int4* s_items = reinterpret_cast<int4*>(reinterpret_cast<unsigned char*>(bars) + 512);
+    uint64_t* sc_full = reinterpret_cast<uint64_t*>(s_items + a.istride);   // SYN: column exponents of an item ready
+    int* s_eb = reinterpret_cast<int*>(sc_full + a.istride);               // [item][5]
+    const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+    const int N = a.N, nh = a.nh, nlat = a.nlat, npair = (nlat + 1) / 2;
+    const int nI = a.cnt[blockIdx.x];
+    for (int i = threadIdx.x; i < a.istride; i += blockDim.x) {
+        s_items[i] = a.items[blockIdx.x * a.istride + i];
+        mbar_init(&sc_full[i], 1);
+    }
+    for (int i = threadIdx.x; i < NS * Q::BBYTES / 16; i += blockDim.x)
+        reinterpret_cast<uint4*>(Bs)[i] = make_uint4(0u, 0u, 0u, 0u);
+    fence_proxy_async_smem();
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(&a_full[s], 1);
+            mbar_init(&b_full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < NACC; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], 128);
+        }
+        *abort = 0;
+    }
+    fence_barrier_init();
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, Q::TCOLS);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    pdl_launch();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        if (elect_one()) {
+            // the table does not depend on the predecessor: stream right away
+            const uint64_t pol = a.evict_first ? policy_evict_first() : policy_evict_last();
+            int it = 0;
+            for (int i = 0; i < nI; ++i) {
+                const int4 itm = s_items[i];
+                const unsigned char* src = a.blocks + size_t(itm.w) * DG_ABYTES;
+                const int k1 = itm.z >> 16;
+                for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, ++it) {
+                    const int s = it % NS;
+                    if (it >= NS && !mbar_wait(&empty[s], ((it / NS) - 1) & 1, abort, a.status)) continue;
+                    if (*abort) continue;
+                    mbar_arrive_expect_tx(&a_full[s], DG_ABYTES);
+                    bulk_g2s(As + s * DG_ABYTES, src + size_t(ks) * DG_ABYTES, DG_ABYTES, &a_full[s], pol);
+                }
+            }
+            for (int k = it - NS; k < it; ++k)
+                if (k >= 0) mbar_wait(&a_full[k % NS], (k / NS) & 1, abort, a.status);
+        }
+    } else if (warp == 1) {
+        if (elect_one()) {
+            int it = 0;
+            for (int i = 0; i < nI; ++i) {
+                const int4 itm = s_items[i];
+                const int buf = i % NACC, k0 = itm.z & 0xFFFF, k1 = itm.z >> 16;
+                bool ok = true;
+                if (i >= NACC) ok = mbar_wait(&acc_empty[buf], (i / NACC - 1) & 1, abort, a.status);
+                tc_fence_after();
+                const uint32_t d = tmem + uint32_t(buf * NG * G);
+                for (int ks = k0; ks < k1; ++ks, ++it) {
+                    const int s = it % NS;
+                    bool okA = mbar_wait(&a_full[s], (it / NS) & 1, abort, a.status);
+                    okA = okA && mbar_wait(&b_full[s], (it / NS) & 1, abort, a.status);
+                    tc_fence_after();
+                    if (ok && okA && !*abort) {
+                        const uint64_t bd = dg_desc(Bs + s * Q::BBYTES);
+                        // the first digit's MMA starts groups 0 .. 7, the zero digit group 8
+                        if (NG > 8 && ks == k0)
+                            mma_bf16(d + 8 * G, dg_desc(As + s * DG_ABYTES),
+                                     dg_desc(Bs + s * Q::BBYTES + 8 * G * 32), idesc_bf16(128, G), 0);
+#pragma unroll
+                        for (int g = 0; g < 7; ++g)
+                            mma_bf16(d + g * G, dg_desc(As + s * DG_ABYTES + g * DG_PLANE), bd,
+                                     idesc_bf16(128, G * (NG - g < 8 ? NG - g : 8)), ks > k0 || g > 0);
+                    }
+                    mma_commit(&empty[s]);
+                }
+                mma_commit(&acc_full[buf]);
+            }
+            if (nI > 0) mbar_wait(&acc_full[(nI - 1) % NACC], ((nI - 1) / NACC) & 1, abort, a.status);
+        }
+    } else if (warp < 6) {
+        pdl_wait();
+        const int quarter = warp & 3;
+        const uint32_t lanes = uint32_t(quarter * 32) << 16;
+        double V[C];   // SYN: this row's sums, over the parts of a split item
+        int xb = 0;    // exchange buffer
+        for (int i = 0; i < nI; ++i) {
+            const int4 itm = s_items[i];
+            const int buf = i % NACC;
+            const bool none = (itm.z & 0xFFFF) >= (itm.z >> 16);   // no nonzero block: the accumulator holds no data
+            const uint32_t d0 = tmem + lanes + uint32_t(buf * NG * G);
+            if constexpr (SYN) {
+                const int m = itm.x & 0xFFFF, par = quarter >> 1, pl = (quarter & 1) * 32 + lane, p = itm.y * 64 + pl;
+                const double inv = p < nh ? a.isin[p] : 0.0, minv = inv * double(m);
+                const int ea = (p < nh ? a.ea[((itm.x >> 17) & 1 ? N + 1 + m : m) * nh + p] : 0) -
+                               ((itm.x >> 19) & 1 ? 55 : 0);
+                if (!((itm.x >> 18) & 1))
+#pragma unroll
+                    for (int c = 0; c < C; ++c) V[c] = 0.0;
+                mbar_wait(&acc_full[buf], (i / NACC) & 1, abort, a.status);
+                tc_fence_after();
+                mbar_wait(&sc_full[i], 0, abort, a.status);
+                {
+                    uint32_t d[8 * NG];
+#pragma unroll
+                    for (int s = 0; s < NG; ++s) tmem_ld8_nowait(d0 + uint32_t(s * G + par * CP), d + 8 * s);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < (C < 8 ? C : 8); ++c) V[c] += none ? 0.0 : dig_val<NG>(d + c, 8, ea + s_eb[5 * i + c / 2]);
+                }
+                if constexpr (C > 8) {
+                    uint32_t d[2 * NG];
+#pragma unroll
+                    for (int s = 0; s < NG; ++s) tmem_ld2_nowait(d0 + uint32_t(s * G + par * CP + 8), d + 2 * s);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 8; c < C; ++c) V[c] += none ? 0.0 : dig_val<NG>(d + c - 8, 2, ea + s_eb[5 * i + c / 2]);
+                }
+                tc_fence_before();
+                mbar_arrive(&acc_empty[buf]);
+                if ((itm.x >> 16) & 1) continue;   // the next item holds the rest
+                // even and odd sums meet: the even warps write north = E + O, the odd ones south = E - O
+                double* mine = xch + ((size_t(xb) * 2 + par) * 64 + pl) * C;
+                const double* other = xch + ((size_t(xb) * 2 + 1 - par) * 64 + pl) * C;
+                xb ^= 1;
+#pragma unroll
+                for (int c = 0; c < C; ++c) mine[c] = V[c];
+                named_bar_sync(1, 128);
+                const int row = par ? nlat - 1 - p : p;
+                if (p >= nh || (par && row == p) || *abort) continue;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    const double gr = par ? other[2 * f] - V[2 * f] : V[2 * f] + other[2 * f];
+                    const double gi = par ? other[2 * f + 1] - V[2 * f + 1] : V[2 * f + 1] + other[2 * f + 1];
+                    double2 o;
+                    if (f == 0) o = make_double2(gr, gi);
+                    else if (f == 1 || f == 3) o = make_double2(-gi * minv, gr * minv);   // (i m / sin) g
+                    else o = make_double2(-gr * inv, -gi * inv);                          // -(1 / sin) g
+                    *reinterpret_cast<double2*>(a.gsyn + gsyn_index(1, f, m, row, N, nlat) * 2) = o;
+                }
+            } else {
+                const int4 pc = a.pieces[4 * itm.x + quarter];
+                const int row = pc.z + lane;
+                const bool in = lane < pc.w;
+                const int ea = in ? a.ea[row] : 0;
+                int eb[NF];
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    const int b = a.emax[f * (N + 1) + pc.x];
+                    eb[f] = b == 2047 ? DG_NAN : b - 1020;
+                }
+                mbar_wait(&acc_full[buf], (i / NACC) & 1, abort, a.status);
+                tc_fence_after();
+                uint32_t d[8 * CP];
+#pragma unroll
+                for (int s = 0; s < 8; ++s) {
+                    if constexpr (CP == 4) tmem_ld4_nowait(d0 + uint32_t(s * G + quarter * CP), d + 4 * s);
+                    else tmem_ld8_nowait(d0 + uint32_t(s * G + quarter * CP), d + 8 * s);
+                }
+                tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive(&acc_empty[buf]);
+                if (!in || *abort) continue;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    const double hr = none ? 0.0 : dig_val<NG>(d + 2 * f, CP, ea + eb[f]);
+                    const double hi = none ? 0.0 : dig_val<NG>(d + 2 * f + 1, CP, ea + eb[f]);
+                    *reinterpret_cast<double2*>(a.hana + size_t(row) * C + 2 * f) = make_double2(hr, hi);
+                }
+            }
+        }
+    } else if (warp < 6 + DG_NB) {
+        // builders: warp 6 + it % NBW writes stage it's column digits
+        const int bw = warp - 6;
+        bool waited = false;
+        int it = 0;
+        if (bw < NBW)
+            for (int i = 0; i < nI; ++i) {
+                const int4 itm = s_items[i];
+                const int k1 = itm.z >> 16;
+                for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, ++it) {
+                    if (it % NBW != bw) continue;
+                    const int s = it % NS;
+                    if (!waited) {
+                        pdl_wait();
+                        waited = true;
+                    }
+                    if constexpr (SYN) mbar_wait(&sc_full[i], 0, abort, a.status);
+                    bool freed = it < NS;   // the slot is waited for after the first loads
+                    constexpr int NT = SYN ? 2 * NF * 8 : 4 * NF * 8;
+#pragma unroll
+                    for (int t0 = 0; t0 < NT; t0 += 32) {
+                        const int task = t0 + lane, w = task & 7;
+                        long long v[4] = {0, 0, 0, 0};   // (re, im) of contracted index 2 w, then 2 w + 1
+                        int col = 0;
+                        if (task < NT) {
+                            if constexpr (SYN) {
+                                const int f = (task >> 3) % NF, par = (task >> 3) / NF, m = itm.x & 0xFFFF;
+                                const int ne = ext_even(N, m), n = par ? ext_odd(N, m) : ne;
+                                const int r0 = ext_off(N, m) + (par ? ne : 0), lo = m > 0 ? m : 1;
+                                const int pk = packed_off(N, m) - lo, j0 = ks * 16 + 2 * w;
+                                const double2* src = f < 3 ? a.alpha : a.beta;
+                                const double sc = f < 3 || m == 0 ? 1.0 : 0.5;
+                                const int kb = 63 - s_eb[5 * i + f];
+                                col = par * CP + 2 * f;
+                                auto A = [&](int K) -> double2 {
+                                    return (K < lo || K > N) ? make_double2(0.0, 0.0) : src[pk + K];
+                                };
+#pragma unroll
+                                for (int e = 0; e < 2; ++e) {
+                                    const int j = j0 + e, K = m + par + 2 * j;
+                                    if (j >= n) continue;
+                                    const double4_32a c = a.prepc[r0 + j];
+                                    double2 b;
+                                    if (f == 2 || f == 4) {
+                                        const double2 dn = A(K - 1), up = A(K + 1);
+                                        b = make_double2(sc * (c.z * dn.x + c.w * up.x), sc * (c.z * dn.y + c.w * up.y));
+                                    } else {
+                                        const double q = f == 0 ? c.x : c.y;
+                                        const double2 x = A(K);
+                                        b = make_double2(sc * (q * x.x), sc * (q * x.y));
+                                    }
+                                    v[2 * e] = f64_to_fx(b.x, kb);
+                                    v[2 * e + 1] = f64_to_fx(b.y, kb);
+                                }
+                            } else {
+                                const int f = (task >> 3) % NF, q = (task >> 3) / NF;
+                                const int4 pc = a.pieces[4 * itm.x + q];
+                                const int m = pc.x, par = pc.y, p = ks * 16 + 2 * w;
+                                const int kb = 63 - (a.emax[f * (N + 1) + m] - 1020);
+                                col = q * CP + 2 * f;
+                                if (pc.w > 0 && p < nh) {
+                                    const double* g = a.gana + (size_t(f) * npair * size_t(N + 1) + m) * 4;
+                                    const size_t ld = size_t(N + 1) * 4;
+                                    const double4_32a no = *reinterpret_cast<const double4_32a*>(g + size_t(p / 2) * ld);
+                                    double2 s0, s1;   // the mirrors of p and p + 1
+                                    if (nlat % 2 == 0) {
+                                        const double4_32a so =
+                                            *reinterpret_cast<const double4_32a*>(g + size_t((nlat - 2 - p) / 2) * ld);
+                                        s0 = make_double2(so.z, so.w);
+                                        s1 = make_double2(so.x, so.y);
+                                    } else {
+                                        // mirrors in different pairs; the equator is its own mirror
+                                        const int q0 = nlat - 1 - p, q1 = nlat - 2 - p;
+                                        s0 = q0 == p ? make_double2(0.0, 0.0)
+                                                     : *reinterpret_cast<const double2*>(g + size_t(q0 / 2) * ld + 2 * (q0 & 1));
+                                        s1 = q1 <= p + 1 ? make_double2(0.0, 0.0)
+                                                         : *reinterpret_cast<const double2*>(g + size_t(q1 / 2) * ld + 2 * (q1 & 1));
+                                    }
+                                    const double sg = par ? -1.0 : 1.0;
+                                    v[0] = f64_to_fx(fma(sg, s0.x, no.x), kb);
+                                    v[1] = f64_to_fx(fma(sg, s0.y, no.y), kb);
+                                    if (p + 1 < nh) {
+                                        v[2] = f64_to_fx(fma(sg, s1.x, no.z), kb);
+                                        v[3] = f64_to_fx(fma(sg, s1.y, no.w), kb);
+                                    }
+                                }
+                            }
+                        }
+                        if (!freed) {
+                            mbar_wait(&empty[s], ((it / NS) - 1) & 1, abort, a.status);
+                            freed = true;
+                        }
+                        if (task < NT && !*abort) {
+                            unsigned char* t = Bs + s * Q::BBYTES;
+                            dig_put(t + dg_off(col, 2 * w), G * 32, v[0], v[2]);
+                            dig_put(t + dg_off(col + 1, 2 * w), G * 32, v[1], v[3]);
+                        }
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&b_full[s]);
+                }
+            }
+    } else if constexpr (SYN) {
+        // column exponents of every item: |b| <= 2^(eb - 1) from the exponents
+        // of alpha and of the coefficient sets
+        pdl_wait();
+        for (int i = 0; i < nI; ++i) {
+            const int m = s_items[i].x & 0xFFFF, lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
+            int e[5] = {0, 0, 0, 0, 0}, top = 0;
+#pragma unroll 4
+            for (int K = lo + lane; K <= N; K += 32) {
+                const short4 c = a.eoff[pk + K];
+                const double2 x = a.alpha[pk + K];
+                const int b = max(f64_bexp(x.x), f64_bexp(x.y));
+                top = max(top, b);
+                e[0] = max(e[0], b + c.x);
+                e[1] = max(e[1], b + c.y);
+                e[2] = max(e[2], b + c.z);
+                if constexpr (NF == 5) {
+                    const double2 y = a.beta[pk + K];
+                    const int d = max(f64_bexp(y.x), f64_bexp(y.y));
+                    top = max(top, d);
+                    e[3] = max(e[3], d + c.y);
+                    e[4] = max(e[4], d + c.z);
+                }
+            }
+            top = __reduce_max_sync(0xffffffffu, top);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+                const int v = __reduce_max_sync(0xffffffffu, e[f]);
+                if (lane == 0) s_eb[5 * i + f] = top == 2047 ? DG_NAN : v - 2 * 1022 + 1;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sc_full[i]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, Q::TCOLS);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// host side
+
+// LPT over one CTA per SM, CTA lists at a fixed stride.  rem (synthesis): the
+// remainder blocks of the lowest orders' first steps; their items become the
+// first step, its remainder and the later steps, one after the other.
+static int dig_schedule(sphnse_plan* P, const std::vector<int4>& items, const int* rem, int ntile, DigSide* D) {
+    std::vector<int> order(items.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = int(i);
+    // an item costs its steps plus about one for its epilogue and start
+    auto cost = [&](int i) { return (items[i].z >> 16) - (items[i].z & 0xFFFF) + 1; };
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
+    const int nc = std::min<int>(P->nsm, int(items.size()));
+    std::vector<std::vector<int4>> bins(nc);
+    std::vector<long> load(nc, 0);
+    for (int idx : order) {
+        const int b = int(std::min_element(load.begin(), load.end()) - load.begin());
+        int4 it = items[idx];
+        const int k0 = it.z & 0xFFFF, k1 = it.z >> 16;
+        if (rem && it.x < DG_SEGM) {
+            if (k0 == 0) {
+                bins[b].push_back(make_int4(it.x | 1 << 16, it.y, 1 << 16, it.w));
+                bins[b].push_back(make_int4(it.x | 1 << 18 | 1 << 19 | (k1 > 1 ? 1 << 16 : 0), it.y, 1 << 16,
+                                            rem[it.x * ntile + it.y]));
+            }
+            it.x |= 1 << 17 | (k0 == 0 ? 1 << 18 : 0);
+            it.z = std::max(k0, 1) | (k1 << 16);
+            if (k0 == 0 && k1 == 1) {
+                load[b] += cost(idx);
+                continue;
+            }
+        }
+        bins[b].push_back(it);
+        load[b] += cost(idx);
+    }
+    D->ncta = nc;
+    D->istride = 1;
+    for (auto& b : bins) D->istride = std::max(D->istride, int(b.size()));
+    std::vector<int4> flat(size_t(nc) * D->istride, make_int4(0, 0, 0, 0));
+    std::vector<int> cnt(nc);
+    for (int c = 0; c < nc; ++c) {
+        cnt[c] = int(bins[c].size());
+        std::copy(bins[c].begin(), bins[c].end(), flat.begin() + size_t(c) * D->istride);
+    }
+    if (cudaMalloc(reinterpret_cast<void**>(&D->items), flat.size() * sizeof(int4)) != cudaSuccess ||
+        cudaMalloc(reinterpret_cast<void**>(&D->cnt), cnt.size() * sizeof(int)) != cudaSuccess)
+        return SPHNSE_E_NOMEM;
+    if (cudaMemcpy(D->items, flat.data(), flat.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(D->cnt, cnt.data(), cnt.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+        return SPHNSE_E_CUDA;
+    return SPHNSE_OK;
+}
+
+void dig_free(sphnse_plan* P) {
+    for (DigSide* D : {&P->dig.syn, &P->dig.ana}) {
+        for (void* q : {static_cast<void*>(D->blocks), static_cast<void*>(D->ea), static_cast<void*>(D->items),
+                        static_cast<void*>(D->cnt), static_cast<void*>(D->pieces)})
+            if (q) cudaFree(q);
+        *D = DigSide();
+    }
+    if (P->dig.eoff) cudaFree(P->dig.eoff);
+    if (P->dig.isin) cudaFree(P->dig.isin);
+    if (P->dig.emax) cudaFree(P->dig.emax);
+    P->dig = DigState();
+}
+
+// Digits, schedules and constants, from the FP64 table [n_ext][nh] on the
+// device (which the digits replace).
+int dig_setup(sphnse_plan* P, const double* d_tab) {
+    const int N = P->N, nh = P->nh, ntile = (nh + 63) / 64;
+    DigState& T = P->dig;
+    auto alloc = [](auto** p, size_t n) { return cudaMalloc(reinterpret_cast<void**>(p), n * sizeof(**p)) == cudaSuccess; };
+    auto up = [](void* d, const void* h, size_t b) { return cudaMemcpy(d, h, b, cudaMemcpyHostToDevice) == cudaSuccess; };
+
+    // synthesis tiles (m, 64 latitudes), steps of 16 degrees of each parity
+    const int nseg = std::min(DG_SEGM, N + 1);
+    std::vector<int> base(size_t(N + 1 + nseg) * ntile);
+    int nblk = 0;
+    for (int m = 0; m <= N; ++m)
+        for (int t = 0; t < ntile; ++t) {
+            base[size_t(m) * ntile + t] = nblk;
+            nblk += (ext_even(N, m) + 15) / 16;
+        }
+    for (size_t i = size_t(N + 1) * ntile; i < base.size(); ++i) base[i] = nblk++;   // remainders
+    // analysis tiles: four pieces of up to 32 rows of one (m, parity)
+    std::vector<int4> pieces;
+    for (int m = 0; m <= N; ++m)
+        for (int par = 0; par < 2; ++par) {
+            const int ne = ext_even(N, m), n = par ? ext_odd(N, m) : ne, r0 = ext_off(N, m) + (par ? ne : 0);
+            for (int r = 0; r < n; r += 32) pieces.push_back(make_int4(m, par, r0 + r, std::min(32, n - r)));
+        }
+    while (pieces.size() % 4) pieces.push_back(make_int4(0, 0, 0, 0));
+    const int atile = int(pieces.size() / 4), aks = (nh + 15) / 16, ablk = atile * aks;
+
+    int *d_base = nullptr, *d_used = nullptr;
+    int rc = SPHNSE_OK;
+    if (!alloc(&T.syn.blocks, size_t(nblk) * DG_ABYTES) || !alloc(&T.ana.blocks, size_t(ablk) * DG_ABYTES) ||
+        !alloc(&T.syn.ea, size_t(N + 1 + DG_SEGM) * nh) || !alloc(&T.ana.ea, size_t(P->n_ext)) ||
+        !alloc(&T.ana.pieces, pieces.size()) || !alloc(&d_base, base.size()) || !alloc(&d_used, size_t(nblk + ablk)) ||
+        !alloc(&T.eoff, size_t(P->n_coeff)) || !alloc(&T.isin, size_t(P->nlat)) || !alloc(&T.emax, size_t(3) * (N + 1)))
+        rc = SPHNSE_E_NOMEM;
+    T.syn.bytes = size_t(nblk) * DG_ABYTES;
+    T.ana.bytes = size_t(ablk) * DG_ABYTES;
+    std::vector<int> used(size_t(nblk) + ablk);
+    if (!rc) {
+        // exponents of the coefficient sets applied to alpha_{K,m}: zeta, theta, and the larger of
+        // alpha_K's two places in the degree-shift set
+        auto bexp = [](double v) { return v == 0.0 ? 0 : std::ilogb(v) + 1023; };
+        std::vector<short4> eoff(P->n_coeff);
+        auto eps = [](int l, int m) {
+            return l <= m ? 0.0 : std::sqrt((double(l) * l - double(m) * m) / (4.0 * l * l - 1.0));
+        };
+        for (int m = 0, i = 0; m <= N; ++m)
+            for (int l = (m > 0 ? m : 1); l <= N; ++l, ++i) {
+                const double sl = std::sqrt(double(l) * (l + 1.0));
+                // alpha_l enters row l + 1 with l eps_{l+1}, row l - 1 with (l + 1) eps_l; the sum of a
+                // row's two terms takes one more bit
+                const double dn = std::max(l * eps(l + 1, m), (l + 1) * eps(l, m)) / sl;
+                eoff[i] = make_short4(short(bexp(sl)), short(bexp(1.0 / sl)), short(bexp(dn) + 1), 0);
+            }
+        std::vector<double> isin(P->nlat);
+        for (int p = 0; p < P->nlat; ++p) isin[p] = 1.0 / P->s[p];
+        if (!up(T.ana.pieces, pieces.data(), pieces.size() * sizeof(int4)) ||
+            !up(d_base, base.data(), base.size() * sizeof(int)) || !up(T.eoff, eoff.data(), eoff.size() * sizeof(short4)) ||
+            !up(T.isin, isin.data(), isin.size() * sizeof(double)) ||
+            cudaMemset(T.emax, 0, size_t(3) * (N + 1) * sizeof(int)) != cudaSuccess ||
+            cudaMemset(d_used, 0, used.size() * sizeof(int)) != cudaSuccess)
+            rc = SPHNSE_E_CUDA;
+    }
+    if (!rc) {
+        k_dig_syn_scale<<<dim3((nh + 127) / 128, N + 1), 128>>>(d_tab, T.syn.ea, N, nh);
+        k_dig_ana_scale<<<(P->n_ext + 3) / 4, 128>>>(d_tab, T.ana.ea, P->n_ext, nh);
+        k_dig_syn<<<dim3((ext_even(N, 0) + 15) / 16, ntile, N + 1), 256>>>(d_tab, T.syn.ea, d_base, T.syn.blocks, d_used,
+                                                                          N, nh, ntile, 0);
+        k_dig_syn<<<dim3(1, ntile, nseg), 256>>>(d_tab, T.syn.ea, d_base + size_t(N + 1) * ntile, T.syn.blocks, d_used,
+                                                 N, nh, ntile, 1);
+        k_dig_ana<<<dim3(aks, atile), 256>>>(d_tab, T.ana.ea, T.ana.pieces, T.ana.blocks, d_used + nblk, nh);
+        if (cudaMemcpy(used.data(), d_used, used.size() * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+            rc = SPHNSE_E_CUDA;
+    }
+    if (d_base) cudaFree(d_base);
+    if (d_used) cudaFree(d_used);
+    if (rc) return rc;
+    // leading steps without a nonzero digit are skipped
+    std::vector<int4> items;
+    for (int m = 0; m <= N; ++m)
+        for (int t = 0; t < ntile; ++t) {
+            const int b = base[size_t(m) * ntile + t], k1 = (ext_even(N, m) + 15) / 16;
+            int k0 = 0;
+            while (k0 < k1 && !used[size_t(b) + k0]) ++k0;
+            items.push_back(make_int4(m, t, k0 | (k1 << 16), b));
+        }
+    if ((rc = dig_schedule(P, items, base.data() + size_t(N + 1) * ntile, ntile, &T.syn))) return rc;
+    items.clear();
+    for (int t = 0; t < atile; ++t) {
+        int k0 = 0;
+        while (k0 < aks && !used[size_t(nblk) + size_t(t) * aks + k0]) ++k0;
+        items.push_back(make_int4(t, 0, k0 | (aks << 16), t * aks));
+    }
+    if ((rc = dig_schedule(P, items, nullptr, 0, &T.ana))) return rc;
+    T.ready = true;
+    return SPHNSE_OK;
+}
+
+static DigArgs dig_args(sphnse_plan* P, const DigSide& D) {
+    DigArgs a{};
+    a.blocks = D.blocks;
+    a.items = D.items;
+    a.cnt = D.cnt;
+    a.istride = D.istride;
+    // tables that fit L2 beside the grid fields stay there between calls
+    a.evict_first = P->dig.syn.bytes + P->dig.ana.bytes > (size_t(48) << 20);
+    a.ea = D.ea;
+    a.status = P->d_status;
+    a.N = P->N;
+    a.nh = P->nh;
+    a.nlat = P->nlat;
+    a.alpha = nullptr;
+    a.prepc = P->d_prepc;
+    a.eoff = P->dig.eoff;
+    a.gsyn = static_cast<double*>(P->d_gsyn);
+    a.isin = P->dig.isin;
+    a.pieces = P->dig.ana.pieces;
+    a.gana = static_cast<const double*>(P->d_gana);
+    a.emax = P->dig.emax;
+    a.hana = static_cast<double*>(P->d_hana);
+    return a;
+}
+
+template <bool SYN, int NF>
+static int dig_launch(sphnse_plan* P, const DigSide& D, const DigArgs& a) {
+    using Q = DigShape<SYN, NF>;
+    const size_t sm = Q::smem(D.istride);
+    if (sm > 227 * 1024) return SPHNSE_E_UNSUPPORTED;
+    allow_dynamic_smem(reinterpret_cast<const void*>(k_dig<SYN, NF>), sm);
+    const int stage = SYN ? SPHNSE_STAGE_SYNTHESIS : SPHNSE_STAGE_ANALYSIS;
+    stage_begin(P, stage);
+    const cudaError_t e = launch_pdl(k_dig<SYN, NF>, dim3(D.ncta), dim3(32 * Q::WARPS), sm, P->stream, a);
+    stage_end(P, stage);
+    return check_cuda(e);
+}
+
+int launch_synthesis_dig(sphnse_plan* P, const double* alpha, const double* beta) {
+    DigArgs a = dig_args(P, P->dig.syn);
+    a.alpha = reinterpret_cast<const double2*>(alpha);
+    a.beta = reinterpret_cast<const double2*>(beta);
+    return beta ? dig_launch<true, 5>(P, P->dig.syn, a) : dig_launch<true, 3>(P, P->dig.syn, a);
+}
+
+int launch_analysis_dig(sphnse_plan* P, int nf) {
+    const DigArgs a = dig_args(P, P->dig.ana);
+    return nf == 3 ? dig_launch<false, 3>(P, P->dig.ana, a) : dig_launch<false, 2>(P, P->dig.ana, a);
+}
+
+}  // namespace sph

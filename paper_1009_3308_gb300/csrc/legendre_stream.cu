@@ -1,4 +1,4 @@
-// Persistent streaming Legendre kernels (CUDA cores, FP64 or FP32).
+// Persistent streaming Legendre kernels (CUDA cores, FP32).
 //
 // The per-order Legendre sums of the RHS (Sec. 4.2; synthesis of the fields
 // of Eq. (app_soln_rep) and (vort_app), analysis = the discrete projection of
@@ -25,13 +25,11 @@
 
 namespace sph {
 
-// pipeline depth: 6 stages of 24 KB for FP32; 4 for FP64 (compute bound and
-// tighter on shared memory)
-template <typename T> __host__ __device__ constexpr int nst() { return sizeof(T) == 4 ? 6 : 4; }
+// pipeline depth: 6 stages of 24 KB
+template <typename T> __host__ __device__ constexpr int nst() { return 6; }
 
 template <typename T> struct Vec;
 template <> struct Vec<float> { using type = float4; static constexpr int n = 4; };
-template <> struct Vec<double> { using type = double2; static constexpr int n = 2; };
 
 template <typename T>
 __device__ __forceinline__ void vload(const T* p, T* out) {
@@ -56,7 +54,7 @@ struct StreamArgs {
     // batches: an item v stands for instance v / (N+1) and order v % (N+1);
     // per-instance strides (elements) of bsyn, gsyn, gana, hana
     size_t sb, sg, sa, sh;
-    int pairs;           // gsyn and gana layout (gsyn_index)
+    int pairs;           // gsyn layout (gsyn_index)
 };
 
 // chunk c of order m: rows [c HR, c HR + HR) of the even and of the odd block
@@ -298,10 +296,10 @@ __global__ void __launch_bounds__(288, 1) k_ana_stream(StreamArgs a) {
         T* S = Ssm + size_t(ii & 1) * 2 * nh * 2 * NF;
         for (int i = ct; i < nh * NF; i += ncons) {
             const int f = i / nh, p = i % nh, pr = nlat - 1 - p;
-            const T* ga = gsrc + gsyn_index(a.pairs, f, m, p, N, nlat) * 2;
+            const T* ga = gsrc + gsyn_index(0, f, m, p, N, nlat) * 2;
             T ar = ga[0], ai = ga[1], br = T(0), bi = T(0);
             if (pr != p) {
-                const T* gb = gsrc + gsyn_index(a.pairs, f, m, pr, N, nlat) * 2;
+                const T* gb = gsrc + gsyn_index(0, f, m, pr, N, nlat) * 2;
                 br = gb[0];
                 bi = gb[1];
             }
@@ -364,15 +362,12 @@ __global__ void __launch_bounds__(288, 1) k_ana_stream(StreamArgs a) {
 // host launchers
 
 template <typename T>
-static constexpr int half_rows() { return sizeof(T) == 4 ? 8 : 4; }
+static constexpr int half_rows() { return 8; }
 
-bool stream_ok(const sphnse_plan* P, int prec) {
-    const int V = prec == SPHNSE_FP64 ? 2 : 4;
-    return P->d_items != nullptr && P->nh % V == 0 && P->nh >= 32;
-}
+bool stream_ok(const sphnse_plan* P) { return P->d_items != nullptr && P->nh % 4 == 0 && P->nh >= 32; }
 
 template <typename T, int NF>
-static int syn_stream_t(sphnse_plan* P, int pairs) {
+static int syn_stream_t(sphnse_plan* P) {
     constexpr int HR = half_rows<T>();
     constexpr int V = Vec<T>::n;
     const int tpg = ((P->nh / V + 31) / 32) * 32;
@@ -383,8 +378,8 @@ static int syn_stream_t(sphnse_plan* P, int pairs) {
                                          size_t(P->nh) * 2 * NF);
     if (sm > 227 * 1024) return SPHNSE_E_UNSUPPORTED;
     allow_dynamic_smem(reinterpret_cast<const void*>(k_syn_stream<T, NF, HR>), sm);
-    StreamArgs a{P->tab[sizeof(T) == 8 ? SPHNSE_FP64 : SPHNSE_FP32].syn, P->d_bsyn, P->d_gsyn, nullptr, nullptr,
-                 P->d_s, P->d_items, P->d_item_off, P->d_status, P->N, P->nh, P->nlat, 0, 0, 0, 0, pairs};
+    StreamArgs a{P->tab[SPHNSE_FP32].syn, P->d_bsyn, P->d_gsyn, nullptr, nullptr,
+                 P->d_s, P->d_items, P->d_item_off, P->d_status, P->N, P->nh, P->nlat, 0, 0, 0, 0, 0};
     stage_begin(P, SPHNSE_STAGE_SYNTHESIS);
     launch_pdl(k_syn_stream<T, NF, HR>, dim3(P->n_cta), dim3(threads), sm, P->stream, a);
     stage_end(P, SPHNSE_STAGE_SYNTHESIS);
@@ -392,7 +387,7 @@ static int syn_stream_t(sphnse_plan* P, int pairs) {
 }
 
 template <typename T, int NF>
-static int ana_stream_t(sphnse_plan* P, int pairs) {
+static int ana_stream_t(sphnse_plan* P) {
     constexpr int HR = half_rows<T>();
     constexpr int QPS = 2 * HR / 4;
     constexpr int NTEAM = 8 / QPS;
@@ -401,23 +396,20 @@ static int ana_stream_t(sphnse_plan* P, int pairs) {
     const size_t sm = 128 + sizeof(T) * (size_t(NST) * 2 * HR * P->nh + size_t(2) * 2 * P->nh * 2 * NF);
     if (sm > 227 * 1024) return SPHNSE_E_UNSUPPORTED;
     allow_dynamic_smem(reinterpret_cast<const void*>(k_ana_stream<T, NF, HR, NTEAM>), sm);
-    StreamArgs a{P->tab[sizeof(T) == 8 ? SPHNSE_FP64 : SPHNSE_FP32].syn, nullptr, nullptr, P->d_gana, P->d_hana,
-                 P->d_s, P->d_items, P->d_item_off, P->d_status, P->N, P->nh, P->nlat, 0, 0, 0, 0, pairs};
+    StreamArgs a{P->tab[SPHNSE_FP32].syn, nullptr, nullptr, P->d_gana, P->d_hana,
+                 P->d_s, P->d_items, P->d_item_off, P->d_status, P->N, P->nh, P->nlat, 0, 0, 0, 0, 0};
     stage_begin(P, SPHNSE_STAGE_ANALYSIS);
     launch_pdl(k_ana_stream<T, NF, HR, NTEAM>, dim3(P->n_cta), dim3(threads), sm, P->stream, a);
     stage_end(P, SPHNSE_STAGE_ANALYSIS);
     return check_cuda(cudaGetLastError());
 }
 
-int launch_synthesis_stream(sphnse_plan* P, int nfields, int prec, int pairs) {
-    if (prec == SPHNSE_FP64)
-        return nfields == 5 ? syn_stream_t<double, 5>(P, pairs) : syn_stream_t<double, 3>(P, pairs);
-    return nfields == 5 ? syn_stream_t<float, 5>(P, pairs) : syn_stream_t<float, 3>(P, pairs);
+int launch_synthesis_stream(sphnse_plan* P, int nfields) {
+    return nfields == 5 ? syn_stream_t<float, 5>(P) : syn_stream_t<float, 3>(P);
 }
 
-int launch_analysis_stream(sphnse_plan* P, int nfields, int prec, int pairs) {
-    if (prec == SPHNSE_FP64) return nfields == 3 ? ana_stream_t<double, 3>(P, pairs) : ana_stream_t<double, 2>(P, pairs);
-    return nfields == 3 ? ana_stream_t<float, 3>(P, pairs) : ana_stream_t<float, 2>(P, pairs);
+int launch_analysis_stream(sphnse_plan* P, int nfields) {
+    return nfields == 3 ? ana_stream_t<float, 3>(P) : ana_stream_t<float, 2>(P);
 }
 
 // FP32 batched streaming passes over instances (items = inst * (N+1) + m)
@@ -429,7 +421,7 @@ int launch_synthesis_stream_batch(sphnse_plan* P, const int* items, const int* i
     const int threads = 32 + 2 * tpg;
     const size_t sm = 128 + sizeof(float) * (size_t(NST) * 2 * HR * P->nh + size_t(2) * (P->N + 2) * 6 +
                                              size_t(P->nh) * 6);
-    if (threads > 512 || sm > 227 * 1024 || !stream_ok(P, SPHNSE_FP32)) return SPHNSE_E_UNSUPPORTED;
+    if (threads > 512 || sm > 227 * 1024 || !stream_ok(P)) return SPHNSE_E_UNSUPPORTED;
     allow_dynamic_smem(reinterpret_cast<const void*>(k_syn_stream<float, 3, HR>), sm);
     StreamArgs a{P->tab[SPHNSE_FP32].syn, bsyn, gsyn, nullptr, nullptr, P->d_s, items, item_off, P->d_status,
                  P->N, P->nh, P->nlat, sb, sg, 0, 0, pairs};
@@ -447,7 +439,7 @@ int launch_analysis_stream_batch(sphnse_plan* P, const int* items, const int* it
     constexpr int NST = nst<float>();
     const int threads = 32 + 32 * QPS * NTEAM;
     const size_t sm = 128 + sizeof(float) * (size_t(NST) * 2 * HR * P->nh + size_t(2) * 2 * P->nh * 4);
-    if (sm > 227 * 1024 || !stream_ok(P, SPHNSE_FP32)) return SPHNSE_E_UNSUPPORTED;
+    if (sm > 227 * 1024 || !stream_ok(P)) return SPHNSE_E_UNSUPPORTED;
     allow_dynamic_smem(reinterpret_cast<const void*>(k_ana_stream<float, 2, HR, NTEAM>), sm);
     StreamArgs a{P->tab[SPHNSE_FP32].syn, nullptr, nullptr, gana, hana, P->d_s, items, item_off, P->d_status,
                  P->N, P->nh, P->nlat, 0, 0, sa, sh, 0};

@@ -61,7 +61,6 @@ static void free_tables(Tables& t) {
     if (t.syn) cudaFree(t.syn);
     if (t.ana) cudaFree(t.ana);
     if (t.syn_lo) cudaFree(t.syn_lo);
-    if (t.ana_lo) cudaFree(t.ana_lo);
     t = Tables();
 }
 
@@ -76,25 +75,27 @@ static void for_each_block(int N, F&& f) {
     }
 }
 
+// one table of converted entries; with_ana: also the analysis fallback's layout
 template <typename T, typename Conv>
-static int upload_pair(sphnse_plan* P, Tables& t, Conv conv, bool lo) {
-    const size_t nh = P->nh, ne = P->n_ext;
-    const size_t count = ne * nh;
-    std::vector<T> syn(count), ana(count);
+static int upload_table(sphnse_plan* P, Tables& t, Conv conv, bool lo, bool with_ana) {
+    const size_t nh = P->nh, count = size_t(P->n_ext) * nh;
+    std::vector<T> syn(count);
     const double* src = P->psyn_host.data();
     for (size_t i = 0; i < count; ++i) syn[i] = conv(src[i], lo);
+    void** dsyn = lo ? &t.syn_lo : &t.syn;
+    if (cudaMalloc(dsyn, count * sizeof(T)) != cudaSuccess) return SPHNSE_E_NOMEM;
+    if (cudaMemcpy(*dsyn, syn.data(), count * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) return SPHNSE_E_CUDA;
+    t.bytes += count * sizeof(T);
+    if (!with_ana) return SPHNSE_OK;
+    std::vector<T> ana(count);
     for_each_block(P->N, [&](int r0, int nr) {
         const size_t base = size_t(r0) * nh;
         for (int j = 0; j < nr; ++j)
             for (size_t p = 0; p < nh; ++p) ana[base + p * nr + j] = syn[base + size_t(j) * nh + p];
     });
-    void** dsyn = lo ? &t.syn_lo : &t.syn;
-    void** dana = lo ? &t.ana_lo : &t.ana;
-    if (cudaMalloc(dsyn, count * sizeof(T)) != cudaSuccess) return SPHNSE_E_NOMEM;
-    if (cudaMalloc(dana, count * sizeof(T)) != cudaSuccess) return SPHNSE_E_NOMEM;
-    if (cudaMemcpy(*dsyn, syn.data(), count * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) return SPHNSE_E_CUDA;
-    if (cudaMemcpy(*dana, ana.data(), count * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) return SPHNSE_E_CUDA;
-    t.bytes += 2 * count * sizeof(T);
+    if (cudaMalloc(&t.ana, count * sizeof(T)) != cudaSuccess) return SPHNSE_E_NOMEM;
+    if (cudaMemcpy(t.ana, ana.data(), count * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) return SPHNSE_E_CUDA;
+    t.bytes += count * sizeof(T);
     return SPHNSE_OK;
 }
 
@@ -103,9 +104,17 @@ int ensure_tables(sphnse_plan* P, int prec) {
     if (t.built) return SPHNSE_OK;
     int rc = SPHNSE_OK;
     if (prec == SPHNSE_FP64) {
-        rc = upload_pair<double>(P, t, [](double v, bool) { return v; }, false);
+        // the digit blocks of the tensor-core sums replace the table
+        const size_t bytes = size_t(P->n_ext) * P->nh * sizeof(double);
+        double* d = nullptr;
+        if (cudaMalloc(reinterpret_cast<void**>(&d), bytes) != cudaSuccess) rc = SPHNSE_E_NOMEM;
+        else if (cudaMemcpy(d, P->psyn_host.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) rc = SPHNSE_E_CUDA;
+        if (rc == SPHNSE_OK) rc = dig_setup(P, d);
+        if (d) cudaFree(d);
+        if (rc == SPHNSE_OK) t.bytes = P->dig.syn.bytes + P->dig.ana.bytes;
+        else dig_free(P);
     } else if (prec == SPHNSE_FP32) {
-        rc = upload_pair<float>(P, t, [](double v, bool) { return float(v); }, false);
+        rc = upload_table<float>(P, t, [](double v, bool) { return float(v); }, false, true);
     } else {
         // BF16 hi + lo split: hi = bf16(v), lo = bf16(v - hi)
         auto conv = [](double v, bool lo) {
@@ -113,8 +122,8 @@ int ensure_tables(sphnse_plan* P, int prec) {
             if (!lo) return hi;
             return __float2bfloat16_rn(float(v - double(__bfloat162float(hi))));
         };
-        rc = upload_pair<__nv_bfloat16>(P, t, conv, false);
-        if (rc == SPHNSE_OK) rc = upload_pair<__nv_bfloat16>(P, t, conv, true);
+        rc = upload_table<__nv_bfloat16>(P, t, conv, false, false);
+        if (rc == SPHNSE_OK) rc = upload_table<__nv_bfloat16>(P, t, conv, true, false);
     }
     if (rc != SPHNSE_OK) {
         free_tables(t);
@@ -147,10 +156,9 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
     int rc;
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);
     if (prec == SPHNSE_FP64) {
-        if ((rc = launch_prep(P, alpha, nullptr, prec))) return rc;
-        if ((rc = launch_synthesis(P, 3, prec, 1))) return rc;
+        if ((rc = launch_synthesis_dig(P, alpha, nullptr))) return rc;
         if ((rc = launch_ring_fx(P, RING_RHS, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-        if ((rc = launch_analysis(P, 2, prec, 1))) return rc;
+        if ((rc = launch_analysis_dig(P, 2))) return rc;
         return launch_finish(P, 0, prec, alpha, forcing, out);
     }
     const bool ring4 = ring4_ok(P);
@@ -161,8 +169,8 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
     if (tc) {
         if ((rc = launch_synthesis_tc(P, alpha, pairs))) return rc;   // builds its coefficient tiles
     } else {
-        if ((rc = launch_prep(P, alpha, nullptr, prec))) return rc;
-        if ((rc = launch_synthesis(P, 3, prec))) return rc;
+        if ((rc = launch_prep(P, alpha, nullptr))) return rc;
+        if ((rc = launch_synthesis(P, 3))) return rc;
     }
     if (ring4) {
         if ((rc = launch_ring4(P, 1, static_cast<const float*>(P->d_gsyn), 0, static_cast<float*>(P->d_gana), 0,
@@ -179,7 +187,7 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
         rc = launch_analysis_finish_tc(P, alpha, forcing, out);
         if (rc != SPHNSE_E_UNSUPPORTED) return rc;
     }
-    if ((rc = tc ? launch_analysis_tc(P, 2) : launch_analysis(P, 2, prec))) return rc;
+    if ((rc = tc ? launch_analysis_tc(P, 2) : launch_analysis(P, 2))) return rc;
     return launch_finish(P, 0, prec, alpha, forcing, out);
 }
 
@@ -189,18 +197,18 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
 int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out) {
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     int rc;
-    if ((rc = launch_prep(P, alpha, w, prec))) return rc;
     if (prec == SPHNSE_FP64) {
-        if ((rc = launch_synthesis(P, 5, prec, 1))) return rc;
+        if ((rc = launch_synthesis_dig(P, alpha, w))) return rc;
         if ((rc = launch_ring_fx(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-        if ((rc = launch_analysis(P, 3, prec, 1))) return rc;
+        if ((rc = launch_analysis_dig(P, 3))) return rc;
         return launch_finish(P, 2, prec, w, nullptr, out);
     }
-    if ((rc = launch_synthesis(P, 5, prec))) return rc;
+    if ((rc = launch_prep(P, alpha, w))) return rc;
+    if ((rc = launch_synthesis(P, 5))) return rc;
     if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 5))) return rc;
     if ((rc = launch_ring(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
     if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 3))) return rc;
-    if ((rc = launch_analysis(P, 3, prec))) return rc;
+    if ((rc = launch_analysis(P, 3))) return rc;
     return launch_finish(P, 2, prec, w, nullptr, out);
 }
 
@@ -216,6 +224,7 @@ static void destroy_plan(sphnse_plan* P) {
     else cudaDeviceSynchronize();
     for (auto& t : P->tab) free_tables(t);
     tc_free(P);
+    dig_free(P);
     host_io_free(P);
     if (P->ng_exec) cudaGraphExecDestroy(P->ng_exec);
     if (P->d_ctl) cudaFree(P->d_ctl);
@@ -355,7 +364,7 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
     if (!rc) rc = dalloc(&P->d_prepc, size_t(P->n_ext) * sizeof(double4_32a));
     if (!rc) rc = dalloc(&P->d_finc32, nc * sizeof(float4));
     if (!rc) rc = dalloc(&P->d_prepc32, size_t(P->n_ext) * sizeof(float4));
-    if (!rc) rc = dalloc(&P->d_bsyn, size_t(P->n_ext) * 10 * sizeof(double));
+    if (!rc) rc = dalloc(&P->d_bsyn, size_t(P->n_ext) * 10 * sizeof(float));
     if (!rc) rc = dalloc(&P->d_gsyn, 5 * sz_g);
     if (!rc) rc = dalloc(&P->d_gana, 3 * sz_g);
     if (!rc) rc = dalloc(&P->d_hana, size_t(P->n_ext) * 6 * sizeof(double));
@@ -519,13 +528,16 @@ int sphnse_grid_fields(sphnse_plan* P, const double* alpha, double* zeta, double
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);
     int rc;
+    if (prec == SPHNSE_FP64) {
+        if ((rc = launch_synthesis_dig(P, alpha, nullptr))) return rc;
+        return launch_ring_fx(P, RING_GRID, nullptr, nullptr, zeta, uth, uph);
+    }
     if (tc) {
         if ((rc = launch_synthesis_tc(P, alpha, 0))) return rc;
     } else {
-        if ((rc = launch_prep(P, alpha, nullptr, prec))) return rc;
-        if ((rc = launch_synthesis(P, 3, prec, prec == SPHNSE_FP64))) return rc;
+        if ((rc = launch_prep(P, alpha, nullptr))) return rc;
+        if ((rc = launch_synthesis(P, 3))) return rc;
     }
-    if (prec == SPHNSE_FP64) return launch_ring_fx(P, RING_GRID, nullptr, nullptr, zeta, uth, uph);
     if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 3))) return rc;
     return launch_ring(P, RING_GRID, nullptr, nullptr, zeta, uth, uph);
 }
@@ -536,13 +548,13 @@ int sphnse_project(sphnse_plan* P, const double* vth, const double* vph, double*
     int rc;
     if (prec == SPHNSE_FP64) {
         if ((rc = launch_ring_fx(P, RING_PROJECT, vth, vph, nullptr, nullptr, nullptr))) return rc;
-        if ((rc = launch_analysis(P, 2, prec, 1))) return rc;
+        if ((rc = launch_analysis_dig(P, 2))) return rc;
         return launch_finish(P, 1, prec, nullptr, nullptr, out);
     }
     if ((rc = launch_ring(P, RING_PROJECT, vth, vph, nullptr, nullptr, nullptr))) return rc;
     if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 2))) return rc;
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);
-    if ((rc = tc ? launch_analysis_tc(P, 2) : launch_analysis(P, 2, prec))) return rc;
+    if ((rc = tc ? launch_analysis_tc(P, 2) : launch_analysis(P, 2))) return rc;
     return launch_finish(P, 1, prec, nullptr, nullptr, out);
 }
 

@@ -94,6 +94,7 @@ struct RingFxArgs {
     double* gout1;
     double* gout2;
     const int4* tw;
+    int* emax;             // [nf][N+1] largest biased exponents of gana (atomic maxima)
     FxPlan plan;
     int early;             // let the successor start its prologue at once
 };
@@ -518,7 +519,12 @@ __global__ void __launch_bounds__(MODE == RING_ADJOINT ? 512 : 288, MODE == RING
         }
 #pragma unroll
         for (int f = 0; f < (MODE == RING_ADJOINT ? 3 : 2); ++f)
+        {
             *reinterpret_cast<double4_32a*>(a.gana + ((size_t(f) * npair + pair) * size_t(N + 1) + m) * 4) = o[f];
+            // the column scales of the analysis
+            atomicMax(a.emax + f * (N + 1) + m,
+                      max(max(f64_bexp(o[f].x), f64_bexp(o[f].y)), max(f64_bexp(o[f].z), f64_bexp(o[f].w))));
+        }
     }
 }
 
@@ -559,6 +565,7 @@ int launch_ring_fx(sphnse_plan* P, int mode, const double* gin0, const double* g
     a.gout1 = gout1;
     a.gout2 = gout2;
     a.tw = P->d_fxtw;
+    a.emax = P->dig.emax;
     stage_begin(P, SPHNSE_STAGE_RING);
     cudaError_t e;
     switch (mode) {
