@@ -1,5 +1,5 @@
 // Longitude ("ring") kernel of the FP64 path in 64-bit fixed point (fx64.cuh),
-// one CTA per pair of Gauss latitudes 2 j, 2 j + 1.
+// one CTA per pair of Gauss latitudes 2 j, 2 j + 1 (ADJOINT: per latitude).
 //
 // RHS (Sec. 4.2: the phi sums of Eqs. (app_soln_rep), (eval_nonlin1) are
 // Fourier sums, evaluated by FFT):
@@ -13,10 +13,14 @@
 // rows of a tangential field; ADJOINT evaluates the transposed linearised
 // product (fields zeta, u_theta, u_phi, v_theta, v_phi).
 //
-// M = nlon = 2^a 3^b; in-place Stockham autosort stages of radix 8, 4, 2, 9
-// and 3 in shared memory.  Every thread holds its butterflies of a stage in
-// registers (8 TPT complex values), the block synchronises, and writes them
-// back.  Spectra are read and written in the latitude-pair-major layout
+// M = nlon = 2^a 3^b; Stockham autosort stages of radix 8, 4, 2, 9 and 3 from
+// one shared-memory buffer to the other, one barrier each.  Small grids are
+// bound by instruction fetch (each instruction runs a few times per CTA: half
+// of the issue slots of the first form, whose in-place stages were unrolled
+// per direction and signal count, waited for instructions at L = 31 .. 255),
+// so one rolled copy of each radix serves both directions: the inverse
+// transform is the forward one with real and imaginary parts exchanged.
+// Spectra are read and written in the latitude-pair-major layout
 // [f][row / 2][m][row % 2] (a CTA's data are contiguous runs, and the
 // order-major side of the Legendre kernels still moves whole 32-byte
 // sectors), so no transpose runs between this kernel and the Legendre sums.
@@ -36,6 +40,7 @@
 // that no FFT intermediate overflows and all 60 bits are used.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -110,82 +115,57 @@ __device__ __forceinline__ cx<fx> fx_ld(const longlong2* p) {
 }
 __device__ __forceinline__ void fx_st(longlong2* p, cx<fx> v) { *p = make_longlong2(v.x.v, v.y.v); }
 
-// One in-place stage of radix R over NSIG signals; a thread's butterflies are
-// t = tid + b NT (signal t / nb, butterfly t mod nb).
-template <int R, int NSIG, int TPT, int S>
-__device__ __forceinline__ void fx_stage(longlong2* buf, int M, int Ns, const int4* tw) {
-    constexpr int MAXB = (8 * TPT + R - 1) / R;
-    // the stage loop holds one copy of this body per radix: without this the
-    // compiler hoists every copy's addresses out of the loop and spills them
-    // (for the same reason an idle thread's values are set to zero below: left
-    // undefined, they count as live around the loop)
-    asm volatile("" : "+r"(M));
-    const int nb = M / R, ld = fx_stride(M), step = M / (Ns * R);
-    cx<fx> v[MAXB][R];
-    int to[MAXB];   // base of the outputs; stride Ns
+// One stage of radix R over nsig signals from entry `from` of the shared array
+// to entry `to`; step = M / (Ns R).
+template <int R>
+__device__ __forceinline__ void fx_stage(longlong2* sm, int from, int to, int nsig, int M, int Ns, int step,
+                                         const int4* tw) {
+    const int nb = M / R, ld = fx_stride(M);
+    const float rns = 1.f / float(Ns);
+#pragma unroll 1
+    for (int u = threadIdx.x; u < nsig * nb; u += blockDim.x) {
+        int t = u, o = 0;   // butterfly and its signal's offset
+        while (t >= nb) {
+            t -= nb;
+            o += ld;
+        }
+        // t / Ns: exact, as t + 1/2 is at least 1 / (2 Ns) away from every multiple
+        const int q = int((float(t) + 0.5f) * rns), k = t - q * Ns;
+        cx<fx> v[R];
 #pragma unroll
-    for (int b = 0; b < MAXB; ++b) {
-        int t = threadIdx.x + b * blockDim.x;
-        if (t < NSIG * nb) {
-            int sg = 0;
+        for (int r = 0; r < R; ++r) v[r] = fx_ld(sm + from + o + fxp(t + r * nb));
+        if (Ns > 1) {
 #pragma unroll
-            for (int i = 1; i < NSIG; ++i)
-                if (t >= nb) {
-                    t -= nb;
-                    ++sg;
-                }
-            const longlong2* src = buf + sg * ld;
-            const int q = t / Ns, k = t - q * Ns;
-            to[b] = sg * M + q * Ns * R + k;   // signal and index, unpadded
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[b][r] = fx_ld(src + fxp(t + r * nb));
-            if (Ns > 1) {
-#pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    const int4 w = tw[k * r * step];
-                    v[b][r] = S > 0 ? fx_cmul(v[b][r], {w.x, w.y}, {-w.z, -w.w})
-                                    : fx_cmul(v[b][r], {w.x, w.y}, {w.z, w.w});
-                }
+            for (int r = 1; r < R; ++r) {
+                const int4 w = tw[k * r * step];
+                v[r] = fx_cmul(v[r], {w.x, w.y}, {w.z, w.w});
             }
-            fx_dft<R, S>(v[b]);
-        } else {
-            to[b] = 0;
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[b][r] = {{0}, {0}};
         }
-    }
-    __syncthreads();
+        fx_dft<R, -1>(v);
 #pragma unroll
-    for (int b = 0; b < MAXB; ++b) {
-        const int t = threadIdx.x + b * blockDim.x;
-        if (t < NSIG * nb) {
-            int i = to[b], sg = 0;
-#pragma unroll
-            for (int j = 1; j < NSIG; ++j)
-                if (i >= M) {
-                    i -= M;
-                    ++sg;
-                }
-            longlong2* dst = buf + sg * ld;
-#pragma unroll
-            for (int r = 0; r < R; ++r) fx_st(dst + fxp(i + r * Ns), v[b][r]);
-        }
+        for (int r = 0; r < R; ++r) fx_st(sm + to + o + fxp(q * Ns * R + k + r * Ns), v[r]);
     }
     __syncthreads();
 }
 
-template <int NSIG, int TPT, int S>
-__device__ __forceinline__ void fx_fft(longlong2* buf, const FxPlan& plan, const int4* tw) {
-    int Ns = 1;
+// Forward transform of nsig signals at entry `from`, `to` the other buffer;
+// returns the entry of the result.
+__device__ __forceinline__ int fx_fft(longlong2* sm, int from, int to, int nsig, const FxPlan& plan, const int4* tw) {
+    int Ns = 1, step = plan.n;
+#pragma unroll 1
     for (int st = 0; st < plan.nst; ++st) {
         const int R = plan.radix[st];
-        if (R == 8) fx_stage<8, NSIG, TPT, S>(buf, plan.n, Ns, tw);
-        else if (R == 4) fx_stage<4, NSIG, TPT, S>(buf, plan.n, Ns, tw);
-        else if (R == 2) fx_stage<2, NSIG, TPT, S>(buf, plan.n, Ns, tw);
-        else if (R == 9) fx_stage<9, NSIG, TPT, S>(buf, plan.n, Ns, tw);
-        else fx_stage<3, NSIG, TPT, S>(buf, plan.n, Ns, tw);
+        if (R == 8) fx_stage<8>(sm, from, to, nsig, plan.n, Ns, step /= 8, tw);
+        else if (R == 4) fx_stage<4>(sm, from, to, nsig, plan.n, Ns, step /= 4, tw);
+        else if (R == 2) fx_stage<2>(sm, from, to, nsig, plan.n, Ns, step /= 2, tw);
+        else if (R == 9) fx_stage<9>(sm, from, to, nsig, plan.n, Ns, step /= 9, tw);
+        else fx_stage<3>(sm, from, to, nsig, plan.n, Ns, step /= 3, tw);
         Ns *= R;
+        const int t = from;
+        from = to;
+        to = t;
     }
+    return from;
 }
 
 // Block reductions of NV small integers per thread into shared slots
@@ -218,332 +198,327 @@ __device__ __forceinline__ int bitlen(unsigned v) { return 32 - __clz(v); }
 __device__ __forceinline__ unsigned hi_abs(long long v) { return unsigned((v ^ (v >> 63)) >> 32); }
 __device__ __forceinline__ unsigned top16_abs(long long v) { return unsigned((v ^ (v >> 63)) >> 44) + 1u; }
 
-// signals of a ring pair: inverse transforms, forward transforms
+// Signals: RHS, GRID: (zeta, u_theta) of each of the CTA's two rings and
+// (u_phi, u_phi) of both; PROJECT: (v_theta, v_phi) of two rings; ADJOINT, one
+// ring per CTA (its shared memory): (zeta, u_theta), (u_phi, v_theta), (v_phi, 0)
+// in, (X_theta, X_phi), (rho, 0) out.
 template <int MODE> struct FxMode {
     static constexpr int NF = MODE == RING_ADJOINT ? 5 : (MODE == RING_PROJECT ? 2 : 3);   // input fields
-    static constexpr int NI = MODE == RING_ADJOINT ? 5 : (MODE == RING_PROJECT ? 0 : 3);   // inverse signals
-    static constexpr int NO = MODE == RING_ADJOINT ? 3 : 2;                                // forward signals
-    static constexpr int NS = NI > NO ? NI : NO;
+    static constexpr int RPC = MODE == RING_ADJOINT ? 1 : 2;                               // rings per CTA
+    static constexpr int NS = MODE == RING_PROJECT ? 2 : 3;                                // signals
+    static constexpr int NV = NF * RPC;                                                    // value f of ring r: RPC f + r
 };
 
-// MODE and TPT (butterfly values per thread / 8) fix the launch shape:
-// blockDim >= NS M / (8 TPT).
-template <int MODE, int TPT>
-__global__ void __launch_bounds__(MODE == RING_ADJOINT ? 512 : 288, MODE == RING_ADJOINT ? 1 : 2) k_ring_fx(RingFxArgs a) {
+template <int MODE>
+__global__ void __launch_bounds__(576, 1) k_ring_fx(RingFxArgs a) {
     using Q = FxMode<MODE>;
-    constexpr int NF = Q::NF, NS = Q::NS;
+    constexpr int NF = Q::NF, NS = Q::NS, RPC = Q::RPC, NV = Q::NV;
     extern __shared__ __align__(16) unsigned char smem_fx[];
-    __shared__ int s_emax[2 * NF];
-    __shared__ unsigned s_sum[2 * NF], s_or[2 * NF], s_sum2[6];
+    __shared__ int s_emax[NV];
+    __shared__ unsigned s_sum[NV], s_or[NV], s_sum2[4];
     const int M = a.M, N = a.N, nlat = a.nlat, ld = fx_stride(M), tid = threadIdx.x, NT = blockDim.x;
-    longlong2* buf = reinterpret_cast<longlong2*>(smem_fx);
-    int4* tw = reinterpret_cast<int4*>(buf + NS * ld);
-    const int pair = blockIdx.x, npair = (nlat + 1) / 2, row0 = 2 * pair;
-    const bool two = row0 + 1 < nlat;
+    longlong2* sm = reinterpret_cast<longlong2*>(smem_fx);
+    int cur = 0;   // the buffer that holds the signals: entries 0 or NS ld
+    int4* tw = reinterpret_cast<int4*>(sm + 2 * NS * ld);
+    const int npair = (nlat + 1) / 2, row0 = RPC * blockIdx.x, pair = row0 / 2;
+    const bool two = RPC == 2 && row0 + 1 < nlat;
     if (a.early) pdl_launch();
     // the plan's constants do not depend on the predecessor
     for (int t = tid; t < M; t += NT) tw[t] = a.tw[t];
-    if (tid < 2 * NF) {
+    if (tid < NV) {
         s_emax[tid] = 0;
         s_sum[tid] = 0u;
         s_or[tid] = 0u;
     }
-    if (tid < 6) s_sum2[tid] = 0u;
-    const double fc[2] = {a.two_omega * a.x[row0], two ? a.two_omega * a.x[row0 + 1] : 0.0};
-    double scale[2] = {MODE == RING_GRID ? 1.0 : a.rw[row0], MODE == RING_GRID ? 1.0 : (two ? a.rw[row0 + 1] : 0.0)};
+    if (tid < 4) s_sum2[tid] = 0u;
+    double fc[RPC], scale[RPC];
+#pragma unroll
+    for (int r = 0; r < RPC; ++r) {
+        const int row = min(row0 + r, nlat - 1);
+        fc[r] = MODE == RING_GRID ? 0.0 : a.two_omega * a.x[row];
+        scale[r] = MODE == RING_GRID ? 1.0 : a.rw[row];
+    }
     pdl_wait();
-    int kf[2 * NF];   // fixed point = value 2^kf, of field f of ring r at 2 f + r
+    int kf[NV];   // fixed point = value 2^kf
+    const double nan = __longlong_as_double(0x7FF8000000000000LL);
 
     if constexpr (MODE != RING_PROJECT) {
-        // a thread owns the orders m = tid + i NT of every field and both rings
-        constexpr int NM = TPT;
-        double x[NM][NF][4];
-        int em[2 * NF];
+        // a thread owns the order m = tid (N < M / 3 <= blockDim) of every field and ring
+        const int m = tid;
+        double x[NV][2];
+        int em[NV];
 #pragma unroll
-        for (int i = 0; i < 2 * NF; ++i) em[i] = 0;
-#pragma unroll
-        for (int i = 0; i < NM; ++i) {
-            const int m = tid + i * NT;
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-                double4_32a g = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-                if (m <= N)
-                    g = *reinterpret_cast<const double4_32a*>(a.gsyn +
-                                                              ((size_t(f) * npair + pair) * size_t(N + 1) + m) * 4);
-                x[i][f][0] = g.x;
-                x[i][f][1] = m == 0 ? 0.0 : g.y;   // fields are real
-                x[i][f][2] = two ? g.z : 0.0;
-                x[i][f][3] = two && m != 0 ? g.w : 0.0;
-                if (f == 0 && m == 0 && MODE != RING_GRID) {   // q = zeta + 2 Omega cos(theta)
-                    x[i][f][0] += fc[0];
-                    x[i][f][2] += fc[1];
-                }
-#pragma unroll
-                for (int r = 0; r < 2; ++r)
-                    em[2 * f + r] = max(em[2 * f + r], max(f64_bexp(x[i][f][2 * r]), f64_bexp(x[i][f][2 * r + 1])));
-            }
-        }
-        __syncthreads();   // the slots are zero
-        red_max<2 * NF>(em, s_emax);
-        __syncthreads();
-        unsigned sm[2 * NF];
-#pragma unroll
-        for (int j = 0; j < 2 * NF; ++j) {
-            const int E = max(s_emax[j], 1);
-            em[j] = E;
-            sm[j] = 0u;
-#pragma unroll
-            for (int i = 0; i < NM; ++i) {
-                const int m = tid + i * NT;
-                const unsigned v = f64_top16(x[i][j / 2][2 * (j & 1)], E) + f64_top16(x[i][j / 2][2 * (j & 1) + 1], E);
-                if (m <= N) sm[j] += m == 0 ? v : 2u * v;
-            }
-        }
-        red_add<2 * NF>(sm, s_sum);
-        // the zero-padded middle of every inverse signal
-        for (int m = N + 1 + tid; m < M - N; m += NT)
-#pragma unroll
-            for (int sg = 0; sg < Q::NI; ++sg) buf[sg * ld + fxp(m)] = make_longlong2(0, 0);
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < 2 * NF; ++j) {
-            kf[j] = 1072 - em[j] + 26 - bitlen(s_sum[j]);
-            // a non-finite input makes its ring's outputs NaN
-            if (em[j] == 2047) scale[j & 1] = __longlong_as_double(0x7FF8000000000000LL);
-        }
-        // signals: RHS, GRID: (zeta, u_theta) of each ring, (u_phi, u_phi) of
-        // both; ADJOINT: (zeta, u_theta), (u_phi, v_theta) of each ring,
-        // (v_phi, v_phi) of both
-#pragma unroll
-        for (int i = 0; i < NM; ++i) {
-            const int m = tid + i * NT;
-            if (m > N) continue;
-            auto put = [&](int sg, int fa, int ra, int fb, int rb) {
-                const long long ax = f64_to_fx(x[i][fa][2 * ra], kf[2 * fa + ra]);
-                const long long ay = f64_to_fx(x[i][fa][2 * ra + 1], kf[2 * fa + ra]);
-                const long long bx = f64_to_fx(x[i][fb][2 * rb], kf[2 * fb + rb]);
-                const long long by = f64_to_fx(x[i][fb][2 * rb + 1], kf[2 * fb + rb]);
-                buf[sg * ld + fxp(m)] = make_longlong2(ax - by, ay + bx);
-                if (m > 0) buf[sg * ld + fxp(M - m)] = make_longlong2(ax + by, bx - ay);
-            };
-            put(0, 0, 0, 1, 0);
-            put(1, 0, 1, 1, 1);
-            if constexpr (MODE == RING_ADJOINT) {
-                put(2, 2, 0, 3, 0);
-                put(3, 2, 1, 3, 1);
-                put(4, 4, 0, 4, 1);
+        for (int f = 0; f < NF; ++f) {
+            const double* g = a.gsyn + ((size_t(f) * npair + pair) * size_t(N + 1) + m) * 4;
+            if constexpr (RPC == 2) {
+                double4_32a v = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+                if (m <= N) v = *reinterpret_cast<const double4_32a*>(g);
+                x[2 * f][0] = v.x;
+                x[2 * f][1] = v.y;
+                x[2 * f + 1][0] = two ? v.z : 0.0;
+                x[2 * f + 1][1] = two ? v.w : 0.0;
             } else {
-                put(2, 2, 0, 2, 1);
+                double2 v = make_double2(0.0, 0.0);
+                if (m <= N) v = *reinterpret_cast<const double2*>(g + 2 * (row0 & 1));
+                x[f][0] = v.x;
+                x[f][1] = v.y;
             }
         }
+        if (m == 0) {
+#pragma unroll
+            for (int j = 0; j < NV; ++j) x[j][1] = 0.0;   // fields are real
+            x[0][0] += fc[0];                             // q = zeta + 2 Omega cos(theta)
+            if constexpr (RPC == 2)
+                if (two) x[1][0] += fc[1];
+        }
+#pragma unroll
+        for (int j = 0; j < NV; ++j) em[j] = max(f64_bexp(x[j][0]), f64_bexp(x[j][1]));
+        __syncthreads();   // the reduction slots are zero, the twiddles in place
+        red_max<NV>(em, s_emax);
         __syncthreads();
-        fx_fft<Q::NI, TPT, +1>(buf, a.plan, tw);
-    }
-
-    if constexpr (MODE == RING_GRID) {
-        for (int q = tid; q < M; q += NT) {
-            const longlong2 B = buf[2 * ld + fxp(q)];
+        unsigned sum[NV];
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                if (r == 1 && !two) break;
-                const longlong2 A = buf[r * ld + fxp(q)];
-                const size_t o = size_t(row0 + r) * M + q;
-                if (a.gout0) a.gout0[o] = f64_scale(__ll2double_rn(A.x) * scale[r], -kf[r]);
-                if (a.gout1) a.gout1[o] = f64_scale(__ll2double_rn(A.y) * scale[r], -kf[2 + r]);
-                if (a.gout2) a.gout2[o] = f64_scale(__ll2double_rn(r ? B.y : B.x) * scale[r], -kf[4 + r]);
+        for (int j = 0; j < NV; ++j) {
+            em[j] = max(s_emax[j], 1);
+            const unsigned v = f64_top16(x[j][0], em[j]) + f64_top16(x[j][1], em[j]);
+            sum[j] = m > N ? 0u : (m == 0 ? v : 2u * v);
+        }
+        red_add<NV>(sum, s_sum);
+        // the zero-padded middle of every signal
+        for (int q = N + 1 + tid; q < M - N; q += NT)
+#pragma unroll
+            for (int sg = 0; sg < NS; ++sg) sm[sg * ld + fxp(q)] = make_longlong2(0, 0);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+            kf[j] = 1072 - em[j] + 26 - bitlen(s_sum[j]);
+            if (em[j] == 2047) scale[j % RPC] = nan;   // a non-finite input: NaN for its ring
+        }
+        if (m <= N) {
+            long long v[NV][2];
+#pragma unroll
+            for (int j = 0; j < NV; ++j) {
+                v[j][0] = f64_to_fx(x[j][0], kf[j]);
+                v[j][1] = f64_to_fx(x[j][1], kf[j]);
+            }
+            // Z = a + i b of two Hermitian spectra, Z_{M-m} = conj(a_m) + i conj(b_m);
+            // stored with real and imaginary parts exchanged (inverse transform)
+            auto put = [&](int sg, long long ax, long long ay, long long bx, long long by) {
+                sm[sg * ld + fxp(m)] = make_longlong2(ay + bx, ax - by);
+                if (m > 0) sm[sg * ld + fxp(M - m)] = make_longlong2(bx - ay, ax + by);
+            };
+            if constexpr (RPC == 2) {
+                put(0, v[0][0], v[0][1], v[2][0], v[2][1]);
+                put(1, v[1][0], v[1][1], v[3][0], v[3][1]);
+                put(2, v[4][0], v[4][1], v[5][0], v[5][1]);
+            } else {
+                put(0, v[0][0], v[0][1], v[1][0], v[1][1]);
+                put(1, v[2][0], v[2][1], v[3][0], v[3][1]);
+                put(2, v[4][0], v[4][1], 0, 0);
             }
         }
-        return;
     }
 
-    // W (fields to transform): value j = 2 c + r, c = 0, 1: the two components
-    // of ring r's signal; ADJOINT also c = 2: rho of ring r
-    constexpr int NW = MODE == RING_ADJOINT ? 6 : 4;
-    constexpr int NQ = (8 * TPT + NS - 1) / NS;   // grid points per thread
+    // W = the fields to transform forward: component c of ring r's signal (ADJOINT: X_theta,
+    // X_phi, rho) at RPC c + r
+    constexpr int NW = MODE == RING_ADJOINT ? 3 : 4;
     int kw[NW];
-    long long w[NQ][NW];
     if constexpr (MODE == RING_PROJECT) {
-        double x[NQ][4];
+        auto grid = [&](int j, int q) {
+            return (j & 1) == 0 || two ? (j / 2 ? a.gin1 : a.gin0)[size_t(row0 + (j & 1)) * M + q] : 0.0;
+        };
         int em[4] = {0, 0, 0, 0};
+        for (int q = tid; q < M; q += NT)
 #pragma unroll
-        for (int i = 0; i < NQ; ++i) {
-            const int q = tid + i * NT;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int c = j / 2, r = j & 1;
-                x[i][j] = 0.0;
-                if (q < M && (r == 0 || two)) x[i][j] = (c ? a.gin1 : a.gin0)[size_t(row0 + r) * M + q];
-                em[j] = max(em[j], f64_bexp(x[i][j]));
-            }
-        }
+            for (int j = 0; j < 4; ++j) em[j] = max(em[j], f64_bexp(grid(j, q)));
         __syncthreads();
         red_max<4>(em, s_emax);
         __syncthreads();
-        unsigned sm[4];
+        unsigned sum[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            em[j] = max(s_emax[j], 1);
-            sm[j] = 0u;
+        for (int j = 0; j < 4; ++j) em[j] = max(s_emax[j], 1);
+        for (int q = tid; q < M; q += NT)
 #pragma unroll
-            for (int i = 0; i < NQ; ++i)
-                if (tid + i * NT < M) sm[j] += f64_top16(x[i][j], em[j]);
-        }
-        red_add<4>(sm, s_sum);
+            for (int j = 0; j < 4; ++j) sum[j] += f64_top16(grid(j, q), em[j]);
+        red_add<4>(sum, s_sum);
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             kw[j] = 1072 - em[j] + 26 - bitlen(s_sum[j]);
-            if (em[j] == 2047) scale[j & 1] = __longlong_as_double(0x7FF8000000000000LL);
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) w[i][j] = f64_to_fx(x[i][j], kw[j]);
+            if (em[j] == 2047) scale[j & 1] = nan;
         }
-    } else {
-        // the grid values of point q: fields 2 f + r
-        auto fields = [&](int q, long long* v) {
-            const longlong2 A0 = buf[fxp(q)], A1 = buf[ld + fxp(q)];
-            v[0] = A0.x; v[1] = A1.x; v[2] = A0.y; v[3] = A1.y;
-            if constexpr (MODE == RING_ADJOINT) {
-                const longlong2 B0 = buf[2 * ld + fxp(q)], B1 = buf[3 * ld + fxp(q)], C = buf[4 * ld + fxp(q)];
-                v[4] = B0.x; v[5] = B1.x; v[6] = B0.y; v[7] = B1.y; v[8] = C.x; v[9] = C.y;
-            } else {
-                const longlong2 B = buf[2 * ld + fxp(q)];
-                v[4] = B.x; v[5] = B.y;
-            }
-        };
-        unsigned om[2 * NF];
+        for (int q = tid; q < M; q += NT)
 #pragma unroll
-        for (int j = 0; j < 2 * NF; ++j) om[j] = 0u;
-        for (int q = tid; q < M; q += NT) {
-            long long v[2 * NF];
-            fields(q, v);
-#pragma unroll
-            for (int j = 0; j < 2 * NF; ++j) om[j] |= hi_abs(v[j]);
-        }
-        red_or<2 * NF>(om, s_or);
-        __syncthreads();
-        int up[2 * NF];   // left shift of a field to |v| < 2^61
-#pragma unroll
-        for (int j = 0; j < 2 * NF; ++j) {
-            up[j] = max(0, 29 - bitlen(s_or[j]));
-            kf[j] += up[j];
-        }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            if constexpr (MODE == RING_RHS) {
-                kw[r] = kf[r] + kf[4 + r] - 62;        // W_theta = -q u_phi
-                kw[2 + r] = kf[r] + kf[2 + r] - 62;    // W_phi = q u_theta
-            } else {
-                kw[r] = kf[r] + kf[8 + r] - 62;        // X_theta = q v_phi
-                kw[2 + r] = kf[r] + kf[6 + r] - 62;    // X_phi = -q v_theta
-                // rho = -v_theta u_phi + v_phi u_theta, at the coarser scale of the two
-                kw[4 + r] = min(kf[6 + r] + kf[4 + r], kf[8 + r] + kf[2 + r]) - 62;
-            }
-        }
-        unsigned sm[NW];
-#pragma unroll
-        for (int j = 0; j < NW; ++j) sm[j] = 0u;
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) {
-            const int q = tid + i * NT;
-#pragma unroll
-            for (int j = 0; j < NW; ++j) w[i][j] = 0;
-            if (q < M) {
-                long long v[2 * NF];
-                fields(q, v);
-#pragma unroll
-                for (int j = 0; j < 2 * NF; ++j) v[j] <<= up[j];
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    if constexpr (MODE == RING_RHS) {
-                        w[i][r] = -fx_mul62(v[r], v[4 + r]);
-                        w[i][2 + r] = fx_mul62(v[r], v[2 + r]);
-                    } else {
-                        w[i][r] = fx_mul62(v[r], v[8 + r]);
-                        w[i][2 + r] = -fx_mul62(v[r], v[6 + r]);
-                        const int d1 = kw[4 + r] + 62 - kf[6 + r] - kf[4 + r];
-                        const int d2 = kw[4 + r] + 62 - kf[8 + r] - kf[2 + r];
-                        w[i][4 + r] = fx_shift(fx_mul62(v[8 + r], v[2 + r]), d2) -
-                                      fx_shift(fx_mul62(v[6 + r], v[4 + r]), d1);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < NW; ++j) sm[j] += top16_abs(w[i][j]);
-            }
-        }
-        red_add<NW>(sm, s_sum2);
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < NW; ++j) {
-            const int sh = 16 - bitlen(s_sum2[j]);
-            kw[j] += sh;
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) w[i][j] = fx_shift(w[i][j], sh);
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) {
-        const int q = tid + i * NT;
-        if (q >= M) continue;
-        buf[fxp(q)] = make_longlong2(w[i][0], w[i][2]);
-        buf[ld + fxp(q)] = make_longlong2(w[i][1], w[i][3]);
-        if constexpr (MODE == RING_ADJOINT) buf[2 * ld + fxp(q)] = make_longlong2(w[i][4], w[i][5]);
+            for (int r = 0; r < 2; ++r)
+                sm[r * ld + fxp(q)] = make_longlong2(f64_to_fx(grid(r, q), kw[r]), f64_to_fx(grid(2 + r, q), kw[2 + r]));
     }
     __syncthreads();
-    fx_fft<Q::NO, TPT, -1>(buf, a.plan, tw);
+
+    // pass 0: inverse transform and product; pass 1: forward transform
+#pragma unroll 1
+    for (int pass = MODE == RING_PROJECT ? 1 : 0; pass < 2; ++pass) {
+        cur = fx_fft(sm, cur, NS * ld - cur, pass == 0 ? NS : 2, a.plan, tw);
+        if (pass == 1) break;
+        const longlong2* in = sm + cur;
+        if constexpr (MODE == RING_GRID) {
+            for (int q = tid; q < M; q += NT) {
+                const longlong2 B = in[2 * ld + fxp(q)];
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    if (r == 1 && !two) break;
+                    const longlong2 A = in[r * ld + fxp(q)];   // (u_theta, zeta)
+                    const size_t o = size_t(row0 + r) * M + q;
+                    if (a.gout0) a.gout0[o] = f64_scale(__ll2double_rn(A.y) * scale[r], -kf[r]);
+                    if (a.gout1) a.gout1[o] = f64_scale(__ll2double_rn(A.x) * scale[r], -kf[2 + r]);
+                    if (a.gout2) a.gout2[o] = f64_scale(__ll2double_rn(r ? B.x : B.y) * scale[r], -kf[4 + r]);
+                }
+            }
+            return;
+        } else if constexpr (MODE != RING_PROJECT) {
+            // the grid values of point q (real and imaginary parts exchanged)
+            auto fields = [&](int q, long long* v) {
+                const longlong2 A = in[fxp(q)], B = in[ld + fxp(q)], C = in[2 * ld + fxp(q)];
+                if constexpr (RPC == 2) {
+                    v[0] = A.y; v[1] = B.y; v[2] = A.x; v[3] = B.x; v[4] = C.y; v[5] = C.x;
+                } else {
+                    v[0] = A.y; v[1] = A.x; v[2] = B.y; v[3] = B.x; v[4] = C.y;
+                }
+            };
+            unsigned om[NV];
+#pragma unroll
+            for (int j = 0; j < NV; ++j) om[j] = 0u;
+            for (int q = tid; q < M; q += NT) {
+                long long v[NV];
+                fields(q, v);
+#pragma unroll
+                for (int j = 0; j < NV; ++j) om[j] |= hi_abs(v[j]);
+            }
+            red_or<NV>(om, s_or);
+            __syncthreads();
+            int up[NV];   // left shift of a field to |v| < 2^61
+#pragma unroll
+            for (int j = 0; j < NV; ++j) {
+                up[j] = max(0, 29 - bitlen(s_or[j]));
+                kf[j] += up[j];
+            }
+            int d1 = 0, d2 = 0;
+            if constexpr (MODE == RING_RHS) {
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    kw[r] = kf[r] + kf[4 + r] - 62;        // W_theta = -q u_phi
+                    kw[2 + r] = kf[r] + kf[2 + r] - 62;    // W_phi = q u_theta
+                }
+            } else {
+                kw[0] = kf[0] + kf[4] - 62;   // X_theta = q v_phi
+                kw[1] = kf[0] + kf[3] - 62;   // X_phi = -q v_theta
+                // rho = -v_theta u_phi + v_phi u_theta, at the coarser scale of the two
+                kw[2] = min(kf[3] + kf[2], kf[4] + kf[1]) - 62;
+                d1 = kw[2] + 62 - kf[3] - kf[2];
+                d2 = kw[2] + 62 - kf[4] - kf[1];
+            }
+            longlong2* out = sm + (NS * ld - cur);
+            unsigned sum[NW];
+#pragma unroll
+            for (int j = 0; j < NW; ++j) sum[j] = 0u;
+            for (int q = tid; q < M; q += NT) {
+                long long v[NV], w[4];
+                fields(q, v);
+#pragma unroll
+                for (int j = 0; j < NV; ++j) v[j] <<= up[j];
+                if constexpr (MODE == RING_RHS) {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        w[r] = -fx_mul62(v[r], v[4 + r]);
+                        w[2 + r] = fx_mul62(v[r], v[2 + r]);
+                    }
+                    out[fxp(q)] = make_longlong2(w[0], w[2]);
+                    out[ld + fxp(q)] = make_longlong2(w[1], w[3]);
+                } else {
+                    w[0] = fx_mul62(v[0], v[4]);
+                    w[1] = -fx_mul62(v[0], v[3]);
+                    w[2] = fx_shift(fx_mul62(v[4], v[1]), d2) - fx_shift(fx_mul62(v[3], v[2]), d1);
+                    out[fxp(q)] = make_longlong2(w[0], w[1]);
+                    out[ld + fxp(q)] = make_longlong2(w[2], 0);
+                }
+#pragma unroll
+                for (int j = 0; j < NW; ++j) sum[j] += top16_abs(w[j]);
+            }
+            red_add<NW>(sum, s_sum2);
+            __syncthreads();
+            int sh[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int j = 0; j < NW; ++j) {
+                sh[j] = 16 - bitlen(s_sum2[j]);
+                kw[j] += sh[j];
+            }
+            // every thread rescales the points it wrote
+            for (int q = tid; q < M; q += NT)
+#pragma unroll
+                for (int sg = 0; sg < 2; ++sg) {
+                    const longlong2 w = out[sg * ld + fxp(q)];
+                    const int jx = RPC == 2 ? sg : 2 * sg, jy = RPC == 2 ? 2 + sg : 1 + 2 * sg;
+                    out[sg * ld + fxp(q)] = make_longlong2(fx_shift(w.x, sh[jx]), fx_shift(w.y, sh[jy]));
+                }
+            cur = NS * ld - cur;
+            __syncthreads();
+        }
+    }
 
     // separate the real spectra: of Z = A + i B, A_m = (Z_m + conj Z_{M-m}) / 2,
     // B_m = (Z_m - conj Z_{M-m}) / (2 i); truncate, weight, store
-    const double sn[2] = {MODE == RING_ADJOINT ? a.s[row0] : 0.0, MODE == RING_ADJOINT && two ? a.s[row0 + 1] : 0.0};
-    for (int m = tid; m <= N; m += NT) {
-        const int mr = m == 0 ? 0 : M - m;
-        double4_32a o[3];
-        auto cv = [&](long long v, double sc, int k) { return f64_scale(__ll2double_rn(v) * sc, -k - 1); };
+    const int m = tid;
+    if (m > N) return;
+    const longlong2* in = sm + cur;
+    const int mr = m == 0 ? 0 : M - m;
+    auto cv = [&](long long v, double sc, int k) { return f64_scale(__ll2double_rn(v) * sc, -k - 1); };
+    // field f of every ring, and the column scales of the analysis
+    auto store = [&](int f, const double4_32a& o) {
+        double* g = a.gana + ((size_t(f) * npair + pair) * size_t(N + 1) + m) * 4;
+        int e = max(f64_bexp(o.x), f64_bexp(o.y));
+        if constexpr (RPC == 2) {
+            *reinterpret_cast<double4_32a*>(g) = o;
+            e = max(e, max(f64_bexp(o.z), f64_bexp(o.w)));
+        } else {
+            *reinterpret_cast<double2*>(g + 2 * (row0 & 1)) = make_double2(o.x, o.y);
+        }
+        atomicMax(a.emax + f * (N + 1) + m, e);
+    };
+    double4_32a o0 = make_double4_32a(0.0, 0.0, 0.0, 0.0), o1 = o0;
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const longlong2 p = buf[r * ld + fxp(m)], z = buf[r * ld + fxp(mr)];
-            const double tx = cv(p.x + z.x, scale[r], kw[r]), ty = cv(p.y - z.y, scale[r], kw[r]);
-            const double fx_ = cv(p.y + z.y, scale[r], kw[2 + r]), fy = cv(z.x - p.x, scale[r], kw[2 + r]);
-            if (r == 0) {
-                o[0].x = tx; o[0].y = ty; o[1].x = fx_; o[1].y = fy;
-            } else {
-                o[0].z = tx; o[0].w = ty; o[1].z = fx_; o[1].w = fy;
-            }
+    for (int r = 0; r < RPC; ++r) {
+        if (r == 1 && !two) break;
+        const longlong2 p = in[r * ld + fxp(m)], z = in[r * ld + fxp(mr)];
+        const double tx = cv(p.x + z.x, scale[r], kw[r]), ty = cv(p.y - z.y, scale[r], kw[r]);
+        const double fx_ = cv(p.y + z.y, scale[r], kw[RPC + r]), fy = cv(z.x - p.x, scale[r], kw[RPC + r]);
+        if (r == 0) {
+            o0.x = tx; o0.y = ty; o1.x = fx_; o1.y = fy;
+        } else {
+            o0.z = tx; o0.w = ty; o1.z = fx_; o1.w = fy;
         }
-        if constexpr (MODE == RING_ADJOINT) {
-            // rho of the two rings: plain quadrature weight (2 pi / M) w_p
-            const longlong2 p = buf[2 * ld + fxp(m)], z = buf[2 * ld + fxp(mr)];
-            o[2].x = cv(p.x + z.x, scale[0] * sn[0], kw[4]);
-            o[2].y = cv(p.y - z.y, scale[0] * sn[0], kw[4]);
-            o[2].z = cv(p.y + z.y, scale[1] * sn[1], kw[5]);
-            o[2].w = cv(z.x - p.x, scale[1] * sn[1], kw[5]);
-        }
-#pragma unroll
-        for (int f = 0; f < (MODE == RING_ADJOINT ? 3 : 2); ++f)
-        {
-            *reinterpret_cast<double4_32a*>(a.gana + ((size_t(f) * npair + pair) * size_t(N + 1) + m) * 4) = o[f];
-            // the column scales of the analysis
-            atomicMax(a.emax + f * (N + 1) + m,
-                      max(max(f64_bexp(o[f].x), f64_bexp(o[f].y)), max(f64_bexp(o[f].z), f64_bexp(o[f].w))));
-        }
+    }
+    store(0, o0);
+    store(1, o1);
+    if constexpr (MODE == RING_ADJOINT) {
+        // rho: plain quadrature weight (2 pi / M) w_p
+        const longlong2 p = in[ld + fxp(m)], z = in[ld + fxp(mr)];
+        const double sc = scale[0] * a.s[row0];
+        o0.x = cv(p.x + z.x, sc, kw[2]);
+        o0.y = cv(p.y - z.y, sc, kw[2]);
+        store(2, o0);
     }
 }
 
-template <int MODE, int TPT>
-static cudaError_t ring_fx_t(sphnse_plan* P, RingFxArgs a) {
-    constexpr int NS = FxMode<MODE>::NS;
-    const int threads = ((NS * a.M + 8 * TPT - 1) / (8 * TPT) + 31) / 32 * 32;
-    const size_t sm = size_t(NS) * fx_stride(a.M) * 16 + size_t(a.M) * 16;
-    allow_dynamic_smem(reinterpret_cast<const void*>(k_ring_fx<MODE, TPT>), sm);
-    const int grid = (a.nlat + 1) / 2;
-    a.early = grid <= 2 * P->nsm;
-    return launch_pdl(k_ring_fx<MODE, TPT>, dim3(grid), dim3(threads), sm, P->stream, a);
-}
-
 template <int MODE>
-static cudaError_t ring_fx_m(sphnse_plan* P, const RingFxArgs& a) {
-    // one butterfly of eight per thread while the block fits its bound
-    constexpr int most = MODE == RING_ADJOINT ? 512 : 288;
-    return FxMode<MODE>::NS * a.M <= 8 * most ? ring_fx_t<MODE, 1>(P, a) : ring_fx_t<MODE, 2>(P, a);
+static cudaError_t ring_fx_t(sphnse_plan* P, RingFxArgs a) {
+    using Q = FxMode<MODE>;
+    // a radix-8 butterfly per thread; every order m <= N < M / 3 needs its own thread
+    const int threads = std::max((Q::NS * a.M / 8 + 31) / 32 * 32, (a.N + 32) / 32 * 32);
+    const size_t sm = size_t(2) * Q::NS * fx_stride(a.M) * 16 + size_t(a.M) * 16;
+    allow_dynamic_smem(reinterpret_cast<const void*>(k_ring_fx<MODE>), sm);
+    const int grid = (a.nlat + Q::RPC - 1) / Q::RPC;
+    // a grid of more than one wave must not start its successor early
+    a.early = grid <= P->nsm * std::max(1, std::min(int((227 * 1024) / (sm + 1024)), 576 / threads));
+    return launch_pdl(k_ring_fx<MODE>, dim3(grid), dim3(threads), sm, P->stream, a);
 }
 
 int launch_ring_fx(sphnse_plan* P, int mode, const double* gin0, const double* gin1, double* gout0, double* gout1,
@@ -569,10 +544,10 @@ int launch_ring_fx(sphnse_plan* P, int mode, const double* gin0, const double* g
     stage_begin(P, SPHNSE_STAGE_RING);
     cudaError_t e;
     switch (mode) {
-        case RING_RHS: e = ring_fx_m<RING_RHS>(P, a); break;
-        case RING_GRID: e = ring_fx_m<RING_GRID>(P, a); break;
-        case RING_PROJECT: e = ring_fx_m<RING_PROJECT>(P, a); break;
-        default: e = ring_fx_m<RING_ADJOINT>(P, a); break;
+        case RING_RHS: e = ring_fx_t<RING_RHS>(P, a); break;
+        case RING_GRID: e = ring_fx_t<RING_GRID>(P, a); break;
+        case RING_PROJECT: e = ring_fx_t<RING_PROJECT>(P, a); break;
+        default: e = ring_fx_t<RING_ADJOINT>(P, a); break;
     }
     stage_end(P, SPHNSE_STAGE_RING);
     return check_cuda(e);
