@@ -259,7 +259,7 @@ struct Bucket {
     int L = 0, nb = 0;
     sphnse_plan* P = nullptr;
     long off = 0;              // first complex entry of the bucket in the concatenated vectors
-    float *bsyn = nullptr, *gsyn = nullptr, *gsyn_r = nullptr, *gana_r = nullptr, *gana = nullptr, *hana = nullptr;
+    float *bsyn = nullptr, *gsyn = nullptr, *gana = nullptr, *hana = nullptr;
     size_t sb = 0, sg = 0, sa = 0, sh = 0;   // per-instance strides (floats)
     int* items = nullptr;
     int* item_off = nullptr;
@@ -322,22 +322,20 @@ int batched_rhs(sphnse_ensemble* E, const double2* x, double2* F) {
         P->stream = E->stream;
         const double* xb = reinterpret_cast<const double*>(x + B.off);
         double* Fb = reinterpret_cast<double*>(F + B.off);
+        const bool ring4 = ring4_ok(P);
+        const int pairs = !ring4;   // layout of the ring kernel's input
         if (B.tc) {
             // all instances of the bucket share every table tile of the synthesis
             if ((rc = launch_prep_tc_batch(P, B.tcb, xb))) return rc;
-            if ((rc = launch_synthesis_tc_batch(P, B.tcb, B.gsyn, B.sg, 0))) return rc;
+            if ((rc = launch_synthesis_tc_batch(P, B.tcb, B.gsyn, B.sg, pairs))) return rc;
         } else {
             if ((rc = launch_prep32_batch(P, B.nb, xb, B.bsyn, B.sb))) return rc;
-            if ((rc = launch_synthesis_stream_batch(P, B.items, B.item_off, B.ncta, B.bsyn, B.sb, B.gsyn, B.sg, 0)))
+            if ((rc = launch_synthesis_stream_batch(P, B.items, B.item_off, B.ncta, B.bsyn, B.sb, B.gsyn, B.sg, pairs)))
                 return rc;
         }
-        if (ring4_ok(P)) {
-            if ((rc = launch_ring4(P, B.nb, B.gsyn, B.sg, B.gana, B.sa, 0))) return rc;
-        } else {
-            if ((rc = launch_transpose(P, B.gsyn, B.gsyn_r, P->N + 1, P->nlat, 3 * B.nb))) return rc;
-            if ((rc = launch_ring_batch(P, B.nb, B.gsyn_r, B.sg, B.gana_r, B.sa))) return rc;
-            if ((rc = launch_transpose(P, B.gana_r, B.gana, P->nlat, P->N + 1, 2 * B.nb))) return rc;
-        }
+        if ((rc = ring4 ? launch_ring4(P, B.nb, B.gsyn, B.sg, B.gana, B.sa, 0)
+                        : launch_ring_batch(P, B.nb, B.gsyn, B.sg, B.gana, B.sa)))
+            return rc;
         if (B.tc) {
             if ((rc = launch_analysis_tc_batch(P, B.tca, B.gana, B.sa, B.hana, B.sh))) return rc;
         } else if ((rc = launch_analysis_stream_batch(P, B.items, B.item_off, B.ncta, B.gana, B.sa, B.hana, B.sh))) {
@@ -395,7 +393,7 @@ void destroy_ens(sphnse_ensemble* E) {
     if (E->ev_in) cudaEventDestroy(E->ev_in);
     if (E->ev_out) cudaEventDestroy(E->ev_out);
     for (auto& B : E->buckets) {
-        void* ptrs[] = {B.bsyn, B.gsyn, B.gsyn_r, B.gana_r, B.gana, B.hana, B.items, B.item_off, B.nu_dev};
+        void* ptrs[] = {B.bsyn, B.gsyn, B.gana, B.hana, B.items, B.item_off, B.nu_dev};
         for (void* q : ptrs)
             if (q) cudaFree(q);
         tc_batch_free(&B.tcb);
@@ -486,7 +484,7 @@ sphnse_ensemble* sphnse_ensemble_create(int n, const int* Ls, const double* nus,
             total += P->n_coeff;
             nub.push_back(nus[i]);
         }
-        const size_t g1 = size_t(P->N + 1) * P->nlat * 2;  // floats in one complex field
+        const size_t g1 = size_t(P->N + 1) * (P->nlat + (P->nlat & 1)) * 2;  // floats in one complex field (whole pairs)
         B.sb = size_t(P->n_ext) * 6;
         B.sg = 3 * g1;
         B.sa = 2 * g1;
@@ -496,8 +494,6 @@ sphnse_ensemble* sphnse_ensemble_create(int n, const int* Ls, const double* nus,
         };
         fal(&B.bsyn, B.sb * B.nb);
         fal(&B.gsyn, B.sg * B.nb);
-        fal(&B.gsyn_r, B.sg * B.nb);
-        fal(&B.gana_r, B.sa * B.nb);
         fal(&B.gana, B.sa * B.nb);
         fal(&B.hana, B.sh * B.nb);
         // LPT over (instance, m) items; costs L + 2 - m; instances interleaved so

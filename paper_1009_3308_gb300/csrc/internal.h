@@ -266,12 +266,9 @@ struct sphnse_plan {
     sph::DigState dig;
 
     // workspaces (sized for the largest field counts: 5 synthesis, 3 analysis)
-    void* d_bsyn = nullptr;      // [n_ext][2 * 5] (re, im) per field, FP32
     void* d_gsyn = nullptr;      // [5][N+1][nlat] complex (m-major)
     void* d_gana = nullptr;      // [3][N+1][nlat] complex (m-major)
     void* d_hana = nullptr;      // [n_ext][2 * 3]
-    void* d_gsyn_r = nullptr;    // FP32 latitude-major copies for the general ring kernel: [5][nlat][N+1]
-    void* d_gana_r = nullptr;    //                                             [3][nlat][N+1]
     double* d_work = nullptr;    // NDF / adjoint vectors (16 x n_coeff complex)
     double* d_grid = nullptr;    // objective: two grid fields (allocated on first use)
     double* d_theta = nullptr;
@@ -327,10 +324,12 @@ namespace sph {
 // ---- launchers (kernels in *.cu) ------------------------------------------
 enum RingMode { RING_RHS = 0, RING_GRID = 1, RING_PROJECT = 2, RING_ADJOINT = 3 };
 
-// FP32 prep: coefficient sets for synthesis.  nsets fields from alpha (3: zeta,
-// theta, phi) and optionally 2 more (theta, phi) from beta scaled by 1/s_m.
-int launch_prep(sphnse_plan* P, const double* alpha, const double* beta);
-int launch_synthesis(sphnse_plan* P, int nfields);   // FP32, order-major
+// FP32 synthesis (coefficient sets built in the kernel; beta: the adjoint's
+// fields 3, 4) and analysis
+int launch_synthesis32(sphnse_plan* P, const double* alpha, const double* beta, int pairs);
+bool ana32_ok(const sphnse_plan* P);
+int launch_analysis32(sphnse_plan* P, int nf);
+int launch_analysis_stream(sphnse_plan* P);   // two fields, FP32, streaming
 int launch_ring(sphnse_plan* P, int mode, const double* gin0, const double* gin1,
                 double* gout0, double* gout1, double* gout2);
 int launch_analysis(sphnse_plan* P, int nfields);
@@ -343,8 +342,6 @@ int launch_analysis_dig(sphnse_plan* P, int nf);
 std::vector<int> ring_fx_twiddles(int nlon);
 int launch_ring_fx(sphnse_plan* P, int mode, const double* gin0, const double* gin1, double* gout0, double* gout1,
                    double* gout2);
-// in [nf][R][Cn] -> out [nf][Cn][R] (complex FP32 entries)
-int launch_transpose(sphnse_plan* P, const void* in, void* out, int R, int Cn, int nf);
 // finish: kind 0 = RHS (F = f - nu lam alpha - N), 1 = projection (N),
 // 2 = adjoint (out = -nu lam w - s_m (N_X + lam^{1/2} H_rho))
 int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha,
@@ -352,7 +349,6 @@ int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha,
 
 int ensure_tables(sphnse_plan* P, int prec);
 bool stream_ok(const sphnse_plan* P);
-int launch_synthesis_stream(sphnse_plan* P, int nfields);
 bool tc_supported(const sphnse_plan* P);
 int launch_analysis_tc(sphnse_plan* P, int nfields);
 // the RHS's analysis (two product fields) with the recombination and update
@@ -394,7 +390,6 @@ int launch_finish32_batch(sphnse_plan* P, int nb, const float* hana, size_t hstr
                           double* out, const double* nu_inst);
 void tc_free(sphnse_plan* P);
 void host_io_free(sphnse_plan* P);
-int launch_analysis_stream(sphnse_plan* P, int nfields);
 void stage_begin(sphnse_plan* P, int stage);
 void stage_end(sphnse_plan* P, int stage);
 int check_cuda(cudaError_t e);

@@ -1,14 +1,12 @@
 // Spectral-side kernels of the RHS F (Eq. (ode)) on CUDA cores:
-//   prep       coefficient sets for synthesis (Eqs. (stok_eig), (vort_app))
-//   synthesis  per-order Legendre sums over the northern nodes, even/odd
-//              split (north = E + O, south = E - O)
+//   prep32     coefficient sets of the FP32 ensembles' synthesis (Eqs.
+//              (stok_eig), (vort_app))
 //   analysis   per-order Legendre sums of the quadrature-weighted Fourier
-//              profiles (Eq. (disc_vec_orth_proj))
+//              profiles (Eq. (disc_vec_orth_proj)), FP32, for numbers of
+//              northern latitudes that legendre_f32.cu does not take
 //   finish     degree-shift recombination and the diagonal Stokes update
 //              (Sec. 4.2: nu lambda_L alpha_{L,m}) plus forcing.
-// Prep, synthesis and analysis serve the FP32 path (the FP64 sums are in
-// legendre_dig.cu), the finish both; the coefficient state in and out is
-// always FP64.
+// The coefficient state in and out is always FP64.
 #include <cuda_runtime.h>
 
 #include "finish.cuh"
@@ -74,73 +72,6 @@ __global__ void __launch_bounds__(128) k_prep32(const double2* __restrict__ alph
         out[7] = c.y * b0.y;
         out[8] = fmaf(c.z, bm.x, c.w * bp.x);
         out[9] = fmaf(c.z, bm.y, c.w * bp.y);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// synthesis: block (p-tile, m); thread = one northern node p.
-//   g_f(theta_p) = sum_K Pt_K^m(x_p) b_{f,K}: even rows E, odd rows O;
-//   north row p: E + O, south row nlat-1-p: E - O.
-// Field scalings: theta fields (i m / sin), phi fields (-1 / sin), zeta none.
-// Output gsyn[f][row][m] complex.
-template <typename T, int NF>
-__global__ void __launch_bounds__(128) k_synthesis(const T* __restrict__ psyn, const T* __restrict__ bsyn,
-                                                    T* __restrict__ gsyn, const double* __restrict__ sinth,
-                                                    int N, int nh, int nlat) {
-    pdl_launch();
-    pdl_wait();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* B = reinterpret_cast<T*>(smem_raw);
-    const int m = blockIdx.y;
-    const int e0 = ext_off(N, m), cnt = ext_count(N, m), ne = ext_even(N, m), no = ext_odd(N, m);
-    for (int i = threadIdx.x; i < cnt * 2 * NF; i += blockDim.x) B[i] = bsyn[size_t(e0) * 2 * NF + i];
-    __syncthreads();
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= nh) return;
-    T ev[2 * NF], od[2 * NF];
-#pragma unroll
-    for (int f = 0; f < 2 * NF; ++f) { ev[f] = T(0); od[f] = T(0); }
-    const T* Pe = psyn + size_t(e0) * nh + p;
-#pragma unroll 4
-    for (int j = 0; j < ne; ++j) {
-        const T pv = __ldg(Pe + size_t(j) * nh);
-        const T* b = B + j * 2 * NF;
-#pragma unroll
-        for (int f = 0; f < 2 * NF; ++f) ev[f] = fma(pv, b[f], ev[f]);
-    }
-    const T* Po = psyn + size_t(e0 + ne) * nh + p;
-#pragma unroll 4
-    for (int j = 0; j < no; ++j) {
-        const T pv = __ldg(Po + size_t(j) * nh);
-        const T* b = B + (ne + j) * 2 * NF;
-#pragma unroll
-        for (int f = 0; f < 2 * NF; ++f) od[f] = fma(pv, b[f], od[f]);
-    }
-    const T inv_s = T(1.0 / sinth[p]);
-    const T mm = T(m);
-#pragma unroll
-    for (int hemi = 0; hemi < 2; ++hemi) {
-        const int row = hemi == 0 ? p : nlat - 1 - p;
-        if (hemi == 1 && row == p) break;  // equator of an odd grid
-        const T sg = hemi == 0 ? T(1) : T(-1);
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-            T gr = ev[2 * f] + sg * od[2 * f];
-            T gi = ev[2 * f + 1] + sg * od[2 * f + 1];
-            T outr, outi;
-            if (f == 0) {
-                outr = gr; outi = gi;
-            } else if (f == 1 || f == 3) {  // (i m / sin) g
-                outr = -mm * gi * inv_s;
-                outi = mm * gr * inv_s;
-            } else {                         // -(1 / sin) g
-                outr = -gr * inv_s;
-                outi = -gi * inv_s;
-            }
-            T* dst = gsyn + gsyn_index(0, f, m, row, N, nlat) * 2;
-            dst[0] = outr;
-            dst[1] = outi;
-        }
     }
 }
 
@@ -307,40 +238,6 @@ __global__ void k_finish32(int kind, const float* __restrict__ hana, int nf, con
 // ---------------------------------------------------------------------------
 // launchers
 
-int launch_prep(sphnse_plan* P, const double* alpha, const double* beta) {
-    const int nf = beta ? 5 : 3;
-    dim3 blk(128), grd((P->N + 2 + 127) / 128, P->N + 1);
-    stage_begin(P, SPHNSE_STAGE_PREP);
-    launch_pdl(k_prep32, grd, blk, 0, P->stream, reinterpret_cast<const double2*>(alpha),
-               reinterpret_cast<const double2*>(beta), static_cast<const float4*>(P->d_prepc32),
-               reinterpret_cast<float*>(P->d_bsyn), P->N, nf, P->n_coeff, size_t(0));
-    stage_end(P, SPHNSE_STAGE_PREP);
-    return check_cuda(cudaGetLastError());
-}
-
-template <typename T, int NF>
-static int synth_t(sphnse_plan* P) {
-    dim3 blk(128), grd((P->nh + 127) / 128, P->N + 1);
-    size_t sm = size_t(P->N + 2) * 2 * NF * sizeof(T);
-    if (sm > 48 * 1024)
-        allow_dynamic_smem(reinterpret_cast<const void*>(k_synthesis<T, NF>), sm);
-    stage_begin(P, SPHNSE_STAGE_SYNTHESIS);
-    launch_pdl_small(P->n_cta, k_synthesis<T, NF>, grd, blk, sm, P->stream,
-               reinterpret_cast<const T*>(P->tab[SPHNSE_FP32].syn),
-               reinterpret_cast<const T*>(P->d_bsyn), reinterpret_cast<T*>(P->d_gsyn),
-               static_cast<const double*>(P->d_s), P->N, P->nh, P->nlat);
-    stage_end(P, SPHNSE_STAGE_SYNTHESIS);
-    return check_cuda(cudaGetLastError());
-}
-
-int launch_synthesis(sphnse_plan* P, int nfields) {
-    if (stream_ok(P)) {
-        int rc = launch_synthesis_stream(P, nfields);
-        if (rc != SPHNSE_E_UNSUPPORTED) return rc;
-    }
-    return nfields == 5 ? synth_t<float, 5>(P) : synth_t<float, 3>(P);
-}
-
 template <typename T, int NF>
 static int anal_t(sphnse_plan* P) {
     const int maxrows = ext_even(P->N, 0);
@@ -358,10 +255,7 @@ static int anal_t(sphnse_plan* P) {
 }
 
 int launch_analysis(sphnse_plan* P, int nfields) {
-    if (stream_ok(P)) {
-        int rc = launch_analysis_stream(P, nfields);
-        if (rc != SPHNSE_E_UNSUPPORTED) return rc;
-    }
+    if (ana32_ok(P)) return launch_analysis32(P, nfields);
     return nfields == 3 ? anal_t<float, 3>(P) : anal_t<float, 2>(P);
 }
 

@@ -1,4 +1,5 @@
-// Persistent streaming Legendre kernels (CUDA cores, FP32).
+// Persistent streaming Legendre kernels of the FP32 ensembles, and of single
+// analyses whose table exceeds L2 (CUDA cores).
 //
 // The per-order Legendre sums of the RHS (Sec. 4.2; synthesis of the fields
 // of Eq. (app_soln_rep) and (vort_app), analysis = the discrete projection of
@@ -366,52 +367,6 @@ static constexpr int half_rows() { return 8; }
 
 bool stream_ok(const sphnse_plan* P) { return P->d_items != nullptr && P->nh % 4 == 0 && P->nh >= 32; }
 
-template <typename T, int NF>
-static int syn_stream_t(sphnse_plan* P) {
-    constexpr int HR = half_rows<T>();
-    constexpr int V = Vec<T>::n;
-    const int tpg = ((P->nh / V + 31) / 32) * 32;
-    const int threads = 32 + 2 * tpg;
-    if (threads > 512) return SPHNSE_E_UNSUPPORTED;
-    constexpr int NST = nst<T>();
-    const size_t sm = 128 + sizeof(T) * (size_t(NST) * 2 * HR * P->nh + size_t(2) * (P->N + 2) * 2 * NF +
-                                         size_t(P->nh) * 2 * NF);
-    if (sm > 227 * 1024) return SPHNSE_E_UNSUPPORTED;
-    allow_dynamic_smem(reinterpret_cast<const void*>(k_syn_stream<T, NF, HR>), sm);
-    StreamArgs a{P->tab[SPHNSE_FP32].syn, P->d_bsyn, P->d_gsyn, nullptr, nullptr,
-                 P->d_s, P->d_items, P->d_item_off, P->d_status, P->N, P->nh, P->nlat, 0, 0, 0, 0, 0};
-    stage_begin(P, SPHNSE_STAGE_SYNTHESIS);
-    launch_pdl(k_syn_stream<T, NF, HR>, dim3(P->n_cta), dim3(threads), sm, P->stream, a);
-    stage_end(P, SPHNSE_STAGE_SYNTHESIS);
-    return check_cuda(cudaGetLastError());
-}
-
-template <typename T, int NF>
-static int ana_stream_t(sphnse_plan* P) {
-    constexpr int HR = half_rows<T>();
-    constexpr int QPS = 2 * HR / 4;
-    constexpr int NTEAM = 8 / QPS;
-    const int threads = 32 + 32 * QPS * NTEAM;
-    constexpr int NST = nst<T>();
-    const size_t sm = 128 + sizeof(T) * (size_t(NST) * 2 * HR * P->nh + size_t(2) * 2 * P->nh * 2 * NF);
-    if (sm > 227 * 1024) return SPHNSE_E_UNSUPPORTED;
-    allow_dynamic_smem(reinterpret_cast<const void*>(k_ana_stream<T, NF, HR, NTEAM>), sm);
-    StreamArgs a{P->tab[SPHNSE_FP32].syn, nullptr, nullptr, P->d_gana, P->d_hana,
-                 P->d_s, P->d_items, P->d_item_off, P->d_status, P->N, P->nh, P->nlat, 0, 0, 0, 0, 0};
-    stage_begin(P, SPHNSE_STAGE_ANALYSIS);
-    launch_pdl(k_ana_stream<T, NF, HR, NTEAM>, dim3(P->n_cta), dim3(threads), sm, P->stream, a);
-    stage_end(P, SPHNSE_STAGE_ANALYSIS);
-    return check_cuda(cudaGetLastError());
-}
-
-int launch_synthesis_stream(sphnse_plan* P, int nfields) {
-    return nfields == 5 ? syn_stream_t<float, 5>(P) : syn_stream_t<float, 3>(P);
-}
-
-int launch_analysis_stream(sphnse_plan* P, int nfields) {
-    return nfields == 3 ? ana_stream_t<float, 3>(P) : ana_stream_t<float, 2>(P);
-}
-
 // FP32 batched streaming passes over instances (items = inst * (N+1) + m)
 int launch_synthesis_stream_batch(sphnse_plan* P, const int* items, const int* item_off, int ncta,
                                   const float* bsyn, size_t sb, float* gsyn, size_t sg, int pairs) {
@@ -429,6 +384,11 @@ int launch_synthesis_stream_batch(sphnse_plan* P, const int* items, const int* i
     launch_pdl(k_syn_stream<float, 3, HR>, dim3(ncta), dim3(threads), sm, P->stream, a);
     stage_end(P, SPHNSE_STAGE_SYNTHESIS);
     return check_cuda(cudaGetLastError());
+}
+
+int launch_analysis_stream(sphnse_plan* P) {
+    return launch_analysis_stream_batch(P, P->d_items, P->d_item_off, P->n_cta, static_cast<const float*>(P->d_gana), 0,
+                                        static_cast<float*>(P->d_hana), 0);
 }
 
 int launch_analysis_stream_batch(sphnse_plan* P, const int* items, const int* item_off, int ncta,

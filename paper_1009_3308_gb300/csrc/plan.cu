@@ -162,25 +162,15 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
         return launch_finish(P, 0, prec, alpha, forcing, out);
     }
     const bool ring4 = ring4_ok(P);
-    // the tensor-core synthesis writes the latitude-pair-major layout the
-    // four-step ring kernel reads contiguously (its epilogue warps are off the
-    // streaming path); the FP32 streaming synthesis keeps the order-major one
-    const int pairs = ring4 && tc;
-    if (tc) {
-        if ((rc = launch_synthesis_tc(P, alpha, pairs))) return rc;   // builds its coefficient tiles
-    } else {
-        if ((rc = launch_prep(P, alpha, nullptr))) return rc;
-        if ((rc = launch_synthesis(P, 3))) return rc;
-    }
-    if (ring4) {
-        if ((rc = launch_ring4(P, 1, static_cast<const float*>(P->d_gsyn), 0, static_cast<float*>(P->d_gana), 0,
-                               pairs)))
-            return rc;
-    } else {
-        if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 3))) return rc;
-        if ((rc = launch_ring(P, RING_RHS, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-        if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 2))) return rc;
-    }
+    // the tensor-core synthesis (its epilogue warps are off the streaming path)
+    // writes the latitude-pair-major layout that the ring kernels read
+    // contiguously; the FP32 one the order-major layout, where the four-step
+    // ring kernel takes it
+    const int pairs = tc || !ring4;
+    if ((rc = tc ? launch_synthesis_tc(P, alpha, pairs) : launch_synthesis32(P, alpha, nullptr, pairs))) return rc;
+    if ((rc = ring4 ? launch_ring4(P, 1, static_cast<const float*>(P->d_gsyn), 0, static_cast<float*>(P->d_gana), 0, pairs)
+                    : launch_ring(P, RING_RHS, nullptr, nullptr, nullptr, nullptr, nullptr)))
+        return rc;
     if (tc) {
         // the finish step runs in the analysis epilogue where its shared
         // memory fits
@@ -203,11 +193,8 @@ int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, dou
         if ((rc = launch_analysis_dig(P, 3))) return rc;
         return launch_finish(P, 2, prec, w, nullptr, out);
     }
-    if ((rc = launch_prep(P, alpha, w))) return rc;
-    if ((rc = launch_synthesis(P, 5))) return rc;
-    if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 5))) return rc;
+    if ((rc = launch_synthesis32(P, alpha, w, 1))) return rc;
     if ((rc = launch_ring(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-    if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 3))) return rc;
     if ((rc = launch_analysis(P, 3))) return rc;
     return launch_finish(P, 2, prec, w, nullptr, out);
 }
@@ -236,8 +223,8 @@ static void destroy_plan(sphnse_plan* P) {
     if (P->d_info) cudaFree(P->d_info);
     if (P->h_info) cudaFreeHost(P->h_info);
     void* ptrs[] = {P->d_items, P->d_item_off, P->d_status,
-                    P->d_x, P->d_s, P->d_isin32, P->d_rw, P->d_tw32, P->d_ftw, P->d_fxtw, P->d_lm, P->d_finc, P->d_prepc, P->d_finc32, P->d_prepc32, P->d_bsyn,
-                    P->d_gsyn, P->d_gana, P->d_hana, P->d_gsyn_r, P->d_gana_r, P->d_grid, P->d_theta, P->d_w, P->d_work, P->d_tmp, P->d_norms};
+                    P->d_x, P->d_s, P->d_isin32, P->d_rw, P->d_tw32, P->d_ftw, P->d_fxtw, P->d_lm, P->d_finc, P->d_prepc, P->d_finc32, P->d_prepc32,
+                    P->d_gsyn, P->d_gana, P->d_hana, P->d_grid, P->d_theta, P->d_w, P->d_work, P->d_tmp, P->d_norms};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (P->h_norms) cudaFreeHost(P->h_norms);
@@ -364,12 +351,9 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
     if (!rc) rc = dalloc(&P->d_prepc, size_t(P->n_ext) * sizeof(double4_32a));
     if (!rc) rc = dalloc(&P->d_finc32, nc * sizeof(float4));
     if (!rc) rc = dalloc(&P->d_prepc32, size_t(P->n_ext) * sizeof(float4));
-    if (!rc) rc = dalloc(&P->d_bsyn, size_t(P->n_ext) * 10 * sizeof(float));
     if (!rc) rc = dalloc(&P->d_gsyn, 5 * sz_g);
     if (!rc) rc = dalloc(&P->d_gana, 3 * sz_g);
     if (!rc) rc = dalloc(&P->d_hana, size_t(P->n_ext) * 6 * sizeof(double));
-    if (!rc) rc = dalloc(&P->d_gsyn_r, 5 * sz_g / 2);   // FP32 only
-    if (!rc) rc = dalloc(&P->d_gana_r, 3 * sz_g / 2);
     if (!rc) rc = dalloc(&P->d_work, 16 * nc * 2 * sizeof(double));
     if (!rc) rc = dalloc(&P->d_tmp, 2 * nc * 2 * sizeof(double));
     if (!rc) rc = dalloc(&P->d_norms, 16 * sizeof(unsigned long long));
@@ -532,13 +516,7 @@ int sphnse_grid_fields(sphnse_plan* P, const double* alpha, double* zeta, double
         if ((rc = launch_synthesis_dig(P, alpha, nullptr))) return rc;
         return launch_ring_fx(P, RING_GRID, nullptr, nullptr, zeta, uth, uph);
     }
-    if (tc) {
-        if ((rc = launch_synthesis_tc(P, alpha, 0))) return rc;
-    } else {
-        if ((rc = launch_prep(P, alpha, nullptr))) return rc;
-        if ((rc = launch_synthesis(P, 3))) return rc;
-    }
-    if ((rc = launch_transpose(P, P->d_gsyn, P->d_gsyn_r, P->N + 1, P->nlat, 3))) return rc;
+    if ((rc = tc ? launch_synthesis_tc(P, alpha, 1) : launch_synthesis32(P, alpha, nullptr, 1))) return rc;
     return launch_ring(P, RING_GRID, nullptr, nullptr, zeta, uth, uph);
 }
 
@@ -552,7 +530,6 @@ int sphnse_project(sphnse_plan* P, const double* vth, const double* vph, double*
         return launch_finish(P, 1, prec, nullptr, nullptr, out);
     }
     if ((rc = launch_ring(P, RING_PROJECT, vth, vph, nullptr, nullptr, nullptr))) return rc;
-    if ((rc = launch_transpose(P, P->d_gana_r, P->d_gana, P->nlat, P->N + 1, 2))) return rc;
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);
     if ((rc = tc ? launch_analysis_tc(P, 2) : launch_analysis(P, 2))) return rc;
     return launch_finish(P, 1, prec, nullptr, nullptr, out);

@@ -1,5 +1,10 @@
 // Longitude ("ring") kernels of the FP32 and BF16x3 paths (the FP64 path's
-// kernel is in ring_fx.cu).  General kernel: one CTA per Gauss latitude theta_p.
+// kernel is in ring_fx.cu).  General kernel: one CTA per pair of Gauss
+// latitudes, half of its threads per ring.  It reads the latitude-pair-major
+// spectra [f][row / 2][m][row % 2] (a CTA's data are contiguous) and writes the
+// order-major ones of the analysis (16 bytes, two latitudes, at a time), so it
+// needs no transposes.  With one latitude per CTA and a transpose kernel on
+// either side the adjoint's ring took 22.5 + 13.5 us at L = 255 (event pairs).
 //
 // RHS mode (Sec. 4.2: the phi sums of Eqs. (app_soln_rep), (eval_nonlin1)
 // are Fourier sums, evaluated by FFT):
@@ -35,16 +40,18 @@ namespace sph {
 // registers, the block synchronises, then writes them to their autosorted
 // positions.  Ns = product of the earlier radices; nsh = log2(Ns) when Ns is
 // a power of two (radix-3 stages run last, so this holds unless M has 3^2).
-// The launch uses blockDim >= M/6, so a thread owns at most MAXB butterflies.
+// A ring's nt threads (rt = 0 .. nt-1) are at least M/6, so a thread owns at
+// most MAXB butterflies.
 template <typename T, typename TW, int R, int NSIG>
-__device__ __forceinline__ void stage(cx<T>* const* buf, int M, int Ns, int nsh, const TW* tw, int sign) {
+__device__ __forceinline__ void stage(cx<T>* const* buf, int M, int Ns, int nsh, const TW* tw, int sign, int rt,
+                                      int nt) {
     constexpr int MAXB = R == 2 ? 3 : (R == 8 ? 1 : 2);
     const int nb = M / R;
     const int twstride = M / (Ns * R);
     cx<T> v[NSIG][MAXB][R];
 #pragma unroll
     for (int b = 0; b < MAXB; ++b) {
-        const int j = threadIdx.x + b * blockDim.x;
+        const int j = rt + b * nt;
         if (j < nb) {
             const int k = nsh >= 0 ? (j & (Ns - 1)) : (j % Ns);
             cx<T> w[R];
@@ -64,7 +71,7 @@ __device__ __forceinline__ void stage(cx<T>* const* buf, int M, int Ns, int nsh,
     __syncthreads();
 #pragma unroll
     for (int b = 0; b < MAXB; ++b) {
-        const int j = threadIdx.x + b * blockDim.x;
+        const int j = rt + b * nt;
         if (j < nb) {
             const int k = nsh >= 0 ? (j & (Ns - 1)) : (j % Ns);
             const int q = nsh >= 0 ? (j >> nsh) : (j / Ns);
@@ -80,16 +87,16 @@ __device__ __forceinline__ void stage(cx<T>* const* buf, int M, int Ns, int nsh,
 
 // Full M-point transform (sign -1 forward, +1 inverse) of NSIG signals in place.
 template <typename T, typename TW, int NSIG>
-__device__ void fft(cx<T>* const* buf, const FFTPlan& plan, const TW* tw, int sign) {
+__device__ void fft(cx<T>* const* buf, const FFTPlan& plan, const TW* tw, int sign, int rt, int nt) {
     const int M = plan.n;
     int Ns = 1;
     for (int st = 0; st < plan.nstages; ++st) {
         const int R = plan.radix[st];
         const int nsh = (Ns & (Ns - 1)) == 0 ? __ffs(Ns) - 1 : -1;
-        if (R == 8) stage<T, TW, 8, NSIG>(buf, M, Ns, nsh, tw, sign);
-        else if (R == 4) stage<T, TW, 4, NSIG>(buf, M, Ns, nsh, tw, sign);
-        else if (R == 2) stage<T, TW, 2, NSIG>(buf, M, Ns, nsh, tw, sign);
-        else stage<T, TW, 3, NSIG>(buf, M, Ns, nsh, tw, sign);
+        if (R == 8) stage<T, TW, 8, NSIG>(buf, M, Ns, nsh, tw, sign, rt, nt);
+        else if (R == 4) stage<T, TW, 4, NSIG>(buf, M, Ns, nsh, tw, sign, rt, nt);
+        else if (R == 2) stage<T, TW, 2, NSIG>(buf, M, Ns, nsh, tw, sign, rt, nt);
+        else stage<T, TW, 3, NSIG>(buf, M, Ns, nsh, tw, sign, rt, nt);
         Ns *= R;
     }
 }
@@ -100,65 +107,75 @@ struct RingArgs {
     const double* x;       // cos(theta)
     const double* s;       // sin(theta)
     const double* rw;      // (2 pi / M) w_p / sin(theta_p)
-    const void* gsyn;      // [nf][nlat][N+1] complex T (row-major)
-    void* gana;            // [nf][nlat][N+1] complex T (row-major)
+    const void* gsyn;      // [nf][pair][N+1][2] complex T
+    void* gana;            // [nf][N+1][nlat] complex T
     const double* gin0;    // grid input rows (PROJECT)
     const double* gin1;
     double* gout0;         // grid output rows (GRID)
     double* gout1;
     double* gout2;
     size_t sgs, sga;       // per-instance strides (complex entries) along gridDim.y
+    int early;             // a grid of one wave: the successor may start its prologue at once
 };
 
 template <typename T, typename TW, int MODE>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_ring(RingArgs a, FFTPlan plan, const TW* __restrict__ tw) {
-    pdl_launch();
-    pdl_wait();
+__global__ void __launch_bounds__(512) k_ring(RingArgs a, FFTPlan plan, const TW* __restrict__ tw) {
+    if (a.early) pdl_launch();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int NBUF = MODE == RING_ADJOINT ? 3 : (MODE == RING_PROJECT ? 1 : 2);
-    cx<T>* buf = reinterpret_cast<cx<T>*>(smem_raw);
+    cx<T>* buf = reinterpret_cast<cx<T>*>(smem_raw);   // [2 rings][NBUF][M]
     // the twiddle table e^{-2 pi i t / M} lives in shared memory after the buffers
-    T* tws = reinterpret_cast<T*>(buf + NBUF * a.M);
+    T* tws = reinterpret_cast<T*>(buf + 2 * NBUF * a.M);
     for (int t = threadIdx.x; t < 2 * a.M; t += blockDim.x) tws[t] = T(tw[t]);
-    const int row = blockIdx.x;
-    const int M = a.M, N = a.N, nlat = a.nlat;
+    const int M = a.M, N = a.N, nlat = a.nlat, pair = blockIdx.x, npair = (nlat + 1) / 2;
+    const int nt = blockDim.x / 2, h = threadIdx.x / nt, rt = threadIdx.x % nt;
+    const int row = 2 * pair + h;                      // this half's ring (h = 1 of an odd grid's last pair: none)
+    const bool two = 2 * pair + 1 < nlat, live = row < nlat;
     const size_t ld = size_t(N + 1);
     const cx<T>* gs = reinterpret_cast<const cx<T>*>(a.gsyn) + size_t(blockIdx.y) * a.sgs;
     cx<T>* ga = reinterpret_cast<cx<T>*>(a.gana) + size_t(blockIdx.y) * a.sga;
-    auto G = [&](int f, int m) -> cx<T> { return gs[(size_t(f) * nlat + row) * ld + m]; };
-
-    cx<T>* src[3] = {buf, buf + M, buf + 2 * M};
+    cx<T>* src[3] = {buf + h * NBUF * M, buf + (h * NBUF + 1) * M, buf + (h * NBUF + 2) * M};
+    pdl_wait();
 
     if constexpr (MODE != RING_PROJECT) {
         // Hermitian spectra of two real fields packed as a + i b:
         //   Z_m = g^a_m + i g^b_m (m <= N);  Z_{M-m} = conj(g^a_m) + i conj(g^b_m)
         const int nsig = MODE == RING_ADJOINT ? 3 : 2;
-        for (int m = threadIdx.x; m < M; m += blockDim.x) {
-            int mm = -1;
-            bool upper = false;
-            if (m <= N) mm = m;
-            else if (m >= M - N) { mm = M - m; upper = true; }
+        for (int m = threadIdx.x; m < M - N; m += blockDim.x) {
             for (int sgi = 0; sgi < nsig; ++sgi) {
                 // fields packed per signal: RHS/GRID (0,1),(2,-); ADJOINT (0,1),(2,3),(4,-)
                 const int fa = 2 * sgi, fb = 2 * sgi + 1;
                 const bool has_b = (MODE == RING_ADJOINT) ? fb <= 4 : fb <= 2;
-                cx<T> z{T(0), T(0)};
-                if (mm >= 0) {
-                    cx<T> ga_ = G(fa, mm);
-                    cx<T> gb_ = has_b ? G(fb, mm) : cx<T>{T(0), T(0)};
-                    if (mm == 0) { ga_.y = T(0); gb_.y = T(0); }
-                    if (!upper) z = {ga_.x - gb_.y, ga_.y + gb_.x};
-                    else        z = {ga_.x + gb_.y, gb_.x - ga_.y};
+                // order m of both rings
+                cx<T> A[2] = {{T(0), T(0)}, {T(0), T(0)}}, Bv[2] = {{T(0), T(0)}, {T(0), T(0)}};
+                if (m <= N) {
+                    const cx<T>* g = gs + ((size_t(fa) * npair + pair) * ld + m) * 2;
+                    const float4 v = *reinterpret_cast<const float4*>(g);
+                    A[0] = {v.x, v.y};
+                    if (two) A[1] = {v.z, v.w};
+                    if (has_b) {
+                        const float4 w = *reinterpret_cast<const float4*>(g + size_t(npair) * ld * 2);
+                        Bv[0] = {w.x, w.y};
+                        if (two) Bv[1] = {w.z, w.w};
+                    }
                 }
-                src[sgi][m] = z;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    cx<T> ga_ = A[r], gb_ = Bv[r];
+                    if (m == 0) { ga_.y = T(0); gb_.y = T(0); }
+                    cx<T>* z = buf + (r * NBUF + sgi) * M;
+                    z[m] = {ga_.x - gb_.y, ga_.y + gb_.x};
+                    if (m > 0 && m <= N) z[M - m] = {ga_.x + gb_.y, gb_.x - ga_.y};
+                }
             }
         }
         __syncthreads();
-        fft<T, T, MODE == RING_ADJOINT ? 3 : 2>(src, plan, tws, +1);
+        fft<T, T, MODE == RING_ADJOINT ? 3 : 2>(src, plan, tws, +1, rt, nt);
     }
 
     if constexpr (MODE == RING_GRID) {
-        for (int q = threadIdx.x; q < M; q += blockDim.x) {
+        if (!live) return;
+        for (int q = rt; q < M; q += nt) {
             if (a.gout0) a.gout0[size_t(row) * M + q] = double(src[0][q].x);
             if (a.gout1) a.gout1[size_t(row) * M + q] = double(src[0][q].y);
             if (a.gout2) a.gout2[size_t(row) * M + q] = double(src[1][q].x);
@@ -168,18 +185,18 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_ring(RingArgs a
 
     constexpr int nout = MODE == RING_ADJOINT ? 2 : 1;
     if constexpr (MODE == RING_RHS) {
-        const T fc = T(a.two_omega * a.x[row]);
-        for (int q = threadIdx.x; q < M; q += blockDim.x) {
+        const T fc = T(a.two_omega * a.x[min(row, nlat - 1)]);
+        for (int q = rt; q < M; q += nt) {
             const T zeta = src[0][q].x, uth = src[0][q].y, uph = src[1][q].x;
             const T qq = zeta + fc;
             src[0][q] = {-qq * uph, qq * uth};
         }
     } else if constexpr (MODE == RING_PROJECT) {
-        for (int q = threadIdx.x; q < M; q += blockDim.x)
-            src[0][q] = {T(a.gin0[size_t(row) * M + q]), T(a.gin1[size_t(row) * M + q])};
+        for (int q = rt; q < M; q += nt)
+            src[0][q] = live ? cx<T>{T(a.gin0[size_t(row) * M + q]), T(a.gin1[size_t(row) * M + q])} : cx<T>{T(0), T(0)};
     } else {  // RING_ADJOINT: fields zeta, u_th, u_ph, v_th, v_ph
-        const T fc = T(a.two_omega * a.x[row]);
-        for (int q = threadIdx.x; q < M; q += blockDim.x) {
+        const T fc = T(a.two_omega * a.x[min(row, nlat - 1)]);
+        for (int q = rt; q < M; q += nt) {
             const T zeta = src[0][q].x, uth = src[0][q].y;
             const T uph = src[1][q].x, vth = src[1][q].y, vph = src[2][q].x;
             const T qq = zeta + fc;
@@ -189,37 +206,61 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_ring(RingArgs a
         }
     }
     __syncthreads();
-    fft<T, T, nout>(src, plan, tws, -1);
+    fft<T, T, nout>(src, plan, tws, -1, rt, nt);
 
-    const T scale = T(a.rw[row]);
-    for (int m = threadIdx.x; m <= N; m += blockDim.x) {
-        const cx<T> p = src[0][m];
-        const cx<T> r = src[0][(M - m) % M];
-        // W = A + i B with A, B real fields: A_m = (Z_m + conj Z_{M-m}) / 2,
-        // B_m = (Z_m - conj Z_{M-m}) / (2 i)
-        cx<T> A{T(0.5) * (p.x + r.x), T(0.5) * (p.y - r.y)};
-        cx<T> B{T(0.5) * (p.y + r.y), T(0.5) * (r.x - p.x)};
-        ga[(size_t(0) * nlat + row) * ld + m] = {A.x * scale, A.y * scale};
-        ga[(size_t(1) * nlat + row) * ld + m] = {B.x * scale, B.y * scale};
-        if constexpr (nout == 2) {
-            // scalar field rho: plain quadrature weight (2 pi / M) w_p
-            const T sc2 = scale * T(a.s[row]);
-            const cx<T> z = src[1][m];
-            ga[(size_t(2) * nlat + row) * ld + m] = {z.x * sc2, z.y * sc2};
+    // both rings of order m at once: two latitudes are 16 bytes of the order-major output
+    const int row0 = 2 * pair;
+    T scale[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) scale[r] = T(a.rw[min(row0 + r, nlat - 1)]);
+    auto put = [&](int f, int m, const cx<T> (&v)[2]) {
+        cx<T>* d = ga + (size_t(f) * ld + m) * nlat + row0;
+        if (nlat % 2 == 0) {
+            *reinterpret_cast<float4*>(d) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+        } else {   // rows of an odd grid are 8-byte aligned
+            d[0] = v[0];
+            if (two) d[1] = v[1];
         }
+    };
+    for (int m = threadIdx.x; m <= N; m += blockDim.x) {
+        cx<T> oA[2], oB[2], oC[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const cx<T>* Z = buf + r * NBUF * M;
+            const cx<T> p = Z[m];
+            const cx<T> q = Z[(M - m) % M];
+            // W = A + i B with A, B real fields: A_m = (Z_m + conj Z_{M-m}) / 2,
+            // B_m = (Z_m - conj Z_{M-m}) / (2 i)
+            cx<T> A{T(0.5) * (p.x + q.x), T(0.5) * (p.y - q.y)};
+            cx<T> Bv{T(0.5) * (p.y + q.y), T(0.5) * (q.x - p.x)};
+            oA[r] = {A.x * scale[r], A.y * scale[r]};
+            oB[r] = {Bv.x * scale[r], Bv.y * scale[r]};
+            if constexpr (nout == 2) {
+                // scalar field rho: plain quadrature weight (2 pi / M) w_p
+                const T sc2 = scale[r] * T(a.s[min(row0 + r, nlat - 1)]);
+                const cx<T> z = Z[M + m];
+                oC[r] = {z.x * sc2, z.y * sc2};
+            }
+        }
+        put(0, m, oA);
+        put(1, m, oB);
+        if constexpr (nout == 2) put(2, m, oC);
     }
 }
 
 template <typename T, typename TW, int MODE>
-static void ring_t(sphnse_plan* P, const RingArgs& a, const TW* tw, int threads, int nb = 1) {
+static void ring_t(sphnse_plan* P, RingArgs a, const TW* tw, int nb = 1) {
     const int nbuf = MODE == RING_ADJOINT ? 3 : (MODE == RING_PROJECT ? 1 : 2);
-    const size_t sm = size_t(nbuf) * P->nlon * sizeof(cx<T>) + size_t(P->nlon) * 2 * sizeof(T);
+    // in-place stages need M / 6 threads per ring (at most 3 butterflies per thread)
+    const int threads = 2 * (((P->nlon / 6 + 31) / 32) * 32);
+    const size_t sm = size_t(2 * nbuf) * P->nlon * sizeof(cx<T>) + size_t(P->nlon) * 2 * sizeof(T);
     allow_dynamic_smem(reinterpret_cast<const void*>(k_ring<T, TW, MODE>), sm);
-    launch_pdl_small(P->n_cta, k_ring<T, TW, MODE>, dim3(P->nlat, nb), dim3(threads), sm, P->stream, a, P->fft, tw);
+    a.early = long(P->nlat + 1) / 2 * nb <= long(P->nsm) * (512 / threads);
+    launch_pdl(k_ring<T, TW, MODE>, dim3((P->nlat + 1) / 2, nb), dim3(threads), sm, P->stream, a, P->fft, tw);
 }
 
-// FP32 RHS ring pass over nb instances (latitude-major buffers with strides)
-int launch_ring_batch(sphnse_plan* P, int nb, const float* gsyn_r, size_t sgs, float* gana_r, size_t sga) {
+// FP32 RHS ring pass over nb instances (latitude-pair-major in, order-major out, with strides)
+int launch_ring_batch(sphnse_plan* P, int nb, const float* gsyn, size_t sgs, float* gana, size_t sga) {
     RingArgs a{};
     a.N = P->N;
     a.M = P->nlon;
@@ -229,25 +270,23 @@ int launch_ring_batch(sphnse_plan* P, int nb, const float* gsyn_r, size_t sgs, f
     a.x = P->d_x;
     a.s = P->d_s;
     a.rw = P->d_rw;
-    a.gsyn = gsyn_r;
-    a.gana = gana_r;
+    a.gsyn = gsyn;
+    a.gana = gana;
     a.sgs = sgs / 2;
     a.sga = sga / 2;
-    int threads = ((P->nlon / 6 + 31) / 32) * 32;
-    if (threads < 32) threads = 32;
     stage_begin(P, SPHNSE_STAGE_RING);
-    ring_t<float, float, RING_RHS>(P, a, P->d_tw32, threads, nb);
+    ring_t<float, float, RING_RHS>(P, a, P->d_tw32, nb);
     stage_end(P, SPHNSE_STAGE_RING);
     return check_cuda(cudaGetLastError());
 }
 
 template <typename T, typename TW>
-static void ring_mode(sphnse_plan* P, int mode, const RingArgs& a, const TW* tw, int threads) {
+static void ring_mode(sphnse_plan* P, int mode, const RingArgs& a, const TW* tw) {
     switch (mode) {
-        case RING_RHS: ring_t<T, TW, RING_RHS>(P, a, tw, threads); break;
-        case RING_GRID: ring_t<T, TW, RING_GRID>(P, a, tw, threads); break;
-        case RING_PROJECT: ring_t<T, TW, RING_PROJECT>(P, a, tw, threads); break;
-        default: ring_t<T, TW, RING_ADJOINT>(P, a, tw, threads); break;
+        case RING_RHS: ring_t<T, TW, RING_RHS>(P, a, tw); break;
+        case RING_GRID: ring_t<T, TW, RING_GRID>(P, a, tw); break;
+        case RING_PROJECT: ring_t<T, TW, RING_PROJECT>(P, a, tw); break;
+        default: ring_t<T, TW, RING_ADJOINT>(P, a, tw); break;
     }
 }
 
@@ -262,19 +301,16 @@ int launch_ring(sphnse_plan* P, int mode, const double* gin0, const double* gin1
     a.x = P->d_x;
     a.s = P->d_s;
     a.rw = P->d_rw;
-    a.gsyn = P->d_gsyn_r;
-    a.gana = P->d_gana_r;
+    a.gsyn = P->d_gsyn;
+    a.gana = P->d_gana;
     a.gin0 = gin0;
     a.gin1 = gin1;
     a.gout0 = gout0;
     a.gout1 = gout1;
     a.gout2 = gout2;
     a.sgs = a.sga = 0;
-    // in-place stages need blockDim >= M / 6 (at most 3 butterflies per thread)
-    int threads = ((P->nlon / 6 + 31) / 32) * 32;
-    if (threads < 32) threads = 32;
     stage_begin(P, SPHNSE_STAGE_RING);
-    ring_mode<float, float>(P, mode, a, P->d_tw32, threads);
+    ring_mode<float, float>(P, mode, a, P->d_tw32);
     stage_end(P, SPHNSE_STAGE_RING);
     return check_cuda(cudaGetLastError());
 }
@@ -385,42 +421,6 @@ int launch_ring4(sphnse_plan* P, int nb, const float* gsyn, size_t sgs, float* g
     }
     stage_end(P, SPHNSE_STAGE_RING);
     return rc;
-}
-
-// ---------------------------------------------------------------------------
-// Tiled transposes between the order-major layout of the Legendre kernels
-// ([f][m][row]) and the latitude-major layout of the ring kernel
-// ([f][row][m]); 32 x 32 complex tiles through shared memory, both sides
-// coalesced.
-
-template <typename C>
-__global__ void __launch_bounds__(256) k_transpose(const C* __restrict__ in, C* __restrict__ out, int R, int Cn) {
-    // no early trigger: several waves at large sizes (see k_prep)
-    pdl_wait();
-    __shared__ C tile[32][33];
-    const int f = blockIdx.z;
-    const C* src = in + size_t(f) * R * Cn;
-    C* dst = out + size_t(f) * R * Cn;
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += 8) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        if (r < R && c < Cn) tile[i][threadIdx.x] = src[size_t(r) * Cn + c];
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += 8) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (r < R && c < Cn) dst[size_t(c) * R + r] = tile[threadIdx.x][i];
-    }
-}
-
-// in: [nf][R][Cn] -> out: [nf][Cn][R]
-int launch_transpose(sphnse_plan* P, const void* in, void* out, int R, int Cn, int nf) {
-    dim3 blk(32, 8), grd((Cn + 31) / 32, (R + 31) / 32, nf);
-    stage_begin(P, SPHNSE_STAGE_TRANSPOSE);
-    launch_pdl_small(P->n_cta, k_transpose<float2>, grd, blk, 0, P->stream, reinterpret_cast<const float2*>(in),
-                   reinterpret_cast<float2*>(out), R, Cn);
-    stage_end(P, SPHNSE_STAGE_TRANSPOSE);
-    return check_cuda(cudaGetLastError());
 }
 
 }  // namespace sph
