@@ -160,10 +160,10 @@ struct DigSide {
 struct DigState {
     DigSide syn, ana;
     short4* eoff = nullptr;            // exponents of the coefficient sets per packed entry
-    double* isin = nullptr;            // 1 / sin(theta_p)
     int* emax = nullptr;               // [3][N+1] largest biased exponents of the ring output; zero
                                        // between calls (the finish kernel clears them)
-    bool ready = false;
+    void* arena = nullptr;             // the allocation of the exponents, pieces and constants
+    void* sched = nullptr;             // ... and of the item lists
 };
 
 // staging of sphnse_rhs_host: two slots, an upload and a download stream
@@ -250,6 +250,7 @@ struct sphnse_plan {
     double* d_x = nullptr;       // cos(theta_p), nlat
     double* d_s = nullptr;       // sin(theta_p), nlat
     float* d_isin32 = nullptr;   // 1 / sin(theta_p) rounded to FP32, nlat
+    double* d_isin = nullptr;    // 1 / sin(theta_p), nlat
     double* d_rw = nullptr;      // (2 pi / M) w_p / sin(theta_p), nlat
     float* d_tw32 = nullptr;     // e^{-2 pi i t / M}, M complex (FP32)
     int4* d_fxtw = nullptr;      // fixed-point twiddles of the FP64 ring kernel, M split Q62 pairs
@@ -338,6 +339,12 @@ int dig_setup(sphnse_plan* P, const double* d_tab);
 void dig_free(sphnse_plan* P);
 int launch_synthesis_dig(sphnse_plan* P, const double* alpha, const double* beta);
 int launch_analysis_dig(sphnse_plan* P, int nf);
+// FP64 sums of small plans (legendre_small.cu): per order, the analysis goes on
+// to the finish step (kind as in launch_finish)
+constexpr int SMALL_NH = 40;
+inline bool small_plan(int nh) { return nh <= SMALL_NH; }
+int launch_synthesis_small(sphnse_plan* P, const double* alpha, const double* beta);
+int launch_analysis_small(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out);
 // the FP64 ring kernel (64-bit fixed point) on the latitude-pair-major buffers
 std::vector<int> ring_fx_twiddles(int nlon);
 int launch_ring_fx(sphnse_plan* P, int mode, const double* gin0, const double* gin1, double* gout0, double* gout1,

@@ -44,6 +44,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "fx64.cuh"
@@ -620,7 +622,8 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
 // LPT over one CTA per SM, CTA lists at a fixed stride.  rem (synthesis): the
 // remainder blocks of the lowest orders' first steps; their items become the
 // first step, its remainder and the later steps, one after the other.
-static int dig_schedule(sphnse_plan* P, const std::vector<int4>& items, const int* rem, int ntile, DigSide* D) {
+static void dig_schedule(sphnse_plan* P, const std::vector<int4>& items, const int* rem, int ntile, DigSide* D,
+                         std::vector<int4>& flat, std::vector<int>& cnt) {
     std::vector<int> order(items.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = int(i);
     // an item costs its steps plus about one for its epilogue and start
@@ -652,42 +655,41 @@ static int dig_schedule(sphnse_plan* P, const std::vector<int4>& items, const in
     D->ncta = nc;
     D->istride = 1;
     for (auto& b : bins) D->istride = std::max(D->istride, int(b.size()));
-    std::vector<int4> flat(size_t(nc) * D->istride, make_int4(0, 0, 0, 0));
-    std::vector<int> cnt(nc);
+    flat.assign(size_t(nc) * D->istride, make_int4(0, 0, 0, 0));
+    cnt.resize(nc);
     for (int c = 0; c < nc; ++c) {
         cnt[c] = int(bins[c].size());
         std::copy(bins[c].begin(), bins[c].end(), flat.begin() + size_t(c) * D->istride);
     }
-    if (cudaMalloc(reinterpret_cast<void**>(&D->items), flat.size() * sizeof(int4)) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(&D->cnt), cnt.size() * sizeof(int)) != cudaSuccess)
-        return SPHNSE_E_NOMEM;
-    if (cudaMemcpy(D->items, flat.data(), flat.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(D->cnt, cnt.data(), cnt.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
-        return SPHNSE_E_CUDA;
-    return SPHNSE_OK;
 }
 
 void dig_free(sphnse_plan* P) {
-    for (DigSide* D : {&P->dig.syn, &P->dig.ana}) {
-        for (void* q : {static_cast<void*>(D->blocks), static_cast<void*>(D->ea), static_cast<void*>(D->items),
-                        static_cast<void*>(D->cnt), static_cast<void*>(D->pieces)})
-            if (q) cudaFree(q);
-        *D = DigSide();
-    }
-    if (P->dig.eoff) cudaFree(P->dig.eoff);
-    if (P->dig.isin) cudaFree(P->dig.isin);
-    if (P->dig.emax) cudaFree(P->dig.emax);
+    for (void* q : {static_cast<void*>(P->dig.syn.blocks), P->dig.arena, P->dig.sched})
+        if (q) cudaFree(q);
     P->dig = DigState();
 }
+
+// parts of one device allocation, 256-byte aligned, with a host image
+struct DigArena {
+    std::vector<unsigned char> host;
+    template <typename T>
+    size_t add(const T* src, size_t n) {   // src null: zeros
+        const size_t o = (host.size() + 255) / 256 * 256;
+        host.resize(o + n * sizeof(T), 0);
+        if (src && n) std::memcpy(host.data() + o, src, n * sizeof(T));
+        return o;
+    }
+    int upload(void** d) const {
+        if (cudaMalloc(d, host.size()) != cudaSuccess) return SPHNSE_E_NOMEM;
+        return cudaMemcpy(*d, host.data(), host.size(), cudaMemcpyHostToDevice) == cudaSuccess ? SPHNSE_OK : SPHNSE_E_CUDA;
+    }
+};
 
 // Digits, schedules and constants, from the FP64 table [n_ext][nh] on the
 // device (which the digits replace).
 int dig_setup(sphnse_plan* P, const double* d_tab) {
     const int N = P->N, nh = P->nh, ntile = (nh + 63) / 64;
     DigState& T = P->dig;
-    auto alloc = [](auto** p, size_t n) { return cudaMalloc(reinterpret_cast<void**>(p), n * sizeof(**p)) == cudaSuccess; };
-    auto up = [](void* d, const void* h, size_t b) { return cudaMemcpy(d, h, b, cudaMemcpyHostToDevice) == cudaSuccess; };
-
     // synthesis tiles (m, 64 latitudes), steps of 16 degrees of each parity
     const int nseg = std::min(DG_SEGM, N + 1);
     std::vector<int> base(size_t(N + 1 + nseg) * ntile);
@@ -708,55 +710,51 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
     while (pieces.size() % 4) pieces.push_back(make_int4(0, 0, 0, 0));
     const int atile = int(pieces.size() / 4), aks = (nh + 15) / 16, ablk = atile * aks;
 
-    int *d_base = nullptr, *d_used = nullptr;
-    int rc = SPHNSE_OK;
-    if (!alloc(&T.syn.blocks, size_t(nblk) * DG_ABYTES) || !alloc(&T.ana.blocks, size_t(ablk) * DG_ABYTES) ||
-        !alloc(&T.syn.ea, size_t(N + 1 + DG_SEGM) * nh) || !alloc(&T.ana.ea, size_t(P->n_ext)) ||
-        !alloc(&T.ana.pieces, pieces.size()) || !alloc(&d_base, base.size()) || !alloc(&d_used, size_t(nblk + ablk)) ||
-        !alloc(&T.eoff, size_t(P->n_coeff)) || !alloc(&T.isin, size_t(P->nlat)) || !alloc(&T.emax, size_t(3) * (N + 1)))
-        rc = SPHNSE_E_NOMEM;
+    // exponents of the coefficient sets applied to alpha_{K,m}: zeta, theta, and the larger of
+    // alpha_K's two places in the degree-shift set
+    auto bexp = [](double v) { return v == 0.0 ? 0 : std::ilogb(v) + 1023; };
+    auto eps = [](int l, int m) {
+        return l <= m ? 0.0 : std::sqrt((double(l) * l - double(m) * m) / (4.0 * l * l - 1.0));
+    };
+    std::vector<short4> eoff(P->n_coeff);
+    for (int m = 0, i = 0; m <= N; ++m)
+        for (int l = (m > 0 ? m : 1); l <= N; ++l, ++i) {
+            const double sl = std::sqrt(double(l) * (l + 1.0));
+            // alpha_l enters row l + 1 with l eps_{l+1}, row l - 1 with (l + 1) eps_l; the sum of a
+            // row's two terms takes one more bit
+            const double dn = std::max(l * eps(l + 1, m), (l + 1) * eps(l, m)) / sl;
+            eoff[i] = make_short4(short(bexp(sl)), short(bexp(1.0 / sl)), short(bexp(dn) + 1), 0);
+        }
+    DigArena A;
+    const size_t o_eas = A.add<int>(nullptr, size_t(N + 1 + DG_SEGM) * nh), o_eaa = A.add<int>(nullptr, P->n_ext);
+    const size_t o_pc = A.add(pieces.data(), pieces.size()), o_base = A.add(base.data(), base.size());
+    const size_t o_eoff = A.add(eoff.data(), eoff.size()), o_emax = A.add<int>(nullptr, size_t(3) * (N + 1));
+    const size_t o_used = A.add<int>(nullptr, size_t(nblk) + ablk);
+    int rc = A.upload(&T.arena);
+    if (rc) return rc;
+    unsigned char* d = static_cast<unsigned char*>(T.arena);
+    T.syn.ea = reinterpret_cast<int*>(d + o_eas);
+    T.ana.ea = reinterpret_cast<int*>(d + o_eaa);
+    T.ana.pieces = reinterpret_cast<int4*>(d + o_pc);
+    T.eoff = reinterpret_cast<short4*>(d + o_eoff);
+    T.emax = reinterpret_cast<int*>(d + o_emax);
+    const int* d_base = reinterpret_cast<const int*>(d + o_base);
+    int* d_used = reinterpret_cast<int*>(d + o_used);
     T.syn.bytes = size_t(nblk) * DG_ABYTES;
     T.ana.bytes = size_t(ablk) * DG_ABYTES;
+    if (cudaMalloc(reinterpret_cast<void**>(&T.syn.blocks), T.syn.bytes + T.ana.bytes) != cudaSuccess)
+        return SPHNSE_E_NOMEM;
+    T.ana.blocks = T.syn.blocks + T.syn.bytes;
+    k_dig_syn_scale<<<dim3((nh + 127) / 128, N + 1), 128>>>(d_tab, T.syn.ea, N, nh);
+    k_dig_ana_scale<<<(P->n_ext + 3) / 4, 128>>>(d_tab, T.ana.ea, P->n_ext, nh);
+    k_dig_syn<<<dim3((ext_even(N, 0) + 15) / 16, ntile, N + 1), 256>>>(d_tab, T.syn.ea, d_base, T.syn.blocks, d_used, N,
+                                                                      nh, ntile, 0);
+    k_dig_syn<<<dim3(1, ntile, nseg), 256>>>(d_tab, T.syn.ea, d_base + size_t(N + 1) * ntile, T.syn.blocks, d_used, N, nh,
+                                             ntile, 1);
+    k_dig_ana<<<dim3(aks, atile), 256>>>(d_tab, T.ana.ea, T.ana.pieces, T.ana.blocks, d_used + nblk, nh);
     std::vector<int> used(size_t(nblk) + ablk);
-    if (!rc) {
-        // exponents of the coefficient sets applied to alpha_{K,m}: zeta, theta, and the larger of
-        // alpha_K's two places in the degree-shift set
-        auto bexp = [](double v) { return v == 0.0 ? 0 : std::ilogb(v) + 1023; };
-        std::vector<short4> eoff(P->n_coeff);
-        auto eps = [](int l, int m) {
-            return l <= m ? 0.0 : std::sqrt((double(l) * l - double(m) * m) / (4.0 * l * l - 1.0));
-        };
-        for (int m = 0, i = 0; m <= N; ++m)
-            for (int l = (m > 0 ? m : 1); l <= N; ++l, ++i) {
-                const double sl = std::sqrt(double(l) * (l + 1.0));
-                // alpha_l enters row l + 1 with l eps_{l+1}, row l - 1 with (l + 1) eps_l; the sum of a
-                // row's two terms takes one more bit
-                const double dn = std::max(l * eps(l + 1, m), (l + 1) * eps(l, m)) / sl;
-                eoff[i] = make_short4(short(bexp(sl)), short(bexp(1.0 / sl)), short(bexp(dn) + 1), 0);
-            }
-        std::vector<double> isin(P->nlat);
-        for (int p = 0; p < P->nlat; ++p) isin[p] = 1.0 / P->s[p];
-        if (!up(T.ana.pieces, pieces.data(), pieces.size() * sizeof(int4)) ||
-            !up(d_base, base.data(), base.size() * sizeof(int)) || !up(T.eoff, eoff.data(), eoff.size() * sizeof(short4)) ||
-            !up(T.isin, isin.data(), isin.size() * sizeof(double)) ||
-            cudaMemset(T.emax, 0, size_t(3) * (N + 1) * sizeof(int)) != cudaSuccess ||
-            cudaMemset(d_used, 0, used.size() * sizeof(int)) != cudaSuccess)
-            rc = SPHNSE_E_CUDA;
-    }
-    if (!rc) {
-        k_dig_syn_scale<<<dim3((nh + 127) / 128, N + 1), 128>>>(d_tab, T.syn.ea, N, nh);
-        k_dig_ana_scale<<<(P->n_ext + 3) / 4, 128>>>(d_tab, T.ana.ea, P->n_ext, nh);
-        k_dig_syn<<<dim3((ext_even(N, 0) + 15) / 16, ntile, N + 1), 256>>>(d_tab, T.syn.ea, d_base, T.syn.blocks, d_used,
-                                                                          N, nh, ntile, 0);
-        k_dig_syn<<<dim3(1, ntile, nseg), 256>>>(d_tab, T.syn.ea, d_base + size_t(N + 1) * ntile, T.syn.blocks, d_used,
-                                                 N, nh, ntile, 1);
-        k_dig_ana<<<dim3(aks, atile), 256>>>(d_tab, T.ana.ea, T.ana.pieces, T.ana.blocks, d_used + nblk, nh);
-        if (cudaMemcpy(used.data(), d_used, used.size() * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-            rc = SPHNSE_E_CUDA;
-    }
-    if (d_base) cudaFree(d_base);
-    if (d_used) cudaFree(d_used);
-    if (rc) return rc;
+    if (cudaMemcpy(used.data(), d_used, used.size() * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return SPHNSE_E_CUDA;
     // leading steps without a nonzero digit are skipped
     std::vector<int4> items;
     for (int m = 0; m <= N; ++m)
@@ -766,15 +764,25 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
             while (k0 < k1 && !used[size_t(b) + k0]) ++k0;
             items.push_back(make_int4(m, t, k0 | (k1 << 16), b));
         }
-    if ((rc = dig_schedule(P, items, base.data() + size_t(N + 1) * ntile, ntile, &T.syn))) return rc;
+    std::vector<int4> fs, fa;
+    std::vector<int> cs, ca;
+    dig_schedule(P, items, base.data() + size_t(N + 1) * ntile, ntile, &T.syn, fs, cs);
     items.clear();
     for (int t = 0; t < atile; ++t) {
         int k0 = 0;
         while (k0 < aks && !used[size_t(nblk) + size_t(t) * aks + k0]) ++k0;
         items.push_back(make_int4(t, 0, k0 | (aks << 16), t * aks));
     }
-    if ((rc = dig_schedule(P, items, nullptr, 0, &T.ana))) return rc;
-    T.ready = true;
+    dig_schedule(P, items, nullptr, 0, &T.ana, fa, ca);
+    DigArena Q;
+    const size_t o_fs = Q.add(fs.data(), fs.size()), o_fa = Q.add(fa.data(), fa.size());
+    const size_t o_cs = Q.add(cs.data(), cs.size()), o_ca = Q.add(ca.data(), ca.size());
+    if ((rc = Q.upload(&T.sched))) return rc;
+    d = static_cast<unsigned char*>(T.sched);
+    T.syn.items = reinterpret_cast<int4*>(d + o_fs);
+    T.ana.items = reinterpret_cast<int4*>(d + o_fa);
+    T.syn.cnt = reinterpret_cast<int*>(d + o_cs);
+    T.ana.cnt = reinterpret_cast<int*>(d + o_ca);
     return SPHNSE_OK;
 }
 
@@ -795,7 +803,7 @@ static DigArgs dig_args(sphnse_plan* P, const DigSide& D) {
     a.prepc = P->d_prepc;
     a.eoff = P->dig.eoff;
     a.gsyn = static_cast<double*>(P->d_gsyn);
-    a.isin = P->dig.isin;
+    a.isin = P->d_isin;
     a.pieces = P->dig.ana.pieces;
     a.gana = static_cast<const double*>(P->d_gana);
     a.emax = P->dig.emax;

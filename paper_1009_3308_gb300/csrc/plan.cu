@@ -104,15 +104,17 @@ int ensure_tables(sphnse_plan* P, int prec) {
     if (t.built) return SPHNSE_OK;
     int rc = SPHNSE_OK;
     if (prec == SPHNSE_FP64) {
-        // the digit blocks of the tensor-core sums replace the table
-        const size_t bytes = size_t(P->n_ext) * P->nh * sizeof(double);
-        double* d = nullptr;
-        if (cudaMalloc(reinterpret_cast<void**>(&d), bytes) != cudaSuccess) rc = SPHNSE_E_NOMEM;
-        else if (cudaMemcpy(d, P->psyn_host.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) rc = SPHNSE_E_CUDA;
-        if (rc == SPHNSE_OK) rc = dig_setup(P, d);
-        if (d) cudaFree(d);
-        if (rc == SPHNSE_OK) t.bytes = P->dig.syn.bytes + P->dig.ana.bytes;
-        else dig_free(P);
+        t.bytes = size_t(P->n_ext) * P->nh * sizeof(double);
+        if (cudaMalloc(&t.syn, t.bytes) != cudaSuccess) rc = SPHNSE_E_NOMEM;
+        else if (cudaMemcpy(t.syn, P->psyn_host.data(), t.bytes, cudaMemcpyHostToDevice) != cudaSuccess) rc = SPHNSE_E_CUDA;
+        if (rc == SPHNSE_OK && !small_plan(P->nh)) {
+            // the digit blocks of the tensor-core sums replace the table
+            rc = dig_setup(P, static_cast<const double*>(t.syn));
+            cudaFree(t.syn);
+            t.syn = nullptr;
+            if (rc == SPHNSE_OK) t.bytes = P->dig.syn.bytes + P->dig.ana.bytes;
+            else dig_free(P);
+        }
     } else if (prec == SPHNSE_FP32) {
         rc = upload_table<float>(P, t, [](double v, bool) { return float(v); }, false, true);
     } else {
@@ -151,15 +153,26 @@ void prefer_max_smem(const void* kernel) {
         cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
 }
 
+// FP64 synthesis (beta: the adjoint's fields 3, 4), and analysis with the
+// finish step: small plans by blocks of one order, larger ones on the tensor
+// cores
+static int synthesis64(sphnse_plan* P, const double* alpha, const double* beta) {
+    return small_plan(P->nh) ? launch_synthesis_small(P, alpha, beta) : launch_synthesis_dig(P, alpha, beta);
+}
+static int analysis64(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out) {
+    if (small_plan(P->nh)) return launch_analysis_small(P, kind, alpha, forcing, out);
+    const int rc = launch_analysis_dig(P, kind == 2 ? 3 : 2);
+    return rc ? rc : launch_finish(P, kind, SPHNSE_FP64, alpha, forcing, out);
+}
+
 int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, double* out) {
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     int rc;
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);
     if (prec == SPHNSE_FP64) {
-        if ((rc = launch_synthesis_dig(P, alpha, nullptr))) return rc;
+        if ((rc = synthesis64(P, alpha, nullptr))) return rc;
         if ((rc = launch_ring_fx(P, RING_RHS, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-        if ((rc = launch_analysis_dig(P, 2))) return rc;
-        return launch_finish(P, 0, prec, alpha, forcing, out);
+        return analysis64(P, 0, alpha, forcing, out);
     }
     const bool ring4 = ring4_ok(P);
     // the tensor-core synthesis (its epilogue warps are off the streaming path)
@@ -188,10 +201,9 @@ int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, dou
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     int rc;
     if (prec == SPHNSE_FP64) {
-        if ((rc = launch_synthesis_dig(P, alpha, w))) return rc;
+        if ((rc = synthesis64(P, alpha, w))) return rc;
         if ((rc = launch_ring_fx(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-        if ((rc = launch_analysis_dig(P, 3))) return rc;
-        return launch_finish(P, 2, prec, w, nullptr, out);
+        return analysis64(P, 2, w, nullptr, out);
     }
     if ((rc = launch_synthesis32(P, alpha, w, 1))) return rc;
     if ((rc = launch_ring(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
@@ -223,7 +235,7 @@ static void destroy_plan(sphnse_plan* P) {
     if (P->d_info) cudaFree(P->d_info);
     if (P->h_info) cudaFreeHost(P->h_info);
     void* ptrs[] = {P->d_items, P->d_item_off, P->d_status,
-                    P->d_x, P->d_s, P->d_isin32, P->d_rw, P->d_tw32, P->d_ftw, P->d_fxtw, P->d_lm, P->d_finc, P->d_prepc, P->d_finc32, P->d_prepc32,
+                    P->d_x, P->d_s, P->d_isin32, P->d_isin, P->d_rw, P->d_tw32, P->d_ftw, P->d_fxtw, P->d_lm, P->d_finc, P->d_prepc, P->d_finc32, P->d_prepc32,
                     P->d_gsyn, P->d_gana, P->d_hana, P->d_grid, P->d_theta, P->d_w, P->d_work, P->d_tmp, P->d_norms};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -340,6 +352,7 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
     if (!rc) rc = dalloc(&P->d_x, nlat * sizeof(double));
     if (!rc) rc = dalloc(&P->d_s, nlat * sizeof(double));
     if (!rc) rc = dalloc(&P->d_isin32, nlat * sizeof(float));
+    if (!rc) rc = dalloc(&P->d_isin, nlat * sizeof(double));
     if (!rc) rc = dalloc(&P->d_rw, nlat * sizeof(double));
     if (!rc) rc = dalloc(&P->d_tw32, tw32.size() * sizeof(float));
     const std::vector<float> ftw = ring4_twiddles(nlon);
@@ -366,8 +379,13 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
     up(P->d_s, P->s.data(), nlat * sizeof(double));
     {
         std::vector<float> isin(nlat);
-        for (int p = 0; p < nlat; ++p) isin[p] = float(1.0 / P->s[p]);
+        std::vector<double> isin64(nlat);
+        for (int p = 0; p < nlat; ++p) {
+            isin64[p] = 1.0 / P->s[p];
+            isin[p] = float(isin64[p]);
+        }
         up(P->d_isin32, isin.data(), nlat * sizeof(float));
+        up(P->d_isin, isin64.data(), nlat * sizeof(double));
     }
     up(P->d_rw, rw.data(), nlat * sizeof(double));
     up(P->d_tw32, tw32.data(), tw32.size() * sizeof(float));
@@ -513,7 +531,7 @@ int sphnse_grid_fields(sphnse_plan* P, const double* alpha, double* zeta, double
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);
     int rc;
     if (prec == SPHNSE_FP64) {
-        if ((rc = launch_synthesis_dig(P, alpha, nullptr))) return rc;
+        if ((rc = synthesis64(P, alpha, nullptr))) return rc;
         return launch_ring_fx(P, RING_GRID, nullptr, nullptr, zeta, uth, uph);
     }
     if ((rc = tc ? launch_synthesis_tc(P, alpha, 1) : launch_synthesis32(P, alpha, nullptr, 1))) return rc;
@@ -526,8 +544,7 @@ int sphnse_project(sphnse_plan* P, const double* vth, const double* vph, double*
     int rc;
     if (prec == SPHNSE_FP64) {
         if ((rc = launch_ring_fx(P, RING_PROJECT, vth, vph, nullptr, nullptr, nullptr))) return rc;
-        if ((rc = launch_analysis_dig(P, 2))) return rc;
-        return launch_finish(P, 1, prec, nullptr, nullptr, out);
+        return analysis64(P, 1, nullptr, nullptr, out);
     }
     if ((rc = launch_ring(P, RING_PROJECT, vth, vph, nullptr, nullptr, nullptr))) return rc;
     const bool tc = P->precision == SPHNSE_BF16X3 && tc_supported(P);

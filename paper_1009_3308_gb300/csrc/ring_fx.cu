@@ -99,7 +99,7 @@ struct RingFxArgs {
     double* gout1;
     double* gout2;
     const int4* tw;
-    int* emax;             // [nf][N+1] largest biased exponents of gana (atomic maxima)
+    int* emax;             // [nf][N+1] largest biased exponents of gana (atomic maxima); null: not needed
     FxPlan plan;
     int early;             // let the successor start its prologue at once
 };
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(576, 1) k_ring_fx(RingFxArgs a) {
         } else {
             *reinterpret_cast<double2*>(g + 2 * (row0 & 1)) = make_double2(o.x, o.y);
         }
-        atomicMax(a.emax + f * (N + 1) + m, e);
+        if (a.emax) atomicMax(a.emax + f * (N + 1) + m, e);
     };
     double4_32a o0 = make_double4_32a(0.0, 0.0, 0.0, 0.0), o1 = o0;
 #pragma unroll
@@ -511,11 +511,15 @@ __global__ void __launch_bounds__(576, 1) k_ring_fx(RingFxArgs a) {
 template <int MODE>
 static cudaError_t ring_fx_t(sphnse_plan* P, RingFxArgs a) {
     using Q = FxMode<MODE>;
-    // a radix-8 butterfly per thread; every order m <= N < M / 3 needs its own thread
-    const int threads = std::max((Q::NS * a.M / 8 + 31) / 32 * 32, (a.N + 32) / 32 * 32);
+    // a radix-8 butterfly per thread; a grid of at most one CTA per SM, whose time
+    // is one thread's chain, takes a radix-3 butterfly and a grid point per thread
+    // (RHS at L = 100, 81 CTAs: 56 -> 46 us; at L = 255, 192 CTAs, 86 -> 92 us);
+    // every order m <= N < M / 3 needs its own thread
+    const int grid = (a.nlat + Q::RPC - 1) / Q::RPC;
+    const int want = grid <= P->nsm ? std::min(Q::NS * a.M / 3, 576) : Q::NS * a.M / 8;
+    const int threads = (std::max(want, a.N + 1) + 31) / 32 * 32;
     const size_t sm = size_t(2) * Q::NS * fx_stride(a.M) * 16 + size_t(a.M) * 16;
     allow_dynamic_smem(reinterpret_cast<const void*>(k_ring_fx<MODE>), sm);
-    const int grid = (a.nlat + Q::RPC - 1) / Q::RPC;
     // a grid of more than one wave must not start its successor early
     a.early = grid <= P->nsm * std::max(1, std::min(int((227 * 1024) / (sm + 1024)), 576 / threads));
     return launch_pdl(k_ring_fx<MODE>, dim3(grid), dim3(threads), sm, P->stream, a);
