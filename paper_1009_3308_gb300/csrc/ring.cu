@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(128, 4) k_ring4(Ring4Args a) {
     __shared__ float s_rw[128 / M2];
     pdl_launch();
     pdl_wait();
-    ring4_rings<M2>(a, blockIdx.x * (128 / M2), blockIdx.y, threadIdx.x, sm4, s_rw, [] { __syncthreads(); });
+    ring4_rings<M2>(a, blockIdx.x * (128 / M2), blockIdx.y, threadIdx.x, sm4, s_rw);
 }
 
 // 256 threads per G = 128 / M2 rings (grids of less than a wave)
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(256, 3) k_ring4w(Ring4Args a) {
     __shared__ float s_rw[128 / M2];
     pdl_launch();
     pdl_wait();
-    ring4w_rings<M2>(a, blockIdx.x * (128 / M2), blockIdx.y, threadIdx.x, sm4, s_rw, [] { __syncthreads(); });
+    ring4w_rings<M2>(a, blockIdx.x * (128 / M2), blockIdx.y, threadIdx.x, sm4, s_rw);
 }
 
 template <int M2>

@@ -22,6 +22,7 @@
 
 #include "fft_small.cuh"
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace sph {
 
@@ -116,14 +117,24 @@ __device__ __forceinline__ cx<float> conjg2(const float2* p) {
     return {v.x, -v.y};
 }
 
+// Barrier over the threads that share rings: a ring's exchanges concern only
+// its own M2 threads (two rings at M2 = 16, ...), so a warp waits for its own
+// rings, not for the whole CTA; a full barrier is left before the final stores,
+// which combine the CTA's latitudes.  H: halves of 128 threads per ring
+// (ring4w_rings).
+template <int M2, int H>
+__device__ __forceinline__ void ring4_sync(int ring_tid) {
+    constexpr int T = M2 < 32 ? 32 : M2;   // threads per half
+    if constexpr (T * H == 32) __syncwarp();
+    else named_bar_sync(1 + ring_tid / T, T * H);
+}
+
 // The RHS ring transform of the G latitudes lat0 .. lat0 + G - 1 of instance
-// inst by 128 threads (tid = 0..127).  sm: ring4_smem<M2>() bytes; s_rw: G
-// floats of shared memory; sync(): a barrier over exactly these 128 threads.
-// The first barrier comes after the spectra are loaded into registers, so
-// consecutive calls may reuse sm.
-template <int M2, typename Sync>
-__device__ __forceinline__ void ring4_rings(const Ring4Args& a, int lat0, int inst, int tid, float2* sm, float* s_rw,
-                                            Sync sync) {
+// inst by a CTA of 128 threads (tid = 0..127).  sm: ring4_smem<M2>() bytes;
+// s_rw: G floats of shared memory.
+template <int M2>
+__device__ __forceinline__ void ring4_rings(const Ring4Args& a, int lat0, int inst, int tid, float2* sm, float* s_rw) {
+    auto sync = [&] { ring4_sync<M2, 1>(tid); };
     using C = R4<M2>;
     constexpr int M = 24 * M2, A = C::A, B = M2 / A, P1 = C::P1, Bp = C::Bp, Q = C::Q, RING = C::RING;
     constexpr int G = 128 / M2, GP = G / 2, B2 = B + 1;
@@ -166,8 +177,6 @@ __device__ __forceinline__ void ring4_rings(const Ring4Args& a, int lat0, int in
             }
         }
     }
-    // the previous call's readers of buf and s_rw are done
-    sync();
     const int r = tid / M2, t = tid % M2;
     const int lat = lat0 + r;
     const float fc = lat < nlat ? a.two_omega * float(a.x[lat]) : 0.f;
@@ -188,7 +197,7 @@ __device__ __forceinline__ void ring4_rings(const Ring4Args& a, int lat0, int in
             }
         }
     }
-    sync();
+    __syncthreads();
     float2* XA = buf + r * RING;
     float2* XB = buf + (G + r) * RING;
 
@@ -339,7 +348,7 @@ __device__ __forceinline__ void ring4_rings(const Ring4Args& a, int lat0, int in
         for (int n1 = 0; n1 < 24; ++n1)
             if (n1 < 8 || n1 >= 16) st2(&XA[t + M2 * n1], y[n1]);
     }
-    sync();
+    __syncthreads();
 
     // separate the two real fields, truncate to m <= N, weight, store
     for (int i = tid; i < ld * GP; i += 128) {
@@ -374,9 +383,9 @@ __device__ __forceinline__ void ring4_rings(const Ring4Args& a, int lat0, int in
 // place in shared memory for the A threads, which take the product and the
 // forward transform alone.  Every signal sees the same operations in the
 // same order as in ring4_rings, so the results are identical.
-template <int M2, typename Sync>
-__device__ __forceinline__ void ring4w_rings(const Ring4Args& a, int lat0, int inst, int tid, float2* sm, float* s_rw,
-                                             Sync sync) {
+template <int M2>
+__device__ __forceinline__ void ring4w_rings(const Ring4Args& a, int lat0, int inst, int tid, float2* sm, float* s_rw) {
+    auto sync = [&] { ring4_sync<M2, 2>(tid % 128); };
     using C = R4<M2>;
     constexpr int M = 24 * M2, A = C::A, B = M2 / A, P1 = C::P1, Bp = C::Bp, Q = C::Q, RING = C::RING;
     constexpr int G = 128 / M2, GP = G / 2, B2 = B + 1;
@@ -414,7 +423,6 @@ __device__ __forceinline__ void ring4w_rings(const Ring4Args& a, int lat0, int i
             }
         }
     }
-    sync();
     const int h = tid / 128, u = tid % 128, r = u / M2, t = u % M2;
     const int lat = lat0 + r;
     const float fc = lat < nlat ? a.two_omega * float(a.x[lat]) : 0.f;
@@ -435,7 +443,7 @@ __device__ __forceinline__ void ring4w_rings(const Ring4Args& a, int lat0, int i
             }
         }
     }
-    sync();
+    __syncthreads();
     float2* XA = buf + r * RING;
     float2* XB = buf + (G + r) * RING;
     float2* X = h ? XB : XA;
@@ -560,7 +568,7 @@ __device__ __forceinline__ void ring4w_rings(const Ring4Args& a, int lat0, int i
         for (int n1 = 0; n1 < 24; ++n1)
             if (n1 < 8 || n1 >= 16) st2(&XA[t + M2 * n1], y[n1]);
     }
-    sync();
+    __syncthreads();
 
     // separate the two real fields, truncate to m <= N, weight, store
     for (int i = tid; i < ld * GP; i += NT) {

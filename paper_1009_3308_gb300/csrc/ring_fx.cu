@@ -41,7 +41,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <climits>
 #include <cmath>
 
 #include "fx64.cuh"
@@ -67,20 +66,42 @@ static bool make_fx_plan(int n, FxPlan* p) {
     return r == 1;
 }
 
-// e^{-2 pi i t / M} as split Q62 pairs (cos hi, cos lo, -sin hi, -sin lo)
+// e^{-2 pi i t / M} as split Q62 pairs (cos hi, cos lo, -sin hi, -sin lo); M is
+// even.  The extended-precision functions, slow where long double is emulated,
+// run at about 2 sqrt(M / 4) angles: a quarter (half) of the circle is their
+// products, the rest reflections.
 std::vector<int> ring_fx_twiddles(int M) {
+    typedef long double ld;
+    std::vector<long long> c(M), s(M);   // cos, sin in Q62
+    const int H = M / 2, top = M % 4 == 0 ? M / 4 : H, B = int(std::sqrt(double(top))) + 1;
+    const ld step = 2.0L * 3.14159265358979323846264338327950288L / M, one = 4611686018427387904.0L;
+    std::vector<ld> uc(B), us(B);
+    for (int a = 0; a < B; ++a) {
+        uc[a] = std::cos(step * a);
+        us[a] = std::sin(step * a);
+    }
+    for (int b = 0; b <= top; b += B) {
+        const ld vc = std::cos(step * b), vs = std::sin(step * b);
+        for (int a = 0; a < B && a + b <= top; ++a) {
+            c[a + b] = llroundl((uc[a] * vc - us[a] * vs) * one);
+            s[a + b] = llroundl((us[a] * vc + uc[a] * vs) * one);
+        }
+    }
+    for (int t = top + 1; t <= H; ++t) {   // reflect at pi / 2
+        c[t] = -c[H - t];
+        s[t] = s[H - t];
+    }
+    for (int t = H + 1; t < M; ++t) {      // and at pi
+        c[t] = c[M - t];
+        s[t] = -s[M - t];
+    }
     std::vector<int> tw(4 * size_t(M));
     for (int t = 0; t < M; ++t) {
-        const long double ang = 2.0L * 3.14159265358979323846264338327950288L * t / M;
-        const fx2 c = fx_split(llroundl(std::cos(ang) * 4611686018427387904.0L));
-        long long sq = llroundl(-std::sin(ang) * 4611686018427387904.0L);
-        // the inverse transform negates both halves of the sine
-        if (fx_split(sq).l == INT_MIN) ++sq;
-        const fx2 s = fx_split(sq);
-        tw[4 * t] = c.h;
-        tw[4 * t + 1] = c.l;
-        tw[4 * t + 2] = s.h;
-        tw[4 * t + 3] = s.l;
+        const fx2 a = fx_split(c[t]), b = fx_split(-s[t]);
+        tw[4 * t] = a.h;
+        tw[4 * t + 1] = a.l;
+        tw[4 * t + 2] = b.h;
+        tw[4 * t + 3] = b.l;
     }
     return tw;
 }
