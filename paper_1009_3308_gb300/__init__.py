@@ -344,6 +344,7 @@ class Ensemble:
         if not h:
             raise SphnseError("sphnse_ensemble_create", -1)
         self._h = ctypes.c_void_p(h)
+        self._views = {}
         self.n = n
         self.Ls = list(Ls)
         self.set("AUTOTUNE", 1 if autotune else 0)
@@ -373,6 +374,7 @@ class Ensemble:
 
     def close(self):
         if getattr(self, "_h", None):
+            self._views.clear()
             _capi.lib().sphnse_ensemble_destroy(self._h)
             self._h = None
 
@@ -405,23 +407,32 @@ class Ensemble:
             self._h, int(i), ctypes.byref(a), ctypes.byref(f), ctypes.byref(nc)))
         return a.value, f.value, nc.value
 
+    def _view(self, i, which):
+        """Instance i's state ('alpha') or last RHS: a tensor over the
+        ensemble's own memory, made once (building it costs more than the copy)."""
+        key = (int(i), which == "alpha")
+        v = self._views.get(key)
+        if v is None:
+            a, f, nc = self._ptrs(i)
+            with _torch().inference_mode(False):
+                v = _wrap(a if which == "alpha" else f, nc * 16).view(_torch().complex128)
+            self._views[key] = v
+        return v
+
     def set_alpha(self, i, alpha):
         """Copy a complex128 CUDA tensor into instance i's state."""
         torch = _torch()
-        a, _, nc = self._ptrs(i)
-        if alpha.numel() != nc:
-            raise ValueError(f"instance {i} has {nc} coefficients")
-        src = alpha.to(self.device, torch.complex128).contiguous()
+        dst = self._view(i, "alpha")
+        if alpha.numel() != dst.numel():
+            raise ValueError(f"instance {i} has {dst.numel()} coefficients")
+        dst.copy_(alpha.detach().to(self.device, torch.complex128).reshape(-1))
         torch.cuda.current_stream(self.device).synchronize()
-        _cudart_copy(a, src.data_ptr(), nc * 16)
 
     def _get_instance(self, i, which="alpha"):
         """Copy of instance i's state ('alpha') or last RHS ('F')."""
         torch = _torch()
-        a, f, nc = self._ptrs(i)
-        out = torch.empty(nc, dtype=torch.complex128, device=self.device)
+        out = self._view(i, which).clone()
         torch.cuda.current_stream(self.device).synchronize()
-        _cudart_copy(out.data_ptr(), a if which == "alpha" else f, nc * 16)
         return out
 
     def rhs(self):
@@ -447,15 +458,6 @@ class Ensemble:
         check("sphnse_ensemble_advance", _capi.lib().sphnse_ensemble_advance(
             self._h, int(nsteps), ctypes.cast(infos, ctypes.c_void_p)))
         return [x.as_dict() for x in infos]
-
-
-def _cudart_copy(dst, src, nbytes):
-    """Device-to-device copy of raw device memory through torch."""
-    torch = _torch()
-    src_t = _wrap(src, nbytes)
-    dst_t = _wrap(dst, nbytes)
-    dst_t.copy_(src_t)
-    torch.cuda.current_stream().synchronize()
 
 
 def _wrap(ptr, nbytes):
