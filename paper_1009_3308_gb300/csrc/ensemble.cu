@@ -94,19 +94,23 @@ __global__ void kb_init(const int2* btab, const InstPar* par, double2* dif, cons
     init_dif_entry(dif + 7 * o, F + o, p.h0, p.n, i);
 }
 
-__global__ void kb_rescale(const int2* btab, const InstPar* par, double2* dif) {
-    INST_PROLOGUE(F_RESCALE)
-    rescale_entry(dif + 7 * o, p.A, p.k, p.n, i);
-}
-
-__global__ void kb_predict(const int2* btab, const InstPar* par, const double2* y, const double2* dif, double2* y0,
-                           double2* psi, double2* d, double2* ynew, unsigned long long* norms) {
-    INST_PROLOGUE_ALL(F_PREDICT)
+// The entry-wise work between two rounds' RHS: the last attempt's accept, the
+// rescale to the new step size and the predictor, each where the instance is
+// flagged (one pass over the differences instead of three launches).
+__global__ void kb_prepare(const int2* btab, const InstPar* par, double2* y, double2* dif, double2* y0, double2* psi,
+                           double2* d, double2* ynew, unsigned long long* norms) {
+    INST_PROLOGUE_ALL(F_ACCEPT | F_RESCALE | F_PREDICT)
     float r[1] = {0.f};
-    // slot 4: ||y / max(|y|, thr)||_inf (FP32, as the corrector's norms)
-    if (i < p.n)
-        r[0] = predict_entry(y + o, dif + 7 * o, p.g, p.k, y0 + o, psi + o, d + o, ynew + o,
-                             fmaxf(float(p.thr), 1e-30f), p.n, i);
+    if (i < p.n) {
+        double2* D = dif + 7 * o;
+        if (p.flags & F_ACCEPT) accept_entry(D, d + o, y + o, ynew + o, p.ka, p.n, i);
+        if (p.flags & F_RESCALE) rescale_entry(D, p.A, p.k, p.n, i);
+        // slot 4: ||y / max(|y|, thr)||_inf (FP32, as the corrector's norms)
+        if (p.flags & F_PREDICT)
+            r[0] = predict_entry(y + o, D, p.g, p.k, y0 + o, psi + o, d + o, ynew + o, fmaxf(float(p.thr), 1e-30f), p.n,
+                                 i);
+    }
+    if (!(p.flags & F_PREDICT)) return;
     const int id[1] = {4};
     block_amax_f<1>(norms + 8 * bt.x, r, id, false);
 }
@@ -269,6 +273,8 @@ struct Bucket {
     TcBatchA tca;              //         and slots of the tensor-core analysis
     bool tc = false;
     double syn_us = 0;         // tuned synthesis duration (0: not tuned)
+    cudaStream_t st = nullptr; // several buckets: this bucket's branch of the batched RHS
+    cudaEvent_t ev = nullptr;
 };
 
 }  // namespace
@@ -285,6 +291,7 @@ struct sphnse_ensemble {
     cudaStream_t stream = nullptr;   // the ensemble's own stream: all work, capture and replay
     cudaStream_t user = nullptr;     // the caller's stream, joined by events at API boundaries
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+    cudaEvent_t ev_fork = nullptr;   // start of the buckets' branches
     std::vector<int> L;
     std::vector<double> nu;
     std::vector<Bucket> buckets;
@@ -315,35 +322,52 @@ struct sphnse_ensemble {
 
 namespace {
 
-int batched_rhs(sphnse_ensemble* E, const double2* x, double2* F) {
+int bucket_rhs(Bucket& B, const double2* x, double2* F) {
     int rc;
-    for (auto& B : E->buckets) {
-        sphnse_plan* P = B.P;
-        P->stream = E->stream;
-        const double* xb = reinterpret_cast<const double*>(x + B.off);
-        double* Fb = reinterpret_cast<double*>(F + B.off);
-        const bool ring4 = ring4_ok(P);
-        const int pairs = !ring4;   // layout of the ring kernel's input
-        if (B.tc) {
-            // all instances of the bucket share every table tile of the synthesis
-            if ((rc = launch_prep_tc_batch(P, B.tcb, xb))) return rc;
-            if ((rc = launch_synthesis_tc_batch(P, B.tcb, B.gsyn, B.sg, pairs))) return rc;
-        } else {
-            if ((rc = launch_prep32_batch(P, B.nb, xb, B.bsyn, B.sb))) return rc;
-            if ((rc = launch_synthesis_stream_batch(P, B.items, B.item_off, B.ncta, B.bsyn, B.sb, B.gsyn, B.sg, pairs)))
-                return rc;
-        }
-        if ((rc = ring4 ? launch_ring4(P, B.nb, B.gsyn, B.sg, B.gana, B.sa, 0)
-                        : launch_ring_batch(P, B.nb, B.gsyn, B.sg, B.gana, B.sa)))
+    sphnse_plan* P = B.P;
+    const double* xb = reinterpret_cast<const double*>(x + B.off);
+    double* Fb = reinterpret_cast<double*>(F + B.off);
+    const bool ring4 = ring4_ok(P);
+    const int pairs = !ring4;   // layout of the ring kernel's input
+    if (B.tc) {
+        // all instances of the bucket share every table tile of the synthesis
+        if ((rc = launch_prep_tc_batch(P, B.tcb, xb))) return rc;
+        if ((rc = launch_synthesis_tc_batch(P, B.tcb, B.gsyn, B.sg, pairs))) return rc;
+    } else {
+        if ((rc = launch_prep32_batch(P, B.nb, xb, B.bsyn, B.sb))) return rc;
+        if ((rc = launch_synthesis_stream_batch(P, B.items, B.item_off, B.ncta, B.bsyn, B.sb, B.gsyn, B.sg, pairs)))
             return rc;
-        if (B.tc) {
-            if ((rc = launch_analysis_tc_batch(P, B.tca, B.gana, B.sa, B.hana, B.sh))) return rc;
-        } else if ((rc = launch_analysis_stream_batch(P, B.items, B.item_off, B.ncta, B.gana, B.sa, B.hana, B.sh))) {
-            return rc;
-        }
-        if ((rc = launch_finish32_batch(P, B.nb, B.hana, B.sh, xb, Fb, B.nu_dev))) return rc;
     }
-    return SPHNSE_OK;
+    if ((rc = ring4 ? launch_ring4(P, B.nb, B.gsyn, B.sg, B.gana, B.sa, 0)
+                    : launch_ring_batch(P, B.nb, B.gsyn, B.sg, B.gana, B.sa)))
+        return rc;
+    if (B.tc) {
+        if ((rc = launch_analysis_tc_batch(P, B.tca, B.gana, B.sa, B.hana, B.sh))) return rc;
+    } else if ((rc = launch_analysis_stream_batch(P, B.items, B.item_off, B.ncta, B.gana, B.sa, B.hana, B.sh))) {
+        return rc;
+    }
+    return launch_finish32_batch(P, B.nb, B.hana, B.sh, xb, Fb, B.nu_dev);
+}
+
+// The buckets are independent: each runs as a branch on its own stream, the
+// largest truncation first, so that the small grids and the launch gaps of one
+// bucket fill with another's work (96 members of L = 63, 127 and 255).
+int batched_rhs(sphnse_ensemble* E, const double2* x, double2* F) {
+    const int nbk = int(E->buckets.size());
+    if (nbk == 1) return bucket_rhs(E->buckets[0], x, F);
+    if (cudaEventRecord(E->ev_fork, E->stream) != cudaSuccess) return SPHNSE_E_CUDA;
+    int rc = SPHNSE_OK;
+    for (int b = nbk - 1; b >= 0; --b) {   // ascending truncations in the list
+        Bucket& B = E->buckets[b];
+        if (cudaStreamWaitEvent(B.st, E->ev_fork, 0) != cudaSuccess) rc = rc ? rc : SPHNSE_E_CUDA;
+        B.P->stream = B.st;
+        if (!rc) rc = bucket_rhs(B, x, F);
+        B.P->stream = E->stream;
+        // (joined on an error too: a capture must not end with an open branch)
+        if (cudaEventRecord(B.ev, B.st) != cudaSuccess || cudaStreamWaitEvent(E->stream, B.ev, 0) != cudaSuccess)
+            rc = rc ? rc : SPHNSE_E_CUDA;
+    }
+    return rc;
 }
 
 int upload_par(sphnse_ensemble* E) {
@@ -392,12 +416,15 @@ void destroy_ens(sphnse_ensemble* E) {
     if (E->d_btab) cudaFree(E->d_btab);
     if (E->ev_in) cudaEventDestroy(E->ev_in);
     if (E->ev_out) cudaEventDestroy(E->ev_out);
+    if (E->ev_fork) cudaEventDestroy(E->ev_fork);
     for (auto& B : E->buckets) {
         void* ptrs[] = {B.bsyn, B.gsyn, B.gana, B.hana, B.items, B.item_off, B.nu_dev};
         for (void* q : ptrs)
             if (q) cudaFree(q);
         tc_batch_free(&B.tcb);
         tc_batch_ana_free(&B.tca);
+        if (B.st) cudaStreamDestroy(B.st);
+        if (B.ev) cudaEventDestroy(B.ev);
         if (B.P) sphnse_plan_destroy(B.P);
     }
     void* ptrs[] = {E->alpha, E->dif, E->y0, E->psi, E->d, E->ynew, E->F, E->d_par, E->d_norms, E->d_sc,
@@ -574,10 +601,18 @@ sphnse_ensemble* sphnse_ensemble_create(int n, const int* Ls, const double* nus,
     }
     if (cudaStreamCreateWithFlags(&E->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&E->ev_in, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&E->ev_out, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&E->ev_out, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&E->ev_fork, cudaEventDisableTiming) != cudaSuccess) {
         destroy_ens(E);
         return nullptr;
     }
+    if (E->buckets.size() > 1)
+        for (auto& B : E->buckets)
+            if (cudaStreamCreateWithFlags(&B.st, cudaStreamNonBlocking) != cudaSuccess ||
+                cudaEventCreateWithFlags(&B.ev, cudaEventDisableTiming) != cudaSuccess) {
+                destroy_ens(E);
+                return nullptr;
+            }
     for (auto& B : E->buckets) B.P->stream = E->stream;
     for (int i = 0; i < n; ++i) {
         InstPar& p = E->par[i];
@@ -851,9 +886,7 @@ static int build_advance_graph(sphnse_ensemble* E) {
     ok = ok && body && cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) ==
                            cudaSuccess;
     if (ok) {
-        kb_accept<<<E->nbt, EB, 0, cs>>>(E->d_btab, E->d_par, E->dif, E->d, E->alpha, E->ynew);
-        kb_rescale<<<E->nbt, EB, 0, cs>>>(E->d_btab, E->d_par, E->dif);
-        kb_predict<<<E->nbt, EB, 0, cs>>>(E->d_btab, E->d_par, E->alpha, E->dif, E->y0, E->psi, E->d, E->ynew,
+        kb_prepare<<<E->nbt, EB, 0, cs>>>(E->d_btab, E->d_par, E->alpha, E->dif, E->y0, E->psi, E->d, E->ynew,
                                            E->d_norms);
         rc = batched_rhs(E, E->ynew, E->F);
         kb_newton<<<E->nbt, EB, 0, cs>>>(E->d_btab, E->d_par, E->F, E->alpha, E->y0, E->psi, E->d, E->ynew, E->dif,

@@ -653,71 +653,13 @@ __global__ void __launch_bounds__(192, 1) k_ana_tc_b(TcAnaBArgs a) {
 // zeta: lam^{1/2} a_K; theta: lam^{-1/2} a_K; phi: c_down a_{K-1} + c_up
 // a_{K+1}, the degree-shift form of sin(theta) d/dtheta, for chunk q of K
 // tile kt of block (m, parity): the 8 degrees K = m + par + 2 j, j = 64 kt +
-// 8 q .. +7.  prep_consts reads the plan's table (before any wait for the
-// predecessor); prep_chunk reads alpha and returns the hi parts of the six
-// columns (v[0..5]), their lo parts (v[6..11]) and, for m = 1, the u_phi at
-// m = 0 column -a_{K,0} (hi v[12], lo v[13]; zero otherwise).  With
+// 8 q .. +7, split over the four lanes (q, p) of the chunk: lane p takes the
+// degrees j = 64 kt + 8 q + 2 p, +1 and returns word p (two bf16) of each row
+// of the chunk: hi parts w[0..5], lo parts w[6..11], and for m = 1 the u_phi
+// at m = 0 column -a_{K,0} w[12] (hi), w[13] (lo) (zero otherwise).  With
 // d/dtheta Pt_K^0 = sqrt(K (K+1)) Pt_K^1 (ladder relation, Condon-Shortley
 // phase), u_phi at m = 0 is -sum_K alpha_{K,0} Pt_K^1: a sum over the
 // order-1 table that needs no division by sin(theta).
-__device__ __forceinline__ void prep_consts(const float4* __restrict__ prepc, int N, int m, int par, int kt, int q,
-                                            float4 (&cf)[8]) {
-    const int ne = ext_even(N, m), n = par ? ext_odd(N, m) : ne;
-    const int j0 = kt * TC_TILE_K + q * 8;
-    const int r0 = ext_off(N, m) + (par ? ne : 0);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) cf[e] = (j0 + e < n) ? prepc[r0 + j0 + e] : make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
-__device__ __forceinline__ void prep_chunk(const double2* __restrict__ alpha, int N, int m, int par, int kt, int q,
-                                           const float4 (&cf)[8], uint4 (&v)[14]) {
-    const int ne = ext_even(N, m), n = par ? ext_odd(N, m) : ne;
-    const int j0 = kt * TC_TILE_K + q * 8;
-    const int lo = m > 0 ? m : 1;
-    const int K0 = m + par + 2 * j0;
-    const int pk = packed_off(N, m) - lo;   // packed index of degree K is pk + K
-    float2 al[17];
-#pragma unroll
-    for (int e = 0; e < 17; ++e) {
-        const int K = K0 - 1 + e;
-        double2 x = make_double2(0.0, 0.0);
-        if (K >= lo && K <= N) x = alpha[pk + K];
-        al[e] = make_float2(f64_to_f32_rn(x.x), f64_to_f32_rn(x.y));
-    }
-    float c6[6][8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        const float2 am = al[2 * e], a0 = al[2 * e + 1], ap = al[2 * e + 2];
-        c6[0][e] = cf[e].x * a0.x;
-        c6[1][e] = cf[e].x * a0.y;
-        c6[2][e] = cf[e].y * a0.x;
-        c6[3][e] = cf[e].y * a0.y;
-        c6[4][e] = fmaf(cf[e].z, am.x, cf[e].w * ap.x);
-        c6[5][e] = fmaf(cf[e].z, am.y, cf[e].w * ap.y);
-    }
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        v[c] = pack_hi(c6[c]);
-        v[6 + c] = pack_lo(c6[c]);
-    }
-    v[12] = v[13] = make_uint4(0u, 0u, 0u, 0u);
-    if (m == 1) {
-        const double2* a0 = alpha + (packed_off(N, 0) - 1);   // a_{K,0} at a0[K], K = 1 .. N (real)
-        float re[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int K = K0 + 2 * e;
-            re[e] = (j0 + e < n && K <= N) ? -f64_to_f32_rn(a0[K].x) : 0.f;
-        }
-        v[12] = pack_hi(re);
-        v[13] = pack_lo(re);
-    }
-}
-
-// The same coefficient sets split over the four lanes (q, p) of a chunk:
-// lane p takes the degrees j = 64 kt + 8 q + 2 p, +1 and returns word p (two
-// bf16) of each row of the chunk: hi parts w[0..5], lo parts w[6..11], the
-// u_phi at m = 0 column (m = 1 only) w[12] (hi), w[13] (lo).
 __device__ __forceinline__ void prep_words(const double2* __restrict__ alpha, const float4* __restrict__ prepc, int N,
                                            int m, int par, int kt, int q, int p, uint32_t (&w)[14]) {
     const int ne = ext_even(N, m), n = par ? ext_odd(N, m) : ne;
@@ -1165,36 +1107,34 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
     }
 }
 
-// B tiles of the batched synthesis: thread (tile, chunk q) of instance
-// blockIdx.y stores the chunk's hi parts in rows r0 .. r0+5 and lo parts in
-// rows r0+6 .. r0+11, r0 = 12 (instance mod ng), of its group's tile, and on
-// order-1 tiles the u_phi at m = 0 column in rows 12 ng + 2 (instance mod
-// ng) (hi, lo); rows past the group's instances stay zero.
+// B tiles of the batched synthesis: a warp per (tile, instance), lane (q, p)
+// word p of chunk q: the hi parts in rows r0 .. r0+5 and the lo parts in rows
+// r0+6 .. r0+11, r0 = 12 (instance mod ng), of its group's tile, and on order-1
+// tiles the u_phi at m = 0 column in rows 12 ng + 2 (instance mod ng) (hi, lo);
+// rows past the group's instances stay zero.  A warp reads consecutive degrees
+// and writes whole 128-byte rows (one thread per chunk, eight degrees apart,
+// took 32 us for 32 instances at L = 255, where 17 MB are read and 34 written).
 __global__ void __launch_bounds__(128) k_prep_tc(const double2* __restrict__ alpha, const float4* __restrict__ prepc,
                                                  unsigned char* __restrict__ btiles, const int2* __restrict__ tinfo,
                                                  int ntiles, int N, int n_coeff, int ng, int brows) {
     pdl_launch();
-    const int g = blockIdx.x * 16 + (threadIdx.x >> 3), q = threadIdx.x & 7;
+    const int g = blockIdx.x * 4 + (threadIdx.x >> 5), q = (threadIdx.x >> 2) & 7, p = threadIdx.x & 3;
     if (g >= ntiles) return;
     const int inst = blockIdx.y;
     alpha += size_t(inst) * n_coeff;
     const int2 ti = tinfo[g];
     const int b = ti.x, kt = ti.y, m = b >> 1, par = b & 1;
-    // the plan's table is read before the wait; alpha may be the
-    // predecessor's output
-    float4 cf[8];
-    prep_consts(prepc, N, m, par, kt, q, cf);
-    pdl_wait();
-    uint4 v[14];
-    prep_chunk(alpha, N, m, par, kt, q, cf, v);
+    pdl_wait();   // alpha may be the predecessor's output
+    uint32_t w[14];
+    prep_words(alpha, prepc, N, m, par, kt, q, p, w);
     const int grp = inst / ng, row0 = 12 * (inst % ng);
     unsigned char* tile = btiles + (size_t(grp) * ntiles + g) * size_t(brows) * TC_TILE_K * 2;
 #pragma unroll
-    for (int c = 0; c < 12; ++c) *reinterpret_cast<uint4*>(tile + sw128_chunk(row0 + c, q)) = v[c];
+    for (int c = 0; c < 12; ++c) *reinterpret_cast<uint32_t*>(tile + sw128_chunk(row0 + c, q) + 4 * p) = w[c];
     if (m == 1) {
         const int rp = 12 * ng + 2 * (inst % ng);
-        *reinterpret_cast<uint4*>(tile + sw128_chunk(rp, q)) = v[12];
-        *reinterpret_cast<uint4*>(tile + sw128_chunk(rp + 1, q)) = v[13];
+        *reinterpret_cast<uint32_t*>(tile + sw128_chunk(rp, q) + 4 * p) = w[12];
+        *reinterpret_cast<uint32_t*>(tile + sw128_chunk(rp + 1, q) + 4 * p) = w[13];
     }
 }
 
@@ -1783,7 +1723,7 @@ void tc_batch_free(TcBatch* B) {
 
 int launch_prep_tc_batch(sphnse_plan* P, const TcBatch& B, const double* alpha) {
     stage_begin(P, SPHNSE_STAGE_PREP);
-    const cudaError_t e = launch_pdl(k_prep_tc, dim3((P->tc.ntiles + 15) / 16, B.nb), dim3(128), 0, P->stream,
+    const cudaError_t e = launch_pdl(k_prep_tc, dim3((P->tc.ntiles + 3) / 4, B.nb), dim3(128), 0, P->stream,
                                      reinterpret_cast<const double2*>(alpha), static_cast<const float4*>(P->d_prepc32),
                                      B.btiles, static_cast<const int2*>(P->tc.tile_info), P->tc.ntiles, P->N,
                                      P->n_coeff, B.ng, B.brows);
