@@ -1,6 +1,6 @@
 // Longitude ("ring") kernels of the FP32 and BF16x3 paths (the FP64 path's
 // kernel is in ring_fx.cu).  General kernel: one CTA per pair of Gauss
-// latitudes, half of its threads per ring.  It reads the latitude-pair-major
+// latitudes.  It reads the latitude-pair-major
 // spectra [f][row / 2][m][row % 2] (a CTA's data are contiguous) and writes the
 // order-major ones of the analysis (16 bytes, two latitudes, at a time), so it
 // needs no transposes.  With one latitude per CTA and a transpose kernel on
@@ -15,9 +15,12 @@
 //   3. forward FFT of W_theta + i W_phi, separation of the two real spectra,
 //      truncation to m = 0..N, scaling by (2 pi / M) w_p / sin(theta_p)
 //      (the quadrature weight of Eq. (quadrule) and the 1/sin of the basis).
-// M = nlon = 2^a 3^b; Stockham autosort radix-8/4/2/3 stages in shared memory
-// (radix 3 last, so every stride Ns before it is a power of two), twiddles
-// e^{-2 pi i t / M} computed in FP64 on the host, staged in shared memory.
+// M = nlon = 2^a 3^b; Stockham autosort radix-8/4/2/3 stages (radix 3 last)
+// from one shared-memory buffer to the other, a butterfly of one signal per
+// thread at a time, one barrier per stage; twiddles e^{-2 pi i t / M} computed
+// in FP64 on the host, staged in shared memory.  (In-place stages holding every
+// signal's butterflies in registers spilled 276 bytes per thread and left half
+// of the threads idle: the adjoint's ring took 24.1 us at L = 255, now 14.3.)
 // Products keep |m| <= 2N and M >= 3N + 2 > 3N, so the truncated m <= N
 // coefficients are alias-free.
 //
@@ -26,6 +29,7 @@
 // ADJOINT evaluates the transposed linearised product (see rhs_adjoint).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "fft_small.cuh"
@@ -35,70 +39,68 @@
 
 namespace sph {
 
-// One in-place Stockham stage of radix R over NSIG signals (buf[s], M points):
-// every thread first reads and transforms all of its butterflies into
-// registers, the block synchronises, then writes them to their autosorted
-// positions.  Ns = product of the earlier radices; nsh = log2(Ns) when Ns is
-// a power of two (radix-3 stages run last, so this holds unless M has 3^2).
-// A ring's nt threads (rt = 0 .. nt-1) are at least M/6, so a thread owns at
-// most MAXB butterflies.
-template <typename T, typename TW, int R, int NSIG>
-__device__ __forceinline__ void stage(cx<T>* const* buf, int M, int Ns, int nsh, const TW* tw, int sign, int rt,
-                                      int nt) {
-    constexpr int MAXB = R == 2 ? 3 : (R == 8 ? 1 : 2);
-    const int nb = M / R;
-    const int twstride = M / (Ns * R);
-    cx<T> v[NSIG][MAXB][R];
+// entry i of a signal: one slot of padding per sixteen keeps the stride-8
+// writes of the first radix-8 stage out of one another's banks
+__device__ __forceinline__ int rpad(int i) { return i + (i >> 4); }
+__host__ __device__ constexpr int ring_stride(int M) { return M + ((M + 15) >> 4); }
+
+// One stage of radix R over the 2 ns signals (ns per ring, rings rs apart),
+// from -> to; Ns = product of the earlier radices, step = M / (Ns R).  FIRST:
+// Ns = 1, every twiddle is 1.
+template <typename T, int R, int SIGN, bool FIRST = false>
+__device__ __forceinline__ void stage(cx<T>* sm, int from, int to, int ns, int rs, int M, int Ns, int step,
+                                      const T* tw) {
+    const int nb = M / R, ld = ring_stride(M);
+    const float rns = 1.f / float(Ns);
+#pragma unroll 1
+    for (int u = threadIdx.x; u < 2 * ns * nb; u += blockDim.x) {
+        int j = u, sg = 0;
+        while (j >= nb) {
+            j -= nb;
+            ++sg;
+        }
+        const int o = sg < ns ? sg * ld : rs + (sg - ns) * ld;
+        // j / Ns: exact, as j + 1/2 is at least 1 / (2 Ns) away from every multiple
+        const int q = int((float(j) + 0.5f) * rns), k = j - q * Ns;
+        cx<T> v[R];
 #pragma unroll
-    for (int b = 0; b < MAXB; ++b) {
-        const int j = rt + b * nt;
-        if (j < nb) {
-            const int k = nsh >= 0 ? (j & (Ns - 1)) : (j % Ns);
-            cx<T> w[R];
+        for (int r = 0; r < R; ++r) v[r] = sm[from + o + rpad(j + r * nb)];
+        if constexpr (!FIRST) {
 #pragma unroll
-            for (int r = 1; r < R; ++r) w[r] = twiddle<T>(tw, k * r * twstride, sign);
-#pragma unroll
-            for (int sg = 0; sg < NSIG; ++sg) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const cx<T> a = buf[sg][j + r * nb];
-                    v[sg][b][r] = r == 0 ? a : cmul(a, w[r]);
-                }
-                dft<T, R>(v[sg][b], sign);
+            for (int r = 1; r < R; ++r) {
+                // which product of a sum is rounded is spelled out, or the compiler picks
+                // it anew for each instance of this loop and results differ between them
+                const cx<T> a = v[r], w = twiddle<T>(tw, k * r * step, SIGN);
+                v[r] = {fmaf(a.x, w.x, -__fmul_rn(a.y, w.y)),
+                        R == 2 && SIGN < 0 ? fmaf(a.x, w.y, __fmul_rn(a.y, w.x)) : fmaf(a.y, w.x, __fmul_rn(a.x, w.y))};
             }
         }
-    }
-    __syncthreads();
+        dft<T, R>(v, SIGN);
 #pragma unroll
-    for (int b = 0; b < MAXB; ++b) {
-        const int j = rt + b * nt;
-        if (j < nb) {
-            const int k = nsh >= 0 ? (j & (Ns - 1)) : (j % Ns);
-            const int q = nsh >= 0 ? (j >> nsh) : (j / Ns);
-            const int idx = q * Ns * R + k;
-#pragma unroll
-            for (int sg = 0; sg < NSIG; ++sg)
-#pragma unroll
-                for (int r = 0; r < R; ++r) buf[sg][idx + r * Ns] = v[sg][b][r];
-        }
+        for (int r = 0; r < R; ++r) sm[to + o + rpad(q * Ns * R + k + r * Ns)] = v[r];
     }
     __syncthreads();
 }
 
-// Full M-point transform (sign -1 forward, +1 inverse) of NSIG signals in place.
-template <typename T, typename TW, int NSIG>
-__device__ void fft(cx<T>* const* buf, const FFTPlan& plan, const TW* tw, int sign, int rt, int nt) {
-    const int M = plan.n;
-    int Ns = 1;
+// Full M-point transforms (SIGN -1 forward, +1 inverse) of the signals at entry
+// `from` of the shared array, `to` the other buffer; returns the result's entry.
+template <typename T, int SIGN>
+__device__ __forceinline__ int fft(cx<T>* sm, int from, int to, int ns, int rs, const FFTPlan& plan, const T* tw) {
+    int Ns = 1, step = plan.n;
+#pragma unroll 1
     for (int st = 0; st < plan.nstages; ++st) {
         const int R = plan.radix[st];
-        const int nsh = (Ns & (Ns - 1)) == 0 ? __ffs(Ns) - 1 : -1;
-        if (R == 8) stage<T, TW, 8, NSIG>(buf, M, Ns, nsh, tw, sign, rt, nt);
-        else if (R == 4) stage<T, TW, 4, NSIG>(buf, M, Ns, nsh, tw, sign, rt, nt);
-        else if (R == 2) stage<T, TW, 2, NSIG>(buf, M, Ns, nsh, tw, sign, rt, nt);
-        else stage<T, TW, 3, NSIG>(buf, M, Ns, nsh, tw, sign, rt, nt);
+        if (R == 8 && st == 0) stage<T, 8, SIGN, true>(sm, from, to, ns, rs, plan.n, 1, step /= 8, tw);
+        else if (R == 8) stage<T, 8, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 8, tw);
+        else if (R == 4) stage<T, 4, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 4, tw);
+        else if (R == 2) stage<T, 2, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 2, tw);
+        else stage<T, 3, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 3, tw);
         Ns *= R;
+        const int t = from;
+        from = to;
+        to = t;
     }
+    return from;
 }
 
 struct RingArgs {
@@ -119,22 +121,22 @@ struct RingArgs {
 };
 
 template <typename T, typename TW, int MODE>
-__global__ void __launch_bounds__(512) k_ring(RingArgs a, FFTPlan plan, const TW* __restrict__ tw) {
+__global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant__ FFTPlan plan,
+                                              const TW* __restrict__ tw) {
     if (a.early) pdl_launch();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int NBUF = MODE == RING_ADJOINT ? 3 : (MODE == RING_PROJECT ? 1 : 2);
-    cx<T>* buf = reinterpret_cast<cx<T>*>(smem_raw);   // [2 rings][NBUF][M]
+    const int M = a.M, N = a.N, nlat = a.nlat, pair = blockIdx.x, npair = (nlat + 1) / 2, row0 = 2 * pair;
+    const int ls = ring_stride(M), rs = NBUF * ls;     // signal and ring strides
+    cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);    // [2 rings][NBUF][ls], twice
+    int cur = 0;                                       // the buffer that holds the signals: entry 0 or 2 rs
     // the twiddle table e^{-2 pi i t / M} lives in shared memory after the buffers
-    T* tws = reinterpret_cast<T*>(buf + 2 * NBUF * a.M);
-    for (int t = threadIdx.x; t < 2 * a.M; t += blockDim.x) tws[t] = T(tw[t]);
-    const int M = a.M, N = a.N, nlat = a.nlat, pair = blockIdx.x, npair = (nlat + 1) / 2;
-    const int nt = blockDim.x / 2, h = threadIdx.x / nt, rt = threadIdx.x % nt;
-    const int row = 2 * pair + h;                      // this half's ring (h = 1 of an odd grid's last pair: none)
-    const bool two = 2 * pair + 1 < nlat, live = row < nlat;
+    T* tws = reinterpret_cast<T*>(sm + 4 * rs);
+    for (int t = threadIdx.x; t < 2 * M; t += blockDim.x) tws[t] = T(tw[t]);
+    const bool two = row0 + 1 < nlat;                  // an odd grid's last pair has one ring
     const size_t ld = size_t(N + 1);
     const cx<T>* gs = reinterpret_cast<const cx<T>*>(a.gsyn) + size_t(blockIdx.y) * a.sgs;
     cx<T>* ga = reinterpret_cast<cx<T>*>(a.gana) + size_t(blockIdx.y) * a.sga;
-    cx<T>* src[3] = {buf + h * NBUF * M, buf + (h * NBUF + 1) * M, buf + (h * NBUF + 2) * M};
     pdl_wait();
 
     if constexpr (MODE != RING_PROJECT) {
@@ -163,53 +165,61 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, FFTPlan plan, const TW
                 for (int r = 0; r < 2; ++r) {
                     cx<T> ga_ = A[r], gb_ = Bv[r];
                     if (m == 0) { ga_.y = T(0); gb_.y = T(0); }
-                    cx<T>* z = buf + (r * NBUF + sgi) * M;
-                    z[m] = {ga_.x - gb_.y, ga_.y + gb_.x};
-                    if (m > 0 && m <= N) z[M - m] = {ga_.x + gb_.y, gb_.x - ga_.y};
+                    cx<T>* z = sm + r * rs + sgi * ls;
+                    z[rpad(m)] = {ga_.x - gb_.y, ga_.y + gb_.x};
+                    if (m > 0 && m <= N) z[rpad(M - m)] = {ga_.x + gb_.y, gb_.x - ga_.y};
                 }
             }
         }
         __syncthreads();
-        fft<T, T, MODE == RING_ADJOINT ? 3 : 2>(src, plan, tws, +1, rt, nt);
+        cur = fft<T, +1>(sm, cur, 2 * rs - cur, nsig, rs, plan, tws);
     }
 
-    if constexpr (MODE == RING_GRID) {
-        if (!live) return;
-        for (int q = rt; q < M; q += nt) {
-            if (a.gout0) a.gout0[size_t(row) * M + q] = double(src[0][q].x);
-            if (a.gout1) a.gout1[size_t(row) * M + q] = double(src[0][q].y);
-            if (a.gout2) a.gout2[size_t(row) * M + q] = double(src[1][q].x);
+    // point q of ring r, both rings over the CTA's threads
+    auto points = [&](auto&& f) {
+        for (int u = threadIdx.x; u < 2 * M; u += blockDim.x) {
+            const int r = u >= M, q = u - r * M;
+            f(r, q, sm + cur + r * rs + rpad(q));
         }
+    };
+    if constexpr (MODE == RING_GRID) {
+        points([&](int r, int q, const cx<T>* z) {
+            if (r && !two) return;
+            const size_t o = size_t(row0 + r) * M + q;
+            if (a.gout0) a.gout0[o] = double(z[0].x);
+            if (a.gout1) a.gout1[o] = double(z[0].y);
+            if (a.gout2) a.gout2[o] = double(z[ls].x);
+        });
         return;
     }
 
     constexpr int nout = MODE == RING_ADJOINT ? 2 : 1;
+    const T fc0 = T(a.two_omega * a.x[row0]), fc1 = T(a.two_omega * a.x[min(row0 + 1, nlat - 1)]);
     if constexpr (MODE == RING_RHS) {
-        const T fc = T(a.two_omega * a.x[min(row, nlat - 1)]);
-        for (int q = rt; q < M; q += nt) {
-            const T zeta = src[0][q].x, uth = src[0][q].y, uph = src[1][q].x;
-            const T qq = zeta + fc;
-            src[0][q] = {-qq * uph, qq * uth};
-        }
+        points([&](int r, int q, cx<T>* z) {
+            const T zeta = z[0].x, uth = z[0].y, uph = z[ls].x;
+            const T qq = zeta + (r ? fc1 : fc0);
+            z[0] = {-qq * uph, qq * uth};
+        });
     } else if constexpr (MODE == RING_PROJECT) {
-        for (int q = rt; q < M; q += nt)
-            src[0][q] = live ? cx<T>{T(a.gin0[size_t(row) * M + q]), T(a.gin1[size_t(row) * M + q])} : cx<T>{T(0), T(0)};
+        points([&](int r, int q, cx<T>* z) {
+            const size_t o = size_t(row0 + r) * M + q;
+            z[0] = r && !two ? cx<T>{T(0), T(0)} : cx<T>{T(a.gin0[o]), T(a.gin1[o])};
+        });
     } else {  // RING_ADJOINT: fields zeta, u_th, u_ph, v_th, v_ph
-        const T fc = T(a.two_omega * a.x[min(row, nlat - 1)]);
-        for (int q = rt; q < M; q += nt) {
-            const T zeta = src[0][q].x, uth = src[0][q].y;
-            const T uph = src[1][q].x, vth = src[1][q].y, vph = src[2][q].x;
-            const T qq = zeta + fc;
+        points([&](int r, int q, cx<T>* z) {
+            const T zeta = z[0].x, uth = z[0].y;
+            const T uph = z[ls].x, vth = z[ls].y, vph = z[2 * ls].x;
+            const T qq = zeta + (r ? fc1 : fc0);
             // X = -q xhat x v = (q v_phi, -q v_theta); rho = v . (xhat x u) = -v_th u_ph + v_ph u_th
-            src[0][q] = {qq * vph, -qq * vth};
-            src[1][q] = {-vth * uph + vph * uth, T(0)};
-        }
+            z[0] = {qq * vph, -qq * vth};
+            z[ls] = {-vth * uph + vph * uth, T(0)};
+        });
     }
     __syncthreads();
-    fft<T, T, nout>(src, plan, tws, -1, rt, nt);
+    cur = fft<T, -1>(sm, cur, 2 * rs - cur, nout, rs, plan, tws);
 
     // both rings of order m at once: two latitudes are 16 bytes of the order-major output
-    const int row0 = 2 * pair;
     T scale[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) scale[r] = T(a.rw[min(row0 + r, nlat - 1)]);
@@ -226,9 +236,9 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, FFTPlan plan, const TW
         cx<T> oA[2], oB[2], oC[2];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            const cx<T>* Z = buf + r * NBUF * M;
-            const cx<T> p = Z[m];
-            const cx<T> q = Z[(M - m) % M];
+            const cx<T>* Z = sm + cur + r * rs;
+            const cx<T> p = Z[rpad(m)];
+            const cx<T> q = Z[rpad(m == 0 ? 0 : M - m)];
             // W = A + i B with A, B real fields: A_m = (Z_m + conj Z_{M-m}) / 2,
             // B_m = (Z_m - conj Z_{M-m}) / (2 i)
             cx<T> A{T(0.5) * (p.x + q.x), T(0.5) * (p.y - q.y)};
@@ -238,7 +248,7 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, FFTPlan plan, const TW
             if constexpr (nout == 2) {
                 // scalar field rho: plain quadrature weight (2 pi / M) w_p
                 const T sc2 = scale[r] * T(a.s[min(row0 + r, nlat - 1)]);
-                const cx<T> z = Z[M + m];
+                const cx<T> z = Z[ls + rpad(m)];
                 oC[r] = {z.x * sc2, z.y * sc2};
             }
         }
@@ -251,11 +261,11 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, FFTPlan plan, const TW
 template <typename T, typename TW, int MODE>
 static void ring_t(sphnse_plan* P, RingArgs a, const TW* tw, int nb = 1) {
     const int nbuf = MODE == RING_ADJOINT ? 3 : (MODE == RING_PROJECT ? 1 : 2);
-    // in-place stages need M / 6 threads per ring (at most 3 butterflies per thread)
-    const int threads = 2 * (((P->nlon / 6 + 31) / 32) * 32);
-    const size_t sm = size_t(2 * nbuf) * P->nlon * sizeof(cx<T>) + size_t(P->nlon) * 2 * sizeof(T);
+    // a radix-8 butterfly of the inverse signals per thread
+    const int threads = std::min(512, std::max(64, (2 * nbuf * P->nlon / 8 + 31) / 32 * 32));
+    const size_t sm = size_t(4 * nbuf) * ring_stride(P->nlon) * sizeof(cx<T>) + size_t(P->nlon) * 2 * sizeof(T);
     allow_dynamic_smem(reinterpret_cast<const void*>(k_ring<T, TW, MODE>), sm);
-    a.early = long(P->nlat + 1) / 2 * nb <= long(P->nsm) * (512 / threads);
+    a.early = long(P->nlat + 1) / 2 * nb <= long(P->nsm) * std::min<long>(512 / threads, (227 << 10) / long(sm + 1024));
     launch_pdl(k_ring<T, TW, MODE>, dim3((P->nlat + 1) / 2, nb), dim3(threads), sm, P->stream, a, P->fft, tw);
 }
 
