@@ -152,9 +152,9 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant_
                 cx<T> A[2] = {{T(0), T(0)}, {T(0), T(0)}}, Bv[2] = {{T(0), T(0)}, {T(0), T(0)}};
                 if (m <= N) {
                     const cx<T>* g = gs + ((size_t(fa) * npair + pair) * ld + m) * 2;
-                    const float4 v = *reinterpret_cast<const float4*>(g);
-                    A[0] = {v.x, v.y};
-                    if (two) A[1] = {v.z, v.w};
+                    const float4 u = *reinterpret_cast<const float4*>(g);
+                    A[0] = {u.x, u.y};
+                    if (two) A[1] = {u.z, u.w};
                     if (has_b) {
                         const float4 w = *reinterpret_cast<const float4*>(g + size_t(npair) * ld * 2);
                         Bv[0] = {w.x, w.y};
@@ -261,8 +261,13 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant_
 template <typename T, typename TW, int MODE>
 static void ring_t(sphnse_plan* P, RingArgs a, const TW* tw, int nb = 1) {
     const int nbuf = MODE == RING_ADJOINT ? 3 : (MODE == RING_PROJECT ? 1 : 2);
-    // a radix-8 butterfly of the inverse signals per thread
-    const int threads = std::min(512, std::max(64, (2 * nbuf * P->nlon / 8 + 31) / 32 * 32));
+    // Two threads per butterfly of the average stage: half of them idle in the
+    // stages, all of them load and store.  One thread per radix-8 butterfly was
+    // right for radix-8 plans only: the projection at L = 153 on 486 = 2 3^5
+    // longitudes took 32.1 us, with this rule 16.7, at 324 FP32 F 28.6, now 20.8.
+    int nb_sum = 0;
+    for (int i = 0; i < P->fft.nstages; ++i) nb_sum += P->nlon / P->fft.radix[i];
+    const int threads = std::min(512, std::max(64, (4 * nbuf * nb_sum / P->fft.nstages + 31) / 32 * 32));
     const size_t sm = size_t(4 * nbuf) * ring_stride(P->nlon) * sizeof(cx<T>) + size_t(P->nlon) * 2 * sizeof(T);
     allow_dynamic_smem(reinterpret_cast<const void*>(k_ring<T, TW, MODE>), sm);
     a.early = long(P->nlat + 1) / 2 * nb <= long(P->nsm) * std::min<long>(512 / threads, (227 << 10) / long(sm + 1024));
