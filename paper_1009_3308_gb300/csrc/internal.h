@@ -51,6 +51,21 @@ __host__ __device__ inline size_t gsyn_index(int pairs, int f, int m, int row, i
 // of them), split by the parity of K - m: even rows first (K = m + 2j,
 // j < ne(m)), then odd rows (K = m + 1 + 2j, j < no(m)).  Degree N+1 is needed
 // by the theta-derivative recombination.
+// sum of a 256-thread block's values (a tree, fixed order) into part[blockIdx.x];
+// every thread of the block calls it
+__device__ __forceinline__ void block_sum256(double s, double* part) {
+#ifdef __CUDA_ARCH__
+    __shared__ double red[256];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+#endif
+}
+
 __host__ __device__ inline int ext_off(int N, int m) { return m * (N + 2) - m * (m - 1) / 2; }
 __host__ __device__ inline int ext_count(int N, int m) { return N + 2 - m; }
 __host__ __device__ inline int ext_even(int N, int m) { return (N + 3 - m) / 2; }
@@ -281,6 +296,7 @@ struct sphnse_plan {
     unsigned* d_status = nullptr;  // device status word (bounded-wait timeouts)
     unsigned long long* d_norms = nullptr;  // 8 reduction slots
     double* h_norms = nullptr;   // pinned host mirror
+    double* h_part = nullptr;    // block partial sums, pinned: kernels write them, the host adds them up
     size_t work_bytes = 0;
 
     // optional per-stage CUDA-event timing on the plan's stream
@@ -344,15 +360,21 @@ int launch_analysis_dig(sphnse_plan* P, int nf);
 constexpr int SMALL_NH = 40;
 inline bool small_plan(int nh) { return nh <= SMALL_NH; }
 int launch_synthesis_small(sphnse_plan* P, const double* alpha, const double* beta);
-int launch_analysis_small(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out);
+int launch_analysis_small(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out,
+                          const double* dot_with = nullptr);
 // the FP64 ring kernel (64-bit fixed point) on the latitude-pair-major buffers
 std::vector<int> ring_fx_twiddles(int nlon);
 int launch_ring_fx(sphnse_plan* P, int mode, const double* gin0, const double* gin1, double* gout0, double* gout1,
                    double* gout2);
+// number of partial sums of <lambda alpha, w> that rhs_adjoint_device leaves
+inline int adjoint_parts(int precision, int nh, int N, int n) {
+    return precision == SPHNSE_FP64 && small_plan(nh) ? N + 1 : (n + 255) / 256;
+}
 // finish: kind 0 = RHS (F = f - nu lam alpha - N), 1 = projection (N),
-// 2 = adjoint (out = -nu lam w - s_m (N_X + lam^{1/2} H_rho))
+// 2 = adjoint (out = -nu lam w - s_m (N_X + lam^{1/2} H_rho)); with dot_with
+// (kind 2) also the partial sums of <lambda dot_with, alpha> into h_part
 int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha,
-                  const double* forcing, double* out);
+                  const double* forcing, double* out, const double* dot_with = nullptr);
 
 int ensure_tables(sphnse_plan* P, int prec);
 bool stream_ok(const sphnse_plan* P);
@@ -453,6 +475,7 @@ inline cudaError_t launch_pdl_small(int n_sm, void (*kernel)(KArgs...), dim3 gri
 
 // whole pipelines
 int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, double* out);
-int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out);
+// parts: also the adjoint_parts() partial sums of <lambda alpha, w> into h_part
+int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out, bool parts = false);
 
 }  // namespace sph

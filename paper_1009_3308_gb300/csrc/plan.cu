@@ -7,6 +7,7 @@
 #include <unordered_map>
 #include <unordered_set>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -159,10 +160,11 @@ void prefer_max_smem(const void* kernel) {
 static int synthesis64(sphnse_plan* P, const double* alpha, const double* beta) {
     return small_plan(P->nh) ? launch_synthesis_small(P, alpha, beta) : launch_synthesis_dig(P, alpha, beta);
 }
-static int analysis64(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out) {
-    if (small_plan(P->nh)) return launch_analysis_small(P, kind, alpha, forcing, out);
+static int analysis64(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out,
+                      const double* dot_with = nullptr) {
+    if (small_plan(P->nh)) return launch_analysis_small(P, kind, alpha, forcing, out, dot_with);
     const int rc = launch_analysis_dig(P, kind == 2 ? 3 : 2);
-    return rc ? rc : launch_finish(P, kind, SPHNSE_FP64, alpha, forcing, out);
+    return rc ? rc : launch_finish(P, kind, SPHNSE_FP64, alpha, forcing, out, dot_with);
 }
 
 int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, double* out) {
@@ -197,18 +199,19 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
 // J(alpha)^T w = -nu lambda w - D_s ( A_u[-(zeta + f) xhat x V] + A_zeta[(xhat x u) . V] ),
 // V = S_u(D_s^{-1} w): the transpose of the linearised product, with the
 // synthesis transpose S^T = D_s A W^{-1} (A the weighted analysis).
-int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out) {
+int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out, bool parts) {
+    const double* dot_with = parts ? alpha : nullptr;
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     int rc;
     if (prec == SPHNSE_FP64) {
         if ((rc = synthesis64(P, alpha, w))) return rc;
         if ((rc = launch_ring_fx(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
-        return analysis64(P, 2, w, nullptr, out);
+        return analysis64(P, 2, w, nullptr, out, dot_with);
     }
     if ((rc = launch_synthesis32(P, alpha, w, 1))) return rc;
     if ((rc = launch_ring(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
     if ((rc = launch_analysis(P, 3))) return rc;
-    return launch_finish(P, 2, prec, w, nullptr, out);
+    return launch_finish(P, 2, prec, w, nullptr, out, dot_with);
 }
 
 }  // namespace sph
@@ -370,8 +373,11 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
     if (!rc) rc = dalloc(&P->d_work, 16 * nc * 2 * sizeof(double));
     if (!rc) rc = dalloc(&P->d_tmp, 2 * nc * 2 * sizeof(double));
     if (!rc) rc = dalloc(&P->d_norms, 16 * sizeof(unsigned long long));
-    if (!rc && cudaMallocHost(reinterpret_cast<void**>(&P->h_norms), 16 * sizeof(double)) != cudaSuccess)
+    // 16 slots, then one partial sum per block of 256 coefficients, per order or per latitude
+    const size_t nparts = std::max({size_t(nc + 255) / 256, size_t(P->N) + 1, size_t(nlat)});
+    if (!rc && cudaMallocHost(reinterpret_cast<void**>(&P->h_norms), (16 + nparts) * sizeof(double)) != cudaSuccess)
         rc = SPHNSE_E_NOMEM;
+    if (!rc) P->h_part = P->h_norms + 16;
     auto up = [&](void* d, const void* h, size_t b) {
         if (!rc && cudaMemcpy(d, h, b, cudaMemcpyHostToDevice) != cudaSuccess) rc = SPHNSE_E_CUDA;
     };
