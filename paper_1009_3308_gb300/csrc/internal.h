@@ -475,7 +475,10 @@ inline cudaError_t launch_pdl_small(int n_sm, void (*kernel)(KArgs...), dim3 gri
 
 // whole pipelines
 int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, double* out);
-// parts: also the adjoint_parts() partial sums of <lambda alpha, w> into h_part
-int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out, bool parts = false);
+// parts: also the adjoint_parts() partial sums of <lambda alpha, w> into h_part;
+// same_alpha: the last use of the plan's buffers was this function with this
+// alpha (the spectra of alpha's fields are still in d_gsyn)
+int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out, bool parts = false,
+                       bool same_alpha = false);
 
 }  // namespace sph

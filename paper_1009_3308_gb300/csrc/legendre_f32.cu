@@ -53,9 +53,10 @@ struct F32Args {
 
 constexpr int F32_U = 16;   // table rows in flight per thread
 
+// NF = 3: the fields of alpha; 5: and the two of beta; 2: those of beta alone
 template <int NF>
 __global__ void __launch_bounds__(128) k_syn32(F32Args a) {
-    constexpr int C = 2 * NF, LD = (C + 3) / 4 * 4;   // coefficient rows padded to 16 bytes
+    constexpr int NA = NF == 2 ? 0 : 3, C = 2 * NF, LD = (C + 3) / 4 * 4;   // coefficient rows padded to 16 bytes
     extern __shared__ __align__(16) float sm32[];
     const int N = a.N, nh = a.nh, nlat = a.nlat, m = blockIdx.y, tid = threadIdx.x;
     const int ne = ext_even(N, m), no = ext_odd(N, m), cnt = ne + no, e0 = ext_off(N, m);
@@ -84,19 +85,21 @@ __global__ void __launch_bounds__(128) k_syn32(F32Args a) {
                 const double2 x = v[pk + Kp];
                 return make_float2(f64_to_f32_rn(x.x) * scale, f64_to_f32_rn(x.y) * scale);
             };
-            const float2 a0 = ld(a.alpha, K, 1.f), am = ld(a.alpha, K - 1, 1.f), ap = ld(a.alpha, K + 1, 1.f);
-            out[0] = c.x * a0.x;
-            out[1] = c.x * a0.y;
-            out[2] = c.y * a0.x;
-            out[3] = c.y * a0.y;
-            out[4] = fmaf(c.z, am.x, c.w * ap.x);
-            out[5] = fmaf(c.z, am.y, c.w * ap.y);
-            if constexpr (NF == 5) {
+            if constexpr (NA == 3) {
+                const float2 a0 = ld(a.alpha, K, 1.f), am = ld(a.alpha, K - 1, 1.f), ap = ld(a.alpha, K + 1, 1.f);
+                out[0] = c.x * a0.x;
+                out[1] = c.x * a0.y;
+                out[2] = c.y * a0.x;
+                out[3] = c.y * a0.y;
+                out[4] = fmaf(c.z, am.x, c.w * ap.x);
+                out[5] = fmaf(c.z, am.y, c.w * ap.y);
+            }
+            if constexpr (NF != 3) {
                 const float2 b0 = ld(a.beta, K, sc), bm = ld(a.beta, K - 1, sc), bp = ld(a.beta, K + 1, sc);
-                out[6] = c.y * b0.x;
-                out[7] = c.y * b0.y;
-                out[8] = fmaf(c.z, bm.x, c.w * bp.x);
-                out[9] = fmaf(c.z, bm.y, c.w * bp.y);
+                out[2 * NA] = c.y * b0.x;
+                out[2 * NA + 1] = c.y * b0.y;
+                out[2 * NA + 2] = fmaf(c.z, bm.x, c.w * bp.x);
+                out[2 * NA + 3] = fmaf(c.z, bm.y, c.w * bp.y);
             }
         }
     }
@@ -135,9 +138,10 @@ __global__ void __launch_bounds__(128) k_syn32(F32Args a) {
     if (p >= nh || (par && row == p)) return;
     const float mm = float(m);
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        const float gr = par ? other[2 * f] - acc[2 * f] : acc[2 * f] + other[2 * f];
-        const float gi = par ? other[2 * f + 1] - acc[2 * f + 1] : acc[2 * f + 1] + other[2 * f + 1];
+    for (int q = 0; q < NF; ++q) {
+        const float gr = par ? other[2 * q] - acc[2 * q] : acc[2 * q] + other[2 * q];
+        const float gi = par ? other[2 * q + 1] - acc[2 * q + 1] : acc[2 * q + 1] + other[2 * q + 1];
+        const int f = q + 3 - NA;
         float2 o;
         if (f == 0) o = make_float2(gr, gi);
         else if (f == 1 || f == 3) o = make_float2(-mm * gi * inv_s, mm * gr * inv_s);   // (i m / sin) g
@@ -267,6 +271,7 @@ static F32Args f32_args(sphnse_plan* P) {
     return a;
 }
 
+// without alpha, the fields of beta only (the others keep their values in d_gsyn)
 int launch_synthesis32(sphnse_plan* P, const double* alpha, const double* beta, int pairs) {
     F32Args a = f32_args(P);
     a.alpha = reinterpret_cast<const double2*>(alpha);
@@ -274,10 +279,12 @@ int launch_synthesis32(sphnse_plan* P, const double* alpha, const double* beta, 
     a.pairs = pairs;
     const dim3 grid((P->nh + 63) / 64, P->N + 1);
     a.early = int(grid.x * grid.y) <= 8 * P->nsm;
-    const size_t sm = (size_t(P->N + 2) * (beta ? 12 : 8) + 128 * (beta ? 10 : 6)) * sizeof(float);
+    const int C = (alpha ? 6 : 0) + (beta ? 4 : 0);
+    const size_t sm = (size_t(P->N + 2) * ((C + 3) / 4 * 4) + 128 * C) * sizeof(float);
     stage_begin(P, SPHNSE_STAGE_SYNTHESIS);
-    const cudaError_t e = beta ? launch_pdl(k_syn32<5>, grid, dim3(128), sm, P->stream, a)
-                               : launch_pdl(k_syn32<3>, grid, dim3(128), sm, P->stream, a);
+    const cudaError_t e = !alpha ? launch_pdl(k_syn32<2>, grid, dim3(128), sm, P->stream, a)
+                          : beta ? launch_pdl(k_syn32<5>, grid, dim3(128), sm, P->stream, a)
+                                 : launch_pdl(k_syn32<3>, grid, dim3(128), sm, P->stream, a);
     stage_end(P, SPHNSE_STAGE_SYNTHESIS);
     return check_cuda(e);
 }

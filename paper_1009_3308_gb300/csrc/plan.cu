@@ -199,7 +199,7 @@ int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, doubl
 // J(alpha)^T w = -nu lambda w - D_s ( A_u[-(zeta + f) xhat x V] + A_zeta[(xhat x u) . V] ),
 // V = S_u(D_s^{-1} w): the transpose of the linearised product, with the
 // synthesis transpose S^T = D_s A W^{-1} (A the weighted analysis).
-int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out, bool parts) {
+int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, double* out, bool parts, bool same_alpha) {
     const double* dot_with = parts ? alpha : nullptr;
     const int prec = P->precision == SPHNSE_FP64 ? SPHNSE_FP64 : SPHNSE_FP32;
     int rc;
@@ -208,7 +208,7 @@ int rhs_adjoint_device(sphnse_plan* P, const double* alpha, const double* w, dou
         if ((rc = launch_ring_fx(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
         return analysis64(P, 2, w, nullptr, out, dot_with);
     }
-    if ((rc = launch_synthesis32(P, alpha, w, 1))) return rc;
+    if ((rc = launch_synthesis32(P, same_alpha ? nullptr : alpha, w, 1))) return rc;
     if ((rc = launch_ring(P, RING_ADJOINT, nullptr, nullptr, nullptr, nullptr, nullptr))) return rc;
     if ((rc = launch_analysis(P, 3))) return rc;
     return launch_finish(P, 2, prec, w, nullptr, out, dot_with);
