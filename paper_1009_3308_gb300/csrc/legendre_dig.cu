@@ -2,10 +2,10 @@
 // digit splitting (the error-free splitting of matrix products of Ozaki,
 // Ogita, Oishi and Rump, Numer. Algorithms 59 (2012)).
 //
-// Every table row is scaled by a power of two to |a| < 1 and cut into seven
+// Every table row is scaled by a power of two to |a| < 0.993 and cut into seven
 // balanced base-256 digits, every coefficient (or profile) column to |b| <=
 // 1/2 and eight digits:  a = sum_i a_i 2^(1 - 8 i),  b = sum_j b_j 2^(1 - 8 j),
-// |a_i|, |b_j| <= 128.  Digits are exact in BF16, their products are integers
+// |a_i|, |b_j| <= 128.  Digits are exact in FP16, their products are integers
 // of at most 2^14, and sums over the contracted index stay below 2^24 in the
 // leading groups, so the tensor core's FP32 accumulators hold them exactly.
 // The products of i + j = s share one accumulator group, s = 2 .. 9 (synthesis:
@@ -19,28 +19,35 @@
 // table against digits 1 .. 9 - i (10 - i) of the columns (N = G (9 - i), G
 // columns per group): with the columns of a group adjacent, those digits are a prefix of
 // the B rows and land on the groups from i + 1 on, a contiguous run of accumulator
-// columns.  The table digits are laid out once per plan in the order the
-// kernels consume them: one 28 KB block per (tile, K step) = 7 planes of 128 x
-// 16 in the un-swizzled core-matrix layout, so a stage is one bulk copy and
-// blocks whose digits are all zero (polar latitudes at high order) are left
-// out.
+// columns.  The table digits are stored once per plan as bytes (digit + 128) in
+// the order the kernels consume them: one 14 KB block per (tile, K step) = 7
+// planes of 128 x 16, one bulk copy each; blocks whose digits are all zero
+// (polar latitudes at high order) are left out.  Four warps expand a block to
+// FP16 (a byte under 0x64 is 1024 + byte; one packed subtraction) straight into
+// tensor memory, where the MMAs take their A operand: written to shared memory
+// instead, the expanded digits cost more than the halved HBM stream saved (L =
+// 511 synthesis 154 us, analysis 107, against 138 and 108 of digits stored in
+// 16 bits).
 //
-// Bound: HBM.  14 bytes per table entry against 8 of the FP64 table, but the
-// FP64 pipe (two operations per clock per SM) needs 10 multiply-adds per entry
-// and RHS: 0.8 ms at L = 511, where the two digit streams take 0.22 ms.
+// Bound: the single-K-step stages, whose barrier waits (150 to 200 cycles even
+// when they pass at once), expansion and MMAs (300 to 400 cycles) leave 870
+// cycles per stage; 7 bytes per table entry stream in 570 at full HBM rate.  The
+// FP64 pipe (two operations per clock per SM) would need 10 multiply-adds per
+// entry and RHS: 0.8 ms at L = 511.
 // Measured (event pairs, GB300) against the FP64 multiply-add kernels and their
-// prep: L = 511 synthesis 558 -> 137 us, analysis 429 -> 111 us; L = 255 96 ->
-// 35, 74 -> 27; L = 100 41 -> 16, 22 -> 12; L = 31 21 -> 13, 10 -> 10.  Errors
-// against 64-bit references are those of the multiply-add kernels or smaller
-// for F, the fields and the projection at 23 sizes (mean over 24 states: u_phi
-// 3.3e-15 and u_theta 8.5e-16 at L = 255, before 3.4e-15 and 1.1e-15).
+// prep, and against 16-bit stored digits: L = 511 synthesis 558 -> 138 -> 100 us,
+// analysis 429 -> 108 -> 78; L = 255 96 -> 37 -> 33, 74 -> 27 -> 21; L = 100
+// 41 -> 17 -> 16, 22 -> 12 -> 12.  Errors against 64-bit references are those of
+// the multiply-add kernels or smaller for F, the fields and the projection at 23
+// sizes (mean over 24 states: u_phi 3.3e-15 and u_theta 8.5e-16 at L = 255,
+// before 3.4e-15 and 1.1e-15).
 //
 // Synthesis tiles: rows 0 .. 63 the even, rows 64 .. 127 the odd degrees of one
 // order on 64 northern latitudes (columns 0 .. G/2-1 of a group belong to the
 // even, the others to the odd degrees), so north = E + O and south = E - O
 // meet in one epilogue.  Analysis tiles: four pieces of up to 32 rows of one
 // (order, parity), one per epilogue warp, each with its own G / 4 columns.
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -54,9 +61,10 @@
 
 namespace sph {
 
-constexpr int DG_PLANE = 128 * 16 * 2;       // 4 KB: 128 rows x 16 of the contracted index
-constexpr int DG_ABYTES = 7 * DG_PLANE;      // one stage of table digits
-constexpr int DG_NB = 6;                     // builder warps
+constexpr int DG_RPLANE = 128 * 16;          // a digit of 128 rows x 16 of the contracted index: bytes digit + 128
+constexpr int DG_RBYTES = 7 * DG_RPLANE;     // one block of the stored table
+constexpr int DG_ACOLS = 7 * 8;              // the same in FP16: columns of tensor memory, a row per lane
+constexpr int DG_NX = 4;                     // stages of it
 constexpr int DG_MINEXP = -30;               // row scales are at least 2^-30 (smaller rows lose digits below 2^-86)
 // Orders below DG_SEGM take their first K step (the lowest degrees) apart,
 // with its own row exponents and with the remainder that its seven digits
@@ -69,19 +77,26 @@ constexpr int DG_MINEXP = -30;               // row scales are at least 2^-30 (s
 constexpr int DG_SEGM = 8;
 constexpr int DG_NAN = 1 << 20;              // exponent of a column with a non-finite entry
 
-// byte offset of element (row, k) of a K = 16 tile: 8 x 8 core matrices of 128
-// bytes, the two of a row group adjacent
+// byte offset of element (row, k) of a K = 16 tile: rows of 32 bytes, the two
+// halves swapped in every second group of four rows (32-byte swizzle)
 __host__ __device__ constexpr int dg_off(int row, int k) {
-    return (row >> 3) * 256 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
+    return row * 32 + (((k >> 3) ^ (row >> 2)) & 1) * 16 + (k & 7) * 2;
 }
-// shared-memory descriptor of that layout: K-major, no swizzle
+// shared-memory descriptor of that layout: K-major, 32-byte swizzle
 __device__ __forceinline__ uint64_t dg_desc(const void* smem_ptr) {
     uint64_t d = 0;
     d |= uint64_t((smem_u32(smem_ptr) & 0x3FFFF) >> 4);
-    d |= uint64_t(128 >> 4) << 16;   // to the next core matrix along K
+    d |= uint64_t(1) << 16;          // leading byte offset (unused with swizzle)
     d |= uint64_t(256 >> 4) << 32;   // to the next 8 rows
     d |= uint64_t(1) << 46;
+    d |= uint64_t(6) << 61;          // 32-byte swizzle
     return d;
+}
+
+// two bytes digit + 128 under 0x64 are the FP16 numbers 1152 + digit
+__device__ __forceinline__ uint32_t dg_half2(uint32_t w) {
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480)));
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 __device__ __forceinline__ int dg_steps(int n) { return (n + 15) / 16; }
@@ -89,8 +104,9 @@ __device__ __forceinline__ int dg_steps(int n) { return (n + 15) / 16; }
 // ---------------------------------------------------------------------------
 // table digits (once per plan)
 
-// row exponents: |P| < 2^e over a row.  Synthesis rows are (m, latitude p)
+// row exponents: |P| < (1 - 2^-7) 2^e over a row, so that the top digit stays below 128.  Synthesis rows are (m, latitude p)
 // over all degrees of the order, analysis rows are the ext rows over p.
+__device__ __forceinline__ int dg_bexp(double x) { return f64_bexp(fma(x, 0x1p-7, x)); }
 __global__ void k_dig_syn_scale(const double* __restrict__ tab, int* __restrict__ ea, int N, int nh) {
     const int m = blockIdx.y, p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= nh) return;
@@ -98,7 +114,7 @@ __global__ void k_dig_syn_scale(const double* __restrict__ tab, int* __restrict_
     const double* t = tab + size_t(ext_off(N, m)) * nh + p;
     int e0 = 0, e1 = 0;   // first step, later steps
     for (int r = 0; r < cnt; ++r) {
-        const int b = f64_bexp(t[size_t(r) * nh]);
+        const int b = dg_bexp(t[size_t(r) * nh]);
         if ((r < ne ? r : r - ne) < 16) e0 = max(e0, b);
         else e1 = max(e1, b);
     }
@@ -110,34 +126,25 @@ __global__ void k_dig_ana_scale(const double* __restrict__ tab, int* __restrict_
     const int r = blockIdx.x * 4 + threadIdx.x / 32;
     if (r >= n_ext) return;
     int e = 0;
-    for (int p = threadIdx.x & 31; p < nh; p += 32) e = max(e, f64_bexp(tab[size_t(r) * nh + p]));
+    for (int p = threadIdx.x & 31; p < nh; p += 32) e = max(e, dg_bexp(tab[size_t(r) * nh + p]));
     e = __reduce_max_sync(0xffffffffu, e);
     if ((threadIdx.x & 31) == 0) ea[r] = max(e - 1022, DG_MINEXP);
 }
 
-// seven digits of eight scaled entries -> one 16-byte chunk per plane; returns whether any is nonzero
+// seven digits of eight scaled entries -> eight bytes of each plane; returns whether any is nonzero
 __device__ __forceinline__ bool dig_store(const double (&x)[8], const int (&e)[8], unsigned char* dst) {
-    long long u[8];
+    unsigned long long w[7] = {0, 0, 0, 0, 0, 0, 0};
     bool any = false;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const long long v = f64_to_fx(x[i], 55 - e[i]);
         any = any || v != 0;
-        u[i] = v + 0x0080808080808080LL;
+        const unsigned long long u = (unsigned long long)v + 0x0080808080808080ULL;
+#pragma unroll
+        for (int d = 0; d < 7; ++d) w[d] |= ((u >> (48 - 8 * d)) & 255) << (8 * i);
     }
 #pragma unroll
-    for (int d = 0; d < 7; ++d) {
-        uint32_t w[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            // the top digit may reach +128: not masked to a byte
-            const int a = int(u[2 * i] >> (48 - 8 * d)), b = int(u[2 * i + 1] >> (48 - 8 * d));
-            const float fa = float((d == 0 ? a : a & 255) - 128), fb = float((d == 0 ? b : b & 255) - 128);
-            const __nv_bfloat162 h = __floats2bfloat162_rn(fa, fb);
-            w[i] = *reinterpret_cast<const uint32_t*>(&h);
-        }
-        *reinterpret_cast<uint4*>(dst + d * DG_PLANE) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
+    for (int d = 0; d < 7; ++d) *reinterpret_cast<unsigned long long*>(dst + d * DG_RPLANE) = w[d];
     return any;
 }
 
@@ -164,7 +171,7 @@ __global__ void __launch_bounds__(256) k_dig_syn(const double* __restrict__ tab,
         }
     }
     const int blk = base[m * ntile + t] + ks;
-    const bool any = dig_store(x, e, out + size_t(blk) * DG_ABYTES + dg_off(row, h * 8));
+    const bool any = dig_store(x, e, out + size_t(blk) * DG_RBYTES + row * 16 + h * 8);
     if (__syncthreads_or(any) && threadIdx.x == 0) used[blk] = 1;
 }
 __global__ void __launch_bounds__(256) k_dig_ana(const double* __restrict__ tab, const int* __restrict__ ea,
@@ -184,14 +191,14 @@ __global__ void __launch_bounds__(256) k_dig_ana(const double* __restrict__ tab,
         e[i] = in ? ea[r] : 0;
     }
     const int blk = tile * nks + ks;
-    const bool any = dig_store(x, e, out + size_t(blk) * DG_ABYTES + dg_off(row, h * 8));
+    const bool any = dig_store(x, e, out + size_t(blk) * DG_RBYTES + row * 16 + h * 8);
     if (__syncthreads_or(any) && threadIdx.x == 0) used[blk] = 1;
 }
 
 // ---------------------------------------------------------------------------
 
 struct DigArgs {
-    const unsigned char* blocks;  // table digits, DG_ABYTES per (tile, step)
+    const unsigned char* blocks;  // table digits, DG_RBYTES per (tile, step)
     const int4* items;            // (m | flags (or analysis tile), latitude tile, first step | end
                                   //  step << 16, first block); flags of the parts of a split item: bit 16
                                   //  another part follows, 17 exponents of the later steps, 18 a part
@@ -224,12 +231,9 @@ __device__ __forceinline__ void dig_put(unsigned char* dst, int stride, long lon
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const uint32_t s0 = j < 4 ? uint32_t(u0 >> 32) : uint32_t(u0), s1 = j < 4 ? uint32_t(u1 >> 32) : uint32_t(u1);
-        // 2^23 + byte, minus 2^23 + 128
-        const int sel = 0x7650 | (3 - (j & 3));
-        const float f0 = __uint_as_float(__byte_perm(s0, 0x4B000000u, sel)) - 8388736.f;
-        const float f1 = __uint_as_float(__byte_perm(s1, 0x4B000000u, sel)) - 8388736.f;
-        const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
-        *reinterpret_cast<uint32_t*>(dst + j * stride) = *reinterpret_cast<const uint32_t*>(&h);
+        const int q = 3 - (j & 3);
+        const uint32_t w = __byte_perm(s0, s1, q | (4 + q) << 8);   // bytes 0 and 2
+        *reinterpret_cast<uint32_t*>(dst + j * stride) = dg_half2(__byte_perm(w, 0x64646464u, 0x4240));
     }
 }
 
@@ -251,6 +255,18 @@ __device__ __forceinline__ double dig_val(const uint32_t* d, int stride, int e) 
     return v == 0 ? 0.0 : f64_scale(__ll2double_rn(v), e - 54 - sh);
 }
 
+// position in a ring of n slots: slot and the parity of its uses
+struct DigRing {
+    int slot = 0;
+    uint32_t phase = 0;
+    __device__ __forceinline__ void next(int n) {
+        if (++slot == n) {
+            slot = 0;
+            phase ^= 1;
+        }
+    }
+};
+
 template <bool SYN, int NF> struct DigShape {
     // columns of one order and parity, padded; group width; pipeline stages
     static constexpr int C = 2 * NF;
@@ -262,33 +278,43 @@ template <bool SYN, int NF> struct DigShape {
     // matters is well below max|a| max|b| (and is then divided by sin(theta))
     static constexpr int NG = SYN ? 9 : 8;
     static constexpr int BBYTES = NG * G * 32;               // eight digits of the columns, SYN: a zero digit
-    static constexpr int NACC = 2 * NG * G <= 512 ? 2 : 1;   // accumulator buffers
-    static constexpr int TCOLS = NACC * NG * G <= 256 ? 256 : 512;
-    static constexpr int NS = G == 16 ? 6 : 5;
+    static constexpr int NACC = 2 * NG * G + DG_NX * DG_ACOLS <= 512 ? 2 : 1;   // accumulator buffers
+    static_assert(NACC * NG * G + DG_NX * DG_ACOLS <= 512, "tensor memory");
+    // ring of stored table blocks (what is in flight from memory) and of column digits
+    static constexpr int NR = SYN && G == 32 ? 8 : 10;
+    static constexpr int NS = SYN ? (NF == 3 ? 9 : 6) : (NF == 2 ? 10 : 6);
     static constexpr int XCH = SYN ? 2 * 128 * C * 8 : 0;   // even and odd sums meet here
-    static constexpr int WARPS = 6 + DG_NB + (SYN ? 1 : 0);
+    // Copy, MMA, 4 epilogue, builder, 4 expander warps, and SYN: column exponents.
+    // A builder takes 4000 to 6000 cycles per stage (load latency, FP64 and 64-bit
+    // integer chains), so there are as many as the registers allow: 20 warps of 96,
+    // where that does not spill, else 16 of 128.
+    static constexpr int NB = SYN ? (NF == 3 ? 9 : 5) : (NF == 2 ? 10 : 6);
+    static constexpr int WARPS = 10 + NB + (SYN ? 1 : 0);
     static constexpr size_t smem(int istride) {
-        return 1024 + size_t(NS) * (DG_ABYTES + BBYTES) + XCH + 512 + size_t(istride) * (16 + 8 + 20);
+        return 1024 + size_t(NR) * DG_RBYTES + size_t(NS) * BBYTES + XCH + 512 + size_t(istride) * (16 + 8 + 20);
     }
 };
 
 template <bool SYN, int NF>
 __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArgs a) {
     using Q = DigShape<SYN, NF>;
-    constexpr int NS = Q::NS, G = Q::G, C = Q::C, CP = Q::CP, NG = Q::NG, NACC = Q::NACC;
-    static_assert(DG_NB >= NS, "every stage of the ring has a builder");
-    constexpr int NBW = NS;   // builders may not run a full ring ahead (one stage each)
+    constexpr int NS = Q::NS, NR = Q::NR, NX = DG_NX, G = Q::G, C = Q::C, CP = Q::CP, NG = Q::NG, NACC = Q::NACC;
+    static_assert(8 * (2 * (NR + NX + NS) + 4) + 8 <= 512, "barriers");
+    constexpr int NB = Q::NB, NBW = NS < NB ? NS : NB;   // a builder per stage, none a full ring ahead
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~uintptr_t(1023));
-    unsigned char* As = smem;
-    unsigned char* Bs = As + NS * DG_ABYTES;
+    unsigned char* Rs = smem;
+    unsigned char* Bs = Rs + NR * DG_RBYTES;
     double* xch = reinterpret_cast<double*>(Bs + NS * Q::BBYTES);
     uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(xch) + Q::XCH);
-    uint64_t* a_full = bars;
-    uint64_t* b_full = a_full + NS;
-    uint64_t* empty = b_full + NS;
-    uint64_t* acc_full = empty + NS;
+    uint64_t* r_full = bars;
+    uint64_t* r_empty = r_full + NR;
+    uint64_t* a_full = r_empty + NR;
+    uint64_t* a_empty = a_full + NX;
+    uint64_t* b_full = a_empty + NX;
+    uint64_t* b_empty = b_full + NS;
+    uint64_t* acc_full = b_empty + NS;
     uint64_t* acc_empty = acc_full + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -306,10 +332,17 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
         reinterpret_cast<uint4*>(Bs)[i] = make_uint4(0u, 0u, 0u, 0u);
     fence_proxy_async_smem();
     if (threadIdx.x == 0) {
+        for (int s = 0; s < NR; ++s) {
+            mbar_init(&r_full[s], 1);
+            mbar_init(&r_empty[s], 4);
+        }
+        for (int s = 0; s < NX; ++s) {
+            mbar_init(&a_full[s], 4);
+            mbar_init(&a_empty[s], 1);
+        }
         for (int s = 0; s < NS; ++s) {
-            mbar_init(&a_full[s], 1);
             mbar_init(&b_full[s], 1);
-            mbar_init(&empty[s], 1);
+            mbar_init(&b_empty[s], 1);
         }
         for (int b = 0; b < NACC; ++b) {
             mbar_init(&acc_full[b], 1);
@@ -319,38 +352,38 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
     }
     fence_barrier_init();
     if (warp == 1) {
-        tmem_alloc(tmem_slot, Q::TCOLS);
+        tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     pdl_launch();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = *tmem_slot, tmemA = tmem + NACC * NG * G;
 
     if (warp == 0) {
         if (elect_one()) {
             // the table does not depend on the predecessor: stream right away
             const uint64_t pol = a.evict_first ? policy_evict_first() : policy_evict_last();
+            DigRing r;
             int it = 0;
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = s_items[i];
-                const unsigned char* src = a.blocks + size_t(itm.w) * DG_ABYTES;
+                const unsigned char* src = a.blocks + size_t(itm.w) * DG_RBYTES;
                 const int k1 = itm.z >> 16;
-                for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, ++it) {
-                    const int s = it % NS;
-                    if (it >= NS && !mbar_wait(&empty[s], ((it / NS) - 1) & 1, abort, a.status)) continue;
+                for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, ++it, r.next(NR)) {
+                    if (it >= NR && !mbar_wait(&r_empty[r.slot], r.phase ^ 1, abort, a.status)) continue;
                     if (*abort) continue;
-                    mbar_arrive_expect_tx(&a_full[s], DG_ABYTES);
-                    bulk_g2s(As + s * DG_ABYTES, src + size_t(ks) * DG_ABYTES, DG_ABYTES, &a_full[s], pol);
+                    mbar_arrive_expect_tx(&r_full[r.slot], DG_RBYTES);
+                    bulk_g2s(Rs + r.slot * DG_RBYTES, src + size_t(ks) * DG_RBYTES, DG_RBYTES, &r_full[r.slot], pol);
                 }
             }
-            for (int k = it - NS; k < it; ++k)
-                if (k >= 0) mbar_wait(&a_full[k % NS], (k / NS) & 1, abort, a.status);
+            for (int k = it - NR; k < it; ++k)
+                if (k >= 0) mbar_wait(&r_full[k % NR], (k / NR) & 1, abort, a.status);
         }
     } else if (warp == 1) {
         if (elect_one()) {
-            int it = 0;
+            DigRing ra, rb;
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = s_items[i];
                 const int buf = i % NACC, k0 = itm.z & 0xFFFF, k1 = itm.z >> 16;
@@ -358,23 +391,23 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                 if (i >= NACC) ok = mbar_wait(&acc_empty[buf], (i / NACC - 1) & 1, abort, a.status);
                 tc_fence_after();
                 const uint32_t d = tmem + uint32_t(buf * NG * G);
-                for (int ks = k0; ks < k1; ++ks, ++it) {
-                    const int s = it % NS;
-                    bool okA = mbar_wait(&a_full[s], (it / NS) & 1, abort, a.status);
-                    okA = okA && mbar_wait(&b_full[s], (it / NS) & 1, abort, a.status);
+                for (int ks = k0; ks < k1; ++ks, ra.next(NX), rb.next(NS)) {
+                    ok = mbar_wait2(&a_full[ra.slot], ra.phase, &b_full[rb.slot], rb.phase, abort, a.status) && ok;
                     tc_fence_after();
-                    if (ok && okA && !*abort) {
-                        const uint64_t bd = dg_desc(Bs + s * Q::BBYTES);
+                    if (ok) {
+                        const unsigned char* B = Bs + rb.slot * Q::BBYTES;
+                        const uint64_t bd = dg_desc(B);
+                        const uint32_t ad = tmemA + ra.slot * DG_ACOLS;
                         // the first digit's MMA starts groups 0 .. 7, the zero digit group 8
                         if (NG > 8 && ks == k0)
-                            mma_bf16(d + 8 * G, dg_desc(As + s * DG_ABYTES),
-                                     dg_desc(Bs + s * Q::BBYTES + 8 * G * 32), idesc_bf16(128, G), 0);
+                            mma_f16_ta(d + 8 * G, ad, dg_desc(B + 8 * G * 32), idesc_f16(128, G), 0);
 #pragma unroll
                         for (int g = 0; g < 7; ++g)
-                            mma_bf16(d + g * G, dg_desc(As + s * DG_ABYTES + g * DG_PLANE), bd,
-                                     idesc_bf16(128, G * (NG - g < 8 ? NG - g : 8)), ks > k0 || g > 0);
+                            mma_f16_ta(d + g * G, ad + g * 8, bd, idesc_f16(128, G * (NG - g < 8 ? NG - g : 8)),
+                                       ks > k0 || g > 0);
                     }
-                    mma_commit(&empty[s]);
+                    mma_commit(&a_empty[ra.slot]);
+                    mma_commit(&b_empty[rb.slot]);
                 }
                 mma_commit(&acc_full[buf]);
             }
@@ -402,21 +435,15 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                 mbar_wait(&acc_full[buf], (i / NACC) & 1, abort, a.status);
                 tc_fence_after();
                 mbar_wait(&sc_full[i], 0, abort, a.status);
-                {
-                    uint32_t d[8 * NG];
 #pragma unroll
-                    for (int s = 0; s < NG; ++s) tmem_ld8_nowait(d0 + uint32_t(s * G + par * CP), d + 8 * s);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int c = 0; c < (C < 8 ? C : 8); ++c) V[c] += none ? 0.0 : dig_val<NG>(d + c, 8, ea + s_eb[5 * i + c / 2]);
-                }
-                if constexpr (C > 8) {
+                for (int f = 0; f < NF; ++f) {
                     uint32_t d[2 * NG];
 #pragma unroll
-                    for (int s = 0; s < NG; ++s) tmem_ld2_nowait(d0 + uint32_t(s * G + par * CP + 8), d + 2 * s);
+                    for (int s = 0; s < NG; ++s) tmem_ld2_nowait(d0 + uint32_t(s * G + par * CP + 2 * f), d + 2 * s);
                     tmem_wait_ld();
-#pragma unroll
-                    for (int c = 8; c < C; ++c) V[c] += none ? 0.0 : dig_val<NG>(d + c - 8, 2, ea + s_eb[5 * i + c / 2]);
+                    const int e = ea + s_eb[5 * i + f];
+                    V[2 * f] += none ? 0.0 : dig_val<NG>(d, 2, e);
+                    V[2 * f + 1] += none ? 0.0 : dig_val<NG>(d + 1, 2, e);
                 }
                 tc_fence_before();
                 mbar_arrive(&acc_empty[buf]);
@@ -471,109 +498,158 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                 }
             }
         }
-    } else if (warp < 6 + DG_NB) {
+    } else if (warp < 6 + NB) {
         // builders: warp 6 + it % NBW writes stage it's column digits
         const int bw = warp - 6;
-        bool waited = false;
+        constexpr int NT = SYN ? 2 * NF * 8 : 4 * NF * 8, TR = (NT + 31) / 32;
+        pdl_wait();
         int it = 0;
         if (bw < NBW)
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = s_items[i];
                 const int k1 = itm.z >> 16;
+                int4 pc[TR];
+                int kb[TR];
+                if constexpr (!SYN) {
+#pragma unroll
+                    for (int r = 0; r < TR; ++r) {
+                        const int task = r * 32 + lane;
+                        pc[r] = task < NT ? a.pieces[4 * itm.x + (task >> 3) / NF] : make_int4(0, 0, 0, 0);
+                    }
+#pragma unroll
+                    for (int r = 0; r < TR; ++r)
+                        kb[r] = 63 - (a.emax[((r * 32 + lane) >> 3) % NF * (N + 1) + pc[r].x] - 1020);
+                }
                 for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, ++it) {
                     if (it % NBW != bw) continue;
                     const int s = it % NS;
-                    if (!waited) {
-                        pdl_wait();
-                        waited = true;
-                    }
-                    if constexpr (SYN) mbar_wait(&sc_full[i], 0, abort, a.status);
-                    bool freed = it < NS;   // the slot is waited for after the first loads
-                    constexpr int NT = SYN ? 2 * NF * 8 : 4 * NF * 8;
+                    // every load of the stage before the first use of one, and before the wait for the slot
+                    double2 x[TR][4];
+                    double sg[TR];
+                    double2 cf[TR][2];
+                    if constexpr (SYN) {
+                        const int m = itm.x & 0xFFFF, ne = ext_even(N, m), lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
 #pragma unroll
-                    for (int t0 = 0; t0 < NT; t0 += 32) {
-                        const int task = t0 + lane, w = task & 7;
-                        long long v[4] = {0, 0, 0, 0};   // (re, im) of contracted index 2 w, then 2 w + 1
-                        int col = 0;
-                        if (task < NT) {
-                            if constexpr (SYN) {
-                                const int f = (task >> 3) % NF, par = (task >> 3) / NF, m = itm.x & 0xFFFF;
-                                const int ne = ext_even(N, m), n = par ? ext_odd(N, m) : ne;
-                                const int r0 = ext_off(N, m) + (par ? ne : 0), lo = m > 0 ? m : 1;
-                                const int pk = packed_off(N, m) - lo, j0 = ks * 16 + 2 * w;
-                                const double2* src = f < 3 ? a.alpha : a.beta;
-                                const double sc = f < 3 || m == 0 ? 1.0 : 0.5;
-                                const int kb = 63 - s_eb[5 * i + f];
-                                col = par * CP + 2 * f;
-                                auto A = [&](int K) -> double2 {
-                                    return (K < lo || K > N) ? make_double2(0.0, 0.0) : src[pk + K];
-                                };
+                        for (int r = 0; r < TR; ++r) {
+                            const int task = r * 32 + lane, w = task & 7, f = (task >> 3) % NF, par = (task >> 3) / NF;
+                            const int n = task < NT ? (par ? ext_odd(N, m) : ne) : 0;
+                            const int r0 = ext_off(N, m) + (par ? ne : 0);
+                            const bool deg = f == 2 || f == 4;   // the degree-shift set
+                            const double2* src = f < 3 ? a.alpha : a.beta;
 #pragma unroll
-                                for (int e = 0; e < 2; ++e) {
-                                    const int j = j0 + e, K = m + par + 2 * j;
-                                    if (j >= n) continue;
-                                    const double4_32a c = a.prepc[r0 + j];
-                                    double2 b;
-                                    if (f == 2 || f == 4) {
-                                        const double2 dn = A(K - 1), up = A(K + 1);
-                                        b = make_double2(sc * (c.z * dn.x + c.w * up.x), sc * (c.z * dn.y + c.w * up.y));
-                                    } else {
-                                        const double q = f == 0 ? c.x : c.y;
-                                        const double2 x = A(K);
-                                        b = make_double2(sc * (q * x.x), sc * (q * x.y));
-                                    }
-                                    v[2 * e] = f64_to_fx(b.x, kb);
-                                    v[2 * e + 1] = f64_to_fx(b.y, kb);
-                                }
-                            } else {
-                                const int f = (task >> 3) % NF, q = (task >> 3) / NF;
-                                const int4 pc = a.pieces[4 * itm.x + q];
-                                const int m = pc.x, par = pc.y, p = ks * 16 + 2 * w;
-                                const int kb = 63 - (a.emax[f * (N + 1) + m] - 1020);
-                                col = q * CP + 2 * f;
-                                if (pc.w > 0 && p < nh) {
-                                    const double* g = a.gana + (size_t(f) * npair * size_t(N + 1) + m) * 4;
-                                    const size_t ld = size_t(N + 1) * 4;
-                                    const double4_32a no = *reinterpret_cast<const double4_32a*>(g + size_t(p / 2) * ld);
-                                    double2 s0, s1;   // the mirrors of p and p + 1
-                                    if (nlat % 2 == 0) {
-                                        const double4_32a so =
-                                            *reinterpret_cast<const double4_32a*>(g + size_t((nlat - 2 - p) / 2) * ld);
-                                        s0 = make_double2(so.z, so.w);
-                                        s1 = make_double2(so.x, so.y);
-                                    } else {
-                                        // mirrors in different pairs; the equator is its own mirror
-                                        const int q0 = nlat - 1 - p, q1 = nlat - 2 - p;
-                                        s0 = q0 == p ? make_double2(0.0, 0.0)
-                                                     : *reinterpret_cast<const double2*>(g + size_t(q0 / 2) * ld + 2 * (q0 & 1));
-                                        s1 = q1 <= p + 1 ? make_double2(0.0, 0.0)
-                                                         : *reinterpret_cast<const double2*>(g + size_t(q1 / 2) * ld + 2 * (q1 & 1));
-                                    }
-                                    const double sg = par ? -1.0 : 1.0;
-                                    v[0] = f64_to_fx(fma(sg, s0.x, no.x), kb);
-                                    v[1] = f64_to_fx(fma(sg, s0.y, no.y), kb);
-                                    if (p + 1 < nh) {
-                                        v[2] = f64_to_fx(fma(sg, s1.x, no.z), kb);
-                                        v[3] = f64_to_fx(fma(sg, s1.y, no.w), kb);
-                                    }
+                            for (int e = 0; e < 2; ++e) {
+                                const int j = ks * 16 + 2 * w + e, K = m + par + 2 * j, K1 = deg ? K - 1 : K, K2 = K + 1;
+                                const double2 z = make_double2(0.0, 0.0);
+                                const double2* c = reinterpret_cast<const double2*>(a.prepc + r0 + j) + deg;
+                                cf[r][e] = j < n ? *c : z;
+                                x[r][2 * e] = j < n && K1 >= lo && K1 <= N ? src[pk + K1] : z;
+                                x[r][2 * e + 1] = deg && j < n && K2 <= N ? src[pk + K2] : z;
+                            }
+                        }
+                        mbar_wait(&sc_full[i], 0, abort, a.status);
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < TR; ++r) {
+                            const int w = lane & 7, f = ((r * 32 + lane) >> 3) % NF, p = ks * 16 + 2 * w;
+                            const double* g = a.gana + (size_t(f) * npair * size_t(N + 1) + pc[r].x) * 4;
+                            const size_t ld = size_t(N + 1) * 4;
+                            const double2 z = make_double2(0.0, 0.0);
+                            sg[r] = pc[r].y ? -1.0 : 1.0;
+                            x[r][0] = x[r][1] = x[r][2] = x[r][3] = z;   // p, p + 1 and their mirrors
+                            if (pc[r].w > 0 && p < nh) {
+                                const double4_32a no = *reinterpret_cast<const double4_32a*>(g + size_t(p / 2) * ld);
+                                x[r][0] = make_double2(no.x, no.y);
+                                if (p + 1 < nh) x[r][1] = make_double2(no.z, no.w);
+                                if (nlat % 2 == 0) {
+                                    const double4_32a so =
+                                        *reinterpret_cast<const double4_32a*>(g + size_t((nlat - 2 - p) / 2) * ld);
+                                    x[r][2] = make_double2(so.z, so.w);
+                                    if (p + 1 < nh) x[r][3] = make_double2(so.x, so.y);
+                                } else {
+                                    // mirrors in different pairs; the equator is its own mirror
+                                    const int q0 = nlat - 1 - p, q1 = nlat - 2 - p;
+                                    if (q0 != p) x[r][2] = *reinterpret_cast<const double2*>(g + size_t(q0 / 2) * ld + 2 * (q0 & 1));
+                                    if (q1 > p + 1) x[r][3] = *reinterpret_cast<const double2*>(g + size_t(q1 / 2) * ld + 2 * (q1 & 1));
                                 }
                             }
                         }
-                        if (!freed) {
-                            mbar_wait(&empty[s], ((it / NS) - 1) & 1, abort, a.status);
-                            freed = true;
-                        }
-                        if (task < NT && !*abort) {
-                            unsigned char* t = Bs + s * Q::BBYTES;
-                            dig_put(t + dg_off(col, 2 * w), G * 32, v[0], v[2]);
-                            dig_put(t + dg_off(col + 1, 2 * w), G * 32, v[1], v[3]);
+                    }
+                    // (re, im) of contracted index 2 w, then 2 w + 1
+                    long long v[TR][4];
+                    int col[TR];
+#pragma unroll
+                    for (int r = 0; r < TR; ++r) {
+                        const int task = r * 32 + lane, f = (task >> 3) % NF, h = (task >> 3) / NF;
+                        col[r] = h * CP + 2 * f;
+                        if constexpr (SYN) {
+                            const bool deg = f == 2 || f == 4;
+                            // beta is scaled by 1 / s_m
+                            const int k = 63 - s_eb[5 * i + f] - (f >= 3 && (itm.x & 0xFFFF) > 0);
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const double c1 = f == 0 || deg ? cf[r][e].x : cf[r][e].y, c2 = cf[r][e].y;
+                                const double2 d = x[r][2 * e], u = x[r][2 * e + 1];
+                                v[r][2 * e] = f64_to_fx(fma(c1, d.x, c2 * u.x), k);
+                                v[r][2 * e + 1] = f64_to_fx(fma(c1, d.y, c2 * u.y), k);
+                            }
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                v[r][2 * e] = f64_to_fx(fma(sg[r], x[r][2 + e].x, x[r][e].x), kb[r]);
+                                v[r][2 * e + 1] = f64_to_fx(fma(sg[r], x[r][2 + e].y, x[r][e].y), kb[r]);
+                            }
                         }
                     }
+                    if (it >= NS) mbar_wait(&b_empty[s], ((it / NS) - 1) & 1, abort, a.status);
+#pragma unroll
+                    for (int r = 0; r < TR; ++r)
+                        if (r * 32 + lane < NT && !*abort) {
+                            unsigned char* t = Bs + s * Q::BBYTES;
+                            const int w = lane & 7;
+                            dig_put(t + dg_off(col[r], 2 * w), G * 32, v[r][0], v[r][2]);
+                            dig_put(t + dg_off(col[r] + 1, 2 * w), G * 32, v[r][1], v[r][3]);
+                        }
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&b_full[s]);
                 }
             }
+    } else if (warp < 10 + NB) {
+        // expanders: 32 rows of every digit from bytes to FP16 in tensor memory
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t lanes = uint32_t((warp & 3) * 32) << 16;
+        DigRing rr, ra;
+        for (int i = 0; i < nI; ++i) {
+            const int4 itm = s_items[i];
+            const int k1 = itm.z >> 16;
+            for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, rr.next(NR), ra.next(NX)) {
+                // (a barrier still in its first phase passes for the one before)
+                mbar_wait2(&r_full[rr.slot], rr.phase, &a_empty[ra.slot], ra.phase ^ 1, abort, a.status);
+                uint4 q[7];
+#pragma unroll
+                for (int d = 0; d < 7; ++d)
+                    q[d] = *reinterpret_cast<const uint4*>(Rs + rr.slot * DG_RBYTES + d * DG_RPLANE + row * 16);
+                tc_fence_after();
+#pragma unroll
+                for (int d = 0; d < 7; ++d) {
+                    const uint32_t in[4] = {q[d].x, q[d].y, q[d].z, q[d].w};
+                    uint32_t h[8];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        h[2 * e] = dg_half2(__byte_perm(in[e], 0x64646464u, 0x4140));
+                        h[2 * e + 1] = dg_half2(__byte_perm(in[e], 0x64646464u, 0x4342));
+                    }
+                    tmem_st8_nowait(tmemA + lanes + uint32_t(ra.slot * DG_ACOLS + d * 8), h);
+                }
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&a_full[ra.slot]);
+                    mbar_arrive(&r_empty[rr.slot]);
+                }
+            }
+        }
     } else if constexpr (SYN) {
         // column exponents of every item: |b| <= 2^(eb - 1) from the exponents
         // of alpha and of the coefficient sets
@@ -581,7 +657,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
         for (int i = 0; i < nI; ++i) {
             const int m = s_items[i].x & 0xFFFF, lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
             int e[5] = {0, 0, 0, 0, 0}, top = 0;
-#pragma unroll 4
+#pragma unroll 8
             for (int K = lo + lane; K <= N; K += 32) {
                 const short4 c = a.eoff[pk + K];
                 const double2 x = a.alpha[pk + K];
@@ -612,7 +688,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, Q::TCOLS);
+        tmem_dealloc(tmem, 512);
     }
 }
 
@@ -740,8 +816,8 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
     T.emax = reinterpret_cast<int*>(d + o_emax);
     const int* d_base = reinterpret_cast<const int*>(d + o_base);
     int* d_used = reinterpret_cast<int*>(d + o_used);
-    T.syn.bytes = size_t(nblk) * DG_ABYTES;
-    T.ana.bytes = size_t(ablk) * DG_ABYTES;
+    T.syn.bytes = size_t(nblk) * DG_RBYTES;
+    T.ana.bytes = size_t(ablk) * DG_RBYTES;
     if (cudaMalloc(reinterpret_cast<void**>(&T.syn.blocks), T.syn.bytes + T.ana.bytes) != cudaSuccess)
         return SPHNSE_E_NOMEM;
     T.ana.blocks = T.syn.blocks + T.syn.bytes;
