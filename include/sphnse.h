@@ -436,13 +436,13 @@ int sphnse_ensemble_advance(sphnse_ensemble* ens, int nsteps, sphnse_step_info* 
 
 /* ---- stage timing ------------------------------------------------------- */
 
-#define SPHNSE_STAGE_PREP       0  /* coefficient sets for synthesis */
+#define SPHNSE_STAGE_PREP       0  /* coefficient sets for synthesis (batches; otherwise part of the synthesis) */
 #define SPHNSE_STAGE_SYNTHESIS  1  /* per-order Legendre synthesis */
 #define SPHNSE_STAGE_RING       2  /* per-latitude FFTs and pointwise product */
 #define SPHNSE_STAGE_ANALYSIS   3  /* per-order Legendre analysis */
 #define SPHNSE_STAGE_FINISH     4  /* recombination and diagonal update */
 #define SPHNSE_STAGE_STEP       5  /* NDF vector kernels (predictor, Newton update, accept) */
-#define SPHNSE_STAGE_TRANSPOSE  6  /* order-major <-> latitude-major transposes */
+#define SPHNSE_STAGE_TRANSPOSE  6  /* never launched: the rings read and write the sums' layouts */
 #define SPHNSE_NSTAGES          7
 
 #define SPHNSE_STAGE_ALL        (-1)

@@ -17,9 +17,10 @@
 //              = A_hi B_hi + A_hi B_lo + A_lo B_hi + A_lo B_lo,
 // the product of the FP32-accurate split operands, accumulated in FP32.
 //
-// Synthesis: the B tiles are written ahead by k_prep_tc (one 2 KB tile per
-// (m, parity, K tile)) and arrive with every A stage by bulk copy; warp 0 is
-// the TMA producer, warp 1 issues the MMAs, warps 2-5 drain the accumulators.
+// Synthesis: warp 0 is the TMA producer, warp 1 issues the MMAs, warps 2-5 drain
+// the accumulators; of one instance warps 6-11 build the stages' B tiles, of a
+// batch k_prep_tc writes them ahead (one 2 KB tile per (m, parity, K tile)) and
+// they arrive with every A stage by bulk copy.
 // Analysis: warps 2-5 build B from the weighted Fourier profiles in 16-byte
 // swizzle chunks, warps 6-9 drain the accumulators, so that neither stalls the
 // MMA issue behind the other.
@@ -39,7 +40,6 @@ namespace sph {
 
 constexpr int TC_TILE_M = 128;    // rows per MMA tile
 constexpr int TC_TILE_K = 64;     // K per smem tile (128 bytes of bf16)
-constexpr int TC_N = 16;          // accumulator columns (B rows)
 constexpr int TC_ATILE = TC_TILE_M * TC_TILE_K * 2;   // 16 KB
 
 // 8 bf16 (hi or lo parts of v[0..7]) packed for one 16-byte swizzle chunk

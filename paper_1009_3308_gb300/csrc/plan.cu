@@ -110,7 +110,11 @@ int ensure_tables(sphnse_plan* P, int prec) {
         else if (cudaMemcpy(t.syn, P->psyn_host.data(), t.bytes, cudaMemcpyHostToDevice) != cudaSuccess) rc = SPHNSE_E_CUDA;
         if (rc == SPHNSE_OK && !small_plan(P->nh)) {
             // the digit blocks of the tensor-core sums replace the table
-            rc = dig_setup(P, static_cast<const double*>(t.syn));
+            try {
+                rc = dig_setup(P, static_cast<const double*>(t.syn));
+            } catch (...) {
+                rc = SPHNSE_E_NOMEM;
+            }
             cudaFree(t.syn);
             t.syn = nullptr;
             if (rc == SPHNSE_OK) t.bytes = P->dig.syn.bytes + P->dig.ana.bytes;
@@ -285,7 +289,7 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
         return nullptr;
     }
     FFTPlan fft;
-    // the ring kernel keeps at most 3 butterflies per thread with <= 256 threads
+    // the ring kernels hold two buffers of every signal of two latitudes in shared memory
     if (!make_fft_plan(nlon, &fft) || nlon > 1536) {
         g_last_error = SPHNSE_E_UNSUPPORTED;
         return nullptr;
