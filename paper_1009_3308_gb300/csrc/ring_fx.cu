@@ -28,9 +28,9 @@
 // Scaling: every real field of a ring is scaled by its own power of two so
 // that the sum of its spectrum's magnitudes is below 2^60 (two shared-memory
 // reductions: the largest exponent, then the sum of the leading 16 bits).
-// Measured on the GB300 (event pairs, RHS): 369 us in FP64 arithmetic, 110 us
-// here at L = 511 (1536 longitudes); 94 and 45 us at L = 255; 41 and 26 us at
-// L = 100 (324 longitudes); 24.5 and 18.4 us at L = 31.  The FP64 form was
+// Measured on the GB300 (event pairs, RHS): 369 us in FP64 arithmetic, 99 us
+// here at L = 511 (1536 longitudes); 94 and 37 us at L = 255; 41 and 20 us at
+// L = 100 (324 longitudes); 24.5 and 14.4 us at L = 31.  The FP64 form was
 // bound by the FP64 pipe; this one by the integer multiply-adds and, for grids
 // of less than a wave, by the chain of stages.  Against 64-bit references the
 // errors of F, the fields and the projection are those of the FP64 form or
