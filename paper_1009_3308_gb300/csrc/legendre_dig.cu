@@ -501,7 +501,13 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
     } else if (warp < 6 + NB) {
         // builders: warp 6 + it % NBW writes stage it's column digits
         const int bw = warp - 6;
-        constexpr int NT = SYN ? 2 * NF * 8 : 4 * NF * 8, TR = (NT + 31) / 32;
+        // Synthesis: task = (parity, field, contracted index), a value per lane, and
+        // two lanes of adjacent indexes exchange real and imaginary parts to write
+        // a word of two each (a word's two indexes per lane left a quarter of the
+        // lanes idle: L = 511 99 us, now 94, L = 255 34, now 32).  Analysis: task = (piece, field, two latitudes).
+        constexpr int NT = SYN ? 2 * NF * 16 : 4 * NF * 8, TR = (NT + 31) / 32;
+        static_assert(NT % 32 == 0 || !SYN, "whole warps");
+        constexpr int XV = SYN ? 2 : 4;   // values loaded per task
         pdl_wait();
         int it = 0;
         if (bw < NBW)
@@ -524,27 +530,23 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                     if (it % NBW != bw) continue;
                     const int s = it % NS;
                     // every load of the stage before the first use of one, and before the wait for the slot
-                    double2 x[TR][4];
+                    double2 x[TR][XV];
                     double sg[TR];
-                    double2 cf[TR][2];
+                    double2 cf[TR];
                     if constexpr (SYN) {
                         const int m = itm.x & 0xFFFF, ne = ext_even(N, m), lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
 #pragma unroll
                         for (int r = 0; r < TR; ++r) {
-                            const int task = r * 32 + lane, w = task & 7, f = (task >> 3) % NF, par = (task >> 3) / NF;
-                            const int n = task < NT ? (par ? ext_odd(N, m) : ne) : 0;
-                            const int r0 = ext_off(N, m) + (par ? ne : 0);
+                            const int task = r * 32 + lane, f = (task >> 4) % NF, par = (task >> 4) / NF;
+                            const int n = par ? ext_odd(N, m) : ne, r0 = ext_off(N, m) + (par ? ne : 0);
                             const bool deg = f == 2 || f == 4;   // the degree-shift set
                             const double2* src = f < 3 ? a.alpha : a.beta;
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const int j = ks * 16 + 2 * w + e, K = m + par + 2 * j, K1 = deg ? K - 1 : K, K2 = K + 1;
-                                const double2 z = make_double2(0.0, 0.0);
-                                const double2* c = reinterpret_cast<const double2*>(a.prepc + r0 + j) + deg;
-                                cf[r][e] = j < n ? *c : z;
-                                x[r][2 * e] = j < n && K1 >= lo && K1 <= N ? src[pk + K1] : z;
-                                x[r][2 * e + 1] = deg && j < n && K2 <= N ? src[pk + K2] : z;
-                            }
+                            const int j = ks * 16 + (task & 15), K = m + par + 2 * j, K1 = deg ? K - 1 : K, K2 = K + 1;
+                            const double2 z = make_double2(0.0, 0.0);
+                            const double2* c = reinterpret_cast<const double2*>(a.prepc + r0 + j) + deg;
+                            cf[r] = j < n ? *c : z;
+                            x[r][0] = j < n && K1 >= lo && K1 <= N ? src[pk + K1] : z;
+                            x[r][1] = deg && j < n && K2 <= N ? src[pk + K2] : z;
                         }
                         mbar_wait(&sc_full[i], 0, abort, a.status);
                     } else {
@@ -574,30 +576,33 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                             }
                         }
                     }
-                    // (re, im) of contracted index 2 w, then 2 w + 1
-                    long long v[TR][4];
+                    // SYN: the words of a column (even lanes the real, odd lanes the imaginary part's);
+                    // else (re, im) of latitude 2 w, then 2 w + 1
+                    long long v[TR][XV];
                     int col[TR];
 #pragma unroll
                     for (int r = 0; r < TR; ++r) {
-                        const int task = r * 32 + lane, f = (task >> 3) % NF, h = (task >> 3) / NF;
-                        col[r] = h * CP + 2 * f;
-                        if constexpr (SYN) {
-                            const bool deg = f == 2 || f == 4;
-                            // beta is scaled by 1 / s_m
-                            const int k = 63 - s_eb[5 * i + f] - (f >= 3 && (itm.x & 0xFFFF) > 0);
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const double c1 = f == 0 || deg ? cf[r][e].x : cf[r][e].y, c2 = cf[r][e].y;
-                                const double2 d = x[r][2 * e], u = x[r][2 * e + 1];
-                                v[r][2 * e] = f64_to_fx(fma(c1, d.x, c2 * u.x), k);
-                                v[r][2 * e + 1] = f64_to_fx(fma(c1, d.y, c2 * u.y), k);
-                            }
-                        } else {
+                        const int task = r * 32 + lane;
+                        if constexpr (!SYN) {
+                            const int f = (task >> 3) % NF, h = (task >> 3) / NF;
+                            col[r] = h * CP + 2 * f;
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
                                 v[r][2 * e] = f64_to_fx(fma(sg[r], x[r][2 + e].x, x[r][e].x), kb[r]);
                                 v[r][2 * e + 1] = f64_to_fx(fma(sg[r], x[r][2 + e].y, x[r][e].y), kb[r]);
                             }
+                        } else {
+                            const int f = (task >> 4) % NF, par = (task >> 4) / NF, odd = lane & 1;
+                            const bool deg = f == 2 || f == 4;
+                            col[r] = par * CP + 2 * f + odd;
+                            // beta is scaled by 1 / s_m
+                            const int k = 63 - s_eb[5 * i + f] - (f >= 3 && (itm.x & 0xFFFF) > 0);
+                            const double c1 = f == 0 || deg ? cf[r].x : cf[r].y, c2 = cf[r].y;
+                            const long long re = f64_to_fx(fma(c1, x[r][0].x, c2 * x[r][1].x), k);
+                            const long long im = f64_to_fx(fma(c1, x[r][0].y, c2 * x[r][1].y), k);
+                            const long long got = __shfl_xor_sync(0xffffffffu, odd ? re : im, 1);
+                            v[r][0] = odd ? got : re;
+                            v[r][1] = odd ? im : got;
                         }
                     }
                     if (it >= NS) mbar_wait(&b_empty[s], ((it / NS) - 1) & 1, abort, a.status);
@@ -605,9 +610,13 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                     for (int r = 0; r < TR; ++r)
                         if (r * 32 + lane < NT && !*abort) {
                             unsigned char* t = Bs + s * Q::BBYTES;
-                            const int w = lane & 7;
-                            dig_put(t + dg_off(col[r], 2 * w), G * 32, v[r][0], v[r][2]);
-                            dig_put(t + dg_off(col[r] + 1, 2 * w), G * 32, v[r][1], v[r][3]);
+                            if constexpr (SYN) {
+                                dig_put(t + dg_off(col[r], lane & 14), G * 32, v[r][0], v[r][1]);
+                            } else {
+                                const int w = lane & 7;
+                                dig_put(t + dg_off(col[r], 2 * w), G * 32, v[r][0], v[r][2]);
+                                dig_put(t + dg_off(col[r] + 1, 2 * w), G * 32, v[r][1], v[r][3]);
+                            }
                         }
                     fence_proxy_async_smem();
                     __syncwarp();
