@@ -30,13 +30,13 @@
 // 16 bits).
 //
 // Bound: the single-K-step stages, whose barrier waits (150 to 200 cycles even
-// when they pass at once), expansion and MMAs (300 to 400 cycles) leave 870
-// cycles per stage; 7 bytes per table entry stream in 570 at full HBM rate.  The
+// when they pass at once), expansion and MMAs (300 to 400 cycles) leave 870 (the
+// synthesis, with longer epilogues and builders, 1070) cycles per stage; 7 bytes per table entry stream in 570 at full HBM rate.  The
 // FP64 pipe (two operations per clock per SM) would need 10 multiply-adds per
 // entry and RHS: 0.8 ms at L = 511.
 // Measured (event pairs, GB300) against the FP64 multiply-add kernels and their
-// prep, and against 16-bit stored digits: L = 511 synthesis 558 -> 138 -> 100 us,
-// analysis 429 -> 108 -> 78; L = 255 96 -> 37 -> 33, 74 -> 27 -> 21; L = 100
+// prep, and against 16-bit stored digits: L = 511 synthesis 558 -> 138 -> 94 us,
+// analysis 429 -> 108 -> 78; L = 255 96 -> 37 -> 32, 74 -> 27 -> 21; L = 100
 // 41 -> 17 -> 16, 22 -> 12 -> 12.  Errors against 64-bit references are those of
 // the multiply-add kernels or smaller for F, the fields and the projection at 23
 // sizes (mean over 24 states: u_phi 3.3e-15 and u_theta 8.5e-16 at L = 255,
