@@ -623,6 +623,10 @@ sphnse_ensemble* sphnse_ensemble_create(int n, const int* Ls, const double* nus,
         p.Omega = Omega;
         p.lm = E->buckets[E->bucket_of[i]].P->d_lm;
     }
+    if (setup_done()) {
+        destroy_ens(E);
+        return nullptr;
+    }
     return E;
 }
 

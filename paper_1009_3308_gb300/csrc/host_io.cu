@@ -67,7 +67,7 @@ int flag_init(HostIO& h) {
     *static_cast<volatile unsigned long long*>(f) = 0ull;
     if (cudaHostGetDevicePointer(reinterpret_cast<void**>(&h.dflag), f, 0) != cudaSuccess ||
         cudaMalloc(reinterpret_cast<void**>(&h.dcnt), sizeof(unsigned)) != cudaSuccess ||
-        cudaMemset(h.dcnt, 0, sizeof(unsigned)) != cudaSuccess) {
+        cudaMemset(h.dcnt, 0, sizeof(unsigned)) != cudaSuccess || setup_done() != SPHNSE_OK) {
         cudaFreeHost(f);
         return SPHNSE_E_NOMEM;
     }

@@ -422,6 +422,8 @@ void host_io_free(sphnse_plan* P);
 void stage_begin(sphnse_plan* P, int stage);
 void stage_end(sphnse_plan* P, int stage);
 int check_cuda(cudaError_t e);
+// end of a set-up: its errors, and the wait for its copies and fills
+int setup_done();
 
 // Ask once per kernel for the largest shared-memory carveout.  An SM runs
 // CTAs of different kernels together only under one L1/shared split: when a

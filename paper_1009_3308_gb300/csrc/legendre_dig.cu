@@ -868,8 +868,7 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
     T.ana.items = reinterpret_cast<int4*>(d + o_fa);
     T.syn.cnt = reinterpret_cast<int*>(d + o_cs);
     T.ana.cnt = reinterpret_cast<int*>(d + o_ca);
-    // the plan's stream need not wait for the default one, and a copy from pageable memory may still be on its way
-    return cudaStreamSynchronize(nullptr) == cudaSuccess ? SPHNSE_OK : SPHNSE_E_CUDA;
+    return SPHNSE_OK;   // (ensure_tables waits for the copies)
 }
 
 static DigArgs dig_args(sphnse_plan* P, const DigSide& D) {

@@ -1291,8 +1291,9 @@ int tc_setup_analysis(sphnse_plan* P, int nf) {
     cudaMemcpy(T.ana_pieces, pieces.data(), pieces.size() * sizeof(int4), cudaMemcpyHostToDevice);
     T.ana_cta = G;
     T.ana_nf = nf;
-    T.ana_ready = true;
-    return check_cuda(cudaGetLastError());
+    const int rc = setup_done();
+    T.ana_ready = rc == SPHNSE_OK;
+    return rc;
 }
 
 template <int NF>
@@ -1445,8 +1446,9 @@ static int tc_setup_analysis_fin(sphnse_plan* P) {
     cudaMemcpy(T.anf_pieces, pieces.data(), pieces.size() * sizeof(int4), cudaMemcpyHostToDevice);
     T.anf_cta = G;
     T.ana_entries = entries;
-    T.anf_ready = true;
-    return check_cuda(cudaGetLastError());
+    rc = setup_done();
+    T.anf_ready = rc == SPHNSE_OK;
+    return rc;
 }
 
 bool tc_rhs_fused(sphnse_plan* P) {
@@ -1605,9 +1607,7 @@ int tc_setup_synthesis(sphnse_plan* P) {
     }
     T.tsyn_bytes = 2 * total * 2;
     T.syn_ready = true;
-    const int rc = tc_batch_init(P, 1, &T.single);
-    if (rc) return rc;
-    return check_cuda(cudaGetLastError());
+    return tc_batch_init(P, 1, &T.single);   // which waits for the copies
 }
 
 static int syn_cluster_capacity(int ns, int cs, size_t smem);
@@ -1712,7 +1712,7 @@ int tc_batch_init(sphnse_plan* P, int nb, TcBatch* B, int ngmax, int nsmax, int 
     T.istride = int(stride);
     T.ncta = G * cs;
     *B = T;
-    return check_cuda(cudaGetLastError());
+    return setup_done();
 }
 
 void tc_batch_free(TcBatch* B) {
@@ -1908,7 +1908,7 @@ int tc_batch_ana_init(sphnse_plan* P, int nb, TcBatchA* B) {
     cudaMemcpy(T.slots, slots.data(), slots.size() * sizeof(int4), cudaMemcpyHostToDevice);
     T.ncta = G;
     *B = T;
-    return check_cuda(cudaGetLastError());
+    return setup_done();
 }
 
 void tc_batch_ana_free(TcBatchA* B) {

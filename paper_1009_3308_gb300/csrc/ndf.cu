@@ -960,6 +960,8 @@ int sphnse_objective(sphnse_plan* P, const double* alpha, const double* target, 
             return SPHNSE_E_NOMEM;
         cudaMemcpy(P->d_theta, P->theta.data(), P->nlat * sizeof(double), cudaMemcpyHostToDevice);
         cudaMemcpy(P->d_w, P->w.data(), P->nlat * sizeof(double), cudaMemcpyHostToDevice);
+        const int rc = setup_done();
+        if (rc) return rc;
     }
     double* uth = P->d_grid;
     double* uph = P->d_grid + gsz;

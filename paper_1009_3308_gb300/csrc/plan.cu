@@ -20,6 +20,17 @@ namespace sph {
 
 int check_cuda(cudaError_t e) { return e == cudaSuccess ? SPHNSE_OK : SPHNSE_E_CUDA; }
 
+// Uploads and fills of a set-up run on the default stream.  A copy from
+// pageable memory may still be on its way when the call returns, a fill always
+// may; the streams that use the data (a caller's side stream, an ensemble's own)
+// need not wait for the default one, and kernels load tables before they wait
+// for their predecessor.
+int setup_done() {
+    const int rc = check_cuda(cudaGetLastError());
+    const int rs = check_cuda(cudaStreamSynchronize(nullptr));
+    return rc ? rc : rs;
+}
+
 static void fold_stage_events(sphnse_plan* P) {
     cudaStreamSynchronize(P->stream);
     for (int s = 0; s < SPHNSE_NSTAGES; ++s) {
@@ -118,7 +129,6 @@ int ensure_tables(sphnse_plan* P, int prec) {
             cudaFree(t.syn);
             t.syn = nullptr;
             if (rc == SPHNSE_OK) t.bytes = P->dig.syn.bytes + P->dig.ana.bytes;
-            else dig_free(P);
         }
     } else if (prec == SPHNSE_FP32) {
         rc = upload_table<float>(P, t, [](double v, bool) { return float(v); }, false, true);
@@ -132,8 +142,11 @@ int ensure_tables(sphnse_plan* P, int prec) {
         rc = upload_table<__nv_bfloat16>(P, t, conv, false, false);
         if (rc == SPHNSE_OK) rc = upload_table<__nv_bfloat16>(P, t, conv, true, false);
     }
+    const int rs = setup_done();   // (the FP64 call also ends the copies of plan creation)
+    if (rc == SPHNSE_OK) rc = rs;
     if (rc != SPHNSE_OK) {
         free_tables(t);
+        if (prec == SPHNSE_FP64) dig_free(P);
         return rc;
     }
     t.built = true;
@@ -569,7 +582,8 @@ int sphnse_sync(sphnse_plan* P) {
     if (cudaMemcpy(&st, P->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost) != cudaSuccess) return SPHNSE_E_CUDA;
     if (st) {
         cudaMemset(P->d_status, 0, sizeof(unsigned));
-        return SPHNSE_E_TIMEOUT;
+        const int rc = setup_done();   // before a kernel that could set it again
+        return rc ? rc : SPHNSE_E_TIMEOUT;
     }
     return SPHNSE_OK;
 }
