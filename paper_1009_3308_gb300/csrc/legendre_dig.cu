@@ -237,6 +237,12 @@ __device__ __forceinline__ void dig_put(unsigned char* dst, int stride, long lon
     }
 }
 
+// the sum over an item without a nonzero digit block, whose accumulator holds no
+// data: 0, but NaN for a column with a non-finite entry (its product with a zero)
+__device__ __forceinline__ double dig_none(int e) {
+    return e >= DG_NAN / 2 ? __longlong_as_double(0x7FF8000000000000LL) : 0.0;
+}
+
 // sum_s D_s 2^(2 - 8 s) 2^e: the groups of one output added exactly, as
 // h 2^-54 + r 2^-70, and rounded once to binary64
 template <int NG>
@@ -248,7 +254,7 @@ __device__ __forceinline__ double dig_val(const uint32_t* d, int stride, int e) 
                         ((long long)g[3] << 16) + ((long long)g[4] << 8) + g[5];
     long long r = (long long)g[6] * 256 + g[7];
     if constexpr (NG > 8) r += (g[8] + 128) >> 8;
-    if (e >= DG_NAN / 2) return __longlong_as_double(0x7FF8000000000000LL);
+    if (e >= DG_NAN / 2) return dig_none(e);
     // as many of r's bits as fit below h (|h| <= 2^61)
     const int sh = min(16, max(0, __clzll(h ^ (h >> 63)) - 3));
     const long long v = (h << sh) + (r >> (16 - sh));
@@ -422,7 +428,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
         for (int i = 0; i < nI; ++i) {
             const int4 itm = s_items[i];
             const int buf = i % NACC;
-            const bool none = (itm.z & 0xFFFF) >= (itm.z >> 16);   // no nonzero block: the accumulator holds no data
+            const bool none = (itm.z & 0xFFFF) >= (itm.z >> 16);   // no nonzero block
             const uint32_t d0 = tmem + lanes + uint32_t(buf * NG * G);
             if constexpr (SYN) {
                 const int m = itm.x & 0xFFFF, par = quarter >> 1, pl = (quarter & 1) * 32 + lane, p = itm.y * 64 + pl;
@@ -442,8 +448,8 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                     for (int s = 0; s < NG; ++s) tmem_ld2_nowait(d0 + uint32_t(s * G + par * CP + 2 * f), d + 2 * s);
                     tmem_wait_ld();
                     const int e = ea + s_eb[5 * i + f];
-                    V[2 * f] += none ? 0.0 : dig_val<NG>(d, 2, e);
-                    V[2 * f + 1] += none ? 0.0 : dig_val<NG>(d + 1, 2, e);
+                    V[2 * f] += none ? dig_none(e) : dig_val<NG>(d, 2, e);
+                    V[2 * f + 1] += none ? dig_none(e) : dig_val<NG>(d + 1, 2, e);
                 }
                 tc_fence_before();
                 mbar_arrive(&acc_empty[buf]);
@@ -492,8 +498,8 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                 if (!in || *abort) continue;
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
-                    const double hr = none ? 0.0 : dig_val<NG>(d + 2 * f, CP, ea + eb[f]);
-                    const double hi = none ? 0.0 : dig_val<NG>(d + 2 * f + 1, CP, ea + eb[f]);
+                    const double hr = none ? dig_none(ea + eb[f]) : dig_val<NG>(d + 2 * f, CP, ea + eb[f]);
+                    const double hi = none ? dig_none(ea + eb[f]) : dig_val<NG>(d + 2 * f + 1, CP, ea + eb[f]);
                     *reinterpret_cast<double2*>(a.hana + size_t(row) * C + 2 * f) = make_double2(hr, hi);
                 }
             }
