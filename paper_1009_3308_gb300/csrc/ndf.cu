@@ -225,16 +225,18 @@ __global__ void k_adj_accept(double2* dbar, const double2* abar, double2* dtot, 
 }
 
 // mu <- mu + (b - mu + c JT) / conj(1 - c J_d); ||b - mu + c JT||_inf (abs) goes
-// to host[0] (first: host[1]), a flag for non-finite values to host[7] (pinned).  The last block
-// writes them and clears the slots, so that an iteration needs no memset and no
-// copy: with alpha's fields kept between iterations, a reverse sweep of ten steps
-// at L = 255 FP32 went from 10.4 to 8.9 ms.
+// to host[0] (first: host[1]), a flag for values beyond the norms' range, in this
+// iteration or an earlier one, to host[7] (pinned).  The last block writes them and
+// clears what the next iteration adds to, so that an iteration needs no memset and
+// no copy: with alpha's fields kept between iterations, a reverse sweep of ten
+// steps at L = 255 FP32 went from 10.4 to 8.9 ms.  slot[5] keeps the first norm:
+// where it is zero mu = 0 is the solution, also with a JT that is not finite.
 __global__ void k_adj_fixpoint(double2* mu, const double2* b, const double2* JT, const int2* lm, double c,
                                double nu, double Omega, unsigned long long* slot, unsigned long long* host, int first,
                                int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double r[1] = {0.0};
-    if (i < n) {
+    if (i < n && (first || __ldcg(slot + 5))) {
         const int L = lm[i].x, m = lm[i].y;
         const double lam = double(L) * (L + 1.0);
         const double mr = 1.0 + c * nu * lam, mi = c * 2.0 * Omega * m * rcp64<2>(lam);  // conj(1 - c J_d)
@@ -262,9 +264,11 @@ __global__ void k_adj_fixpoint(double2* mu, const double2* b, const double2* JT,
     __syncthreads();
     if (threadIdx.x != 0 || atomicAdd(slot + 6, 1ull) != gridDim.x - 1) return;
     __threadfence();
-    host[first ? 1 : 0] = __ldcg(slot);
+    const unsigned long long norm = __ldcg(slot);
+    host[first ? 1 : 0] = norm;
     host[7] = __ldcg(slot + 7);
-    slot[0] = slot[6] = slot[7] = 0ull;
+    if (first) slot[5] = norm;
+    slot[0] = slot[6] = 0ull;
 }
 
 // y0bar = abar + mu - dtot;  dbar_j += g_j (-mu) + y0bar (j < k);  abar = y0bar;
