@@ -2,45 +2,57 @@
 // digit splitting (the error-free splitting of matrix products of Ozaki,
 // Ogita, Oishi and Rump, Numer. Algorithms 59 (2012)).
 //
-// Every table row is scaled by a power of two to |a| < 0.993 and cut into seven
-// balanced base-256 digits, every coefficient (or profile) column to |b| <=
-// 1/2 and eight digits:  a = sum_i a_i 2^(1 - 8 i),  b = sum_j b_j 2^(1 - 8 j),
-// |a_i|, |b_j| <= 128.  Digits are exact in FP16, their products are integers
-// of at most 2^14, and sums over the contracted index stay below 2^24 in the
-// leading groups, so the tensor core's FP32 accumulators hold them exactly.
-// The products of i + j = s share one accumulator group, s = 2 .. 9 (synthesis:
-// .. 10):
+// Every table row is scaled by a power of two to |a| < 0.993, every coefficient
+// (or profile) column to |b| <= 1/2, and both are cut into eight balanced
+// base-256 digits:  a = sum_i a_i 2^(1 - 8 i),  b = sum_j b_j 2^(1 - 8 j),
+// |a_i|, |b_j| <= 128.  The products of i + j = s share one accumulator group,
+// s = 2 .. 10:
 //     sum_k a b = sum_s 2^(2 - 8 s) D_s,   D_s = sum_{i + j = s} sum_k a_i b_j,
-// and the epilogue adds the groups in integers.  What is left out (the eighth
-// digit of a, products with larger i + j) is about 2^-57 of max|a| |b| per term;
-// an FP64 multiply-add chain over 256 terms rounds to about 2^-50 of max|a| max|b|.
+// and the epilogue adds the groups in integers.  Digits are exact in FP16, their
+// products are integers of at most 2^14, and D_s of the four leading groups stays
+// below 2^24 for the 384 terms of the largest plan, so that the FP32
+// accumulators hold it exactly; from s = 6 on a bound of 2^25.3 is above that,
+// but digits past the first are spread out (their sums reach about 2^20), and one
+// rounding there would be 2^-45 of a group's weight 2^(2 - 48).
 //
-// Per K = 16 step one tile of 128 table rows takes seven MMAs, digit i of the
-// table against digits 1 .. 9 - i (10 - i) of the columns (N = G (9 - i), G
+// Error.  Relative to max|a| max|b| of a row and a column, digits end at 2^-64
+// and the products left out (i + j > 10) add up to about 2^-67.  A multiply-add
+// chain errs relative to the largest product |a_k b_k|, which is far smaller
+// where a state's low degrees meet polar rows: there Pt_K^m rises with K like
+// K^(m + 1/2), the spectrum falls, and the result is divided by sin(theta).
+// Eight table digits cover the 2^9 of 1/sin(theta) at L = 511; with seven the
+// largest error of u_theta for the mode (9, 8) was 5.1e-15 of its maximum, with
+// eight 2.5e-16 as in a multiply-add chain.  For the columns the degrees of an
+// order are balanced: table entries of degree K are divided, coefficient sets
+// multiplied by 2^t, t = floor(log2(K + 1)) (dig_shift); without it a spectrum
+// falling like l^-4 lost a factor of four (order 1 at L = 511).  What stays below
+// the chain's precision are results smaller than 2^-60 of max|a| max|b|: the
+// projection of a field that lives on polar rows in one order above about ten.
+//
+// Per K = 16 step one tile of 128 table rows takes eight MMAs, digit i of the
+// table against digits 1 .. 10 - i of the columns (N = G (10 - i), G
 // columns per group): with the columns of a group adjacent, those digits are a prefix of
 // the B rows and land on the groups from i + 1 on, a contiguous run of accumulator
 // columns.  The table digits are stored once per plan as bytes (digit + 128) in
-// the order the kernels consume them: one 14 KB block per (tile, K step) = 7
+// the order the kernels consume them: one 16 KB block per (tile, K step) = 8
 // planes of 128 x 16, one bulk copy each; blocks whose digits are all zero
 // (polar latitudes at high order) are left out.  Four warps expand a block to
 // FP16 (a byte under 0x64 is 1024 + byte; one packed subtraction) straight into
 // tensor memory, where the MMAs take their A operand: written to shared memory
-// instead, the expanded digits cost more than the halved HBM stream saved (L =
-// 511 synthesis 154 us, analysis 107, against 138 and 108 of digits stored in
-// 16 bits).
+// instead, the expanded digits cost more than the halved HBM stream saved.
 //
 // Bound: the single-K-step stages, whose barrier waits (150 to 200 cycles even
-// when they pass at once), expansion and MMAs (300 to 400 cycles) leave 870 (the
-// synthesis, with longer epilogues and builders, 1070) cycles per stage; 7 bytes per table entry stream in 570 at full HBM rate.  The
+// when they pass at once), expansion and MMAs leave about 1000 cycles per stage;
+// eight bytes per table entry stream in 650 at full HBM rate.  The
 // FP64 pipe (two operations per clock per SM) would need 10 multiply-adds per
 // entry and RHS: 0.8 ms at L = 511.
 // Measured (event pairs, GB300) against the FP64 multiply-add kernels and their
-// prep, and against 16-bit stored digits: L = 511 synthesis 558 -> 138 -> 94 us,
-// analysis 429 -> 108 -> 78; L = 255 96 -> 37 -> 32, 74 -> 27 -> 21; L = 100
-// 41 -> 17 -> 16, 22 -> 12 -> 12.  Errors against 64-bit references are those of
-// the multiply-add kernels or smaller for F, the fields and the projection at 23
-// sizes (mean over 24 states: u_phi 3.3e-15 and u_theta 8.5e-16 at L = 255,
-// before 3.4e-15 and 1.1e-15).
+// prep: L = 511 synthesis 558 -> 94 us, analysis 429 -> 80; L = 255 96 -> 30,
+// 74 -> 22; L = 100 41 -> 15, 22 -> 13.  Errors of the sums against extended
+// precision, emulated for single modes, exponential and power-law spectra at L =
+// 53, 100, 255 and 511, 8 to 18 orders each: the largest and the mean error of
+// every field are at most 1.1 times those of the multiply-add chain and mostly
+// smaller (two states of order 0 at L = 100: 1.2 times).
 //
 // Synthesis tiles: rows 0 .. 63 the even, rows 64 .. 127 the odd degrees of one
 // order on 64 northern latitudes (columns 0 .. G/2-1 of a group belong to the
@@ -61,20 +73,13 @@
 
 namespace sph {
 
+constexpr int DG_ND = 8;                     // digits of the table and of the columns
+constexpr int DG_NG = 9;                     // accumulator groups i + j = 2 .. 10
 constexpr int DG_RPLANE = 128 * 16;          // a digit of 128 rows x 16 of the contracted index: bytes digit + 128
-constexpr int DG_RBYTES = 7 * DG_RPLANE;     // one block of the stored table
-constexpr int DG_ACOLS = 7 * 8;              // the same in FP16: columns of tensor memory, a row per lane
-constexpr int DG_NX = 4;                     // stages of it
-constexpr int DG_MINEXP = -30;               // row scales are at least 2^-30 (smaller rows lose digits below 2^-86)
-// Orders below DG_SEGM take their first K step (the lowest degrees) apart,
-// with its own row exponents and with the remainder that its seven digits
-// leave of the table as a second block of digits; the epilogue adds the parts.
-// At the poles Pt_K^m grows like K^(m + 1/2), so with one exponent per row the
-// largest coefficients, at the lowest degrees, would meet table entries 2^13
-// below the row's maximum (L = 511, m = 1); at m = 0 the degree-shift sum of
-// u_phi cancels there; and the division by sin(theta) carries these errors
-// into u (u_theta 2.4e-15 against 1.3e-15 of the FP64 sums at L = 511).
-constexpr int DG_SEGM = 8;
+constexpr int DG_RBYTES = DG_ND * DG_RPLANE; // one block of the stored table
+constexpr int DG_ACOLS = DG_ND * 8;          // the same in FP16: columns of tensor memory, a row per lane
+constexpr int DG_NX = 3;                     // stages of it
+constexpr int DG_MINEXP = -22;               // row scales are at least 2^-22 (smaller rows lose digits below 2^-86)
 constexpr int DG_NAN = 1 << 20;              // exponent of a column with a non-finite entry
 
 // byte offset of element (row, k) of a K = 16 tile: rows of 32 bytes, the two
@@ -112,15 +117,12 @@ __global__ void k_dig_syn_scale(const double* __restrict__ tab, int* __restrict_
     if (p >= nh) return;
     const int ne = ext_even(N, m), cnt = ext_count(N, m);
     const double* t = tab + size_t(ext_off(N, m)) * nh + p;
-    int e0 = 0, e1 = 0;   // first step, later steps
+    int e = 0;
     for (int r = 0; r < cnt; ++r) {
-        const int b = dg_bexp(t[size_t(r) * nh]);
-        if ((r < ne ? r : r - ne) < 16) e0 = max(e0, b);
-        else e1 = max(e1, b);
+        const int K = r < ne ? m + 2 * r : m + 1 + 2 * (r - ne);
+        e = max(e, dg_bexp(t[size_t(r) * nh]) - dig_shift(K));
     }
-    if (m >= DG_SEGM) e0 = e1 = max(e0, e1);
-    ea[m * nh + p] = max(e0 - 1022, DG_MINEXP);
-    if (m < DG_SEGM) ea[(N + 1 + m) * nh + p] = max(e1 - 1022, DG_MINEXP);
+    ea[m * nh + p] = max(e - 1022, DG_MINEXP);
 }
 __global__ void k_dig_ana_scale(const double* __restrict__ tab, int* __restrict__ ea, int n_ext, int nh) {
     const int r = blockIdx.x * 4 + threadIdx.x / 32;
@@ -131,44 +133,39 @@ __global__ void k_dig_ana_scale(const double* __restrict__ tab, int* __restrict_
     if ((threadIdx.x & 31) == 0) ea[r] = max(e - 1022, DG_MINEXP);
 }
 
-// seven digits of eight scaled entries -> eight bytes of each plane; returns whether any is nonzero
+// the digits of eight scaled entries -> eight bytes of each plane; returns whether any is nonzero
 __device__ __forceinline__ bool dig_store(const double (&x)[8], const int (&e)[8], unsigned char* dst) {
-    unsigned long long w[7] = {0, 0, 0, 0, 0, 0, 0};
+    unsigned long long w[DG_ND] = {};
     bool any = false;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        const long long v = f64_to_fx(x[i], 55 - e[i]);
+        const long long v = f64_to_fx(x[i], 63 - e[i]);
         any = any || v != 0;
-        const unsigned long long u = (unsigned long long)v + 0x0080808080808080ULL;
+        const unsigned long long u = (unsigned long long)v + 0x8080808080808080ULL;
 #pragma unroll
-        for (int d = 0; d < 7; ++d) w[d] |= ((u >> (48 - 8 * d)) & 255) << (8 * i);
+        for (int d = 0; d < DG_ND; ++d) w[d] |= ((u >> (56 - 8 * d)) & 255) << (8 * i);
     }
 #pragma unroll
-    for (int d = 0; d < 7; ++d) *reinterpret_cast<unsigned long long*>(dst + d * DG_RPLANE) = w[d];
+    for (int d = 0; d < DG_ND; ++d) *reinterpret_cast<unsigned long long*>(dst + d * DG_RPLANE) = w[d];
     return any;
 }
 
 // block = (step, latitude tile, order): thread = (row, half of the step)
 __global__ void __launch_bounds__(256) k_dig_syn(const double* __restrict__ tab, const int* __restrict__ ea,
                                                  const int* __restrict__ base, unsigned char* __restrict__ out,
-                                                 int* __restrict__ used, int N, int nh, int ntile, int remainder) {
+                                                 int* __restrict__ used, int N, int nh, int ntile) {
     const int m = blockIdx.z, t = blockIdx.y, ks = blockIdx.x, ne = ext_even(N, m);
     if (ks >= dg_steps(ne)) return;
     const int row = threadIdx.x & 127, h = threadIdx.x >> 7, par = row >> 6, p = t * 64 + (row & 63);
     const int n = par ? ext_odd(N, m) : ne;
     const double* src = tab + size_t(ext_off(N, m) + (par ? ne : 0)) * nh + p;
-    const int mr = m < DG_SEGM && ks > 0 ? N + 1 + m : m;   // row of exponents
     double x[8];
     int e[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int j = ks * 16 + h * 8 + i;
         x[i] = j < n && p < nh ? src[size_t(j) * nh] : 0.0;
-        e[i] = p < nh ? ea[mr * nh + p] : 0;
-        if (remainder) {   // what the seven digits leave (exact: x has 53 bits)
-            x[i] -= scalbn(double(f64_to_fx(x[i], 55 - e[i])), e[i] - 55);
-            e[i] -= 55;
-        }
+        e[i] = p < nh ? ea[m * nh + p] + dig_shift(m + par + 2 * j) : 0;
     }
     const int blk = base[m * ntile + t] + ks;
     const bool any = dig_store(x, e, out + size_t(blk) * DG_RBYTES + row * 16 + h * 8);
@@ -199,10 +196,8 @@ __global__ void __launch_bounds__(256) k_dig_ana(const double* __restrict__ tab,
 
 struct DigArgs {
     const unsigned char* blocks;  // table digits, DG_RBYTES per (tile, step)
-    const int4* items;            // (m | flags (or analysis tile), latitude tile, first step | end
-                                  //  step << 16, first block); flags of the parts of a split item: bit 16
-                                  //  another part follows, 17 exponents of the later steps, 18 a part
-                                  //  precedes, 19 remainder of the first step (exponents lower by 55)
+    const int4* items;            // (m or analysis tile, latitude tile, first step | end step << 16,
+                                  //  first block)
     const int* cnt;               // items of every CTA, at c * istride
     int istride;
     int evict_first;              // the digits exceed what L2 can keep
@@ -245,17 +240,15 @@ __device__ __forceinline__ double dig_none(int e) {
 
 // sum_s D_s 2^(2 - 8 s) 2^e: the groups of one output added exactly, as
 // h 2^-54 + r 2^-70, and rounded once to binary64
-template <int NG>
 __device__ __forceinline__ double dig_val(const uint32_t* d, int stride, int e) {
-    int g[NG];
+    int g[DG_NG];
 #pragma unroll
-    for (int s = 0; s < NG; ++s) g[s] = __float2int_rn(__uint_as_float(d[s * stride]));
+    for (int s = 0; s < DG_NG; ++s) g[s] = __float2int_rn(__uint_as_float(d[s * stride]));
     const long long h = ((long long)g[0] << 40) + ((long long)g[1] << 32) + ((long long)g[2] << 24) +
                         ((long long)g[3] << 16) + ((long long)g[4] << 8) + g[5];
-    long long r = (long long)g[6] * 256 + g[7];
-    if constexpr (NG > 8) r += (g[8] + 128) >> 8;
+    const long long r = (long long)g[6] * 256 + g[7] + ((g[8] + 128) >> 8);
     if (e >= DG_NAN / 2) return dig_none(e);
-    // as many of r's bits as fit below h (|h| <= 2^61)
+    // as many of r's bits as fit below h (|h| < 2^62: 384 terms of at most 1/2)
     const int sh = min(16, max(0, __clzll(h ^ (h >> 63)) - 3));
     const long long v = (h << sh) + (r >> (16 - sh));
     return v == 0 ? 0.0 : f64_scale(__ll2double_rn(v), e - 54 - sh);
@@ -278,14 +271,9 @@ template <bool SYN, int NF> struct DigShape {
     static constexpr int C = 2 * NF;
     static constexpr int CP = SYN ? (C <= 8 ? 8 : 16) : (C <= 4 ? 4 : 8);
     static constexpr int G = SYN ? 2 * CP : 4 * CP;
-    // accumulator groups i + j = 2 .. NG + 1.  The synthesis takes one more:
-    // near the poles the rows of the lowest orders grow like K^(m + 1/2), so a
-    // row's maximum meets the small high-degree coefficients, and the sum that
-    // matters is well below max|a| max|b| (and is then divided by sin(theta))
-    static constexpr int NG = SYN ? 9 : 8;
-    static constexpr int BBYTES = NG * G * 32;               // eight digits of the columns, SYN: a zero digit
-    static constexpr int NACC = 2 * NG * G + DG_NX * DG_ACOLS <= 512 ? 2 : 1;   // accumulator buffers
-    static_assert(NACC * NG * G + DG_NX * DG_ACOLS <= 512, "tensor memory");
+    static constexpr int BBYTES = DG_NG * G * 32;            // eight digits of the columns and a zero digit
+    static constexpr int NACC = 2 * DG_NG * G + DG_NX * DG_ACOLS <= 512 ? 2 : 1;   // accumulator buffers
+    static_assert(NACC * DG_NG * G + DG_NX * DG_ACOLS <= 512, "tensor memory");
     // ring of stored table blocks (what is in flight from memory) and of column digits
     static constexpr int NR = SYN && G == 32 ? 8 : 10;
     static constexpr int NS = SYN ? (NF == 3 ? 9 : 6) : (NF == 2 ? 10 : 6);
@@ -304,7 +292,7 @@ template <bool SYN, int NF> struct DigShape {
 template <bool SYN, int NF>
 __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArgs a) {
     using Q = DigShape<SYN, NF>;
-    constexpr int NS = Q::NS, NR = Q::NR, NX = DG_NX, G = Q::G, C = Q::C, CP = Q::CP, NG = Q::NG, NACC = Q::NACC;
+    constexpr int NS = Q::NS, NR = Q::NR, NX = DG_NX, G = Q::G, C = Q::C, CP = Q::CP, NG = DG_NG, NACC = Q::NACC;
     static_assert(8 * (2 * (NR + NX + NS) + 4) + 8 <= 512, "barriers");
     constexpr int NB = Q::NB, NBW = NS < NB ? NS : NB;   // a builder per stage, none a full ring ahead
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -405,10 +393,10 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                         const uint64_t bd = dg_desc(B);
                         const uint32_t ad = tmemA + ra.slot * DG_ACOLS;
                         // the first digit's MMA starts groups 0 .. 7, the zero digit group 8
-                        if (NG > 8 && ks == k0)
+                        if (ks == k0)
                             mma_f16_ta(d + 8 * G, ad, dg_desc(B + 8 * G * 32), idesc_f16(128, G), 0);
 #pragma unroll
-                        for (int g = 0; g < 7; ++g)
+                        for (int g = 0; g < DG_ND; ++g)
                             mma_f16_ta(d + g * G, ad + g * 8, bd, idesc_f16(128, G * (NG - g < 8 ? NG - g : 8)),
                                        ks > k0 || g > 0);
                     }
@@ -423,7 +411,6 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
         pdl_wait();
         const int quarter = warp & 3;
         const uint32_t lanes = uint32_t(quarter * 32) << 16;
-        double V[C];   // SYN: this row's sums, over the parts of a split item
         int xb = 0;    // exchange buffer
         for (int i = 0; i < nI; ++i) {
             const int4 itm = s_items[i];
@@ -431,13 +418,10 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
             const bool none = (itm.z & 0xFFFF) >= (itm.z >> 16);   // no nonzero block
             const uint32_t d0 = tmem + lanes + uint32_t(buf * NG * G);
             if constexpr (SYN) {
-                const int m = itm.x & 0xFFFF, par = quarter >> 1, pl = (quarter & 1) * 32 + lane, p = itm.y * 64 + pl;
+                const int m = itm.x, par = quarter >> 1, pl = (quarter & 1) * 32 + lane, p = itm.y * 64 + pl;
                 const double inv = p < nh ? a.isin[p] : 0.0, minv = inv * double(m);
-                const int ea = (p < nh ? a.ea[((itm.x >> 17) & 1 ? N + 1 + m : m) * nh + p] : 0) -
-                               ((itm.x >> 19) & 1 ? 55 : 0);
-                if (!((itm.x >> 18) & 1))
-#pragma unroll
-                    for (int c = 0; c < C; ++c) V[c] = 0.0;
+                const int ea = p < nh ? a.ea[m * nh + p] : 0;
+                double V[C];   // this row's sums
                 mbar_wait(&acc_full[buf], (i / NACC) & 1, abort, a.status);
                 tc_fence_after();
                 mbar_wait(&sc_full[i], 0, abort, a.status);
@@ -448,12 +432,11 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                     for (int s = 0; s < NG; ++s) tmem_ld2_nowait(d0 + uint32_t(s * G + par * CP + 2 * f), d + 2 * s);
                     tmem_wait_ld();
                     const int e = ea + s_eb[5 * i + f];
-                    V[2 * f] += none ? dig_none(e) : dig_val<NG>(d, 2, e);
-                    V[2 * f + 1] += none ? dig_none(e) : dig_val<NG>(d + 1, 2, e);
+                    V[2 * f] = none ? dig_none(e) : dig_val(d, 2, e);
+                    V[2 * f + 1] = none ? dig_none(e) : dig_val(d + 1, 2, e);
                 }
                 tc_fence_before();
                 mbar_arrive(&acc_empty[buf]);
-                if ((itm.x >> 16) & 1) continue;   // the next item holds the rest
                 // even and odd sums meet: the even warps write north = E + O, the odd ones south = E - O
                 double* mine = xch + ((size_t(xb) * 2 + par) * 64 + pl) * C;
                 const double* other = xch + ((size_t(xb) * 2 + 1 - par) * 64 + pl) * C;
@@ -486,22 +469,33 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                 }
                 mbar_wait(&acc_full[buf], (i / NACC) & 1, abort, a.status);
                 tc_fence_after();
-                uint32_t d[8 * CP];
+                double H[C];
+                if constexpr (CP == 4) {
+                    uint32_t d[NG * CP];
 #pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    if constexpr (CP == 4) tmem_ld4_nowait(d0 + uint32_t(s * G + quarter * CP), d + 4 * s);
-                    else tmem_ld8_nowait(d0 + uint32_t(s * G + quarter * CP), d + 8 * s);
+                    for (int s = 0; s < NG; ++s) tmem_ld4_nowait(d0 + uint32_t(s * G + quarter * CP), d + CP * s);
+                    tmem_wait_ld();
+                    tc_fence_before();
+                    mbar_arrive(&acc_empty[buf]);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) H[c] = none ? dig_none(ea + eb[c / 2]) : dig_val(d + c, CP, ea + eb[c / 2]);
+                } else {
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) {
+                        uint32_t d[2 * NG];
+#pragma unroll
+                        for (int s = 0; s < NG; ++s) tmem_ld2_nowait(d0 + uint32_t(s * G + quarter * CP + 2 * f), d + 2 * s);
+                        tmem_wait_ld();
+                        H[2 * f] = none ? dig_none(ea + eb[f]) : dig_val(d, 2, ea + eb[f]);
+                        H[2 * f + 1] = none ? dig_none(ea + eb[f]) : dig_val(d + 1, 2, ea + eb[f]);
+                    }
+                    tc_fence_before();
+                    mbar_arrive(&acc_empty[buf]);
                 }
-                tmem_wait_ld();
-                tc_fence_before();
-                mbar_arrive(&acc_empty[buf]);
                 if (!in || *abort) continue;
 #pragma unroll
-                for (int f = 0; f < NF; ++f) {
-                    const double hr = none ? dig_none(ea + eb[f]) : dig_val<NG>(d + 2 * f, CP, ea + eb[f]);
-                    const double hi = none ? dig_none(ea + eb[f]) : dig_val<NG>(d + 2 * f + 1, CP, ea + eb[f]);
-                    *reinterpret_cast<double2*>(a.hana + size_t(row) * C + 2 * f) = make_double2(hr, hi);
-                }
+                for (int f = 0; f < NF; ++f)
+                    *reinterpret_cast<double2*>(a.hana + size_t(row) * C + 2 * f) = make_double2(H[2 * f], H[2 * f + 1]);
             }
         }
     } else if (warp < 6 + NB) {
@@ -540,7 +534,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                     double sg[TR];
                     double2 cf[TR];
                     if constexpr (SYN) {
-                        const int m = itm.x & 0xFFFF, ne = ext_even(N, m), lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
+                        const int m = itm.x, ne = ext_even(N, m), lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
 #pragma unroll
                         for (int r = 0; r < TR; ++r) {
                             const int task = r * 32 + lane, f = (task >> 4) % NF, par = (task >> 4) / NF;
@@ -602,7 +596,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                             const bool deg = f == 2 || f == 4;
                             col[r] = par * CP + 2 * f + odd;
                             // beta is scaled by 1 / s_m
-                            const int k = 63 - s_eb[5 * i + f] - (f >= 3 && (itm.x & 0xFFFF) > 0);
+                            const int k = 63 - s_eb[5 * i + f] - (f >= 3 && itm.x > 0);
                             const double c1 = f == 0 || deg ? cf[r].x : cf[r].y, c2 = cf[r].y;
                             const long long re = f64_to_fx(fma(c1, x[r][0].x, c2 * x[r][1].x), k);
                             const long long im = f64_to_fx(fma(c1, x[r][0].y, c2 * x[r][1].y), k);
@@ -640,21 +634,24 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
             for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, rr.next(NR), ra.next(NX)) {
                 // (a barrier still in its first phase passes for the one before)
                 mbar_wait2(&r_full[rr.slot], rr.phase, &a_empty[ra.slot], ra.phase ^ 1, abort, a.status);
-                uint4 q[7];
-#pragma unroll
-                for (int d = 0; d < 7; ++d)
-                    q[d] = *reinterpret_cast<const uint4*>(Rs + rr.slot * DG_RBYTES + d * DG_RPLANE + row * 16);
                 tc_fence_after();
 #pragma unroll
-                for (int d = 0; d < 7; ++d) {
-                    const uint32_t in[4] = {q[d].x, q[d].y, q[d].z, q[d].w};
-                    uint32_t h[8];
+                for (int d0 = 0; d0 < DG_ND; d0 += 4) {
+                    uint4 q[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        h[2 * e] = dg_half2(__byte_perm(in[e], 0x64646464u, 0x4140));
-                        h[2 * e + 1] = dg_half2(__byte_perm(in[e], 0x64646464u, 0x4342));
+                    for (int d = 0; d < 4; ++d)
+                        q[d] = *reinterpret_cast<const uint4*>(Rs + rr.slot * DG_RBYTES + (d0 + d) * DG_RPLANE + row * 16);
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) {
+                        const uint32_t in[4] = {q[d].x, q[d].y, q[d].z, q[d].w};
+                        uint32_t h[8];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            h[2 * e] = dg_half2(__byte_perm(in[e], 0x64646464u, 0x4140));
+                            h[2 * e + 1] = dg_half2(__byte_perm(in[e], 0x64646464u, 0x4342));
+                        }
+                        tmem_st8_nowait(tmemA + lanes + uint32_t(ra.slot * DG_ACOLS + (d0 + d) * 8), h);
                     }
-                    tmem_st8_nowait(tmemA + lanes + uint32_t(ra.slot * DG_ACOLS + d * 8), h);
                 }
                 tmem_wait_st();
                 tc_fence_before();
@@ -670,7 +667,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
         // of alpha and of the coefficient sets
         pdl_wait();
         for (int i = 0; i < nI; ++i) {
-            const int m = s_items[i].x & 0xFFFF, lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
+            const int m = s_items[i].x, lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
             int e[5] = {0, 0, 0, 0, 0}, top = 0;
 #pragma unroll 8
             for (int K = lo + lane; K <= N; K += 32) {
@@ -710,11 +707,9 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
 // ---------------------------------------------------------------------------
 // host side
 
-// LPT over one CTA per SM, CTA lists at a fixed stride.  rem (synthesis): the
-// remainder blocks of the lowest orders' first steps; their items become the
-// first step, its remainder and the later steps, one after the other.
-static void dig_schedule(sphnse_plan* P, const std::vector<int4>& items, const int* rem, int ntile, DigSide* D,
-                         std::vector<int4>& flat, std::vector<int>& cnt) {
+// LPT over one CTA per SM, CTA lists at a fixed stride
+static void dig_schedule(sphnse_plan* P, const std::vector<int4>& items, DigSide* D, std::vector<int4>& flat,
+                         std::vector<int>& cnt) {
     std::vector<int> order(items.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = int(i);
     // an item costs its steps plus about one for its epilogue and start
@@ -725,22 +720,7 @@ static void dig_schedule(sphnse_plan* P, const std::vector<int4>& items, const i
     std::vector<long> load(nc, 0);
     for (int idx : order) {
         const int b = int(std::min_element(load.begin(), load.end()) - load.begin());
-        int4 it = items[idx];
-        const int k0 = it.z & 0xFFFF, k1 = it.z >> 16;
-        if (rem && it.x < DG_SEGM) {
-            if (k0 == 0) {
-                bins[b].push_back(make_int4(it.x | 1 << 16, it.y, 1 << 16, it.w));
-                bins[b].push_back(make_int4(it.x | 1 << 18 | 1 << 19 | (k1 > 1 ? 1 << 16 : 0), it.y, 1 << 16,
-                                            rem[it.x * ntile + it.y]));
-            }
-            it.x |= 1 << 17 | (k0 == 0 ? 1 << 18 : 0);
-            it.z = std::max(k0, 1) | (k1 << 16);
-            if (k0 == 0 && k1 == 1) {
-                load[b] += cost(idx);
-                continue;
-            }
-        }
-        bins[b].push_back(it);
+        bins[b].push_back(items[idx]);
         load[b] += cost(idx);
     }
     D->ncta = nc;
@@ -782,15 +762,13 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
     const int N = P->N, nh = P->nh, ntile = (nh + 63) / 64;
     DigState& T = P->dig;
     // synthesis tiles (m, 64 latitudes), steps of 16 degrees of each parity
-    const int nseg = std::min(DG_SEGM, N + 1);
-    std::vector<int> base(size_t(N + 1 + nseg) * ntile);
+    std::vector<int> base(size_t(N + 1) * ntile);
     int nblk = 0;
     for (int m = 0; m <= N; ++m)
         for (int t = 0; t < ntile; ++t) {
             base[size_t(m) * ntile + t] = nblk;
             nblk += (ext_even(N, m) + 15) / 16;
         }
-    for (size_t i = size_t(N + 1) * ntile; i < base.size(); ++i) base[i] = nblk++;   // remainders
     // analysis tiles: four pieces of up to 32 rows of one (m, parity)
     std::vector<int4> pieces;
     for (int m = 0; m <= N; ++m)
@@ -812,12 +790,14 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
         for (int l = (m > 0 ? m : 1); l <= N; ++l, ++i) {
             const double sl = std::sqrt(double(l) * (l + 1.0));
             // alpha_l enters row l + 1 with l eps_{l+1}, row l - 1 with (l + 1) eps_l; the sum of a
-            // row's two terms takes one more bit
-            const double dn = std::max(l * eps(l + 1, m), (l + 1) * eps(l, m)) / sl;
-            eoff[i] = make_short4(short(bexp(sl)), short(bexp(1.0 / sl)), short(bexp(dn) + 1), 0);
+            // row's two terms takes one more bit; the sets of degree K are scaled by 2^dig_shift(K)
+            const double dn = std::max(std::ldexp(l * eps(l + 1, m), dig_shift(l + 1)),
+                                       std::ldexp((l + 1) * eps(l, m), dig_shift(l - 1))) / sl;
+            const int t = dig_shift(l);
+            eoff[i] = make_short4(short(bexp(sl) + t), short(bexp(1.0 / sl) + t), short(bexp(dn) + 1), 0);
         }
     DigArena A;
-    const size_t o_eas = A.add<int>(nullptr, size_t(N + 1 + DG_SEGM) * nh), o_eaa = A.add<int>(nullptr, P->n_ext);
+    const size_t o_eas = A.add<int>(nullptr, size_t(N + 1) * nh), o_eaa = A.add<int>(nullptr, P->n_ext);
     const size_t o_pc = A.add(pieces.data(), pieces.size()), o_base = A.add(base.data(), base.size());
     const size_t o_eoff = A.add(eoff.data(), eoff.size()), o_emax = A.add<int>(nullptr, size_t(3) * (N + 1));
     const size_t o_used = A.add<int>(nullptr, size_t(nblk) + ablk);
@@ -839,9 +819,7 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
     k_dig_syn_scale<<<dim3((nh + 127) / 128, N + 1), 128>>>(d_tab, T.syn.ea, N, nh);
     k_dig_ana_scale<<<(P->n_ext + 3) / 4, 128>>>(d_tab, T.ana.ea, P->n_ext, nh);
     k_dig_syn<<<dim3((ext_even(N, 0) + 15) / 16, ntile, N + 1), 256>>>(d_tab, T.syn.ea, d_base, T.syn.blocks, d_used, N,
-                                                                      nh, ntile, 0);
-    k_dig_syn<<<dim3(1, ntile, nseg), 256>>>(d_tab, T.syn.ea, d_base + size_t(N + 1) * ntile, T.syn.blocks, d_used, N, nh,
-                                             ntile, 1);
+                                                                      nh, ntile);
     k_dig_ana<<<dim3(aks, atile), 256>>>(d_tab, T.ana.ea, T.ana.pieces, T.ana.blocks, d_used + nblk, nh);
     std::vector<int> used(size_t(nblk) + ablk);
     if (cudaMemcpy(used.data(), d_used, used.size() * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -857,14 +835,14 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
         }
     std::vector<int4> fs, fa;
     std::vector<int> cs, ca;
-    dig_schedule(P, items, base.data() + size_t(N + 1) * ntile, ntile, &T.syn, fs, cs);
+    dig_schedule(P, items, &T.syn, fs, cs);
     items.clear();
     for (int t = 0; t < atile; ++t) {
         int k0 = 0;
         while (k0 < aks && !used[size_t(nblk) + size_t(t) * aks + k0]) ++k0;
         items.push_back(make_int4(t, 0, k0 | (aks << 16), t * aks));
     }
-    dig_schedule(P, items, nullptr, 0, &T.ana, fa, ca);
+    dig_schedule(P, items, &T.ana, fa, ca);
     DigArena Q;
     const size_t o_fs = Q.add(fs.data(), fs.size()), o_fa = Q.add(fa.data(), fa.size());
     const size_t o_cs = Q.add(cs.data(), cs.size()), o_ca = Q.add(ca.data(), ca.size());

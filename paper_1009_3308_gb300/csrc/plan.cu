@@ -416,7 +416,6 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
     if (!ftw.empty()) up(P->d_ftw, ftw.data(), ftw.size() * sizeof(float));
     up(P->d_lm, lm.data(), nc * sizeof(int2));
     up(P->d_finc, finc.data(), nc * sizeof(double4_32a));
-    up(P->d_prepc, prepc.data(), size_t(P->n_ext) * sizeof(double4_32a));
     {
         std::vector<float4> f32(nc), p32(P->n_ext);
         for (size_t i = 0; i < nc; ++i)
@@ -426,6 +425,14 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
         up(P->d_finc32, f32.data(), nc * sizeof(float4));
         up(P->d_prepc32, p32.data(), size_t(P->n_ext) * sizeof(float4));
     }
+    if (!small_plan(P->nh))   // exact: powers of two
+        for (int m = 0; m <= L; ++m)
+            for (int K = m; K <= L + 1; ++K) {
+                double4_32a& c = prepc[ext_row(L, m, K)];
+                const double f = std::ldexp(1.0, dig_shift(K));
+                c = make_double4_32a(f * c.x, f * c.y, f * c.z, f * c.w);
+            }
+    up(P->d_prepc, prepc.data(), size_t(P->n_ext) * sizeof(double4_32a));
     // LPT schedule of the orders m (cost L + 2 - m table rows) over one
     // persistent CTA per SM for the streaming Legendre kernels
     if (!rc) {
