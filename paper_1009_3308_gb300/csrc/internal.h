@@ -176,7 +176,8 @@ struct DigState {
     DigSide syn, ana;
     short4* eoff = nullptr;            // exponents of the coefficient sets per packed entry
     int* emax = nullptr;               // [3][N+1] largest biased exponents of the ring output; zero
-                                       // between calls (the finish kernel clears them)
+                                       // between calls (the finish kernel clears them, or
+                                       // dig_clear_exponents where it could not be launched)
     void* arena = nullptr;             // the allocation of the exponents, pieces and constants
     void* sched = nullptr;             // ... and of the item lists
 };
@@ -363,6 +364,7 @@ int dig_setup(sphnse_plan* P, const double* d_tab);
 void dig_free(sphnse_plan* P);
 int launch_synthesis_dig(sphnse_plan* P, const double* alpha, const double* beta);
 int launch_analysis_dig(sphnse_plan* P, int nf);
+void dig_clear_exponents(sphnse_plan* P);
 // FP64 sums of small plans (legendre_small.cu): per order, the analysis goes on
 // to the finish step (kind as in launch_finish)
 constexpr int SMALL_NH = 40;

@@ -900,6 +900,10 @@ int launch_synthesis_dig(sphnse_plan* P, const double* alpha, const double* beta
     return beta ? dig_launch<true, 5>(P, P->dig.syn, a) : dig_launch<true, 3>(P, P->dig.syn, a);
 }
 
+void dig_clear_exponents(sphnse_plan* P) {
+    cudaMemsetAsync(P->dig.emax, 0, size_t(3) * (P->N + 1) * sizeof(int), P->stream);
+}
+
 int launch_analysis_dig(sphnse_plan* P, int nf) {
     const DigArgs a = dig_args(P, P->dig.ana);
     return nf == 3 ? dig_launch<false, 3>(P, P->dig.ana, a) : dig_launch<false, 2>(P, P->dig.ana, a);

@@ -14,6 +14,7 @@
 #include <limits>
 #include <new>
 
+#include "chain.h"
 #include "internal.h"
 
 namespace sph {
@@ -180,8 +181,9 @@ static int synthesis64(sphnse_plan* P, const double* alpha, const double* beta) 
 static int analysis64(sphnse_plan* P, int kind, const double* alpha, const double* forcing, double* out,
                       const double* dot_with = nullptr) {
     if (small_plan(P->nh)) return launch_analysis_small(P, kind, alpha, forcing, out, dot_with);
-    const int rc = launch_analysis_dig(P, kind == 2 ? 3 : 2);
-    return rc ? rc : launch_finish(P, kind, SPHNSE_FP64, alpha, forcing, out, dot_with);
+    return chain_or_reset([&] { return launch_analysis_dig(P, kind == 2 ? 3 : 2); },
+                          [&] { return launch_finish(P, kind, SPHNSE_FP64, alpha, forcing, out, dot_with); },
+                          [&] { dig_clear_exponents(P); });
 }
 
 int rhs_device(sphnse_plan* P, const double* alpha, const double* forcing, double* out) {
