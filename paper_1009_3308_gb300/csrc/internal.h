@@ -273,7 +273,7 @@ struct sphnse_plan {
     float* d_ftw = nullptr;      // four-step ring kernel twiddles (M = 24 M2), FP32
     int2* d_lm = nullptr;        // (L, m) of each packed entry
     double4_32a* d_prepc = nullptr;  // per ext row (m, K): (lam_K^{1/2}, lam_K^{-1/2}, c_down, c_up), times
-                                     // 2^dig_shift(K) on plans of the digit sums
+                                     // 2^dig_shift(L, K) on plans of the digit sums
     float4* d_prepc32 = nullptr; // FP32 copies of the two coefficient tables
     float4* d_finc32 = nullptr;
     double4_32a* d_finc = nullptr;   // per packed (L, m): (lam^{-1/2}, L eps_{L+1,m} lam^{-1/2},
@@ -353,10 +353,14 @@ int launch_ring(sphnse_plan* P, int mode, const double* gin0, const double* gin1
                 double* gout0, double* gout1, double* gout2);
 int launch_analysis(sphnse_plan* P, int nfields);
 // Power of two by which the digit sums divide the table entries of degree K and
-// multiply its coefficient sets (prepc holds the factor): floor(log2(K + 1)).
-__host__ __device__ inline int dig_shift(int K) {
-    int t = 0;
+// multiply its coefficient sets (prepc holds the factor): floor(log2(K + 1)), less
+// its largest value and four.  With that a coefficient overflows only where it
+// exceeds the largest number 2^4 times, and the bound on it that flags an overflow
+// (it is at most 2^4 too large) flags none that binary64 holds.
+__host__ __device__ inline int dig_shift(int N, int K) {
+    int t = -4;
     for (++K; K > 1; K >>= 1) ++t;
+    for (N += 2; N > 1; N >>= 1) --t;
     return t;
 }
 // FP64 Legendre sums on the tensor cores (beta: the adjoint's fields 3, 4; nf analysis fields)

@@ -24,8 +24,8 @@
 // largest error of u_theta for the mode (9, 8) was 5.1e-15 of its maximum, with
 // eight 2.5e-16 as in a multiply-add chain.  For the columns the degrees of an
 // order are balanced: table entries of degree K are divided, coefficient sets
-// multiplied by 2^t, t = floor(log2(K + 1)) (dig_shift); without it a spectrum
-// falling like l^-4 lost a factor of four (order 1 at L = 511).  What stays below
+// multiplied by 2^t, t = floor(log2(K + 1)) up to a constant (dig_shift); without it
+// a spectrum falling like l^-4 lost a factor of four (order 1 at L = 511).  What stays below
 // the chain's precision are results smaller than 2^-60 of max|a| max|b|: the
 // projection of a field that lives on polar rows in one order above about ten.
 //
@@ -120,9 +120,9 @@ __global__ void k_dig_syn_scale(const double* __restrict__ tab, int* __restrict_
     int e = 0;
     for (int r = 0; r < cnt; ++r) {
         const int K = r < ne ? m + 2 * r : m + 1 + 2 * (r - ne);
-        e = max(e, dg_bexp(t[size_t(r) * nh]) - dig_shift(K));
+        e = max(e, dg_bexp(t[size_t(r) * nh]) - dig_shift(N, K));
     }
-    ea[m * nh + p] = max(e - 1022, DG_MINEXP);
+    ea[m * nh + p] = max(e - 1022, DG_MINEXP - dig_shift(N, 0));   // of entries scaled up by -dig_shift
 }
 __global__ void k_dig_ana_scale(const double* __restrict__ tab, int* __restrict__ ea, int n_ext, int nh) {
     const int r = blockIdx.x * 4 + threadIdx.x / 32;
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(256) k_dig_syn(const double* __restrict__ tab,
     for (int i = 0; i < 8; ++i) {
         const int j = ks * 16 + h * 8 + i;
         x[i] = j < n && p < nh ? src[size_t(j) * nh] : 0.0;
-        e[i] = p < nh ? ea[m * nh + p] + dig_shift(m + par + 2 * j) : 0;
+        e[i] = p < nh ? ea[m * nh + p] + dig_shift(N, m + par + 2 * j) : 0;
     }
     const int blk = base[m * ntile + t] + ks;
     const bool any = dig_store(x, e, out + size_t(blk) * DG_RBYTES + row * 16 + h * 8);
@@ -516,6 +516,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                 const int k1 = itm.z >> 16;
                 int4 pc[TR];
                 int kb[TR];
+                bool big = false;   // analysis: a sum of two x may exceed the largest number
                 if constexpr (!SYN) {
 #pragma unroll
                     for (int r = 0; r < TR; ++r) {
@@ -525,6 +526,10 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
 #pragma unroll
                     for (int r = 0; r < TR; ++r)
                         kb[r] = 63 - (a.emax[((r * 32 + lane) >> 3) % NF * (N + 1) + pc[r].x] - 1020);
+#pragma unroll
+                    for (int r = 0; r < TR; ++r) big = big || kb[r] < 63 - 1025;
+#pragma unroll
+                    for (int r = 0; r < TR; ++r) kb[r] += big;
                 }
                 for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, ++it) {
                     if (it % NBW != bw) continue;
@@ -575,6 +580,12 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                                 }
                             }
                         }
+                    }
+                    if (!SYN && big) {
+#pragma unroll
+                        for (int r = 0; r < TR; ++r)
+#pragma unroll
+                            for (int e = 0; e < XV; ++e) x[r][e] = make_double2(0.5 * x[r][e].x, 0.5 * x[r][e].y);
                     }
                     // SYN: the words of a column (even lanes the real, odd lanes the imaginary part's);
                     // else (re, im) of latitude 2 w, then 2 w + 1
@@ -664,7 +675,9 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
         }
     } else if constexpr (SYN) {
         // column exponents of every item: |b| <= 2^(eb - 1) from the exponents
-        // of alpha and of the coefficient sets
+        // of alpha and of the coefficient sets; NaN for a column that may hold a
+        // number beyond the largest (see dig_shift; looking at the products here
+        // cost 2.5 us at L = 511)
         pdl_wait();
         for (int i = 0; i < nI; ++i) {
             const int m = s_items[i].x, lo = m > 0 ? m : 1, pk = packed_off(N, m) - lo;
@@ -689,8 +702,8 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
             top = __reduce_max_sync(0xffffffffu, top);
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
-                const int v = __reduce_max_sync(0xffffffffu, e[f]);
-                if (lane == 0) s_eb[5 * i + f] = top == 2047 ? DG_NAN : v - 2 * 1022 + 1;
+                const int v = __reduce_max_sync(0xffffffffu, e[f]) - 2 * 1022 + 1;
+                if (lane == 0) s_eb[5 * i + f] = top == 2047 || v > 1024 ? DG_NAN : v;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sc_full[i]);
@@ -790,10 +803,10 @@ int dig_setup(sphnse_plan* P, const double* d_tab) {
         for (int l = (m > 0 ? m : 1); l <= N; ++l, ++i) {
             const double sl = std::sqrt(double(l) * (l + 1.0));
             // alpha_l enters row l + 1 with l eps_{l+1}, row l - 1 with (l + 1) eps_l; the sum of a
-            // row's two terms takes one more bit; the sets of degree K are scaled by 2^dig_shift(K)
-            const double dn = std::max(std::ldexp(l * eps(l + 1, m), dig_shift(l + 1)),
-                                       std::ldexp((l + 1) * eps(l, m), dig_shift(l - 1))) / sl;
-            const int t = dig_shift(l);
+            // row's two terms takes one more bit; the sets of degree K are scaled by 2^dig_shift(N, K)
+            const double dn = std::max(std::ldexp(l * eps(l + 1, m), dig_shift(N, l + 1)),
+                                       std::ldexp((l + 1) * eps(l, m), dig_shift(N, l - 1))) / sl;
+            const int t = dig_shift(N, l);
             eoff[i] = make_short4(short(bexp(sl) + t), short(bexp(1.0 / sl) + t), short(bexp(dn) + 1), 0);
         }
     DigArena A;

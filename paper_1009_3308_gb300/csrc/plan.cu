@@ -431,7 +431,7 @@ sphnse_plan* sphnse_plan_create(int L, int nlat, int nlon, double nu, double Ome
         for (int m = 0; m <= L; ++m)
             for (int K = m; K <= L + 1; ++K) {
                 double4_32a& c = prepc[ext_row(L, m, K)];
-                const double f = std::ldexp(1.0, dig_shift(K));
+                const double f = std::ldexp(1.0, dig_shift(L, K));
                 c = make_double4_32a(f * c.x, f * c.y, f * c.z, f * c.w);
             }
     up(P->d_prepc, prepc.data(), size_t(P->n_ext) * sizeof(double4_32a));

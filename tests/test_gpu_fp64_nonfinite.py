@@ -1,9 +1,10 @@
-"""Non-finite values through the FP64 transforms, on plans of
+"""Non-finite and overflowing values through the FP64 transforms, on plans of
 the tensor-core sums (more than 40 northern latitudes) and of the small ones.
 
 A non-finite coefficient reaches every latitude (its product with the table
 does, also where the table underflows), and a plan gives the same results after
-such a call as before it."""
+such a call as before it.  What overflows is infinite or NaN, never a finite
+number that is wrong."""
 import numpy as np
 import pytest
 
@@ -55,3 +56,33 @@ def test_nonfinite_coefficient_reaches_every_output(L, nlon, m, l, bad):
     assert not fin(plan.project(vb, v[1])).all(dim=1).any()
     for f, r in zip(ops, ref):
         assert torch.equal(f(_dev(a), _dev(w)), r)
+
+
+@pytest.mark.parametrize("size", [0.4, 1.0, 2.5, 20.0, 64.0])
+@pytest.mark.parametrize("L,nlon", [(255, 768), (100, 324), (53, 162), (33, 108)])
+def test_overflowing_vorticity(L, nlon, size):
+    # one zonal mode, its vorticity coefficient about size 2^1023
+    plan = _plan(L, nlon, 0.0, 0.0)
+    a = np.zeros(plan.n_coeff, np.complex128)
+    a[L - 1] = min(size / L, 1.9) * 2.0 ** 1023
+    exact, got = plan.grid_fields(_dev(a * 2.0 ** -64)), plan.grid_fields(_dev(a))
+    ok = torch.isfinite(got[0])
+    big = exact[0] * 2.0 ** 64
+    assert torch.equal(got[0][ok], big[ok])
+    if size <= 1.0:   # the coefficient is finite: so is what it gives away from overflowing latitudes
+        assert torch.equal(ok.all(dim=1), torch.isfinite(big).all(dim=1))
+    else:
+        assert not bool(ok.all())
+
+
+@pytest.mark.parametrize("L,nlon", [(100, 324), (53, 162), (33, 108)])
+def test_overflowing_product(L, nlon):
+    # without viscosity and rotation F is quadratic
+    plan = _plan(L, nlon, 0.0, 0.0)
+    a = coefficients(L, 31, 3.0 / L)
+    ref = torch.view_as_real(plan.rhs(_dev(a)))
+    for e in range(504, 524):
+        got = torch.view_as_real(plan.rhs(_dev(a * 2.0 ** e)))
+        ok = torch.isfinite(got)
+        assert torch.equal(got[ok], (ref * 2.0 ** 500 * 2.0 ** (2 * e - 500))[ok]), e
+    assert not bool(ok.any())
