@@ -257,10 +257,11 @@ __global__ void __launch_bounds__(576, 1) k_ring_fx(RingFxArgs a) {
     for (int r = 0; r < RPC; ++r) {
         const int row = min(row0 + r, nlat - 1);
         fc[r] = MODE == RING_GRID ? 0.0 : a.two_omega * a.x[row];
-        scale[r] = MODE == RING_GRID ? 1.0 : a.rw[row];
+        scale[r] = MODE == RING_GRID ? 0.0 : a.rw[row];
     }
     pdl_wait();
     int kf[NV];   // fixed point = value 2^kf
+    unsigned bad = 0;   // GRID: fields (bits, in the order of kf) with a non-finite input
     const double nan = __longlong_as_double(0x7FF8000000000000LL);
 
     if constexpr (MODE != RING_PROJECT) {
@@ -313,7 +314,9 @@ __global__ void __launch_bounds__(576, 1) k_ring_fx(RingFxArgs a) {
 #pragma unroll
         for (int j = 0; j < NV; ++j) {
             kf[j] = 1072 - em[j] + 26 - bitlen(s_sum[j]);
-            if (em[j] == 2047) scale[j % RPC] = nan;   // a non-finite input: NaN for its ring
+            // a non-finite input: NaN for its ring, on the grid for that field of it
+            if (MODE == RING_GRID) bad |= em[j] == 2047 ? 1u << j : 0u;
+            else if (em[j] == 2047) scale[j % RPC] = nan;
         }
         if (m <= N) {
             long long v[NV][2];
@@ -389,9 +392,10 @@ __global__ void __launch_bounds__(576, 1) k_ring_fx(RingFxArgs a) {
                     if (r == 1 && !two) break;
                     const longlong2 A = in[r * ld + fxp(q)];   // (u_theta, zeta)
                     const size_t o = size_t(row0 + r) * M + q;
-                    if (a.gout0) a.gout0[o] = f64_scale(__ll2double_rn(A.y) * scale[r], -kf[r]);
-                    if (a.gout1) a.gout1[o] = f64_scale(__ll2double_rn(A.x) * scale[r], -kf[2 + r]);
-                    if (a.gout2) a.gout2[o] = f64_scale(__ll2double_rn(r ? B.x : B.y) * scale[r], -kf[4 + r]);
+                    auto val = [&](long long v, int j) { return bad >> j & 1 ? nan : f64_scale(__ll2double_rn(v), -kf[j]); };
+                    if (a.gout0) a.gout0[o] = val(A.y, r);
+                    if (a.gout1) a.gout1[o] = val(A.x, 2 + r);
+                    if (a.gout2) a.gout2[o] = val(r ? B.x : B.y, 4 + r);
                 }
             }
             return;

@@ -69,6 +69,10 @@ def test_overflowing_vorticity(L, nlon, size):
     ok = torch.isfinite(got[0])
     big = exact[0] * 2.0 ** 64
     assert torch.equal(got[0][ok], big[ok])
+    for k in (1, 2):   # the velocity is in range where the vorticity is not
+        b = exact[k] * 2.0 ** 64
+        assert bool(torch.isfinite(b).any()) and torch.equal(torch.isfinite(got[k]), torch.isfinite(b))
+        assert torch.equal(got[k][torch.isfinite(b)], b[torch.isfinite(b)])
     if size <= 1.0:   # the coefficient is finite: so is what it gives away from overflowing latitudes
         assert torch.equal(ok.all(dim=1), torch.isfinite(big).all(dim=1))
     else:
