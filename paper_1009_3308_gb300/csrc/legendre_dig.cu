@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
             // the table does not depend on the predecessor: stream right away
             const uint64_t pol = a.evict_first ? policy_evict_first() : policy_evict_last();
             DigRing r;
-            int it = 0;
+            int it = 0, end = 0;   // blocks, and those requested (all, unless a wait ran out)
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = s_items[i];
                 const unsigned char* src = a.blocks + size_t(itm.w) * DG_RBYTES;
@@ -368,12 +368,12 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                 for (int ks = itm.z & 0xFFFF; ks < k1; ++ks, ++it, r.next(NR)) {
                     if (it >= NR && !mbar_wait(&r_empty[r.slot], r.phase ^ 1, abort, a.status)) continue;
                     if (*abort) continue;
+                    end = it + 1;
                     mbar_arrive_expect_tx(&r_full[r.slot], DG_RBYTES);
                     bulk_g2s(Rs + r.slot * DG_RBYTES, src + size_t(ks) * DG_RBYTES, DG_RBYTES, &r_full[r.slot], pol);
                 }
             }
-            for (int k = it - NR; k < it; ++k)
-                if (k >= 0) mbar_wait(&r_full[k % NR], (k / NR) & 1, abort, a.status);
+            for (int k = max(0, end - NR); k < end; ++k) mbar_drain(&r_full[k % NR], (k / NR) & 1, a.status);
         }
     } else if (warp == 1) {
         if (elect_one()) {
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                 }
                 mma_commit(&acc_full[buf]);
             }
-            if (nI > 0) mbar_wait(&acc_full[(nI - 1) % NACC], ((nI - 1) / NACC) & 1, abort, a.status);
+            if (nI > 0) mbar_drain(&acc_full[(nI - 1) % NACC], ((nI - 1) / NACC) & 1, a.status);
         }
     } else if (warp < 6) {
         pdl_wait();

@@ -66,7 +66,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return false;
 }
 
-// The same for two barriers: both are polled before either result is used (a
+// Bounded wait at the end of a role for what it has in flight, bulk copies into the
+// CTA's shared memory or MMAs on its tensor memory: these finish by themselves, so
+// it goes on when abort is set (the CTA must not exit under them).
+__device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity, unsigned* status) {
+    for (uint32_t i = 0; i < SPH_WAIT_LIMIT; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
+    if (status) atomicOr(status, SPH_STATUS_TIMEOUT);
+    return false;
+}
+
+// mbar_wait for two barriers: both are polled before either result is used (a
 // poll that succeeds at once takes 150 to 200 cycles in a busy CTA).
 __device__ __forceinline__ bool mbar_wait2(uint64_t* bar0, uint32_t parity0, uint64_t* bar1, uint32_t parity1,
                                            volatile int* abort, unsigned* status) {
