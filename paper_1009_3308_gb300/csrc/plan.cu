@@ -132,7 +132,7 @@ int ensure_tables(sphnse_plan* P, int prec) {
             if (rc == SPHNSE_OK) t.bytes = P->dig.syn.bytes + P->dig.ana.bytes;
         }
     } else if (prec == SPHNSE_FP32) {
-        rc = upload_table<float>(P, t, [](double v, bool) { return float(v); }, false, true);
+        rc = upload_table<float>(P, t, [](double v, bool) { return float(v); }, false, !ana32_ok(P));
     } else {
         // BF16 hi + lo split: hi = bf16(v), lo = bf16(v - hi)
         auto conv = [](double v, bool lo) {
