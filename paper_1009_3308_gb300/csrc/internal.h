@@ -41,16 +41,12 @@ __host__ __device__ inline void packed_lm(int N, int i, int& L, int& m) {
 
 // Complex index of (field f, order m, latitude row) in a synthesis output:
 // order-major [f][m][row], or latitude-pair-major [f][row / 2][m][row % 2]
-// (pairs != 0), the layout the four-step ring kernel reads contiguously.
+// (pairs != 0), the layout the ring kernels read contiguously.
 __host__ __device__ inline size_t gsyn_index(int pairs, int f, int m, int row, int N, int nlat) {
     return pairs ? ((size_t(f) * ((nlat + 1) / 2) + row / 2) * size_t(N + 1) + m) * 2 + (row & 1)
                  : (size_t(f) * (N + 1) + m) * size_t(nlat) + row;
 }
 
-// Extended-degree ("ext") rows: for each m the degrees K = m..N+1 (n_m = N+2-m
-// of them), split by the parity of K - m: even rows first (K = m + 2j,
-// j < ne(m)), then odd rows (K = m + 1 + 2j, j < no(m)).  Degree N+1 is needed
-// by the theta-derivative recombination.
 // sum of a 256-thread block's values (a tree, fixed order) into part[blockIdx.x];
 // every thread of the block calls it
 __device__ __forceinline__ void block_sum256(double s, double* part) {
@@ -66,6 +62,10 @@ __device__ __forceinline__ void block_sum256(double s, double* part) {
 #endif
 }
 
+// Extended-degree ("ext") rows: for each m the degrees K = m..N+1 (n_m = N+2-m
+// of them), split by the parity of K - m: even rows first (K = m + 2j,
+// j < ne(m)), then odd rows (K = m + 1 + 2j, j < no(m)).  Degree N+1 is needed
+// by the theta-derivative recombination.
 __host__ __device__ inline int ext_off(int N, int m) { return m * (N + 2) - m * (m - 1) / 2; }
 __host__ __device__ inline int ext_count(int N, int m) { return N + 2 - m; }
 __host__ __device__ inline int ext_even(int N, int m) { return (N + 3 - m) / 2; }
@@ -284,8 +284,8 @@ struct sphnse_plan {
     sph::DigState dig;
 
     // workspaces (sized for the largest field counts: 5 synthesis, 3 analysis)
-    void* d_gsyn = nullptr;      // [5][N+1][nlat] complex (m-major)
-    void* d_gana = nullptr;      // [3][N+1][nlat] complex (m-major)
+    void* d_gsyn = nullptr;      // [5] spectra of the fields, layout gsyn_index(pairs, ...)
+    void* d_gana = nullptr;      // [3] weighted spectra: FP64 latitude-pair-major, else [N+1][nlat]
     void* d_hana = nullptr;      // [n_ext][2 * 3]
     double* d_work = nullptr;    // NDF / adjoint vectors (16 x n_coeff complex)
     double* d_grid = nullptr;    // objective: two grid fields (allocated on first use)
@@ -299,7 +299,6 @@ struct sphnse_plan {
     unsigned long long* d_norms = nullptr;  // 8 reduction slots
     double* h_norms = nullptr;   // pinned host mirror
     double* h_part = nullptr;    // block partial sums, pinned: kernels write them, the host adds them up
-    size_t work_bytes = 0;
 
     // optional per-stage CUDA-event timing on the plan's stream
     unsigned timing = 0;         // bit mask of timed stages

@@ -22,43 +22,33 @@ namespace sph {
 //   field 2 (phi):   (K-1) eps_{K,m} a_{K-1} - (K+2) eps_{K+1,m} a_{K+1}
 // (sin(theta) d/dtheta Pt_L^m = L eps_{L+1,m} Pt_{L+1}^m - (L+1) eps_{L,m} Pt_{L-1}^m
 //  regrouped by degree).  The coefficients come precomputed per row, c =
-// (lam^{1/2}, lam^{-1/2}, c_down, c_up).  With beta (adjoint): fields 3, 4 are
-// the theta/phi sets of beta / s_m, s_m = 1 (m = 0) or 2.
-// FP32-path prep: alpha_K is converted once per row and its degree
+// (lam^{1/2}, lam^{-1/2}, c_down, c_up).  alpha_K is converted once per row and its degree
 // neighbours come from shared memory; the arithmetic is FP32 (the FP32 path
 // contracts in FP32 anyway), keeping the weak FP64 pipe for the state only.
-__global__ void __launch_bounds__(128) k_prep32(const double2* __restrict__ alpha, const double2* __restrict__ beta,
-                                                const float4* __restrict__ prepc, float* __restrict__ bsyn, int N,
-                                                int nf, int ncoef, size_t bstride) {
-    __shared__ float2 sa[130], sb[130];
+__global__ void __launch_bounds__(128) k_prep32(const double2* __restrict__ alpha, const float4* __restrict__ prepc,
+                                                float* __restrict__ bsyn, int N, int ncoef, size_t bstride) {
+    __shared__ float2 sa[130];
     pdl_launch();
     pdl_wait();   // alpha may be the predecessor's output
     // batch of instances along gridDim.z (fixed strides between instances)
     alpha += size_t(blockIdx.z) * ncoef;
-    if (beta) beta += size_t(blockIdx.z) * ncoef;
     bsyn += size_t(blockIdx.z) * bstride;
     const int m = blockIdx.y, t = threadIdx.x;
     const int K0 = m + blockIdx.x * 128, K = K0 + t;
     const int lo = m > 0 ? m : 1;
-    const float sc = m == 0 ? 1.f : 0.5f;
-    auto ld = [&](const double2* v, int Kp, float scale) -> float2 {
+    auto ld = [&](int Kp) -> float2 {
         if (Kp < lo || Kp > N) return make_float2(0.f, 0.f);
-        const double2 c = v[packed_index(N, m, Kp)];
-        return make_float2(float(c.x) * scale, float(c.y) * scale);
+        const double2 c = alpha[packed_index(N, m, Kp)];
+        return make_float2(float(c.x), float(c.y));
     };
-    sa[t + 1] = ld(alpha, K, 1.f);
-    if (t == 0) sa[0] = ld(alpha, K0 - 1, 1.f);
-    if (t == 127) sa[129] = ld(alpha, K0 + 128, 1.f);
-    if (nf == 5) {
-        sb[t + 1] = ld(beta, K, sc);
-        if (t == 0) sb[0] = ld(beta, K0 - 1, sc);
-        if (t == 127) sb[129] = ld(beta, K0 + 128, sc);
-    }
+    sa[t + 1] = ld(K);
+    if (t == 0) sa[0] = ld(K0 - 1);
+    if (t == 127) sa[129] = ld(K0 + 128);
     __syncthreads();
     if (K > N + 1) return;
     const int row = ext_row(N, m, K);
     const float4 c = prepc[row];
-    float* out = bsyn + size_t(row) * (2 * nf);
+    float* out = bsyn + size_t(row) * 6;
     const float2 a0 = sa[t + 1], am = sa[t], ap = sa[t + 2];
     out[0] = c.x * a0.x;
     out[1] = c.x * a0.y;
@@ -66,13 +56,6 @@ __global__ void __launch_bounds__(128) k_prep32(const double2* __restrict__ alph
     out[3] = c.y * a0.y;
     out[4] = fmaf(c.z, am.x, c.w * ap.x);
     out[5] = fmaf(c.z, am.y, c.w * ap.y);
-    if (nf == 5) {
-        const float2 b0 = sb[t + 1], bm = sb[t], bp = sb[t + 2];
-        out[6] = c.y * b0.x;
-        out[7] = c.y * b0.y;
-        out[8] = fmaf(c.z, bm.x, c.w * bp.x);
-        out[9] = fmaf(c.z, bm.y, c.w * bp.y);
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -81,13 +64,13 @@ __global__ void __launch_bounds__(128) k_prep32(const double2* __restrict__ alph
 // p' the mirror row; the table block is [nh][rows] so that threads of a warp
 // read consecutive degrees.  G already carries (2 pi / M) w_p / sin(theta_p)
 // (and sin(theta_p) for the scalar adjoint field).
-template <typename T, int NF>
-__global__ void __launch_bounds__(128) k_analysis(const T* __restrict__ pana, const T* __restrict__ gana,
-                                                   T* __restrict__ hana, int N, int nh, int nlat) {
+template <int NF>
+__global__ void __launch_bounds__(128) k_analysis(const float* __restrict__ pana, const float* __restrict__ gana,
+                                                   float* __restrict__ hana, int N, int nh, int nlat) {
     pdl_launch();
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* S = reinterpret_cast<T*>(smem_raw);  // [nh][2 NF]
+    float* S = reinterpret_cast<float*>(smem_raw);  // [nh][2 NF]
     const int m = blockIdx.y, par = blockIdx.z;
     const int ne = ext_even(N, m), no = ext_odd(N, m);
     const int nrows = par ? no : ne;
@@ -96,10 +79,10 @@ __global__ void __launch_bounds__(128) k_analysis(const T* __restrict__ pana, co
     for (int i = threadIdx.x; i < nh * NF; i += blockDim.x) {
         const int p = i / NF, f = i % NF;
         const int pr = nlat - 1 - p;
-        const T* a = gana + gsyn_index(0, f, m, p, N, nlat) * 2;
-        T ar = a[0], ai = a[1], br = T(0), bi = T(0);
+        const float* a = gana + gsyn_index(0, f, m, p, N, nlat) * 2;
+        float ar = a[0], ai = a[1], br = 0.f, bi = 0.f;
         if (pr != p) {
-            const T* b = gana + gsyn_index(0, f, m, pr, N, nlat) * 2;
+            const float* b = gana + gsyn_index(0, f, m, pr, N, nlat) * 2;
             br = b[0];
             bi = b[1];
         }
@@ -109,18 +92,18 @@ __global__ void __launch_bounds__(128) k_analysis(const T* __restrict__ pana, co
     __syncthreads();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= nrows) return;
-    T acc[2 * NF];
+    float acc[2 * NF];
 #pragma unroll
-    for (int f = 0; f < 2 * NF; ++f) acc[f] = T(0);
-    const T* Pa = pana + size_t(rowstart) * nh + j;
+    for (int f = 0; f < 2 * NF; ++f) acc[f] = 0.f;
+    const float* Pa = pana + size_t(rowstart) * nh + j;
 #pragma unroll 4
     for (int p = 0; p < nh; ++p) {
-        const T pv = __ldg(Pa + size_t(p) * nrows);
-        const T* sp = S + p * 2 * NF;
+        const float pv = __ldg(Pa + size_t(p) * nrows);
+        const float* sp = S + p * 2 * NF;
 #pragma unroll
         for (int f = 0; f < 2 * NF; ++f) acc[f] = fma(pv, sp[f], acc[f]);
     }
-    T* dst = hana + size_t(rowstart + j) * 2 * NF;
+    float* dst = hana + size_t(rowstart + j) * 2 * NF;
 #pragma unroll
     for (int f = 0; f < 2 * NF; ++f) dst[f] = acc[f];
 }
@@ -143,8 +126,7 @@ __device__ __forceinline__ double lam_dot(int L, double2 a, double2 b) {
     return double(L) * (L + 1.0) * (a.x * b.x + a.y * b.y);
 }
 
-template <typename T>
-__global__ void k_finish(int kind, const T* __restrict__ hana, int nf, const double2* __restrict__ alpha,
+__global__ void k_finish(int kind, const double* __restrict__ hana, int nf, const double2* __restrict__ alpha,
                          const double2* __restrict__ forcing, double2* __restrict__ out,
                          const int2* __restrict__ lm, const double4_32a* __restrict__ finc, int N, double nu,
                          int n, double omega_d, int* __restrict__ emax, const double2* dot_with,
@@ -158,15 +140,15 @@ __global__ void k_finish(int kind, const T* __restrict__ hana, int nf, const dou
     if (i >= n) return;
     const int L = lm[i].x, m = lm[i].y;
     const double4_32a c = finc[i];
-    const T* hL = hana + size_t(ext_row(N, m, L)) * 2 * nf;
-    const T* hU = hana + size_t(ext_row(N, m, L + 1)) * 2 * nf;
-    const double htr = double(hL[0]), hti = double(hL[1]);
-    const double hur = double(hU[2]), hui = double(hU[3]);
+    const double* hL = hana + size_t(ext_row(N, m, L)) * 2 * nf;
+    const double* hU = hana + size_t(ext_row(N, m, L + 1)) * 2 * nf;
+    const double htr = hL[0], hti = hL[1];
+    const double hur = hU[2], hui = hU[3];
     double hdr = 0.0, hdi = 0.0;
     if (L - 1 >= m) {
-        const T* hD = hana + size_t(ext_row(N, m, L - 1)) * 2 * nf;
-        hdr = double(hD[2]);
-        hdi = double(hD[3]);
+        const double* hD = hana + size_t(ext_row(N, m, L - 1)) * 2 * nf;
+        hdr = hD[2];
+        hdi = hD[3];
     }
     const double cm = c.x * m;
     const double nr = cm * hti - (c.y * hur - c.z * hdr);
@@ -189,8 +171,8 @@ __global__ void k_finish(int kind, const T* __restrict__ hana, int nf, const dou
         const double2 wv = alpha[i];
         const double sm = m == 0 ? 1.0 : 2.0;
         const double sl = lam * c.x;  // lambda^{1/2}
-        r.x = -nu * lam * wv.x - sm * (nr + sl * double(hL[4]));
-        r.y = -nu * lam * wv.y - sm * (ni + sl * double(hL[5]));
+        r.x = -nu * lam * wv.x - sm * (nr + sl * hL[4]);
+        r.y = -nu * lam * wv.y - sm * (ni + sl * hL[5]);
     }
     out[i] = r;
 }
@@ -252,25 +234,25 @@ __global__ void k_finish32(int kind, const float* __restrict__ hana, int nf, con
 // ---------------------------------------------------------------------------
 // launchers
 
-template <typename T, int NF>
+template <int NF>
 static int anal_t(sphnse_plan* P) {
     const int maxrows = ext_even(P->N, 0);
     dim3 blk(128), grd((maxrows + 127) / 128, P->N + 1, 2);
-    size_t sm = size_t(P->nh) * 2 * NF * sizeof(T);
+    size_t sm = size_t(P->nh) * 2 * NF * sizeof(float);
     if (sm > 48 * 1024) {
-        allow_dynamic_smem(reinterpret_cast<const void*>(k_analysis<T, NF>), sm);
+        allow_dynamic_smem(reinterpret_cast<const void*>(k_analysis<NF>), sm);
     }
     stage_begin(P, SPHNSE_STAGE_ANALYSIS);
-    launch_pdl_small(P->n_cta, k_analysis<T, NF>, grd, blk, sm, P->stream,
-               reinterpret_cast<const T*>(P->tab[SPHNSE_FP32].ana),
-               reinterpret_cast<const T*>(P->d_gana), reinterpret_cast<T*>(P->d_hana), P->N, P->nh, P->nlat);
+    launch_pdl_small(P->n_cta, k_analysis<NF>, grd, blk, sm, P->stream,
+               reinterpret_cast<const float*>(P->tab[SPHNSE_FP32].ana),
+               reinterpret_cast<const float*>(P->d_gana), reinterpret_cast<float*>(P->d_hana), P->N, P->nh, P->nlat);
     stage_end(P, SPHNSE_STAGE_ANALYSIS);
     return check_cuda(cudaGetLastError());
 }
 
 int launch_analysis(sphnse_plan* P, int nfields) {
     if (ana32_ok(P)) return launch_analysis32(P, nfields);
-    return nfields == 3 ? anal_t<float, 3>(P) : anal_t<float, 2>(P);
+    return nfields == 3 ? anal_t<3>(P) : anal_t<2>(P);
 }
 
 int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha, const double* forcing,
@@ -282,7 +264,7 @@ int launch_finish(sphnse_plan* P, int kind, int prec, const double* alpha, const
     dim3 blk(256), grd((n + 255) / 256);
     stage_begin(P, SPHNSE_STAGE_FINISH);
     if (prec == SPHNSE_FP64)
-        launch_pdl_small(P->n_cta, k_finish<double>, grd, blk, 0, P->stream, kind, static_cast<const double*>(P->d_hana), nf,
+        launch_pdl_small(P->n_cta, k_finish, grd, blk, 0, P->stream, kind, static_cast<const double*>(P->d_hana), nf,
                                                      reinterpret_cast<const double2*>(alpha),
                                                      reinterpret_cast<const double2*>(forcing),
                                                      reinterpret_cast<double2*>(out), P->d_lm, P->d_finc, P->N, P->nu, n,
@@ -302,8 +284,7 @@ int launch_prep32_batch(sphnse_plan* P, int nb, const double* alpha, float* bsyn
     dim3 blk(128), grd((P->N + 2 + 127) / 128, P->N + 1, nb);
     stage_begin(P, SPHNSE_STAGE_PREP);
     launch_pdl(k_prep32, grd, blk, 0, P->stream, reinterpret_cast<const double2*>(alpha),
-               static_cast<const double2*>(nullptr), static_cast<const float4*>(P->d_prepc32), bsyn, P->N, 3,
-               P->n_coeff, bstride);
+               static_cast<const float4*>(P->d_prepc32), bsyn, P->N, P->n_coeff, bstride);
     stage_end(P, SPHNSE_STAGE_PREP);
     return check_cuda(cudaGetLastError());
 }

@@ -47,9 +47,9 @@ __host__ __device__ constexpr int ring_stride(int M) { return M + ((M + 15) >> 4
 // One stage of radix R over the 2 ns signals (ns per ring, rings rs apart),
 // from -> to; Ns = product of the earlier radices, step = M / (Ns R).  FIRST:
 // Ns = 1, every twiddle is 1.
-template <typename T, int R, int SIGN, bool FIRST = false>
-__device__ __forceinline__ void stage(cx<T>* sm, int from, int to, int ns, int rs, int M, int Ns, int step,
-                                      const T* tw) {
+template <int R, int SIGN, bool FIRST = false>
+__device__ __forceinline__ void stage(cx<float>* sm, int from, int to, int ns, int rs, int M, int Ns, int step,
+                                      const float* tw) {
     const int nb = M / R, ld = ring_stride(M);
     const float rns = 1.f / float(Ns);
 #pragma unroll 1
@@ -62,7 +62,7 @@ __device__ __forceinline__ void stage(cx<T>* sm, int from, int to, int ns, int r
         const int o = sg < ns ? sg * ld : rs + (sg - ns) * ld;
         // j / Ns: exact, as j + 1/2 is at least 1 / (2 Ns) away from every multiple
         const int q = int((float(j) + 0.5f) * rns), k = j - q * Ns;
-        cx<T> v[R];
+        cx<float> v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = sm[from + o + rpad(j + r * nb)];
         if constexpr (!FIRST) {
@@ -70,12 +70,12 @@ __device__ __forceinline__ void stage(cx<T>* sm, int from, int to, int ns, int r
             for (int r = 1; r < R; ++r) {
                 // which product of a sum is rounded is spelled out, or the compiler picks
                 // it anew for each instance of this loop and results differ between them
-                const cx<T> a = v[r], w = twiddle<T>(tw, k * r * step, SIGN);
+                const cx<float> a = v[r], w = twiddle<float>(tw, k * r * step, SIGN);
                 v[r] = {fmaf(a.x, w.x, -__fmul_rn(a.y, w.y)),
                         R == 2 && SIGN < 0 ? fmaf(a.x, w.y, __fmul_rn(a.y, w.x)) : fmaf(a.y, w.x, __fmul_rn(a.x, w.y))};
             }
         }
-        dft<T, R>(v, SIGN);
+        dft<float, R>(v, SIGN);
 #pragma unroll
         for (int r = 0; r < R; ++r) sm[to + o + rpad(q * Ns * R + k + r * Ns)] = v[r];
     }
@@ -84,17 +84,17 @@ __device__ __forceinline__ void stage(cx<T>* sm, int from, int to, int ns, int r
 
 // Full M-point transforms (SIGN -1 forward, +1 inverse) of the signals at entry
 // `from` of the shared array, `to` the other buffer; returns the result's entry.
-template <typename T, int SIGN>
-__device__ __forceinline__ int fft(cx<T>* sm, int from, int to, int ns, int rs, const FFTPlan& plan, const T* tw) {
+template <int SIGN>
+__device__ __forceinline__ int fft(cx<float>* sm, int from, int to, int ns, int rs, const FFTPlan& plan, const float* tw) {
     int Ns = 1, step = plan.n;
 #pragma unroll 1
     for (int st = 0; st < plan.nstages; ++st) {
         const int R = plan.radix[st];
-        if (R == 8 && st == 0) stage<T, 8, SIGN, true>(sm, from, to, ns, rs, plan.n, 1, step /= 8, tw);
-        else if (R == 8) stage<T, 8, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 8, tw);
-        else if (R == 4) stage<T, 4, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 4, tw);
-        else if (R == 2) stage<T, 2, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 2, tw);
-        else stage<T, 3, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 3, tw);
+        if (R == 8 && st == 0) stage<8, SIGN, true>(sm, from, to, ns, rs, plan.n, 1, step /= 8, tw);
+        else if (R == 8) stage<8, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 8, tw);
+        else if (R == 4) stage<4, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 4, tw);
+        else if (R == 2) stage<2, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 2, tw);
+        else stage<3, SIGN>(sm, from, to, ns, rs, plan.n, Ns, step /= 3, tw);
         Ns *= R;
         const int t = from;
         from = to;
@@ -104,13 +104,13 @@ __device__ __forceinline__ int fft(cx<T>* sm, int from, int to, int ns, int rs, 
 }
 
 struct RingArgs {
-    int N, M, nlat, mode;
+    int N, M, nlat;
     double two_omega;
     const double* x;       // cos(theta)
     const double* s;       // sin(theta)
     const double* rw;      // (2 pi / M) w_p / sin(theta_p)
-    const void* gsyn;      // [nf][pair][N+1][2] complex T
-    void* gana;            // [nf][N+1][nlat] complex T
+    const void* gsyn;      // [nf][pair][N+1][2] complex float
+    void* gana;            // [nf][N+1][nlat] complex float
     const double* gin0;    // grid input rows (PROJECT)
     const double* gin1;
     double* gout0;         // grid output rows (GRID)
@@ -120,23 +120,23 @@ struct RingArgs {
     int early;             // a grid of one wave: the successor may start its prologue at once
 };
 
-template <typename T, typename TW, int MODE>
+template <int MODE>
 __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant__ FFTPlan plan,
-                                              const TW* __restrict__ tw) {
+                                              const float* __restrict__ tw) {
     if (a.early) pdl_launch();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int NBUF = MODE == RING_ADJOINT ? 3 : (MODE == RING_PROJECT ? 1 : 2);
     const int M = a.M, N = a.N, nlat = a.nlat, pair = blockIdx.x, npair = (nlat + 1) / 2, row0 = 2 * pair;
     const int ls = ring_stride(M), rs = NBUF * ls;     // signal and ring strides
-    cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);    // [2 rings][NBUF][ls], twice
+    cx<float>* sm = reinterpret_cast<cx<float>*>(smem_raw);    // [2 rings][NBUF][ls], twice
     int cur = 0;                                       // the buffer that holds the signals: entry 0 or 2 rs
     // the twiddle table e^{-2 pi i t / M} lives in shared memory after the buffers
-    T* tws = reinterpret_cast<T*>(sm + 4 * rs);
-    for (int t = threadIdx.x; t < 2 * M; t += blockDim.x) tws[t] = T(tw[t]);
+    float* tws = reinterpret_cast<float*>(sm + 4 * rs);
+    for (int t = threadIdx.x; t < 2 * M; t += blockDim.x) tws[t] = tw[t];
     const bool two = row0 + 1 < nlat;                  // an odd grid's last pair has one ring
     const size_t ld = size_t(N + 1);
-    const cx<T>* gs = reinterpret_cast<const cx<T>*>(a.gsyn) + size_t(blockIdx.y) * a.sgs;
-    cx<T>* ga = reinterpret_cast<cx<T>*>(a.gana) + size_t(blockIdx.y) * a.sga;
+    const cx<float>* gs = reinterpret_cast<const cx<float>*>(a.gsyn) + size_t(blockIdx.y) * a.sgs;
+    cx<float>* ga = reinterpret_cast<cx<float>*>(a.gana) + size_t(blockIdx.y) * a.sga;
     pdl_wait();
 
     if constexpr (MODE != RING_PROJECT) {
@@ -149,9 +149,9 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant_
                 const int fa = 2 * sgi, fb = 2 * sgi + 1;
                 const bool has_b = (MODE == RING_ADJOINT) ? fb <= 4 : fb <= 2;
                 // order m of both rings
-                cx<T> A[2] = {{T(0), T(0)}, {T(0), T(0)}}, Bv[2] = {{T(0), T(0)}, {T(0), T(0)}};
+                cx<float> A[2] = {{0.f, 0.f}, {0.f, 0.f}}, Bv[2] = {{0.f, 0.f}, {0.f, 0.f}};
                 if (m <= N) {
-                    const cx<T>* g = gs + ((size_t(fa) * npair + pair) * ld + m) * 2;
+                    const cx<float>* g = gs + ((size_t(fa) * npair + pair) * ld + m) * 2;
                     const float4 u = *reinterpret_cast<const float4*>(g);
                     A[0] = {u.x, u.y};
                     if (two) A[1] = {u.z, u.w};
@@ -163,16 +163,16 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant_
                 }
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
-                    cx<T> ga_ = A[r], gb_ = Bv[r];
-                    if (m == 0) { ga_.y = T(0); gb_.y = T(0); }
-                    cx<T>* z = sm + r * rs + sgi * ls;
+                    cx<float> ga_ = A[r], gb_ = Bv[r];
+                    if (m == 0) { ga_.y = 0.f; gb_.y = 0.f; }
+                    cx<float>* z = sm + r * rs + sgi * ls;
                     z[rpad(m)] = {ga_.x - gb_.y, ga_.y + gb_.x};
                     if (m > 0 && m <= N) z[rpad(M - m)] = {ga_.x + gb_.y, gb_.x - ga_.y};
                 }
             }
         }
         __syncthreads();
-        cur = fft<T, +1>(sm, cur, 2 * rs - cur, nsig, rs, plan, tws);
+        cur = fft<+1>(sm, cur, 2 * rs - cur, nsig, rs, plan, tws);
     }
 
     // point q of ring r, both rings over the CTA's threads
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant_
         }
     };
     if constexpr (MODE == RING_GRID) {
-        points([&](int r, int q, const cx<T>* z) {
+        points([&](int r, int q, const cx<float>* z) {
             if (r && !two) return;
             const size_t o = size_t(row0 + r) * M + q;
             if (a.gout0) a.gout0[o] = double(z[0].x);
@@ -194,37 +194,37 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant_
     }
 
     constexpr int nout = MODE == RING_ADJOINT ? 2 : 1;
-    const T fc0 = T(a.two_omega * a.x[row0]), fc1 = T(a.two_omega * a.x[min(row0 + 1, nlat - 1)]);
+    const float fc0 = float(a.two_omega * a.x[row0]), fc1 = float(a.two_omega * a.x[min(row0 + 1, nlat - 1)]);
     if constexpr (MODE == RING_RHS) {
-        points([&](int r, int q, cx<T>* z) {
-            const T zeta = z[0].x, uth = z[0].y, uph = z[ls].x;
-            const T qq = zeta + (r ? fc1 : fc0);
+        points([&](int r, int q, cx<float>* z) {
+            const float zeta = z[0].x, uth = z[0].y, uph = z[ls].x;
+            const float qq = zeta + (r ? fc1 : fc0);
             z[0] = {-qq * uph, qq * uth};
         });
     } else if constexpr (MODE == RING_PROJECT) {
-        points([&](int r, int q, cx<T>* z) {
+        points([&](int r, int q, cx<float>* z) {
             const size_t o = size_t(row0 + r) * M + q;
-            z[0] = r && !two ? cx<T>{T(0), T(0)} : cx<T>{T(a.gin0[o]), T(a.gin1[o])};
+            z[0] = r && !two ? cx<float>{0.f, 0.f} : cx<float>{float(a.gin0[o]), float(a.gin1[o])};
         });
     } else {  // RING_ADJOINT: fields zeta, u_th, u_ph, v_th, v_ph
-        points([&](int r, int q, cx<T>* z) {
-            const T zeta = z[0].x, uth = z[0].y;
-            const T uph = z[ls].x, vth = z[ls].y, vph = z[2 * ls].x;
-            const T qq = zeta + (r ? fc1 : fc0);
+        points([&](int r, int q, cx<float>* z) {
+            const float zeta = z[0].x, uth = z[0].y;
+            const float uph = z[ls].x, vth = z[ls].y, vph = z[2 * ls].x;
+            const float qq = zeta + (r ? fc1 : fc0);
             // X = -q xhat x v = (q v_phi, -q v_theta); rho = v . (xhat x u) = -v_th u_ph + v_ph u_th
             z[0] = {qq * vph, -qq * vth};
-            z[ls] = {-vth * uph + vph * uth, T(0)};
+            z[ls] = {-vth * uph + vph * uth, 0.f};
         });
     }
     __syncthreads();
-    cur = fft<T, -1>(sm, cur, 2 * rs - cur, nout, rs, plan, tws);
+    cur = fft<-1>(sm, cur, 2 * rs - cur, nout, rs, plan, tws);
 
     // both rings of order m at once: two latitudes are 16 bytes of the order-major output
-    T scale[2];
+    float scale[2];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) scale[r] = T(a.rw[min(row0 + r, nlat - 1)]);
-    auto put = [&](int f, int m, const cx<T> (&v)[2]) {
-        cx<T>* d = ga + (size_t(f) * ld + m) * nlat + row0;
+    for (int r = 0; r < 2; ++r) scale[r] = float(a.rw[min(row0 + r, nlat - 1)]);
+    auto put = [&](int f, int m, const cx<float> (&v)[2]) {
+        cx<float>* d = ga + (size_t(f) * ld + m) * nlat + row0;
         if (nlat % 2 == 0) {
             *reinterpret_cast<float4*>(d) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
         } else {   // rows of an odd grid are 8-byte aligned
@@ -233,22 +233,22 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant_
         }
     };
     for (int m = threadIdx.x; m <= N; m += blockDim.x) {
-        cx<T> oA[2], oB[2], oC[2];
+        cx<float> oA[2], oB[2], oC[2];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            const cx<T>* Z = sm + cur + r * rs;
-            const cx<T> p = Z[rpad(m)];
-            const cx<T> q = Z[rpad(m == 0 ? 0 : M - m)];
+            const cx<float>* Z = sm + cur + r * rs;
+            const cx<float> p = Z[rpad(m)];
+            const cx<float> q = Z[rpad(m == 0 ? 0 : M - m)];
             // W = A + i B with A, B real fields: A_m = (Z_m + conj Z_{M-m}) / 2,
             // B_m = (Z_m - conj Z_{M-m}) / (2 i)
-            cx<T> A{T(0.5) * (p.x + q.x), T(0.5) * (p.y - q.y)};
-            cx<T> Bv{T(0.5) * (p.y + q.y), T(0.5) * (q.x - p.x)};
+            cx<float> A{0.5f * (p.x + q.x), 0.5f * (p.y - q.y)};
+            cx<float> Bv{0.5f * (p.y + q.y), 0.5f * (q.x - p.x)};
             oA[r] = {A.x * scale[r], A.y * scale[r]};
             oB[r] = {Bv.x * scale[r], Bv.y * scale[r]};
             if constexpr (nout == 2) {
                 // scalar field rho: plain quadrature weight (2 pi / M) w_p
-                const T sc2 = scale[r] * T(a.s[min(row0 + r, nlat - 1)]);
-                const cx<T> z = Z[ls + rpad(m)];
+                const float sc2 = scale[r] * float(a.s[min(row0 + r, nlat - 1)]);
+                const cx<float> z = Z[ls + rpad(m)];
                 oC[r] = {z.x * sc2, z.y * sc2};
             }
         }
@@ -258,8 +258,8 @@ __global__ void __launch_bounds__(512) k_ring(RingArgs a, const __grid_constant_
     }
 }
 
-template <typename T, typename TW, int MODE>
-static void ring_t(sphnse_plan* P, RingArgs a, const TW* tw, int nb = 1) {
+template <int MODE>
+static void ring_t(sphnse_plan* P, RingArgs a, const float* tw, int nb = 1) {
     const int nbuf = MODE == RING_ADJOINT ? 3 : (MODE == RING_PROJECT ? 1 : 2);
     // Two threads per butterfly of the average stage: half of them idle in the
     // stages, all of them load and store.  One thread per radix-8 butterfly was
@@ -268,10 +268,10 @@ static void ring_t(sphnse_plan* P, RingArgs a, const TW* tw, int nb = 1) {
     int nb_sum = 0;
     for (int i = 0; i < P->fft.nstages; ++i) nb_sum += P->nlon / P->fft.radix[i];
     const int threads = std::min(512, std::max(64, (4 * nbuf * nb_sum / P->fft.nstages + 31) / 32 * 32));
-    const size_t sm = size_t(4 * nbuf) * ring_stride(P->nlon) * sizeof(cx<T>) + size_t(P->nlon) * 2 * sizeof(T);
-    allow_dynamic_smem(reinterpret_cast<const void*>(k_ring<T, TW, MODE>), sm);
+    const size_t sm = size_t(4 * nbuf) * ring_stride(P->nlon) * sizeof(cx<float>) + size_t(P->nlon) * 2 * sizeof(float);
+    allow_dynamic_smem(reinterpret_cast<const void*>(k_ring<MODE>), sm);
     a.early = long(P->nlat + 1) / 2 * nb <= long(P->nsm) * std::min<long>(512 / threads, (227 << 10) / long(sm + 1024));
-    launch_pdl(k_ring<T, TW, MODE>, dim3((P->nlat + 1) / 2, nb), dim3(threads), sm, P->stream, a, P->fft, tw);
+    launch_pdl(k_ring<MODE>, dim3((P->nlat + 1) / 2, nb), dim3(threads), sm, P->stream, a, P->fft, tw);
 }
 
 // FP32 RHS ring pass over nb instances (latitude-pair-major in, order-major out, with strides)
@@ -280,7 +280,6 @@ int launch_ring_batch(sphnse_plan* P, int nb, const float* gsyn, size_t sgs, flo
     a.N = P->N;
     a.M = P->nlon;
     a.nlat = P->nlat;
-    a.mode = RING_RHS;
     a.two_omega = 2.0 * P->Omega;
     a.x = P->d_x;
     a.s = P->d_s;
@@ -290,18 +289,17 @@ int launch_ring_batch(sphnse_plan* P, int nb, const float* gsyn, size_t sgs, flo
     a.sgs = sgs / 2;
     a.sga = sga / 2;
     stage_begin(P, SPHNSE_STAGE_RING);
-    ring_t<float, float, RING_RHS>(P, a, P->d_tw32, nb);
+    ring_t<RING_RHS>(P, a, P->d_tw32, nb);
     stage_end(P, SPHNSE_STAGE_RING);
     return check_cuda(cudaGetLastError());
 }
 
-template <typename T, typename TW>
-static void ring_mode(sphnse_plan* P, int mode, const RingArgs& a, const TW* tw) {
+static void ring_mode(sphnse_plan* P, int mode, const RingArgs& a, const float* tw) {
     switch (mode) {
-        case RING_RHS: ring_t<T, TW, RING_RHS>(P, a, tw); break;
-        case RING_GRID: ring_t<T, TW, RING_GRID>(P, a, tw); break;
-        case RING_PROJECT: ring_t<T, TW, RING_PROJECT>(P, a, tw); break;
-        default: ring_t<T, TW, RING_ADJOINT>(P, a, tw); break;
+        case RING_RHS: ring_t<RING_RHS>(P, a, tw); break;
+        case RING_GRID: ring_t<RING_GRID>(P, a, tw); break;
+        case RING_PROJECT: ring_t<RING_PROJECT>(P, a, tw); break;
+        default: ring_t<RING_ADJOINT>(P, a, tw); break;
     }
 }
 
@@ -311,7 +309,6 @@ int launch_ring(sphnse_plan* P, int mode, const double* gin0, const double* gin1
     a.N = P->N;
     a.M = P->nlon;
     a.nlat = P->nlat;
-    a.mode = mode;
     a.two_omega = mode == RING_RHS && P->coriolis_split ? 0.0 : 2.0 * P->Omega;
     a.x = P->d_x;
     a.s = P->d_s;
@@ -325,7 +322,7 @@ int launch_ring(sphnse_plan* P, int mode, const double* gin0, const double* gin1
     a.gout2 = gout2;
     a.sgs = a.sga = 0;
     stage_begin(P, SPHNSE_STAGE_RING);
-    ring_mode<float, float>(P, mode, a, P->d_tw32);
+    ring_mode(P, mode, a, P->d_tw32);
     stage_end(P, SPHNSE_STAGE_RING);
     return check_cuda(cudaGetLastError());
 }
