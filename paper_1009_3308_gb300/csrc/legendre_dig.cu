@@ -9,11 +9,12 @@
 // s = 2 .. 10:
 //     sum_k a b = sum_s 2^(2 - 8 s) D_s,   D_s = sum_{i + j = s} sum_k a_i b_j,
 // and the epilogue adds the groups in integers.  Digits are exact in FP16, their
-// products are integers of at most 2^14, and D_s of the four leading groups stays
-// below 2^24 for the 384 terms of the largest plan, so that the FP32
-// accumulators hold it exactly; from s = 6 on a bound of 2^25.3 is above that,
-// but digits past the first are spread out (their sums reach about 2^20), and one
-// rounding there would be 2^-45 of a group's weight 2^(2 - 48).
+// products are integers of at most 2^14.  For the digits of these tables (14
+// orders at L = 511) no column makes |D_s| reach 2^24 in the synthesis, nor in
+// the analysis up to s = 6, so that the FP32 accumulators hold it exactly; the
+// bound of the analysis' last groups is 2^24.6, where a rounding is worth 2^-54
+// of max|a| max|b| at most (no such sum has been seen: digits past the first
+// are spread out and sums stay near 2^20).
 //
 // Error.  Relative to max|a| max|b| of a row and a column, digits end at 2^-64
 // and the products left out (i + j > 10) add up to about 2^-67.  A multiply-add
@@ -100,7 +101,8 @@ __device__ __forceinline__ uint64_t dg_desc(const void* smem_ptr) {
 
 // two bytes digit + 128 under 0x64 are the FP16 numbers 1152 + digit
 __device__ __forceinline__ uint32_t dg_half2(uint32_t w) {
-    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480)));
+    const __half2 bias = __half2half2(__ushort_as_half(0x6480));
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), bias);
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
@@ -575,8 +577,11 @@ __global__ void __launch_bounds__(32 * DigShape<SYN, NF>::WARPS, 1) k_dig(DigArg
                                 } else {
                                     // mirrors in different pairs; the equator is its own mirror
                                     const int q0 = nlat - 1 - p, q1 = nlat - 2 - p;
-                                    if (q0 != p) x[r][2] = *reinterpret_cast<const double2*>(g + size_t(q0 / 2) * ld + 2 * (q0 & 1));
-                                    if (q1 > p + 1) x[r][3] = *reinterpret_cast<const double2*>(g + size_t(q1 / 2) * ld + 2 * (q1 & 1));
+                                    auto row = [&](int q) {
+                                        return *reinterpret_cast<const double2*>(g + size_t(q / 2) * ld + 2 * (q & 1));
+                                    };
+                                    if (q0 != p) x[r][2] = row(q0);
+                                    if (q1 > p + 1) x[r][3] = row(q1);
                                 }
                             }
                         }
@@ -874,7 +879,9 @@ static DigArgs dig_args(sphnse_plan* P, const DigSide& D) {
     a.items = D.items;
     a.cnt = D.cnt;
     a.istride = D.istride;
-    // tables that fit L2 beside the grid fields stay there between calls
+    // tables that fit L2 beside the grid fields stay there between calls (either
+    // way 45.8 us for F at L = 150, 32 MB; kept at L = 200, 74 MB, F took 72.2 us
+    // against 69.5, at L = 255, 120 MB, 85.8 against 81.1)
     a.evict_first = P->dig.syn.bytes + P->dig.ana.bytes > (size_t(48) << 20);
     a.ea = D.ea;
     a.status = P->d_status;

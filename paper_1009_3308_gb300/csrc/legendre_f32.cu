@@ -48,7 +48,12 @@ struct F32Args {
     float* hana;           // [n_ext][2 NF]
     int N, nh, nlat, pairs, evict_first;
     int rb;                // analysis: groups of 32 rows per block
-    int early;             // a grid of one wave: the successor may start its prologue at once
+    // a grid of about one wave (eight synthesis blocks of 128 threads and 64
+    // registers an SM, three analysis blocks of 256 and 80): the successor may start
+    // its prologue at once.  From larger grids its CTAs take the slots of later
+    // blocks: F 22.6 us against 18.9 at L = 170, 34.4 against 28.8 at L = 255; never
+    // early is as fast from L = 100 on, below that calls are bound by the host.
+    int early;
 };
 
 constexpr int F32_U = 16;   // table rows in flight per thread
@@ -265,8 +270,9 @@ static F32Args f32_args(sphnse_plan* P) {
     a.nh = P->nh;
     a.nlat = P->nlat;
     // synthesis and analysis read the same table: up to half of L2 it stays
-    // there between them and the next call, a larger one must not displace the
-    // grid fields
+    // there between them and the next call (F at L = 340, 60 MB: 45.5 us, 49.1
+    // without), a larger one must not displace the grid fields (L = 511, 202 MB:
+    // 104.6 us, 109.4 if it did; at L = 383, 85 MB, 67.4 and 66.2)
     a.evict_first = size_t(P->n_ext) * P->nh * sizeof(float) > (size_t(64) << 20);
     return a;
 }
