@@ -68,7 +68,7 @@ __device__ void produce(const StreamArgs& a, float* stages, uint64_t* full, uint
     const uint64_t pol = policy_evict_first();
     const float* tab = reinterpret_cast<const float*>(a.table);
     const size_t rowb = size_t(a.nh) * sizeof(float);
-    int it = 0;
+    int it = 0, end = 0;   // stages, and those requested
     for (int ii = n_items_begin; ii < n_items_end; ++ii) {
         const int m = a.items[ii] % (a.N + 1);
         const int ne = ext_even(a.N, m), no = ext_odd(a.N, m), e0 = ext_off(a.N, m);
@@ -78,6 +78,7 @@ __device__ void produce(const StreamArgs& a, float* stages, uint64_t* full, uint
             const uint32_t ph = (it / NST) & 1;
             if (it >= NST && !mbar_wait(&empty[s], ph ^ 1, abort, a.status)) continue;
             if (*abort) continue;
+            end = it + 1;
             int ce, co;
             chunk_rows(ne, no, c, HR, &ce, &co);
             float* dst = stages + size_t(s) * 2 * HR * a.nh;
@@ -88,11 +89,7 @@ __device__ void produce(const StreamArgs& a, float* stages, uint64_t* full, uint
         }
     }
     // wait for the copies still in flight before leaving (bounded)
-    const int last = it;
-    for (int k = last - NST; k < last; ++k) {
-        if (k < 0) continue;
-        mbar_wait(&full[k % NST], (k / NST) & 1, abort, a.status);
-    }
+    for (int k = max(0, end - NST); k < end; ++k) mbar_drain(&full[k % NST], (k / NST) & 1, a.status);
 }
 
 // ---------------------------------------------------------------------------

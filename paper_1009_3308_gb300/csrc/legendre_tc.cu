@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(FIN ? 448 : 320, 1) k_ana_tc(TcAnaArgs a) {
         if (elect_one()) {
             // the tables do not depend on the predecessor: stream them right away
             const uint64_t pol = policy_evict_first();
-            int it = 0;
+            int it = 0, end = 0;   // stages, and those requested (all, unless a wait ran out)
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = a.items[ib + i];
                 // FIN: the box height of the item's rows (16 (bj + 1)) and its map
@@ -196,13 +196,13 @@ __global__ void __launch_bounds__(FIN ? 448 : 320, 1) k_ana_tc(TcAnaArgs a) {
                     if (it >= ANS && !mbar_wait(&a_empty[s], ((it / ANS) - 1) & 1, abort, a.status))
                         continue;
                     if (*abort) continue;
+                    end = it + 1;
                     mbar_arrive_expect_tx(&a_full[s], abytes);
                     tma_load_2d(A_hi + s * TC_ATILE, a.map_hi + bj, kt * TC_TILE_K, itm.x, &a_full[s], pol);
                     tma_load_2d(A_lo + s * TC_ATILE, a.map_lo + bj, kt * TC_TILE_K, itm.x, &a_full[s], pol);
                 }
             }
-            for (int k = it - ANS; k < it; ++k)
-                if (k >= 0) mbar_wait(&a_full[k % ANS], (k / ANS) & 1, abort, a.status);
+            for (int k = max(0, end - ANS); k < end; ++k) mbar_drain(&a_full[k % ANS], (k / ANS) & 1, a.status);
         }
     } else if (warp == 1) {
         if (elect_one()) {
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(FIN ? 448 : 320, 1) k_ana_tc(TcAnaArgs a) {
                 mma_commit(&acc_full[buf]);
                 mma_commit(&b_empty[buf]);
             }
-            if (nI > 0) mbar_wait(&acc_full[(nI - 1) & 1], ((nI - 1) >> 1) & 1, abort, a.status);
+            if (nI > 0) mbar_drain(&acc_full[(nI - 1) & 1], ((nI - 1) >> 1) & 1, a.status);
         }
     } else if (warp < 6) {
         // B builders: task (piece, K tile, chunk q of 8 latitudes, field f)
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(192, 1) k_ana_tc_b(TcAnaBArgs a) {
         // read once
         const uint64_t pol = policy_evict_last();
         const uint64_t polb = policy_evict_first();
-        int it = 0;
+        int it = 0, end = 0;
         for (int i = 0; i < nI; ++i) {
             const int4 itm = a.items[ib + i];
             int4 sl = make_int4(0, 0, 0, 0);
@@ -570,6 +570,7 @@ __global__ void __launch_bounds__(192, 1) k_ana_tc_b(TcAnaBArgs a) {
                 }
                 go = __shfl_sync(0xffffffffu, go, 0);
                 if (!go) continue;
+                end = it + 1;
                 if (lane == 0) {
                     tma_load_2d(A_hi + s * TC_ATILE, a.map_hi, kt * TC_TILE_K, itm.x * TC_TILE_M, &a_full[s], pol);
                     tma_load_2d(A_lo + s * TC_ATILE, a.map_lo, kt * TC_TILE_K, itm.x * TC_TILE_M, &a_full[s], pol);
@@ -581,8 +582,8 @@ __global__ void __launch_bounds__(192, 1) k_ana_tc_b(TcAnaBArgs a) {
             }
         }
         if (lane == 0)
-            for (int k = it - TC_ANAB_NS; k < it; ++k)
-                if (k >= 0) mbar_wait(&a_full[k % TC_ANAB_NS], (k / TC_ANAB_NS) & 1, abort, a.status);
+            for (int k = max(0, end - TC_ANAB_NS); k < end; ++k)
+                mbar_drain(&a_full[k % TC_ANAB_NS], (k / TC_ANAB_NS) & 1, a.status);
     } else if (warp == 1) {
         if (elect_one()) {
             int it = 0;
@@ -611,7 +612,7 @@ __global__ void __launch_bounds__(192, 1) k_ana_tc_b(TcAnaBArgs a) {
                 }
                 mma_commit(&acc_full[buf]);
             }
-            if (nI > 0) mbar_wait(&acc_full[(nI - 1) & 1], ((nI - 1) >> 1) & 1, abort, a.status);
+            if (nI > 0) mbar_drain(&acc_full[(nI - 1) & 1], ((nI - 1) >> 1) & 1, a.status);
         }
     } else {
         // epilogue: slot j of the item -> columns 8 j .. 8 j + 7 (hi, then lo parts)
@@ -857,7 +858,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
             // first coefficient loads would otherwise queue behind every
             // CTA's full pipeline of table requests
             const uint64_t pol = policy_evict_first();
-            int it = 0;
+            int it = 0, end = 0;
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = item_meta(i);
                 const int m = itm.x, mt = itm.y;
@@ -869,6 +870,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
                         if (it == 1 && !mbar_wait(&a_full[0], 0, abort, a.status)) continue;
                         if (it >= ns && !mbar_wait(&a_empty[s], ((it / ns) - 1) & 1, abort, a.status)) continue;
                         if (*abort) continue;
+                        end = it + 1;
                         const bool last = kt == nkt - 1;
                         const int w = last ? tw : TC_TILE_K;
                         const int mi = last ? a.nblk + b : b;
@@ -878,8 +880,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
                     }
                 }
             }
-            for (int k = it - ns; k < it; ++k)
-                if (k >= 0) mbar_wait(&a_full[k % ns], (k / ns) & 1, abort, a.status);
+            for (int k = max(0, end - ns); k < end; ++k) mbar_drain(&a_full[k % ns], (k / ns) & 1, a.status);
         }
     } else if (warp == 0) {
         if (elect_one()) {
@@ -892,7 +893,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
             const uint64_t polb = policy_evict_last();
             const unsigned char* pend[NS];
             bool waited = false;
-            int it = 0;
+            int it = 0, end = 0;
             for (int i = 0; i < nI; ++i) {
                 const int4 itm = item_meta(i);
                 const int m = itm.x, mt = itm.y, g = itm.z * CS + crank;
@@ -914,6 +915,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
                             if (!mbar_wait(&a_empty[s], ((it / ns) - 1) & 1, abort, a.status)) continue;
                         }
                         if (*abort) continue;
+                        end = it + 1;
                         const bool last = kt == nkt - 1;
                         const int w = last ? tw : TC_TILE_K;
                         const int mi = last ? a.nblk + b : b;
@@ -942,8 +944,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
                 for (int j = 0; j < it && j < ns; ++j)
                     if (!*abort) bulk_g2s(Bs + j * bbytes, pend[j], uint32_t(bbytes), &a_full[j], polb);
             }
-            for (int k = it - ns; k < it; ++k)
-                if (k >= 0) mbar_wait(&a_full[k % ns], (k / ns) & 1, abort, a.status);
+            for (int k = max(0, end - ns); k < end; ++k) mbar_drain(&a_full[k % ns], (k / ns) & 1, a.status);
         }
     } else if (warp == 1) {
         if (elect_one()) {
@@ -980,7 +981,7 @@ __global__ void __launch_bounds__(SINGLE ? 192 + 32 * TC_SYN_BUILDERS : 192, 1) 
                 }
                 mma_commit(&acc_full[buf]);
             }
-            if (nI > 0) mbar_wait(&acc_full[(nI - 1) % NACC], ((nI - 1) / NACC) & 1, abort, a.status);
+            if (nI > 0) mbar_drain(&acc_full[(nI - 1) % NACC], ((nI - 1) / NACC) & 1, a.status);
         }
     } else if (warp < 6) {
         pdl_wait();

@@ -68,9 +68,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 
 // Bounded wait at the end of a role for what it has in flight, bulk copies into the
 // CTA's shared memory or MMAs on its tensor memory: these finish by themselves, so
-// it goes on when abort is set (the CTA must not exit under them).
+// it goes on when abort is set (the CTA must not exit under them), for a time that
+// no copy or MMA takes.
 __device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity, unsigned* status) {
-    for (uint32_t i = 0; i < SPH_WAIT_LIMIT; ++i)
+    constexpr uint32_t limit = SPH_WAIT_LIMIT < (1u << 16) ? SPH_WAIT_LIMIT : 1u << 16;
+    for (uint32_t i = 0; i < limit; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     if (status) atomicOr(status, SPH_STATUS_TIMEOUT);
     return false;
