@@ -225,18 +225,16 @@ __global__ void k_adj_accept(double2* dbar, const double2* abar, double2* dtot, 
 }
 
 // mu <- mu + (b - mu + c JT) / conj(1 - c J_d); ||b - mu + c JT||_inf (abs) goes
-// to host[0] (first: host[1]), a flag for values beyond the norms' range, in this
-// iteration or an earlier one, to host[7] (pinned).  The last block writes them and
-// clears what the next iteration adds to, so that an iteration needs no memset and
-// no copy: with alpha's fields kept between iterations, a reverse sweep of ten
-// steps at L = 255 FP32 went from 10.4 to 8.9 ms.  slot[5] keeps the first norm:
-// where it is zero mu = 0 is the solution, also with a JT that is not finite.
+// to host[0] (first: host[1]), a flag for values beyond the norms' range to host[7]
+// (first: host[6]; pinned).  The last block writes them and clears the slots, so
+// that an iteration needs no memset and no copy: with alpha's fields kept between
+// iterations, a reverse sweep of ten steps at L = 255 FP32 went from 10.4 to 8.9 ms.
 __global__ void k_adj_fixpoint(double2* mu, const double2* b, const double2* JT, const int2* lm, double c,
                                double nu, double Omega, unsigned long long* slot, unsigned long long* host, int first,
                                int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double r[1] = {0.0};
-    if (i < n && (first || __ldcg(slot + 5))) {
+    if (i < n) {
         const int L = lm[i].x, m = lm[i].y;
         const double lam = double(L) * (L + 1.0);
         const double mr = 1.0 + c * nu * lam, mi = c * 2.0 * Omega * m * rcp64<2>(lam);  // conj(1 - c J_d)
@@ -264,11 +262,9 @@ __global__ void k_adj_fixpoint(double2* mu, const double2* b, const double2* JT,
     __syncthreads();
     if (threadIdx.x != 0 || atomicAdd(slot + 6, 1ull) != gridDim.x - 1) return;
     __threadfence();
-    const unsigned long long norm = __ldcg(slot);
-    host[first ? 1 : 0] = norm;
-    host[7] = __ldcg(slot + 7);
-    if (first) slot[5] = norm;
-    slot[0] = slot[6] = 0ull;
+    host[first ? 1 : 0] = __ldcg(slot);
+    host[first ? 6 : 7] = __ldcg(slot + 7);
+    slot[0] = slot[6] = slot[7] = 0ull;
 }
 
 // y0bar = abar + mu - dtot;  dbar_j += g_j (-mu) + y0bar (j < k);  abar = y0bar;
@@ -912,22 +908,29 @@ int sphnse_adjoint_step_explicit(sphnse_plan* P, double h, int k, double h_dif_b
     double prev = 0.0;
     unsigned long long* hn = reinterpret_cast<unsigned long long*>(P->h_norms);
     if ((rc = clear_norms(P))) return rc;
+    auto fixpoint = [&](int first) {
+        stage_begin(P, SPHNSE_STAGE_STEP);
+        k_adj_fixpoint<<<grid(n), 256, 0, P->stream>>>(W.mu, W.dtot, W.jt, P->d_lm, c, P->nu, P->Omega,
+                                                       P->d_norms, hn, first, n);
+        stage_end(P, SPHNSE_STAGE_STEP);
+        return check_cuda(cudaGetLastError());
+    };
     for (int it = 0; it < 200; ++it) {
         if (it > 0 && (rc = rhs_adjoint_device(P, alpha_next, reinterpret_cast<const double*>(W.mu),
                                                reinterpret_cast<double*>(W.jt), false, it > 1)))
             return rc;
-        stage_begin(P, SPHNSE_STAGE_STEP);
-        k_adj_fixpoint<<<grid(n), 256, 0, P->stream>>>(W.mu, W.dtot, W.jt, P->d_lm, c, P->nu, P->Omega,
-                                                       P->d_norms, hn, it == 0, n);
-        stage_end(P, SPHNSE_STAGE_STEP);
-        if ((rc = check_cuda(cudaGetLastError()))) return rc;
+        if ((rc = fixpoint(it == 0))) return rc;
         if (it == 0) continue;   // its norm, the scale, is read with the next one
         if (cudaStreamSynchronize(P->stream) != cudaSuccess) return SPHNSE_E_CUDA;
-        if (hn[7]) return SPHNSE_E_NONFINITE;
         const double r = d2u_max(hn[0]), scale = d2u_max(hn[1]);
+        if (hn[6] || (hn[7] && scale != 0.0)) return SPHNSE_E_NONFINITE;
+        if (scale == 0.0) {   // mu = 0, also where J^T 0 was not finite
+            if ((rc = fixpoint(1))) return rc;
+            break;
+        }
         // converged, or stalled at the rounding level of the contractions
         const bool stalled = P->precision != SPHNSE_FP64 && it >= 3 && r > 0.8 * prev;
-        if (r <= 1e-14 * scale || scale == 0.0 || stalled) break;
+        if (r <= 1e-14 * scale || stalled) break;
         prev = r;
     }
     Coef g;
