@@ -43,9 +43,9 @@
 // instead, the expanded digits cost more than the halved HBM stream saved.
 //
 // Bound: the single-K-step stages, whose barrier waits (150 to 200 cycles even
-// when they pass at once), expansion and MMAs leave about 1000 cycles per stage;
-// eight bytes per table entry stream in 650 at full HBM rate.  The
-// FP64 pipe (two operations per clock per SM) would need 10 multiply-adds per
+// when they pass at once), expansion and MMAs take about 1070 (synthesis) and 890
+// (analysis) cycles per 16 KB block, which streams in 760 at the measured copy rate
+// (6.8 TB/s).  The FP64 pipe (two operations per clock per SM) would need 10 multiply-adds per
 // entry and RHS: 0.8 ms at L = 511.
 // Measured (event pairs, GB300) against the FP64 multiply-add kernels and their
 // prep: L = 511 synthesis 558 -> 94 us, analysis 429 -> 80; L = 255 96 -> 30,
