@@ -355,7 +355,8 @@ int launch_analysis(sphnse_plan* P, int nfields);
 // multiply its coefficient sets (prepc holds the factor): floor(log2(K + 1)), less
 // its largest value and four.  With that a coefficient overflows only where it
 // exceeds the largest number 2^4 times, and the bound on it that flags an overflow
-// (it is at most 2^4 too large) flags none that binary64 holds.
+// (it is at most 2^4 too large) flags none that binary64 holds.  (In exchange, sets
+// whose largest entry is below 2^-1009 lose bits to subnormal numbers.)
 __host__ __device__ inline int dig_shift(int N, int K) {
     int t = -4;
     for (++K; K > 1; K >>= 1) ++t;
